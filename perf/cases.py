@@ -324,8 +324,8 @@ def tolerance(case):
     """Packed values, metadata, scales, integer sums and the roundings behind them are defined bit for bit by the
     interface, and every path to them gives the same.  Only the scale search compares sums of double precision whose
     order is left open: a tie to the last bits may fall to a neighbouring candidate (1/64 of the scale) in a row here
-    and there; with the sums in another order none of
-    the 82944 rows of the listed case chose otherwise, and a row or two are allowed for."""
+    and there; with the sums in another order none of the 82944 rows of the listed case chose otherwise, and a row or two
+    are allowed for."""
     if case["kind"] == "project" and case["scale"] == "dist":
         return {"rel": 1e-4, "max": 0.02, "differ": 1e-4}
     return "exact"
