@@ -204,18 +204,21 @@ __device__ __forceinline__ void store_half_row128(uint8_t* tile, int row, int ha
         *reinterpret_cast<uint4*>(base + (((half * 4 + c) ^ x) << 4)) = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
 }
 
-// Hardware metadata words (4 per k-block) of one row from its canonical metadata.
-__device__ __forceinline__ uint4 hw_meta(int pat, const uint8_t* msrc, const uint32_t* lut) {
-    if (pat == P24_4) return ldg16(msrc);
+// Hardware metadata words (4 per k-block) of one row from its canonical metadata: the load and the conversion apart, so
+// that the loads of several k-blocks can be in flight together.
+__device__ __forceinline__ uint4 meta_raw(int pat, const uint8_t* msrc) {
+    if (meta_bytes(pat) == 16) return ldg16(msrc);
+    const uint2 m = ldg8(msrc);
+    return make_uint4(m.x, m.y, 0u, 0u);
+}
+__device__ __forceinline__ uint4 hw_meta(int pat, const uint4 m, const uint32_t* lut) {
+    if (pat == P24_4) return m;
     uint32_t h[4] = {0, 0, 0, 0};
+    const uint32_t mw[4] = {m.x, m.y, m.z, m.w};
     if (pat == P28_8 || pat == P28_4) {
-        const uint4 m = ldg16(msrc);
-        const uint32_t mw[4] = {m.x, m.y, m.z, m.w};
 #pragma unroll
         for (int u = 0; u < 16; ++u) h[u >> 2] |= (lut[kLut28 + ((mw[u >> 2] >> ((u & 3) * 8)) & 0x77u)] >> 16) << ((u & 3) * 8);
     } else {
-        const uint2 m = ldg8(msrc);
-        const uint32_t mw[2] = {m.x, m.y};
         const int base = (pat == P14_8 || pat == P14_4) ? kLut14 : kLut18;
         const uint32_t mask = base == kLut14 ? 0xFu : 0x7u;
 #pragma unroll

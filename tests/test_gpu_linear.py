@@ -62,6 +62,13 @@ def test_ragged_out_and_no_bias(n, m, bits):
     _run(5, 70, 128, 8, n, m, bits)
 
 
+@pytest.mark.parametrize("n,m,bits", [(2, 4, 8), (2, 8, 4), (1, 4, 8)])
+@pytest.mark.parametrize("K", [128, 896, 1152, 2176, 8192])
+def test_metadata_batches(n, m, bits, K):
+    # metadata goes to TMEM in batches of eight (four) k-blocks: less than one batch, a remainder, the longest reduction
+    _run(40, 64, K, 200, n, m, bits)
+
+
 @pytest.mark.parametrize("n,m,bits", ALL_MODES)
 def test_bert_base_attention_projection(n, m, bits):
     # 128 tokens x 768 -> 768 (the small single-GEMM configuration)
