@@ -197,6 +197,231 @@ __device__ __forceinline__ void store_bytes_slow(uint8_t* dst, const unsigned* w
         if (i < nbytes) dst[i] = (uint8_t)(w[i >> 2] >> ((i & 3) * 8));
 }
 
+// ---------------------------------------------------------------------------------------------
+// ADMM-Dist scale (Sec. 3.3.1, "Minimize Quantization Distance"): per output channel the scale that
+// minimises the squared distance E_j between the N:M-projected channel and its quantised form, searched
+// over the candidates s_j = fl32(s_max * (64 - j) / 64), j = 0 .. ncand-1 (s_max = the ADMM-Max scale;
+// lowest j on equal distance).  The decision is taken on distances held in double, in two steps:
+//
+// 1. All candidates in single precision, in units of s_max: y = |v| / s_max, code magnitude k =
+//    min(rne(y * 64 / (64 - j)), end code of v's sign), d = y - k * (64 - j) / 64, sum of d * d: five
+//    operations per candidate and kept value, four of them as packed pairs.  Per value |d| is within
+//    eps = 2^(b - 1) * 2^-19 of the exact distance: y and 64 / (64 - j) carry relative errors of 1.5 * 2^-23 and 2^-24 and
+//    the real scale s_j one of 2^-24, which move d by less than 2^(b - 1) * 2^-21 when the code is the true one; the
+//    code differs only where the quotient is within 2^(b - 1) * 3 * 2^-23 of a tie, and there the two
+//    distances differ by twice that.  By the triangle inequality the root of the exact E_j is within
+//    eps * sqrt(values) of the root of the computed one, whose sums (at most 80 roundings of non-negative terms) are
+//    good to 2^-17 relative.
+// 2. A candidate whose lower bound exceeds another's upper bound cannot win.  Usually one is left (about 96 of
+//    100 rows of 768 weights at 4 bits); otherwise those that are left are evaluated in double from the fp32
+//    weights (code from the IEEE quotient, d = v - s_j * code and E += d * d as two FMAs, s_j * code being exact in double) and
+//    compared.  Scales outside [2^-126, 2^125] and non-finite rows skip step 1.
+//
+// A row spans `wpr` warps; the partial sums of its warps are added in a fixed order, so the result is
+// deterministic.  Evaluating every candidate in double took 14.8 instructions per candidate and value, among them
+// a quarter-rate conversion: 85 M weights at 2:4 / 4 bit and 32 candidates, search alone 1050 us before, 405 us now.
+// ---------------------------------------------------------------------------------------------
+template <int N, int M>
+__device__ __forceinline__ void kept_values(const float* v, float* sel) {
+    if constexpr (N == M) {
+#pragma unroll
+        for (int p = 0; p < M; ++p) sel[p] = v[p];
+    } else if constexpr ((N == 1) || (N == 2 && M == 8)) {
+        unsigned selp[N];
+        select_passes<N, M>(v, sel, selp);
+    } else {
+        float a[M];
+#pragma unroll
+        for (int p = 0; p < M; ++p) a[p] = fabsf(v[p]);
+        const unsigned mask = keep_mask<N, M>(a);
+        if constexpr (N == 2 && M == 4) {
+            const bool b0 = mask & 1u, b1 = mask & 2u, b2 = mask & 4u, b3 = mask & 8u;
+            sel[0] = b0 ? v[0] : (b1 ? v[1] : v[2]);
+            sel[1] = b3 ? v[3] : (b2 ? v[2] : v[1]);
+        } else {
+#pragma unroll
+            for (int c = 0; c < N; ++c) sel[c] = 0.0f;
+#pragma unroll
+            for (int p = 0; p < M; ++p) {
+                const bool kept = (mask >> p) & 1u;
+                const int before = __popc(mask & ((1u << p) - 1u));
+#pragma unroll
+                for (int c = 0; c < N; ++c)
+                    if (c <= p && (M - p) >= (N - c)) sel[c] = (kept && before == c) ? v[p] : sel[c];
+            }
+        }
+    }
+}
+
+
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// The kept values of this lane, from the warp's tile.
+template <int N, int M>
+__device__ __forceinline__ void lane_kept_values(const float4* mytile, int lane, float* x) {
+    constexpr int G = 32 / M;
+    float v[32];
+#pragma unroll
+    for (int jj = 0; jj < 8; ++jj) {
+        const float4 t = mytile[lane * 8 + (jj ^ (lane & 7))];
+        v[jj * 4 + 0] = t.x; v[jj * 4 + 1] = t.y; v[jj * 4 + 2] = t.z; v[jj * 4 + 3] = t.w;
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g) kept_values<N, M>(v + g * M, x + g * N);
+}
+
+// Distance of candidate j in double over the warp's chunk (every lane returns the sum over the lanes).
+template <int N, int M, int BITS>
+__device__ __noinline__ double dist_exact(const float4* mytile, int lane, float smax, int j) {
+    constexpr int KN = 32 / M * N;
+    constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
+    constexpr float kLo = -(float)(1 << (BITS - 1)) - 0.49f, kHi = qmax + 0.49f;
+    constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
+    float x[KN];
+    lane_kept_values<N, M>(mytile, lane, x);
+    const float sj = __fmul_rn(smax, (float)(64 - j) * 0.015625f);
+    const double nsd = -(double)sj;
+    double e0 = 0.0, e1 = 0.0;
+#pragma unroll 4
+    for (int i = 0; i < KN; ++i) {
+        const float qc = fminf(fmaxf(__fdiv_rn(x[i], sj), kLo), kHi);
+        const float r = __fsub_rn(__fadd_rn(qc, kMagic), kMagic);  // nearest-even integer of qc
+        const double d = fma(nsd, (double)r, (double)x[i]);
+        if (i & 1) e1 = fma(d, d, e1); else e0 = fma(d, d, e0);
+    }
+    double e = e0 + e1;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    return e;
+}
+
+// Winning candidate of this warp's row.  `red_e` holds 32 doubles per warp of the block.  Every warp of the block calls it
+// (block-wide barriers when a row spans warps).
+template <int N, int M, int BITS>
+__device__ __forceinline__ int dist_search(const float4* mytile, int lane, int w, int wpr, int row_in_block, bool row_ok,
+                                           float smax, bool bad, int ncand, double* red_e) {
+    constexpr int KN = 32 / M * N;                    // kept values per lane
+    constexpr float qend = (float)(1 << (BITS - 1));  // magnitude of the negative end code
+    constexpr float kMagic = 12582912.0f;             // 1.5 * 2^23: adding it rounds to the nearest-even integer
+    constexpr float kEps = qend * 1.9073486328125e-6f;  // 2^(b - 1) * 2^-19
+    const float inf = __int_as_float(0x7f800000);
+    const bool usable = !bad && smax >= 1.17549435e-38f && smax <= 4.25e37f;  // 1 / s_max is a normal number
+    float mine = inf;  // lane j: candidate j's distance in units of s_max^2
+    if (usable && row_ok) {
+        uint64_t y[KN / 2];
+        float lim[KN];
+        {
+            float x[KN];
+            lane_kept_values<N, M>(mytile, lane, x);
+            const float r0 = __frcp_rn(smax);
+#pragma unroll
+            for (int i = 0; i < KN; ++i) lim[i] = kMagic + (x[i] < 0.0f ? qend : qend - 1.0f);
+#pragma unroll
+            for (int i = 0; i < KN / 2; ++i) y[i] = pack_f32x2(fabsf(__fmul_rn(x[2 * i], r0)), fabsf(__fmul_rn(x[2 * i + 1], r0)));
+        }
+        const float my_inv = __frcp_rn((float)(64 - lane) * 0.015625f);  // 64 / (64 - j) of candidate j = lane
+        const uint64_t magic2 = pack_f32x2(kMagic, kMagic), nmagic2 = pack_f32x2(-kMagic, -kMagic);
+        // eight candidates at a time; their sums over the lanes by a transposing butterfly (lane l ends up with
+        // candidate 8 * group + (l >> 2)), of which lane l keeps group l & 3's
+        float kept = inf;
+#pragma unroll 1
+        for (int g = 0; g < 4; ++g) {
+            if (8 * g >= ncand) break;
+            float e[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float inv = __shfl_sync(0xffffffffu, my_inv, 8 * g + k);
+                const float na = (float)(8 * g + k - 64) * 0.015625f;  // -(64 - j) / 64
+                const uint64_t inv2 = pack_f32x2(inv, inv), na2 = pack_f32x2(na, na);
+                uint64_t acc = 0;
+#pragma unroll
+                for (int i = 0; i < KN / 2; ++i) {
+                    float t0, t1;
+                    unpack_f32x2(fma_f32x2(y[i], inv2, magic2), t0, t1);
+                    const uint64_t code = add_f32x2(pack_f32x2(fminf(t0, lim[2 * i]), fminf(t1, lim[2 * i + 1])), nmagic2);
+                    const uint64_t d = fma_f32x2(na2, code, y[i]);
+                    acc = fma_f32x2(d, d, acc);
+                }
+                float a0, a1;
+                unpack_f32x2(acc, a0, a1);
+                e[k] = a0 + a1;
+            }
+#pragma unroll
+            for (int h = 4; h >= 1; h >>= 1) {
+                const bool up = lane & (4 * h);
+#pragma unroll
+                for (int k = 0; k < h; ++k) {
+                    const float keep = up ? e[k + h] : e[k], give = up ? e[k] : e[k + h];
+                    e[k] = keep + __shfl_xor_sync(0xffffffffu, give, 4 * h);
+                }
+            }
+            e[0] += __shfl_xor_sync(0xffffffffu, e[0], 2);
+            e[0] += __shfl_xor_sync(0xffffffffu, e[0], 1);
+            if ((lane & 3) == g) kept = e[0];
+        }
+        mine = __shfl_sync(0xffffffffu, kept, ((lane & 7) << 2) | (lane >> 3));  // candidate j to lane j
+    }
+    if (wpr > 1) {
+        float* red_f = reinterpret_cast<float*>(red_e);
+        red_f[w * 32 + lane] = mine;
+        __syncthreads();
+        mine = 0.0f;
+        for (int c = 0; c < wpr; ++c) mine += red_f[(row_in_block * wpr + c) * 32 + lane];
+        __syncthreads();  // the array is used again below
+    }
+    // candidates that the bounds leave
+    const float slack = kEps * sqrtf((float)(KN * 32 * wpr));
+    const float root = sqrtf(mine), lo = fmaxf(root - slack, 0.0f);
+    float best = lane < ncand ? (root + slack) * (root + slack) * 1.0000153f : inf;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+    const bool left = lane < ncand && (!usable || lo * lo * 0.9999847f <= best);
+    const unsigned mask = row_ok ? __ballot_sync(0xffffffffu, left) : 1u;
+    const bool single = (mask & (mask - 1u)) == 0u;
+    if (single && wpr == 1) return __ffs(mask) - 1;
+    double exact = __longlong_as_double(0x7ff0000000000000ll);
+    if (!single) {
+        for (unsigned m = mask; m; m &= m - 1u) {
+            const int j = __ffs(m) - 1;
+            const double e = dist_exact<N, M, BITS>(mytile, lane, smax, j);
+            if (lane == j) exact = e;
+        }
+    }
+    if (wpr > 1) {
+        red_e[w * 32 + lane] = exact;
+        __syncthreads();
+        if (single) return __ffs(mask) - 1;
+        exact = 0.0;
+        for (int c = 0; c < wpr; ++c) exact += red_e[(row_in_block * wpr + c) * 32 + lane];
+    }
+    int bj = lane;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double oe = __shfl_xor_sync(0xffffffffu, exact, o);
+        const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+        const bool take = (oe < exact) || (oe == exact && oj < bj);
+        exact = take ? oe : exact;
+        bj = take ? oj : bj;
+    }
+    bj = __shfl_sync(0xffffffffu, bj, 0);
+    return bj < ncand ? bj : 0;  // only when every distance is NaN or infinite (non-finite input)
+}
+
 // N == M: dense (quantise only, no metadata), processed in groups of 4.
 // DENSE_OUT: the ADMM step / STE forward form.  Besides (or instead of: values, meta and scales may then be
 // null) the packed outputs the kernel writes Z = s * code as dense fp32, zero where pruned, and, when
@@ -264,10 +489,11 @@ __device__ __forceinline__ unsigned units_of(const PackJobDev& job, int warps) {
 // Everything after the load: `mytile` holds the warp's chunk of V = W + U in the swizzled layout, `amax` and
 // `poison` are the lane's running |max| and non-finite detector.  `red` is this unit's slot array for the row
 // maximum across the warps of a row.  Every warp of the block calls it (block-wide barrier when a row spans warps).
-template <int N, int M, int BITS, bool DENSE_OUT>
+template <int N, int M, int BITS, bool DENSE_OUT, bool DIST = false>
 __device__ __forceinline__ void pack_finish(const PackJobDev& job, const UnitPos& up, int lane, int w, float4* mytile,
                                             float* red, const uint16_t* pos48, float amax, float poison, uint32_t* status,
-                                            float* __restrict__ Zout, float* __restrict__ Unext, int group_mode, int group_rows) {
+                                            float* __restrict__ Zout, float* __restrict__ Unext, int group_mode, int group_rows,
+                                            double* red_e = nullptr) {
     constexpr bool kDense = (N == M);
     constexpr int G = 32 / M;                          // groups per lane
     constexpr int F = (M == 4) ? 2 : 4;                // metadata field width
@@ -304,8 +530,12 @@ __device__ __forceinline__ void pack_finish(const PackJobDev& job, const UnitPos
     // ---- ADMM-Max scale ---------------------------------------------------------------------
     constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
     // group-wise quantisation hands the scale in (one per row, equal within a group of rows)
-    const float s = group_mode == kGroupScalesGiven ? job.scales[row_ok ? row : 0]
-                                                    : ((amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax));
+    float s = !DIST && group_mode == kGroupScalesGiven ? job.scales[row_ok ? row : 0]
+                                                       : ((amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax));
+    if constexpr (DIST) {  // group_rows carries the number of candidate scales
+        const int best = dist_search<N, M, BITS>(mytile, lane, w, wpr, row_in_block, row_ok, s, bad, group_rows, red_e);
+        s = __fmul_rn(s, (float)(64 - best) * 0.015625f);
+    }
     if (row_ok && chunk == 0 && lane == 0 && (!DENSE_OUT || job.scales)) job.scales[row] = s;
     const float rs = __frcp_rn(s);  // correctly rounded reciprocal, once per row
     const bool fast_ok = (s >= 1.17549435e-38f) && (s <= 4.25e37f);  // rs is a normal number
@@ -523,8 +753,8 @@ __device__ __forceinline__ void load_chunk_staged(const PackJobDev& job, const U
 enum { kDirect = 0, kStaged2 = 1, kAhead = 2 };
 __host__ __device__ constexpr int pack_blocks_per_sm(int pipe) { return pipe == kStaged2 ? 3 : 8; }
 
-template <int N, int M, int BITS, int MAXT, bool DENSE_OUT = false, int PIPE = kDirect>
-__global__ void __launch_bounds__(MAXT, PIPE != kDirect ? pack_blocks_per_sm(PIPE) : (MAXT == 128 ? (DENSE_OUT ? 4 : 8) : 1))
+template <int N, int M, int BITS, int MAXT, bool DENSE_OUT = false, int PIPE = kDirect, bool DIST = false>
+__global__ void __launch_bounds__(MAXT, PIPE != kDirect ? pack_blocks_per_sm(PIPE) : (MAXT == 128 ? (DENSE_OUT || DIST ? 4 : 8) : 1))
 pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constant__ PackJobInline inl, uint32_t* status,
             float* __restrict__ Zout, float* __restrict__ Unext, const DenseOutDev* __restrict__ dense_jobs,
             int group_mode, int group_rows, unsigned nunits) {
@@ -583,6 +813,7 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
             job = njob; index = nindex;
         }
     } else if constexpr (PIPE == kDirect) {
+        double* red_e = DIST ? reinterpret_cast<double*>(pos48 + 256) : nullptr;  // 32 per warp
         int index = 0;
         const PackJobDev job = find_job(jobs, njobs, inl, blockIdx.x, index);
         if constexpr (DENSE_OUT) {
@@ -592,8 +823,8 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
         float4* mytile = tile + w * 256;
         float amax = 0.0f, poison = 0.0f;
         load_chunk_global(job, up, lane, mytile, amax, poison);
-        pack_finish<N, M, BITS, DENSE_OUT>(job, up, lane, w, mytile, red, pos48, amax, poison, status, Zout, Unext,
-                                          group_mode, group_rows);
+        pack_finish<N, M, BITS, DENSE_OUT, DIST>(job, up, lane, w, mytile, red, pos48, amax, poison, status, Zout, Unext,
+                                                group_mode, group_rows, red_e);
     } else {
         uint64_t* bars = reinterpret_cast<uint64_t*>(pos48 + 256);       // [warps][2]
         volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 2 * warps);
@@ -734,109 +965,25 @@ static int launch_group_scales(const float* W, const float* U, int out, int in, 
     return NM_OK;
 }
 
-// ---------------------------------------------------------------------------------------------
-// ADMM-Dist scale (Sec. 3.3.1, "Minimize Quantization Distance"): per output channel the scale that
-// minimises the squared distance between the N:M-projected channel and its quantised form, searched
-// over the candidates s_j = fl32(s_max * (64 - j) / 64), j = 0 .. ncand-1 (s_max = the ADMM-Max scale;
-// lowest j on equal distance).  The kernel writes the winning scale to `scales`; the projection /
-// packing kernel then runs with the scales handed in.
-//
-// Same decomposition as pack_kernel: a warp owns 1024 consecutive weights, a lane 32 consecutive ones,
-// of which it keeps G*N in registers (as fp32 for the quantiser, as fp64 for the distance).  Per
-// candidate and kept value: the code from the reciprocal product (true division when the quotient is
-// within 2^-15 of a rounding tie or the scale is outside the range where the reciprocal is accurate),
-// converted to a double, then d = v - s*code and E += d*d as two fp64 FMAs (the
-// product s*code is exact in double).  E is summed per lane, over the lanes by a butterfly, over the
-// warps of a row through shared memory: a fixed order, so the result is deterministic.  The work is
-// bound by instruction issue (about 15 instructions per candidate and kept value), not by HBM.
-// ---------------------------------------------------------------------------------------------
-template <int N, int M>
-__device__ __forceinline__ void kept_values(const float* v, float* sel) {
-    if constexpr (N == M) {
-#pragma unroll
-        for (int p = 0; p < M; ++p) sel[p] = v[p];
-    } else if constexpr ((N == 1) || (N == 2 && M == 8)) {
-        unsigned selp[N];
-        select_passes<N, M>(v, sel, selp);
-    } else {
-        float a[M];
-#pragma unroll
-        for (int p = 0; p < M; ++p) a[p] = fabsf(v[p]);
-        const unsigned mask = keep_mask<N, M>(a);
-        if constexpr (N == 2 && M == 4) {
-            const bool b0 = mask & 1u, b1 = mask & 2u, b2 = mask & 4u, b3 = mask & 8u;
-            sel[0] = b0 ? v[0] : (b1 ? v[1] : v[2]);
-            sel[1] = b3 ? v[3] : (b2 ? v[2] : v[1]);
-        } else {
-#pragma unroll
-            for (int c = 0; c < N; ++c) sel[c] = 0.0f;
-#pragma unroll
-            for (int p = 0; p < M; ++p) {
-                const bool kept = (mask >> p) & 1u;
-                const int before = __popc(mask & ((1u << p) - 1u));
-#pragma unroll
-                for (int c = 0; c < N; ++c)
-                    if (c <= p && (M - p) >= (N - c)) sel[c] = (kept && before == c) ? v[p] : sel[c];
-            }
-        }
-    }
-}
-
+// The search alone (nm_dist_scales), and in front of the projection for rows of more than 4096 weights, whose blocks have too
+// few registers per thread for both: writes the winning scale to `scales`.
 template <int N, int M, int BITS, int MAXT>
-__global__ void __launch_bounds__(MAXT, MAXT == 128 ? (32 / M * N > 16 ? 4 : 5) : 1) dist_scale_kernel(const PackJobDev* __restrict__ jobs, int njobs,
-                                                                              PackJobDev single, uint32_t* status, int ncand,
+__global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1) dist_scale_kernel(const PackJobDev* __restrict__ jobs, int njobs,
+                                                                              const __grid_constant__ PackJobInline inl,
+                                                                              uint32_t* status, int ncand,
                                                                               int32_t* __restrict__ cand_out) {
-    constexpr int G = 32 / M;
-    constexpr int KN = G * N;  // kept values per lane
     extern __shared__ float4 tile[];  // [warps][256] float4, [warps][32] doubles, [warps] floats
     const int warps = blockDim.x >> 5;
     double* red_e = reinterpret_cast<double*>(tile + warps * 256);
     float* red = reinterpret_cast<float*>(red_e + warps * 32);
-
-    PackJobDev job;
-    if (jobs) {
-        int lo = 0, hi = njobs - 1;  // last job whose unit_begin <= blockIdx.x
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (jobs[mid].unit_begin <= blockIdx.x) lo = mid; else hi = mid - 1;
-        }
-        job = jobs[lo];
-    } else {
-        job = single;
-    }
+    int index = 0;
+    const PackJobDev job = find_job(jobs, njobs, inl, blockIdx.x, index);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const UnitPos up = unit_pos(job, blockIdx.x, w, warps);
     const int wpr = 1 << job.wpr_log2;
-    const int row_in_block = w >> job.wpr_log2, chunk = w & (wpr - 1);
-    const int rows_per_block = warps >> job.wpr_log2;
-    const long long row = (long long)(blockIdx.x - job.unit_begin) * rows_per_block + row_in_block;
-    const bool row_ok = row < job.out;
-    const int in4 = job.in >> 2;
-
-    // ---- V = W + U (coalesced; kept in cache for the projection pass that follows), |max|, transpose ----
     float4* mytile = tile + w * 256;
     float amax = 0.0f, poison = 0.0f;
-    {
-        const float4* W4 = reinterpret_cast<const float4*>(job.W) + (row_ok ? row * in4 : 0);
-        const float4* U4 = job.U ? reinterpret_cast<const float4*>(job.U) + (row_ok ? row * in4 : 0) : nullptr;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int f = chunk * 256 + j * 32 + lane;
-            float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (row_ok && f < in4) {
-                t = __ldg(W4 + f);
-                if (U4) {
-                    const float4 u = __ldg(U4 + f);
-                    t.x = __fadd_rn(t.x, u.x); t.y = __fadd_rn(t.y, u.y);
-                    t.z = __fadd_rn(t.z, u.z); t.w = __fadd_rn(t.w, u.w);
-                }
-            }
-            amax = fmaxf(amax, fmaxf(fmaxf(fabsf(t.x), fabsf(t.y)), fmaxf(fabsf(t.z), fabsf(t.w))));
-            poison = __fmaf_rn(t.x, 0.0f, poison); poison = __fmaf_rn(t.y, 0.0f, poison);
-            poison = __fmaf_rn(t.z, 0.0f, poison); poison = __fmaf_rn(t.w, 0.0f, poison);
-            const int fl = j * 32 + lane, owner = fl >> 3, jj = fl & 7;
-            mytile[owner * 8 + (jj ^ (owner & 7))] = t;
-        }
-    }
+    load_chunk_global(job, up, lane, mytile, amax, poison);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     const bool bad = __any_sync(0xffffffffu, poison != poison) || !(amax <= 3.402823466e+38f);
@@ -844,84 +991,16 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? (32 / M * N > 16 ? 4 : 5) 
     if (wpr > 1) {
         if (lane == 0) red[w] = amax;
         __syncthreads();
-        for (int c = 0; c < wpr; ++c) amax = fmaxf(amax, red[row_in_block * wpr + c]);
+        for (int c = 0; c < wpr; ++c) amax = fmaxf(amax, red[up.row_in_block * wpr + c]);
     } else {
         __syncwarp();
     }
-
-    // ---- this lane's kept values (columns beyond the row were loaded as zeros: they add nothing) --------
-    float x[KN];
-    double xd[KN];
-    {
-        float v[32];
-#pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-            const float4 t = mytile[lane * 8 + (jj ^ (lane & 7))];
-            v[jj * 4 + 0] = t.x; v[jj * 4 + 1] = t.y; v[jj * 4 + 2] = t.z; v[jj * 4 + 3] = t.w;
-        }
-#pragma unroll
-        for (int g = 0; g < G; ++g) kept_values<N, M>(v + g * M, x + g * N);
-#pragma unroll
-        for (int i = 0; i < KN; ++i) xd[i] = (double)x[i];
-    }
-
     constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
-    constexpr float kLo = -(float)(1 << (BITS - 1)) - 0.49f, kHi = qmax + 0.49f;
-    constexpr float kMagic = 12582912.0f;             // 1.5 * 2^23 = 0x4B400000
     const float smax = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
-    double mine = __longlong_as_double(0x7ff0000000000000ll);  // lane j ends up with candidate j's distance
-    for (int j = 0; j < ncand; ++j) {
-        const float sj = __fmul_rn(smax, (float)(64 - j) * 0.015625f);
-        const float rj = __frcp_rn(sj);
-        const double nsd = -(double)sj;
-        // outside [2^-126, 2^125] the reciprocal is subnormal, infinite or the product loses bits
-        const bool fast_ok = (sj >= 1.17549435e-38f) && (sj <= 4.25e37f);
-        // fast pass: code from the reciprocal product; the rounded quotient (an integer-valued float) goes to
-        // the fp64 pipe through one conversion
-        bool near_tie = !fast_ok;
-        double e0 = 0.0, e1 = 0.0;
-#pragma unroll
-        for (int i = 0; i < KN; ++i) {
-            const float qc = fminf(fmaxf(__fmul_rn(x[i], rj), kLo), kHi);
-            const float r = __fsub_rn(__fadd_rn(qc, kMagic), kMagic);  // nearest-even integer of qc
-            near_tie |= !(fabsf(__fsub_rn(qc, r)) <= 0.49996948f);
-            const double d = fma(nsd, (double)r, xd[i]);
-            if (i & 1) e1 = fma(d, d, e1); else e0 = fma(d, d, e0);
-        }
-        if (near_tie) {  // some quotient of this lane sits next to a rounding tie: the whole candidate again, exactly
-            e0 = 0.0; e1 = 0.0;
-#pragma unroll
-            for (int i = 0; i < KN; ++i) {
-                const float qc = fminf(fmaxf(__fdiv_rn(x[i], sj), kLo), kHi);
-                const float r = __fsub_rn(__fadd_rn(qc, kMagic), kMagic);
-                const double d = fma(nsd, (double)r, xd[i]);
-                if (i & 1) e1 = fma(d, d, e1); else e0 = fma(d, d, e0);
-            }
-        }
-        double e = e0 + e1;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-        if (lane == j) mine = e;
-    }
-    if (wpr > 1) {
-        red_e[w * 32 + lane] = mine;
-        __syncthreads();
-        mine = 0.0;
-        for (int c = 0; c < wpr; ++c) mine += red_e[(row_in_block * wpr + c) * 32 + lane];
-    }
-    int bj = lane;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double oe = __shfl_xor_sync(0xffffffffu, mine, o);
-        const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
-        const bool take = (oe < mine) || (oe == mine && oj < bj);
-        mine = take ? oe : mine;
-        bj = take ? oj : bj;
-    }
-    if (bj >= ncand) bj = 0;  // only when every distance is NaN or infinite (non-finite input, flagged above)
-    if (row_ok && chunk == 0 && lane == 0) {
-        job.scales[row] = __fmul_rn(smax, (float)(64 - bj) * 0.015625f);
-        if (cand_out) cand_out[row] = bj;
+    const int bj = dist_search<N, M, BITS>(mytile, lane, w, wpr, up.row_in_block, up.row_ok, smax, bad, ncand, red_e);
+    if (up.row_ok && up.chunk == 0 && lane == 0) {
+        job.scales[up.row] = __fmul_rn(smax, (float)(64 - bj) * 0.015625f);
+        if (cand_out) cand_out[up.row] = bj;
     }
 }
 
@@ -929,7 +1008,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? (32 / M * N > 16 ? 4 : 5) 
 // host side
 // ---------------------------------------------------------------------------------------------
 using PackFnPtr = void (*)(const PackJobDev*, int, const PackJobInline, uint32_t*, float*, float*, const DenseOutDev*, int, int, unsigned);
-struct PackFn { PackFnPtr fn; int form; };  // kernel and its form (kDirect, kStaged2, kAhead)
+struct PackFn { PackFnPtr fn; int form; bool dist = false; };  // kernel, its form (kDirect, kStaged2, kAhead), with the scale search
 
 // nm_debug_set_option("pack_form"): 0 = automatic, 1 = kDirect, 2 = kStaged2, 3 = kAhead for blocks of four warps.
 int g_pack_form = 0;
@@ -1015,7 +1094,7 @@ static int launch_table(PackFn k, const PackJobDev* jobs_dev, int njobs, const P
     // and the abort flag, and a grid that stays resident
     const bool staged = k.form == kStaged2, persistent = k.form != kDirect;
     size_t smem = (size_t)warps * ((staged ? 1024 : 256) * sizeof(float4) + 2 * sizeof(float)) + 512 +
-                  (staged ? (size_t)warps * 16 + 16 : 0);
+                  (staged ? (size_t)warps * 16 + 16 : 0) + (k.dist ? (size_t)warps * 32 * sizeof(double) : 0);
     const PackFnPtr fn = k.fn;
     if (smem > 48 * 1024) {  // the attribute is set once per kernel and device
         struct Done { const void* fn; int dev; };
@@ -1046,7 +1125,7 @@ static int launch(PackFn fn, const PackJobDev* jobs_dev, int njobs, const PackJo
     return launch_table(fn, jobs_dev, njobs, inl, blocks, warps, status, stream, Z, U_next, dense_jobs, group_mode, group_rows);
 }
 
-using DistFn = void (*)(const PackJobDev*, int, PackJobDev, uint32_t*, int, int32_t*);
+using DistFn = void (*)(const PackJobDev*, int, const PackJobInline, uint32_t*, int, int32_t*);
 
 template <int N, int M>
 static DistFn pick_dist_bits(int bits, int warps) {
@@ -1070,9 +1149,28 @@ static int launch_dist(DistFn fn, const PackJobDev* jobs_dev, int njobs, const P
     size_t smem = (size_t)warps * (256 * sizeof(float4) + 32 * sizeof(double) + sizeof(float));
     if (smem > 48 * 1024)
         NM_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    fn<<<blocks, warps * 32, smem, stream>>>(jobs_dev, njobs, single, status, ncand, cand);
+    PackJobInline inl{};
+    inl.j[0] = single;
+    fn<<<blocks, warps * 32, smem, stream>>>(jobs_dev, njobs, inl, status, ncand, cand);
     NM_CUDA_TRY(cudaGetLastError());
     return NM_OK;
+}
+
+// Search and projection in one kernel (blocks of four warps): the search keeps the row in shared memory, so W and U are read
+// once: 85 M weights at 2:4 / 4 bit 533 us against 405 + 156 us for the search followed by the projection.
+template <int N, int M, bool DENSE_OUT>
+static PackFn pick_dist_pack_bits(int bits) {
+    return bits == 8 ? PackFn{(PackFnPtr)pack_kernel<N, M, 8, 128, DENSE_OUT, kDirect, true>, kDirect, true}
+                     : PackFn{(PackFnPtr)pack_kernel<N, M, 4, 128, DENSE_OUT, kDirect, true>, kDirect, true};
+}
+
+template <bool DENSE_OUT>
+static PackFn pick_dist_pack(int n, int m, int bits) {
+    if (n == m) return pick_dist_pack_bits<4, 4, DENSE_OUT>(bits);
+    if (m == 4) return n == 1 ? pick_dist_pack_bits<1, 4, DENSE_OUT>(bits) : pick_dist_pack_bits<2, 4, DENSE_OUT>(bits);
+    if (n == 1) return pick_dist_pack_bits<1, 8, DENSE_OUT>(bits);
+    if (n == 2) return pick_dist_pack_bits<2, 8, DENSE_OUT>(bits);
+    return pick_dist_pack_bits<4, 8, DENSE_OUT>(bits);
 }
 
 // One matrix: the ADMM-Dist scales into job.scales (and the winning candidate numbers into `cand`).
@@ -1082,6 +1180,23 @@ static int launch_dist_single(const nm_pack_job_t& j, int ncand, int32_t* cand, 
     const int rows_per_block = warps >> d.wpr_log2;
     const unsigned blocks = (unsigned)((j.out + rows_per_block - 1) / rows_per_block);
     return launch_dist(pick_dist(j.n, j.m, j.bits, warps), nullptr, 0, d, blocks, warps, status, stream, ncand, cand);
+}
+
+// One matrix: search and projection.
+template <bool DENSE_OUT>
+static int launch_dist_project_single(const nm_pack_job_t& j, int ncand, uint32_t* status, cudaStream_t stream,
+                                      float* Z = nullptr, float* U_next = nullptr) {
+    PackJobDev d = to_dev(j);
+    const int warps = std::max(kPackMinWarps, 1 << d.wpr_log2);
+    const int rows_per_block = warps >> d.wpr_log2;
+    const unsigned blocks = (unsigned)((j.out + rows_per_block - 1) / rows_per_block);
+    if (warps <= kPackMinWarps)
+        return launch(pick_dist_pack<DENSE_OUT>(j.n, j.m, j.bits), nullptr, 0, d, blocks, warps, status, stream, Z, U_next, nullptr,
+                      kGroupNone, ncand);
+    int rc = launch_dist_single(j, ncand, nullptr, status, stream);
+    if (rc != NM_OK) return rc;
+    return launch(pick_kernel<DENSE_OUT>(j.n, j.m, j.bits, warps, blocks), nullptr, 0, d, blocks, warps, status, stream, Z, U_next,
+                  nullptr, kGroupScalesGiven, 0);
 }
 
 // Shared by the batched entry points: groups the jobs that can share one launch (same pattern, code width
@@ -1169,22 +1284,25 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
             NM_CUDA_TRY(cudaGetLastError());
         }
     }
-    if (dist_ncand > 0) {
-        // ADMM-Dist: the scale search writes every job's scales, the projection below takes them
-        for (size_t g = 0; g < keys.size(); ++g) {
-            const nm::PackJobDev* dev = reinterpret_cast<const nm::PackJobDev*>(ws) + group_first[g];
-            int rc = nm::launch_dist(nm::pick_dist(keys[g].n, keys[g].m, keys[g].bits, keys[g].warps), dev,
-                                     (int)groups[g].size(), nm::PackJobDev{}, group_blocks[g], keys[g].warps, status, s,
-                                     dist_ncand, nullptr);
-            if (rc != NM_OK) return rc;
-        }
-    }
     for (size_t g = 0; g < keys.size(); ++g) {
         const nm::PackJobDev* dev = reinterpret_cast<const nm::PackJobDev*>(ws) + group_first[g];
-        int rc = nm::launch(nm::pick_kernel<DENSE_OUT>(keys[g].n, keys[g].m, keys[g].bits, keys[g].warps, group_blocks[g]), dev,
-                            (int)groups[g].size(), nm::PackJobDev{}, group_blocks[g], keys[g].warps,
-                            status, s, nullptr, nullptr, DENSE_OUT ? dense_dev + group_first[g] : nullptr,
+        const Key& k = keys[g];
+        const int count = (int)groups[g].size();
+        const DenseOutDev* dense_g = DENSE_OUT ? dense_dev + group_first[g] : nullptr;
+        int rc;
+        if (dist_ncand > 0 && k.warps <= kPackMinWarps) {  // ADMM-Dist: search and projection in one kernel
+            rc = nm::launch(nm::pick_dist_pack<DENSE_OUT>(k.n, k.m, k.bits), dev, count, nm::PackJobDev{}, group_blocks[g], k.warps,
+                            status, s, nullptr, nullptr, dense_g, kGroupNone, dist_ncand);
+        } else {
+            if (dist_ncand > 0) {  // the search writes every job's scales, the projection takes them
+                rc = nm::launch_dist(nm::pick_dist(k.n, k.m, k.bits, k.warps), dev, count, nm::PackJobDev{}, group_blocks[g], k.warps,
+                                     status, s, dist_ncand, nullptr);
+                if (rc != NM_OK) return rc;
+            }
+            rc = nm::launch(nm::pick_kernel<DENSE_OUT>(k.n, k.m, k.bits, k.warps, group_blocks[g]), dev, count, nm::PackJobDev{},
+                            group_blocks[g], k.warps, status, s, nullptr, nullptr, dense_g,
                             (grouped || dist_ncand > 0) ? kGroupScalesGiven : kGroupNone, group_rows);
+        }
         if (rc != NM_OK) return rc;
     }
     return NM_OK;
@@ -1291,14 +1409,7 @@ int nm_project_pack_dist(const float* W, const float* U, int out, int in, int n,
     if (rc != NM_OK) return rc;
     if (ncand < 1 || ncand > NM_DIST_MAX_CANDIDATES) return NM_ERR_SHAPE;
     if (out == 0 || in == 0) return NM_OK;
-    rc = nm::launch_dist_single(j, ncand, nullptr, status, (cudaStream_t)stream);
-    if (rc != NM_OK) return rc;
-    nm::PackJobDev d = nm::to_dev(j);
-    int warps = std::max(nm::kPackMinWarps, 1 << d.wpr_log2);
-    int rows_per_block = warps >> d.wpr_log2;
-    unsigned blocks = (unsigned)((out + rows_per_block - 1) / rows_per_block);
-    return nm::launch(nm::pick_kernel(n, m, bits, warps, blocks), nullptr, 0, d, blocks, warps, status, (cudaStream_t)stream,
-                      nullptr, nullptr, nullptr, nm::kGroupScalesGiven, 0);
+    return nm::launch_dist_project_single<false>(j, ncand, status, (cudaStream_t)stream);
 }
 
 int nm_admm_project_dist(const float* W, const float* U, int out, int in, int n, int m, int bits, int ncand,
@@ -1310,14 +1421,7 @@ int nm_admm_project_dist(const float* W, const float* U, int out, int in, int n,
     if (ncand < 1 || ncand > NM_DIST_MAX_CANDIDATES) return NM_ERR_SHAPE;
     if (out == 0 || in == 0) return NM_OK;
     nm_pack_job_t j{W, U, out, in, n, m, bits, values, meta, scales};
-    rc = nm::launch_dist_single(j, ncand, nullptr, status, (cudaStream_t)stream);
-    if (rc != NM_OK) return rc;
-    nm::PackJobDev d = nm::to_dev(j);
-    int warps = std::max(nm::kPackMinWarps, 1 << d.wpr_log2);
-    int rows_per_block = warps >> d.wpr_log2;
-    unsigned blocks = (unsigned)((out + rows_per_block - 1) / rows_per_block);
-    return nm::launch(nm::pick_kernel<true>(n, m, bits, warps, blocks), nullptr, 0, d, blocks, warps, status,
-                      (cudaStream_t)stream, Z, U_next, nullptr, nm::kGroupScalesGiven, 0);
+    return nm::launch_dist_project_single<true>(j, ncand, status, (cudaStream_t)stream, Z, U_next);
 }
 
 int nm_project_pack_dist_batched(const nm_pack_job_t* jobs, int njobs, int ncand, void* ws, size_t ws_bytes,

@@ -130,6 +130,25 @@ def test_one_candidate_is_admm_max_and_extreme_magnitudes():
             assert (c == 0).all() and (s == 1.0).all()
 
 
+@pytest.mark.parametrize("k", [16, 1024, 1040, 2064, 4096])  # one, two and four warps per row, with and without a remainder
+@pytest.mark.parametrize("n,m,bits", [(2, 4, 4), (1, 8, 4), (4, 4, 8)])
+def test_rows_that_the_single_precision_bounds_cannot_decide(n, m, bits, k):
+    """Rows where several candidates stay within the bounds of the single-precision pass, and rows that skip it."""
+    W, _ = wl.pack_sweep_matrix(13, k, 11, k)
+    W[0] = 0.0                                            # every distance is 0: candidate 0
+    W[1] = np.float32(0.25) * np.sign(W[1])               # one magnitude: codes at the end of the range, clipped from j = 1 on
+    W[2] *= np.float32(2.0 ** -124)                       # scale below the range of the reciprocal
+    W[3] *= np.float32(2.0 ** 122)                        # ... and near its upper end
+    W[4] = np.where(np.arange(k) % 4 == 0, W[4], 0.0)     # mostly zeros
+    W[5, 1:] = 0.0                                        # a single value
+    W[6] = np.round(W[6] * 64.0) / 64.0                   # coarse grid: quotients on rounding ties
+    W[7] = W[8]                                           # equal rows choose equally
+    _check_pack(W, None, n, m, bits, 32)
+    s, c, rc = _gpu_dist_scales(W, None, n, m, bits, 32)
+    assert rc == 0 and c[0] == 0 and s[0] == 1.0 and c[7] == c[8]
+    _check_choice(W, None, n, m, bits, 32, s, c)
+
+
 @pytest.mark.parametrize("n,m,bits", [(2, 4, 4), (1, 4, 8), (4, 8, 4), (4, 4, 4)])
 def test_admm_step_dist_dense_outputs(n, m, bits):
     import paper_2206_15014_b200 as nm
