@@ -1,11 +1,9 @@
 // N:M magnitude projection + per-channel symmetric quantisation + packing (one HBM pass).
 //
-// Work decomposition: a warp owns a chunk of 1024 consecutive weights of one row; a row is
-// covered by 1, 2, 4 ... 32 warps of the same block.  Loads are coalesced 16-byte accesses
-// (lane l, step j -> float4 number j*32+l of the chunk); the sum V = W + U goes through a
-// swizzled shared-memory tile so that afterwards every lane holds 32 CONSECUTIVE values (8 groups
-// of 4 or 4 groups of 8).  From there everything is lane-local: the lane's share of the packed
-// values and of the metadata is a whole number of bytes, written with one vector store each.
+// Work decomposition: a row is covered by 1, 2, 4 ... 32 warps of the same block, a warp by up to four steps of 256
+// consecutive weights, of which every lane holds eight (32 bytes: one load per operand and step).  Eight consecutive weights
+// are whole groups of four or eight, so everything after the row maximum is lane-local and stays in registers; the
+// codes and the index fields of a step are one store each, coalesced over the warp.
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 #include <cuda_runtime.h>
@@ -65,7 +63,26 @@ int pack_set_skip_unit(int unit) {
 // `scales`; take the scales found in `scales`.
 enum { kGroupNone = 0, kGroupMaxPass = 1, kGroupScalesGiven = 2 };
 
-__device__ __forceinline__ float4 ld_stream(const float4* p) { return __ldcs(p); }
+// Eight consecutive floats that are not read again: one 32-byte access, or two of 16 bytes where the rows are only aligned to those.
+__device__ __forceinline__ void ld8(const float* p, float* x) {
+    asm volatile("ld.global.cs.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7]) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void ld4(const float* p, float* x) {
+    const float4 t = __ldcs(reinterpret_cast<const float4*>(p));
+    x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w;
+}
+__device__ __forceinline__ void st8(float* p, const float* x) {
+    asm volatile("st.global.cs.v8.f32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};" ::"f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "f"(x[4]),
+                 "f"(x[5]), "f"(x[6]), "f"(x[7]), "l"(p) : "memory");
+}
+__device__ __forceinline__ void st4(float* p, const float* x) { __stcs(reinterpret_cast<float4*>(p), make_float4(x[0], x[1], x[2], x[3])); }
+// max(|a|, |b|, m), NaN if any is NaN
+__device__ __forceinline__ float max_abs_nan(float a, float b, float m) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(fabsf(a)), "f"(fabsf(b)), "f"(m));
+    return r;
+}
 
 // Bit mask of the positions kept in one group: position i is kept iff fewer than N others beat it,
 // where j beats i when |v_j| > |v_i|, or |v_j| == |v_i| and j < i.
@@ -105,17 +122,15 @@ __device__ __forceinline__ void select_passes(const float* v, float* sel, unsign
 // Two of four by a tournament on the pairs (0,1) and (2,3).  With "larger magnitude first, lower index first
 // among equals" the two kept positions are 0 and 1 when the smaller of the first pair is >= the larger of the
 // second, 2 and 3 when the smaller of the second pair is > the larger of the first, and otherwise the larger of
-// each pair (the first one of a pair on equality).  Kept values and positions come out in ascending position.
-__device__ __forceinline__ void select_2_of_4(const float* v, float* sel, unsigned* selp) {
-    const float a0 = fabsf(v[0]), a1 = fabsf(v[1]), a2 = fabsf(v[2]), a3 = fabsf(v[3]);
-    const bool i01 = a1 > a0, i23 = a3 > a2;
-    const float hi01 = fmaxf(a0, a1), lo01 = fminf(a0, a1), hi23 = fmaxf(a2, a3), lo23 = fminf(a2, a3);
-    const bool both01 = lo01 >= hi23, both23 = lo23 > hi01;
-    const float w01 = i01 ? v[1] : v[0], w23 = i23 ? v[3] : v[2];
+// each pair (the first one of a pair on equality).  Kept values in ascending position; returns the index nibble.
+__device__ __forceinline__ unsigned select_2_of_4(const float* v, float* sel) {
+    const bool i01 = fabsf(v[1]) > fabsf(v[0]), i23 = fabsf(v[3]) > fabsf(v[2]);
+    const float w01 = i01 ? v[1] : v[0], l01 = i01 ? v[0] : v[1], w23 = i23 ? v[3] : v[2], l23 = i23 ? v[2] : v[3];
+    const bool both01 = fabsf(l01) >= fabsf(w23), both23 = fabsf(l23) > fabsf(w01);
     sel[0] = both01 ? v[0] : (both23 ? v[2] : w01);
     sel[1] = both01 ? v[1] : (both23 ? v[3] : w23);
-    selp[0] = both01 ? 0u : (both23 ? 2u : (i01 ? 1u : 0u));
-    selp[1] = both01 ? 1u : (both23 ? 3u : (i23 ? 3u : 2u));
+    const unsigned mixed = (i01 ? 9u : 8u) + (i23 ? 4u : 0u);
+    return both01 ? 0x4u : (both23 ? 0xEu : mixed);
 }
 
 template <int N, int M>
@@ -175,26 +190,6 @@ __device__ __forceinline__ unsigned keep_mask(const float* a) {
 #pragma unroll
     for (int i = 0; i < M; ++i) mask |= (rank[i] < N ? 1u : 0u) << i;
     return mask;
-}
-
-template <int NBYTES>
-__device__ __forceinline__ void store_bytes_vec(uint8_t* dst, const unsigned* w) {
-    if constexpr (NBYTES == 2) *reinterpret_cast<uint16_t*>(dst) = (uint16_t)w[0];
-    else if constexpr (NBYTES == 4) *reinterpret_cast<uint32_t*>(dst) = w[0];
-    else if constexpr (NBYTES == 8) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
-    else if constexpr (NBYTES == 16) *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-    else {
-        static_assert(NBYTES == 32, "unexpected lane share");
-        reinterpret_cast<uint4*>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-        reinterpret_cast<uint4*>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
-    }
-}
-
-template <int MAXBYTES>
-__device__ __forceinline__ void store_bytes_slow(uint8_t* dst, const unsigned* w, int nbytes) {
-#pragma unroll
-    for (int i = 0; i < MAXBYTES; ++i)
-        if (i < nbytes) dst[i] = (uint8_t)(w[i >> 2] >> ((i & 3) * 8));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -271,38 +266,26 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
     return d;
 }
 
-// The kept values of this lane, from the warp's tile.
-template <int N, int M>
-__device__ __forceinline__ void lane_kept_values(const float4* mytile, int lane, float* x) {
-    constexpr int G = 32 / M;
-    float v[32];
-#pragma unroll
-    for (int jj = 0; jj < 8; ++jj) {
-        const float4 t = mytile[lane * 8 + (jj ^ (lane & 7))];
-        v[jj * 4 + 0] = t.x; v[jj * 4 + 1] = t.y; v[jj * 4 + 2] = t.z; v[jj * 4 + 3] = t.w;
-    }
-#pragma unroll
-    for (int g = 0; g < G; ++g) kept_values<N, M>(v + g * M, x + g * N);
-}
-
-// Distance of candidate j in double over the warp's chunk (every lane returns the sum over the lanes).
+// Distance of candidate j in double over the warp's part of the row (every lane returns the sum over the lanes).
 template <int N, int M, int BITS>
-__device__ __noinline__ double dist_exact(const float4* mytile, int lane, float smax, int j) {
-    constexpr int KN = 32 / M * N;
+__device__ __forceinline__ double dist_exact(const float* v, float smax, int j) {
     constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
     constexpr float kLo = -(float)(1 << (BITS - 1)) - 0.49f, kHi = qmax + 0.49f;
     constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
-    float x[KN];
-    lane_kept_values<N, M>(mytile, lane, x);
     const float sj = __fmul_rn(smax, (float)(64 - j) * 0.015625f);
     const double nsd = -(double)sj;
     double e0 = 0.0, e1 = 0.0;
-#pragma unroll 4
-    for (int i = 0; i < KN; ++i) {
-        const float qc = fminf(fmaxf(__fdiv_rn(x[i], sj), kLo), kHi);
-        const float r = __fsub_rn(__fadd_rn(qc, kMagic), kMagic);  // nearest-even integer of qc
-        const double d = fma(nsd, (double)r, (double)x[i]);
-        if (i & 1) e1 = fma(d, d, e1); else e0 = fma(d, d, e0);
+#pragma unroll
+    for (int g = 0; g < 32 / M; ++g) {
+        float x[N];
+        kept_values<N, M>(v + g * M, x);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const float qc = fminf(fmaxf(__fdiv_rn(x[i], sj), kLo), kHi);
+            const float r = __fsub_rn(__fadd_rn(qc, kMagic), kMagic);  // nearest-even integer of qc
+            const double d = fma(nsd, (double)r, (double)x[i]);
+            if ((g * N + i) & 1) e1 = fma(d, d, e1); else e0 = fma(d, d, e0);
+        }
     }
     double e = e0 + e1;
 #pragma unroll
@@ -313,9 +296,9 @@ __device__ __noinline__ double dist_exact(const float4* mytile, int lane, float 
 // Winning candidate of this warp's row.  `red_e` holds 32 doubles per warp of the block.  Every warp of the block calls it
 // (block-wide barriers when a row spans warps).
 template <int N, int M, int BITS>
-__device__ __forceinline__ int dist_search(const float4* mytile, int lane, int w, int wpr, int row_in_block, bool row_ok,
+__device__ __forceinline__ int dist_search(const float* v, int steps, int lane, int w, int wpr, int row_in_block, bool row_ok,
                                            float smax, bool bad, int ncand, double* red_e) {
-    constexpr int KN = 32 / M * N;                    // kept values per lane
+    constexpr int KN = 32 / M * N, KS = KN / 4;       // kept values per lane, and per step
     constexpr float qend = (float)(1 << (BITS - 1));  // magnitude of the negative end code
     constexpr float kMagic = 12582912.0f;             // 1.5 * 2^23: adding it rounds to the nearest-even integer
     constexpr float kEps = qend * 1.9073486328125e-6f;  // 2^(b - 1) * 2^-19
@@ -327,7 +310,8 @@ __device__ __forceinline__ int dist_search(const float4* mytile, int lane, int w
         float lim[KN];
         {
             float x[KN];
-            lane_kept_values<N, M>(mytile, lane, x);
+#pragma unroll
+            for (int g = 0; g < 32 / M; ++g) kept_values<N, M>(v + g * M, x + g * N);
             const float r0 = __frcp_rn(smax);
 #pragma unroll
             for (int i = 0; i < KN; ++i) lim[i] = kMagic + (x[i] < 0.0f ? qend : qend - 1.0f);
@@ -336,45 +320,57 @@ __device__ __forceinline__ int dist_search(const float4* mytile, int lane, int w
         }
         const float my_inv = __frcp_rn((float)(64 - lane) * 0.015625f);  // 64 / (64 - j) of candidate j = lane
         const uint64_t magic2 = pack_f32x2(kMagic, kMagic), nmagic2 = pack_f32x2(-kMagic, -kMagic);
-        // eight candidates at a time; their sums over the lanes by a transposing butterfly (lane l ends up with
-        // candidate 8 * group + (l >> 2)), of which lane l keeps group l & 3's
+        // kTrip candidates a trip, their sums over the lanes by a transposing butterfly: lane l ends up with candidate
+        // kTrip * g + l / (32 / kTrip) of trip g and keeps trip l % (32 / kTrip)'s.  Eight a trip where a lane keeps 16 values (85 M
+        // weights at 2:4 / 4 bit 457 us, with two 504); two where it keeps more or fewer: the body of eight no longer fits
+        // the instruction cache (4:4 / 8 bit 276 -> 260 us), or its registers cost occupancy (1:4 144 -> 126).
+        constexpr int kTrip = KN == 16 ? 8 : 2, kLanes = 32 / kTrip;
         float kept = inf;
 #pragma unroll 1
-        for (int g = 0; g < 4; ++g) {
-            if (8 * g >= ncand) break;
-            float e[8];
+        for (int g = 0; kTrip * g < ncand; ++g) {
+            float e[kTrip];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const float inv = __shfl_sync(0xffffffffu, my_inv, 8 * g + k);
-                const float na = (float)(8 * g + k - 64) * 0.015625f;  // -(64 - j) / 64
+            for (int k = 0; k < kTrip; ++k) {
+                const float inv = __shfl_sync(0xffffffffu, my_inv, kTrip * g + k);
+                const float na = (float)(kTrip * g + k - 64) * 0.015625f;  // -(64 - j) / 64
                 const uint64_t inv2 = pack_f32x2(inv, inv), na2 = pack_f32x2(na, na);
                 uint64_t acc = 0;
-#pragma unroll
-                for (int i = 0; i < KN / 2; ++i) {
+                auto add = [&](int i) {
                     float t0, t1;
                     unpack_f32x2(fma_f32x2(y[i], inv2, magic2), t0, t1);
                     const uint64_t code = add_f32x2(pack_f32x2(fminf(t0, lim[2 * i]), fminf(t1, lim[2 * i + 1])), nmagic2);
                     const uint64_t d = fma_f32x2(na2, code, y[i]);
                     acc = fma_f32x2(d, d, acc);
+                };
+                if constexpr (KS >= 4) {
+#pragma unroll
+                    for (int st = 0; st < 4; ++st)
+                        if (st < steps) {  // steps beyond the warp's columns hold zeros
+#pragma unroll
+                            for (int i = st * KS / 2; i < (st + 1) * KS / 2; ++i) add(i);
+                        }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < KN / 2; ++i) add(i);
                 }
                 float a0, a1;
                 unpack_f32x2(acc, a0, a1);
                 e[k] = a0 + a1;
             }
 #pragma unroll
-            for (int h = 4; h >= 1; h >>= 1) {
-                const bool up = lane & (4 * h);
+            for (int h = kTrip / 2; h >= 1; h >>= 1) {
+                const bool up = lane & (kLanes * h);
 #pragma unroll
                 for (int k = 0; k < h; ++k) {
                     const float keep = up ? e[k + h] : e[k], give = up ? e[k] : e[k + h];
-                    e[k] = keep + __shfl_xor_sync(0xffffffffu, give, 4 * h);
+                    e[k] = keep + __shfl_xor_sync(0xffffffffu, give, kLanes * h);
                 }
             }
-            e[0] += __shfl_xor_sync(0xffffffffu, e[0], 2);
-            e[0] += __shfl_xor_sync(0xffffffffu, e[0], 1);
-            if ((lane & 3) == g) kept = e[0];
+#pragma unroll
+            for (int o = kLanes / 2; o > 0; o >>= 1) e[0] += __shfl_xor_sync(0xffffffffu, e[0], o);
+            if (lane % kLanes == g) kept = e[0];
         }
-        mine = __shfl_sync(0xffffffffu, kept, ((lane & 7) << 2) | (lane >> 3));  // candidate j to lane j
+        mine = __shfl_sync(0xffffffffu, kept, (lane % kTrip) * kLanes + lane / kTrip);  // candidate j to lane j
     }
     if (wpr > 1) {
         float* red_f = reinterpret_cast<float*>(red_e);
@@ -398,7 +394,7 @@ __device__ __forceinline__ int dist_search(const float4* mytile, int lane, int w
     if (!single) {
         for (unsigned m = mask; m; m &= m - 1u) {
             const int j = __ffs(m) - 1;
-            const double e = dist_exact<N, M, BITS>(mytile, lane, smax, j);
+            const double e = dist_exact<N, M, BITS>(v, smax, j);
             if (lane == j) exact = e;
         }
     }
@@ -422,23 +418,11 @@ __device__ __forceinline__ int dist_search(const float4* mytile, int lane, int w
     return bj < ncand ? bj : 0;  // only when every distance is NaN or infinite (non-finite input)
 }
 
-// N == M: dense (quantise only, no metadata), processed in groups of 4.
-// DENSE_OUT: the ADMM step / STE forward form.  Besides (or instead of: values, meta and scales may then be
-// null) the packed outputs the kernel writes Z = s * code as dense fp32, zero where pruned, and, when
-// U_next is not null, the dual update U_next = (W + U) - Z.  Both go back through the shared-memory
-// tile so that the stores are as coalesced as the loads.
-//
-// A "unit" is what one block does at a time: `warps >> wpr_log2` rows of one job, one 1024-value chunk per warp.
-// PIPE (blocks of four warps): the grid is persistent, block b takes the units b, b + gridDim.x, ...; every warp
-// fetches the chunk of its NEXT unit (W and U, 4 KB each) with two bulk copies into the other half of a
-// double buffer in shared memory while it works on the current one, so that loading and arithmetic overlap
-// inside a warp and not only between blocks that happen to be out of step.  Without PIPE one block = one unit
-// and the chunk is loaded with 16-byte global loads.
-
-// Where a warp stands inside a unit of a job.
+// Where a warp stands inside a unit of a job.  A "unit" is what one block does at a time: `warps >> wpr_log2` rows of one job.
 struct UnitPos {
     long long row;
-    int chunk, row_in_block, elems;  // elems: values of the chunk that lie inside the row (0 when the row does not exist)
+    int first, steps, elems;  // first column of the warp, its steps of 256 columns, its columns inside the row (0 when the row does not exist)
+    int chunk, row_in_block;
     bool row_ok;
 };
 
@@ -449,7 +433,9 @@ __device__ __forceinline__ UnitPos unit_pos(const PackJobDev& job, unsigned unit
     u.chunk = w & (wpr - 1);
     u.row = (long long)(unit - job.unit_begin) * (warps >> job.wpr_log2) + u.row_in_block;
     u.row_ok = u.row < job.out;
-    u.elems = u.row_ok ? max(0, min(1024, job.in - u.chunk * 1024)) : 0;
+    u.steps = (((job.in + 255) >> 8) + wpr - 1) >> job.wpr_log2;  // at most 4
+    u.first = u.chunk * u.steps * 256;
+    u.elems = u.row_ok ? max(0, min(u.steps * 256, job.in - u.first)) : 0;
     return u;
 }
 
@@ -486,349 +472,404 @@ __device__ __forceinline__ unsigned units_of(const PackJobDev& job, int warps) {
     return (unsigned)((job.out + rpb - 1) / rpb);
 }
 
-// Everything after the load: `mytile` holds the warp's chunk of V = W + U in the swizzled layout, `amax` and
-// `poison` are the lane's running |max| and non-finite detector.  `red` is this unit's slot array for the row
-// maximum across the warps of a row.  Every warp of the block calls it (block-wide barrier when a row spans warps).
-template <int N, int M, int BITS, bool DENSE_OUT, bool DIST = false>
-__device__ __forceinline__ void pack_finish(const PackJobDev& job, const UnitPos& up, int lane, int w, float4* mytile,
-                                            float* red, const uint16_t* pos48, float amax, float poison, uint32_t* status,
-                                            float* __restrict__ Zout, float* __restrict__ Unext, int group_mode, int group_rows,
-                                            double* red_e = nullptr) {
-    constexpr bool kDense = (N == M);
-    constexpr int G = 32 / M;                          // groups per lane
-    constexpr int F = (M == 4) ? 2 : 4;                // metadata field width
-    constexpr int VBITS = G * N * BITS;                // value bits per lane (16 .. 256)
-    constexpr int VWORDS = (VBITS + 31) / 32;
-    constexpr int MBITS = kDense ? 0 : G * N * F;      // metadata bits per lane (0, 16, 32, 64)
-    constexpr int MWORDS = kDense ? 1 : (MBITS + 31) / 32;
-    const int wpr = 1 << job.wpr_log2;
-    const int row_in_block = up.row_in_block, chunk = up.chunk;
-    const long long row = up.row;
-    const bool row_ok = up.row_ok;
-    const int in4 = job.in >> 2;
+// Maximum magnitude of the row that this warp works on, from the lanes' shares `v` (zeros outside the row).  `bad`: the warp's part
+// holds a value that is not finite; the maximum of such a row leaves its NaNs out.  `red`: one slot per warp of the
+// block.  Every warp of the block calls it (block-wide barrier when a row spans warps).
+__device__ __forceinline__ float row_max(const float* v, int lane, int w, int wpr, int row_in_block, float* red,
+                                         uint32_t* status, bool& bad) {
+    float amax = 0.0f;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    const bool bad = __any_sync(0xffffffffu, poison != poison) || !(amax <= 3.402823466e+38f);
-    if (bad && lane == 0 && status) atomicOr(status, NM_STATUS_NONFINITE);
+    for (int i = 0; i < 16; ++i) amax = max_abs_nan(v[2 * i], v[2 * i + 1], amax);
+    bad = __any_sync(0xffffffffu, !(amax <= 3.402823466e+38f));
+    if (bad) {
+        if (lane == 0 && status) atomicOr(status, NM_STATUS_NONFINITE);
+        amax = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) amax = fmaxf(amax, fabsf(v[i]));
+    }
+    amax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(amax)));
     if (wpr > 1) {
         if (lane == 0) red[w] = amax;
         __syncthreads();
         for (int c = 0; c < wpr; ++c) amax = fmaxf(amax, red[row_in_block * wpr + c]);
-    } else {
-        __syncwarp();
     }
+    return amax;
+}
+
+// The code of x at the scale s as a float, 1.5 * 2^23 + OFFSET + code, from the IEEE quotient (Eq. 5: rounded half to even, clamped).
+template <int BITS, int OFFSET>
+__device__ __noinline__ float code_exact(float x, float s) {
+    constexpr float kLo = -(float)(1 << (BITS - 1)) - 0.49f, kHi = (float)((1 << (BITS - 1)) - 1) + 0.49f;
+    return __fadd_rn(fminf(fmaxf(__fdiv_rn(x, s), kLo), kHi), 12582912.0f + (float)OFFSET);
+}
+
+template <int BYTES>
+__device__ __forceinline__ void store_lane(uint8_t* dst, const unsigned* w) {
+    if constexpr (BYTES == 1) *dst = (uint8_t)w[0];
+    else if constexpr (BYTES == 2) *reinterpret_cast<uint16_t*>(dst) = (uint16_t)w[0];
+    else if constexpr (BYTES == 4) *reinterpret_cast<uint32_t*>(dst) = w[0];
+    else { static_assert(BYTES == 8, "lane share"); *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]); }
+}
+
+// Everything after the row maximum (row_max): `v` holds the lane's share of V = W + U (eight values per step, zeros outside the row).
+//
+// N == M: dense (quantise only, no metadata), processed in groups of 4.
+// DENSE_OUT: the ADMM step / STE forward form.  Besides (or instead of: values, meta and scales may then be
+// null) the packed outputs the kernel writes Z = s * code as dense fp32, zero where pruned, and, when
+// U_next is not null, the dual update U_next = (W + U) - Z, both as coalesced as the loads.
+// CLIP: the scale may be smaller than the row's maximum asks for (a searched scale), so codes are clamped; a scale from the
+// row's or its group's maximum leaves nothing to clamp.
+//
+// Codes: t = fma(v, RN(1 / s), 1.5 * 2^23) rounds the product to the nearest-even integer, r = t - 1.5 * 2^23 is that
+// integer, and f = fma(v, RN(1 / s), -r) its distance.  The product is within 2^-16 of the IEEE quotient over the code range,
+// so the code is the quotient's unless |f| is within 2^-15 of a half (6 values in 100000), which is looked at
+// once per step; those lanes, and rows with a scale outside the range where RN(1 / s) is a normal number or with a
+// non-finite value, take the division.
+template <int N, int M, int BITS, bool DENSE_OUT, bool CLIP>
+__device__ __forceinline__ void pack_row(const PackJobDev& job, const UnitPos& up, int lane, const float* v, float s, bool bad,
+                                         const uint16_t* pos48, float* scratch, float* __restrict__ Zout,
+                                         float* __restrict__ Unext, bool wide) {
+    constexpr bool kDense = (N == M);
+    constexpr int G = 8 / M;                           // groups per lane and step
+    constexpr int F = (M == 4) ? 2 : 4;                // metadata field width
+    constexpr int KS = G * N;                          // kept values per lane and step
+    constexpr int VBITS = KS * BITS;                   // value bits per lane and step (4 .. 64)
+    constexpr int VWORDS = (VBITS + 31) / 32;
+    constexpr int MBITS = kDense ? 0 : KS * F;         // metadata bits per lane and step (0, 4, 8, 16)
+    constexpr int kOffset = BITS == 4 ? 8 : 0;         // 4-bit codes are collected as unsigned nibbles code + 8
+    constexpr float kMagic = 12582912.0f + (float)kOffset;
+    constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
+    const long long row = up.row;
+    const float rs = __frcp_rn(s);  // correctly rounded reciprocal, once per row
+    const bool fast_ok = !bad && (s >= 1.17549435e-38f) && (s <= 4.25e37f);  // rs is a normal number
+
+    const unsigned mrow_bytes = job.mrow_words * 4u;
+    uint8_t* const vrow = (!DENSE_OUT || job.values) ? job.values + (size_t)row * job.vrow_bytes : nullptr;
+    uint8_t* const mrow = kDense || (DENSE_OUT && !job.meta) ? nullptr : reinterpret_cast<uint8_t*>(job.meta + (size_t)row * job.mrow_words);
+    constexpr int VB = VBITS >= 8 ? VBITS / 8 : 1;     // bytes of a lane's (or pair of lanes') codes
+    const bool vec_ok = VB == 1 || (job.vrow_bytes % VB == 0);  // the values start on a 16-byte boundary
+
+#pragma unroll
+    for (int st = 0; st < 4; ++st) {
+        if (st >= up.steps) break;
+        const int col = up.first + st * 256 + lane * 8;             // first column of this lane
+        const int nvals = max(0, min(8, job.in - col));             // columns inside the row: 0, 4 or 8
+        const float* x8 = v + st * 8;
+        float sel[KS];
+        unsigned mbits = 0;
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const float* x = x8 + g * M;
+            float* k = sel + g * N;
+            if constexpr (kDense) {
+#pragma unroll
+                for (int p = 0; p < M; ++p) k[p] = x[p];
+            } else if constexpr (N == 2 && M == 4) {
+                mbits |= select_2_of_4(x, k) << (4 * g);
+            } else if constexpr (N == 4) {
+                // four of eight: the keep mask indexes a table whose entry is the four positions, i.e. the group's
+                // metadata; the kept values are fetched by position from a column of shared memory of this lane
+                float a[M];
+#pragma unroll
+                for (int p = 0; p < M; ++p) { a[p] = fabsf(x[p]); scratch[p * 32 + lane] = x[p]; }
+                mbits = pos48[keep_mask<N, M>(a)];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) k[c] = scratch[((mbits >> (4 * c)) & 7u) * 32 + lane];
+            } else {
+                unsigned selp[N];
+                select_passes<N, M>(x, k, selp);
+#pragma unroll
+                for (int c = 0; c < N; ++c) mbits |= selp[c] << ((g * N + c) * F);
+            }
+        }
+        float t[KS], worst = 0.0f;
+#pragma unroll
+        for (int c = 0; c < KS; ++c) {
+            t[c] = __fmaf_rn(sel[c], rs, kMagic);
+            worst = fmaxf(worst, fabsf(__fmaf_rn(sel[c], rs, -__fsub_rn(t[c], kMagic))));
+            if (CLIP) t[c] = fminf(fmaxf(t[c], kMagic - qmax - 1.0f), kMagic + qmax);
+        }
+        if (!(worst <= 0.49996948f) || !fast_ok) {
+#pragma unroll
+            for (int c = 0; c < KS; ++c) t[c] = code_exact<BITS, kOffset>(sel[c], s);
+        }
+        if (nvals == 0) {  // past the end of the row: zeros in the metadata's padding
+#pragma unroll
+            for (int c = 0; c < KS; ++c) t[c] = kMagic;
+            mbits = 0;
+        } else if (M == 4 && nvals == 4) {
+            mbits &= (1u << (MBITS / 2)) - 1u;
+        }
+
+        // ---- dense outputs (ADMM step) -----------------------------------------------------------
+        if constexpr (DENSE_OUT) {
+            float z[8];
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+#pragma unroll
+                for (int p = 0; p < M; ++p) {
+                    if constexpr (kDense) {
+                        z[g * M + p] = __fmul_rn(s, __fsub_rn(t[g * M + p], kMagic));
+                    } else {
+                        float zp = 0.0f;
+#pragma unroll
+                        for (int c = 0; c < N; ++c) {
+                            const unsigned pos = (mbits >> ((g * N + c) * F)) & (unsigned)(M - 1);
+                            zp = pos == (unsigned)p ? __fmul_rn(s, __fsub_rn(t[g * N + c], kMagic)) : zp;
+                        }
+                        z[g * M + p] = zp;
+                    }
+                }
+            float* zp = Zout + (size_t)row * job.in + col;
+            if (wide) {
+                if (nvals == 8) st8(zp, z);
+            } else {
+                if (nvals >= 4) st4(zp, z);
+                if (nvals == 8) st4(zp + 4, z + 4);
+            }
+            if (Unext) {
+                float* np = Unext + (size_t)row * job.in + col;
+                float u[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) u[i] = __fsub_rn(x8[i], z[i]);  // (W + U) - Z
+                if (wide) {
+                    if (nvals == 8) st8(np, u);
+                } else {
+                    if (nvals >= 4) st4(np, u);
+                    if (nvals == 8) st4(np + 4, u + 4);
+                }
+            }
+        }
+
+        // ---- packed outputs ------------------------------------------------------------------------
+        const int unit8 = col >> 3;  // number of the lane's eight columns in the row
+        if (vrow) {
+            unsigned vw[VWORDS];
+            if constexpr (BITS == 8) {
+                auto b = [&](int c) { return __float_as_uint(t[c < KS ? c : 0]); };
+#pragma unroll
+                for (int i = 0; i < VWORDS; ++i)  // the low bytes of up to four codes
+                    vw[i] = __byte_perm(__byte_perm(b(4 * i), b(4 * i + 1), 0x0040), __byte_perm(b(4 * i + 2), b(4 * i + 3), 0x0040), 0x5410);
+            } else {
+                // sum of (0x4B400000 + nibble) << 4 c, less the sum of the constants, modulo 2^32
+                unsigned acc = 0, base = 0, flip = 0;
+#pragma unroll
+                for (int c = 0; c < KS; ++c) {
+                    acc += __float_as_uint(t[c]) << (4 * c);
+                    base += 0x4B400000u << (4 * c);
+                    flip |= 8u << (4 * c);
+                }
+                vw[0] = (acc - base) ^ flip;  // code + 8 to two's complement
+            }
+            if constexpr (VBITS == 4) {  // two lanes share a byte
+                const unsigned other = __shfl_down_sync(0xffffffffu, vw[0], 1);
+                if ((lane & 1) == 0 && nvals > 0) vrow[unit8 >> 1] = (uint8_t)(vw[0] | (other << 4));
+            } else {
+                uint8_t* dst = vrow + (size_t)unit8 * (VBITS / 8);
+                if (nvals == 8 && vec_ok) store_lane<VB>(dst, vw);
+                else {
+                    const int nb = nvals * VBITS / 64;
+#pragma unroll
+                    for (int i = 0; i < VB; ++i)
+                        if (i < nb) dst[i] = (uint8_t)(vw[i >> 2] >> ((i & 3) * 8));
+                }
+            }
+        }
+        if constexpr (!kDense) {
+            if (mrow) {
+                if constexpr (MBITS == 4) {
+                    const unsigned other = __shfl_down_sync(0xffffffffu, mbits, 1);
+                    if ((lane & 1) == 0 && (unsigned)(unit8 >> 1) < mrow_bytes) mrow[unit8 >> 1] = (uint8_t)(mbits | (other << 4));
+                } else {
+                    constexpr int MB = MBITS / 8;
+                    if ((unsigned)unit8 * MB < mrow_bytes) store_lane<MB>(mrow + (size_t)unit8 * MB, &mbits);
+                }
+            }
+        }
+    }
+}
+
+// From the loaded row to its outputs.  `red`: this unit's slots for row_max.  Every warp of the block calls it.
+template <int N, int M, int BITS, bool DENSE_OUT, bool DIST = false>
+__device__ __forceinline__ void pack_finish(const PackJobDev& job, const UnitPos& up, int lane, int w, const float* v,
+                                            float* red, const uint16_t* pos48, float* scratch, uint32_t* status,
+                                            float* __restrict__ Zout, float* __restrict__ Unext, bool wide, int group_mode, int group_rows,
+                                            double* red_e = nullptr) {
+    const int wpr = 1 << job.wpr_log2;
+    bool bad;
+    const float amax = row_max(v, lane, w, wpr, up.row_in_block, red, status, bad);
 
     // ---- group-wise scales, first pass: fold this row's maximum into the first entry of its group -----
     if (group_mode == kGroupMaxPass) {
-        if (row_ok && chunk == 0 && lane == 0) {
+        if (up.row_ok && up.chunk == 0 && lane == 0) {
             const int G = (group_rows <= 0 || group_rows > job.out) ? job.out : group_rows;
-            atomicMax(reinterpret_cast<unsigned*>(job.scales) + (size_t)(row / G) * G, __float_as_uint(amax));
+            atomicMax(reinterpret_cast<unsigned*>(job.scales) + (size_t)(up.row / G) * G, __float_as_uint(amax));
         }
         return;
     }
 
     // ---- ADMM-Max scale ---------------------------------------------------------------------
     constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
-    // group-wise quantisation hands the scale in (one per row, equal within a group of rows)
-    float s = !DIST && group_mode == kGroupScalesGiven ? job.scales[row_ok ? row : 0]
-                                                       : ((amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax));
+    float s;
+    if (!DIST && group_mode == kGroupScalesGiven) {
+        // one scale per row, equal within a group of rows, or searched before (rows of more than 4096 weights)
+        if (!up.row_ok) return;
+        s = job.scales[up.row];
+        pack_row<N, M, BITS, DENSE_OUT, true>(job, up, lane, v, s, bad, pos48, scratch, Zout, Unext, wide);
+        return;
+    }
+    s = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
     if constexpr (DIST) {  // group_rows carries the number of candidate scales
-        const int best = dist_search<N, M, BITS>(mytile, lane, w, wpr, row_in_block, row_ok, s, bad, group_rows, red_e);
+        const int best = dist_search<N, M, BITS>(v, up.steps, lane, w, wpr, up.row_in_block, up.row_ok, s, bad, group_rows, red_e);
         s = __fmul_rn(s, (float)(64 - best) * 0.015625f);
     }
-    if (row_ok && chunk == 0 && lane == 0 && (!DENSE_OUT || job.scales)) job.scales[row] = s;
-    const float rs = __frcp_rn(s);  // correctly rounded reciprocal, once per row
-    const bool fast_ok = (s >= 1.17549435e-38f) && (s <= 4.25e37f);  // rs is a normal number
+    if (!up.row_ok) return;
+    if (up.chunk == 0 && lane == 0 && (!DENSE_OUT || job.scales)) job.scales[up.row] = s;
+    pack_row<N, M, BITS, DENSE_OUT, DIST>(job, up, lane, v, s, bad, pos48, scratch, Zout, Unext, wide);
+}
 
-    // ---- this lane's 32 consecutive values ----------------------------------------------------
-    float v[32];
+// Loads the lane's share of V = W + U straight from global memory.  `wide`: 32-byte accesses are aligned and rows end on them.
+__device__ __forceinline__ void load_global(const PackJobDev& job, const UnitPos& up, int lane, bool wide, float* v) {
+    const size_t at = (size_t)(up.row_ok ? up.row : 0) * job.in + up.first + lane * 8;
+    const float* W = job.W + at;
+    const float* U = job.U ? job.U + at : nullptr;
 #pragma unroll
-    for (int jj = 0; jj < 8; ++jj) {
-        float4 t = mytile[lane * 8 + (jj ^ (lane & 7))];
-        v[jj * 4 + 0] = t.x; v[jj * 4 + 1] = t.y; v[jj * 4 + 2] = t.z; v[jj * 4 + 3] = t.w;
-    }
-    const int lane_first = chunk * 1024 + lane * 32;             // first column of this lane
-    const int nvals = max(0, min(32, job.in - lane_first));      // columns inside the row
-    if (!DENSE_OUT && (!row_ok || nvals == 0)) return;
-    float z[DENSE_OUT ? 32 : 1];  // dequantised projection of this lane's values (DENSE_OUT)
-    if constexpr (DENSE_OUT) {
+    for (int i = 0; i < 32; ++i) v[i] = 0.0f;
+    const int mine = up.elems - lane * 8;  // columns from this lane's first one to the end of the warp's part
+    if (wide) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) z[i] = 0.0f;
-    }
-
-    unsigned vw[VWORDS], mw[MWORDS];
+        for (int st = 0; st < 4; ++st)
+            if (st * 256 < mine) ld8(W + st * 256, v + st * 8);
+        if (U) {
 #pragma unroll
-    for (int i = 0; i < VWORDS; ++i) vw[i] = 0;
+            for (int st = 0; st < 4; ++st)
+                if (st * 256 < mine) {
+                    float u[8];
+                    ld8(U + st * 256, u);
 #pragma unroll
-    for (int i = 0; i < MWORDS; ++i) mw[i] = 0;
-
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        if (g * M < nvals) {
-            if constexpr (kDense) {
-#pragma unroll
-                for (int p = 0; p < M; ++p) {
-                    const int pos = (g * M + p) * BITS;
-                    const int code = quantise_shared_scale<BITS>(v[g * M + p], s, rs, fast_ok);
-                    vw[pos >> 5] |= ((unsigned)code & ((1u << BITS) - 1u)) << (pos & 31);
-                    if constexpr (DENSE_OUT) z[g * M + p] = __fmul_rn(s, (float)code);
+                    for (int i = 0; i < 8; ++i) v[st * 8 + i] = __fadd_rn(v[st * 8 + i], u[i]);
                 }
-            } else {
-                float sel[N];
-                unsigned selp[N];
-#pragma unroll
-                for (int c = 0; c < N; ++c) { sel[c] = 0.0f; selp[c] = 0; }
-                constexpr bool kPasses = (N == 1) || (N == 2 && M == 8) || (N == 2 && M == 4);
-                unsigned mask = 0;
-                if constexpr (N == 2 && M == 4) {
-                    select_2_of_4(v + g * M, sel, selp);
-                } else if constexpr (kPasses) {
-                    select_passes<N, M>(v + g * M, sel, selp);
-                } else {
-                    float a[M];
-#pragma unroll
-                    for (int p = 0; p < M; ++p) a[p] = fabsf(v[g * M + p]);
-                    mask = keep_mask<N, M>(a);
-                }
-                // compaction: slot c receives the c-th kept position (ascending)
-                if constexpr (kPasses) {
-                } else if constexpr (N == 4 && M == 8) {
-                    const unsigned pos4 = pos48[mask];
-                    const float* tile_f = reinterpret_cast<const float*>(mytile);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        selp[c] = (pos4 >> (4 * c)) & 7u;
-                        const unsigned e = (unsigned)(g * 8) + selp[c];  // element of this lane, in the tile's swizzle
-                        sel[c] = tile_f[(lane * 8 + ((e >> 2) ^ (lane & 7))) * 4 + (e & 3u)];
-                    }
-                } else {
-#pragma unroll
-                for (int p = 0; p < M; ++p) {
-                    const bool kept = (mask >> p) & 1u;
-                    const int before = __popc(mask & ((1u << p) - 1u));
-#pragma unroll
-                    for (int c = 0; c < N; ++c) {
-                        // position p can only land in slot c if c <= p and enough positions remain
-                        if (c <= p && (M - p) >= (N - c)) {
-                            const bool hit = kept && before == c;
-                            sel[c] = hit ? v[g * M + p] : sel[c];
-                            selp[c] = hit ? (unsigned)p : selp[c];
-                        }
-                    }
-                }
-                }
-#pragma unroll
-                for (int c = 0; c < N; ++c) {
-                    const int vpos = (g * N + c) * BITS, mpos = (g * N + c) * F;
-                    const int code = quantise_shared_scale<BITS>(sel[c], s, rs, fast_ok);
-                    vw[vpos >> 5] |= ((unsigned)code & ((1u << BITS) - 1u)) << (vpos & 31);
-                    mw[mpos >> 5] |= selp[c] << (mpos & 31);
-                    if constexpr (DENSE_OUT) {
-                        const float zc = __fmul_rn(s, (float)code);
-#pragma unroll
-                        for (int p = 0; p < M; ++p) z[g * M + p] = (selp[c] == (unsigned)p) ? zc : z[g * M + p];
-                    }
-                }
-            }
         }
-    }
-
-    // ---- dense outputs (ADMM step): back through the tile, then coalesced 16-byte stores --------
-    if constexpr (DENSE_OUT) {
-        auto write_back = [&](const float* x, float* dst_base) {
+    } else {
 #pragma unroll
-            for (int jj = 0; jj < 8; ++jj)
-                mytile[lane * 8 + (jj ^ (lane & 7))] = make_float4(x[jj * 4], x[jj * 4 + 1], x[jj * 4 + 2], x[jj * 4 + 3]);
-            __syncwarp();
-            float4* D4 = reinterpret_cast<float4*>(dst_base) + (row_ok ? row * in4 : 0);
+        for (int h = 0; h < 8; ++h)
+            if ((h >> 1) * 256 + (h & 1) * 4 < mine) ld4(W + (h >> 1) * 256 + (h & 1) * 4, v + h * 4);
+        if (U) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int fl = j * 32 + lane, owner = fl >> 3, jj = fl & 7, f = chunk * 256 + fl;
-                const float4 t = mytile[owner * 8 + (jj ^ (owner & 7))];
-                if (row_ok && f < in4) __stcs(D4 + f, t);
-            }
-            __syncwarp();
-        };
-        write_back(z, Zout);
-        if (Unext) {
+            for (int h = 0; h < 8; ++h)
+                if ((h >> 1) * 256 + (h & 1) * 4 < mine) {
+                    float u[4];
+                    ld4(U + (h >> 1) * 256 + (h & 1) * 4, u);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = __fsub_rn(v[i], z[i]);  // (W + U) - Z
-            write_back(v, Unext);
-        }
-        if (!row_ok || nvals == 0) return;
-    }
-
-    // ---- stores -----------------------------------------------------------------------------
-    const int lane_global = chunk * 32 + lane;
-    const bool full = (nvals == 32);
-    if (!DENSE_OUT || job.values) {
-        constexpr int LB = VBITS / 8;
-        uint8_t* dst = job.values + (size_t)row * job.vrow_bytes + (size_t)lane_global * LB;
-        if (full && (reinterpret_cast<uintptr_t>(dst) % (LB < 16 ? LB : 16)) == 0) store_bytes_vec<LB>(dst, vw);
-        else store_bytes_slow<LB>(dst, vw, nvals / M * N * BITS / 8);
-    }
-    if constexpr (!kDense) {
-        if (DENSE_OUT && !job.meta) return;
-        constexpr int MB = MBITS / 8;
-        const unsigned lane_off = (unsigned)lane_global * MB;
-        const unsigned row_bytes = job.mrow_words * 4u;
-        uint8_t* dst = reinterpret_cast<uint8_t*>(job.meta + (size_t)row * job.mrow_words) + lane_off;
-        const bool last = (lane_first + 32 >= job.in);  // lane holding the end of the row
-        if (full && !last && (reinterpret_cast<uintptr_t>(dst) % MB) == 0) {  // aligned vector store
-            store_bytes_vec<MB>(dst, mw);
-        } else {
-            // the last lane also writes the zero padding up to the row's word boundary
-            const unsigned wpad[3] = {mw[0], MWORDS > 1 ? mw[MWORDS - 1] : 0u, 0u};
-            store_bytes_slow<MB + 4>(dst, wpad, last ? (int)min(row_bytes - lane_off, (unsigned)(MB + 4)) : MB);
+                    for (int i = 0; i < 4; ++i) v[h * 4 + i] = __fadd_rn(v[h * 4 + i], u[i]);
+                }
         }
     }
 }
 
-// Loads the warp's chunk with coalesced 16-byte global loads, leaves V = W + U in `mytile` (swizzled).
-__device__ __forceinline__ void load_chunk_global(const PackJobDev& job, const UnitPos& up, int lane, float4* mytile,
-                                                  float& amax, float& poison) {
-    const int in4 = job.in >> 2;
-    const float4* W4 = reinterpret_cast<const float4*>(job.W) + (up.row_ok ? up.row * in4 : 0);
-    const float4* U4 = job.U ? reinterpret_cast<const float4*>(job.U) + (up.row_ok ? up.row * in4 : 0) : nullptr;
-    float4 v[8];
+// The same from the part of the row that the bulk copies left in shared memory (`wbuf`, `ubuf`: up to 1024 floats each).
+// Every other group of four lanes reads its two 16-byte halves in the other order, so that no two lanes of a
+// quarter warp meet in a bank.
+__device__ __forceinline__ void load_staged(const PackJobDev& job, const UnitPos& up, int lane, const float* wbuf,
+                                            const float* ubuf, float* v) {
+    const bool swap = lane & 4;
+    const int a = lane * 8 + (swap ? 4 : 0), b = lane * 8 + (swap ? 0 : 4);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        int f = up.chunk * 256 + j * 32 + lane;
-        v[j] = (up.row_ok && f < in4) ? ld_stream(W4 + f) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    if (U4) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            int f = up.chunk * 256 + j * 32 + lane;
-            if (up.row_ok && f < in4) {
-                float4 u = ld_stream(U4 + f);
-                v[j].x = __fadd_rn(v[j].x, u.x); v[j].y = __fadd_rn(v[j].y, u.y);
-                v[j].z = __fadd_rn(v[j].z, u.z); v[j].w = __fadd_rn(v[j].w, u.w);
+    for (int st = 0; st < 4; ++st) {
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+        if (st * 256 + a < up.elems) x = *reinterpret_cast<const float4*>(wbuf + st * 256 + a);
+        if (st * 256 + b < up.elems) y = *reinterpret_cast<const float4*>(wbuf + st * 256 + b);
+        if (job.U) {
+            if (st * 256 + a < up.elems) {
+                const float4 u = *reinterpret_cast<const float4*>(ubuf + st * 256 + a);
+                x.x = __fadd_rn(x.x, u.x); x.y = __fadd_rn(x.y, u.y); x.z = __fadd_rn(x.z, u.z); x.w = __fadd_rn(x.w, u.w);
+            }
+            if (st * 256 + b < up.elems) {
+                const float4 u = *reinterpret_cast<const float4*>(ubuf + st * 256 + b);
+                y.x = __fadd_rn(y.x, u.x); y.y = __fadd_rn(y.y, u.y); y.z = __fadd_rn(y.z, u.z); y.w = __fadd_rn(y.w, u.w);
             }
         }
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        amax = fmaxf(amax, fmaxf(fmaxf(fabsf(v[j].x), fabsf(v[j].y)), fmaxf(fabsf(v[j].z), fabsf(v[j].w))));
-        poison = __fmaf_rn(v[j].x, 0.0f, poison); poison = __fmaf_rn(v[j].y, 0.0f, poison);
-        poison = __fmaf_rn(v[j].z, 0.0f, poison); poison = __fmaf_rn(v[j].w, 0.0f, poison);
-        int fl = j * 32 + lane, owner = fl >> 3, jj = fl & 7;
-        mytile[owner * 8 + (jj ^ (owner & 7))] = v[j];
+        float* o = v + st * 8;
+        o[0] = swap ? y.x : x.x; o[1] = swap ? y.y : x.y; o[2] = swap ? y.z : x.z; o[3] = swap ? y.w : x.w;
+        o[4] = swap ? x.x : y.x; o[5] = swap ? x.y : y.y; o[6] = swap ? x.z : y.z; o[7] = swap ? x.w : y.w;
     }
 }
 
-// The same from the chunk that the bulk copies left in shared memory (`wbuf`, `ubuf`: 256 float4 each, in
-// memory order); V = W + U replaces W in place, swizzled inside each 128-byte row.
-__device__ __forceinline__ void load_chunk_staged(const PackJobDev& job, const UnitPos& up, int lane, float4* wbuf,
-                                                  const float4* ubuf, float& amax, float& poison) {
-    const int n4 = up.elems >> 2;  // float4 of the chunk that the copy brought
-    float4 v[8];
+// Whether the rows of a job can be moved in 32-byte accesses.
+__device__ __forceinline__ bool wide_rows(const PackJobDev& job, const float* Z, const float* U_next) {
+    return (((uintptr_t)job.W | (uintptr_t)job.U | (uintptr_t)Z | (uintptr_t)U_next) & 31u) == 0 && (job.in & 7) == 0;
+}
+
+// Four of eight: table from the 8-bit keep mask to its four positions (4-bit fields, ascending), which is also the group's
+// metadata.
+__device__ __forceinline__ void fill_positions(uint16_t* pos48) {
+    for (unsigned mk = threadIdx.x; mk < 256; mk += blockDim.x) {
+        unsigned r = 0, c = 0;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int fl = j * 32 + lane;
-        v[j] = fl < n4 ? wbuf[fl] : make_float4(0.f, 0.f, 0.f, 0.f);
-        if (job.U && fl < n4) {
-            const float4 u = ubuf[fl];
-            v[j].x = __fadd_rn(v[j].x, u.x); v[j].y = __fadd_rn(v[j].y, u.y);
-            v[j].z = __fadd_rn(v[j].z, u.z); v[j].w = __fadd_rn(v[j].w, u.w);
-        }
-    }
-    __syncwarp();  // every lane has read its part before the rows are rewritten in place
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        amax = fmaxf(amax, fmaxf(fmaxf(fabsf(v[j].x), fabsf(v[j].y)), fmaxf(fabsf(v[j].z), fabsf(v[j].w))));
-        poison = __fmaf_rn(v[j].x, 0.0f, poison); poison = __fmaf_rn(v[j].y, 0.0f, poison);
-        poison = __fmaf_rn(v[j].z, 0.0f, poison); poison = __fmaf_rn(v[j].w, 0.0f, poison);
-        int fl = j * 32 + lane, owner = fl >> 3, jj = fl & 7;
-        wbuf[owner * 8 + (jj ^ (owner & 7))] = v[j];
+        for (unsigned p8 = 0; p8 < 8; ++p8)
+            if ((mk >> p8) & 1u) { r |= p8 << (4 * (c & 3u)); ++c; }
+        pos48[mk] = (uint16_t)r;
     }
 }
 
-// Forms of the kernel.  kDirect: one block = one unit, 16-byte global loads.  kStaged2: persistent, two chunk
-// buffers per warp (16 KB), the next unit's copies are issued before the current unit is touched; for the forms that
-// keep using the tile to the end of the unit (4:8, dense outputs).
-// kAhead: persistent, 16-byte global loads as in kDirect, but every warp first asks for its NEXT unit's chunk to be
-// brought into L2 (a bulk prefetch: no registers, no shared memory), so that DRAM streams from the first cycle on and
-// the loads of all units but the first are L2 hits.
-enum { kDirect = 0, kStaged2 = 1, kAhead = 2 };
-__host__ __device__ constexpr int pack_blocks_per_sm(int pipe) { return pipe == kStaged2 ? 3 : 8; }
+// Forms of the kernel.  kDirect: one block = one unit, global loads.  kStaged2: persistent, two buffers of up to 1024 values
+// of W and U per warp (16 KB); every warp fetches its part of its NEXT unit with two bulk copies into the other buffer
+// while it works on the current one, so that loading and arithmetic overlap inside a warp and not only between
+// blocks that happen to be out of step.
+enum { kDirect = 0, kStaged2 = 1 };
+constexpr int kStagedBlocksPerSm = 3;
+// Resident blocks of four warps that the registers are cut for (kDirect).  Eight (64 registers) for the plain projection: with five
+// or six, more of a warp's loads are in flight, but 85 M weights in four formats take 125 / 116 us instead of 104, the
+// 24-layer sweep 436 / 441 instead of 403.  Dense outputs six (738 us; five and four the same).  The search four, and
+// six where a lane keeps at most eight values.
+template <int N, int M, bool DENSE_OUT, bool DIST>
+constexpr int kDirectBlocksPerSm = DIST ? (32 / M * N <= 8 ? 6 : 4) : DENSE_OUT ? 6 : 8;
 
 template <int N, int M, int BITS, int MAXT, bool DENSE_OUT = false, int PIPE = kDirect, bool DIST = false>
-__global__ void __launch_bounds__(MAXT, PIPE != kDirect ? pack_blocks_per_sm(PIPE) : (MAXT == 128 ? (DENSE_OUT || DIST ? 4 : 8) : 1))
+__global__ void __launch_bounds__(MAXT, PIPE != kDirect ? kStagedBlocksPerSm : (MAXT == 128 ? kDirectBlocksPerSm<N, M, DENSE_OUT, DIST> : 1))
 pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constant__ PackJobInline inl, uint32_t* status,
             float* __restrict__ Zout, float* __restrict__ Unext, const DenseOutDev* __restrict__ dense_jobs,
             int group_mode, int group_rows, unsigned nunits) {
-    static_assert(PIPE == kDirect || MAXT == 128, "the staged forms are built for blocks of four warps");
-    // staged: [warps][2 buffers][W, U][256] float4; else [warps][256] float4.  Then [2][warps] floats for the row
-    // maximum, 256 u16 (4:8 positions), and for the staged forms [warps][2] mbarriers and the abort flag.
+    static_assert(PIPE == kDirect || (MAXT == 128 && N == 2 && M == 4 && !DENSE_OUT && !DIST), "see staged_form");
+    // staged: [warps][2 buffers][W, U][1024] floats.  Then (DIST) [warps][32] doubles, [2][warps] floats for the row maximum, (4:8) the
+    // position table and [warps][8][32] floats, (staged) [warps][2] mbarriers and the abort flag.
     extern __shared__ float4 tile[];
     const int warps = blockDim.x >> 5;
-    float* red = reinterpret_cast<float*>(tile + warps * (PIPE == kStaged2 ? 1024 : 256));
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint8_t* at = reinterpret_cast<uint8_t*>(tile) + (PIPE == kStaged2 ? warps * 16384 : 0);
+    double* red_e = reinterpret_cast<double*>(at);
+    if (DIST) at += warps * 256;
+    float* red = reinterpret_cast<float*>(at);
+    at += warps * 8;
+    uint16_t* pos48 = nullptr;
+    float* scratch = nullptr;
     // a kernel launched as this one's programmatic dependent may begin its set-up on SMs this grid has left
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // four of eight: table from the 8-bit keep mask to its four positions (4-bit fields, ascending), which is
-    // also the group's metadata; the kept values are then fetched from the warp's tile by position
-    uint16_t* pos48 = reinterpret_cast<uint16_t*>(red + 2 * warps);
     if constexpr (N == 4 && M == 8) {
-        for (unsigned mk = threadIdx.x; mk < 256; mk += blockDim.x) {
-            unsigned r = 0, c = 0;
-#pragma unroll
-            for (unsigned p8 = 0; p8 < 8; ++p8)
-                if ((mk >> p8) & 1u) { r |= p8 << (4 * (c & 3u)); ++c; }
-            pos48[mk] = (uint16_t)r;
-        }
+        pos48 = reinterpret_cast<uint16_t*>(at);
+        at += 512;
+        scratch = reinterpret_cast<float*>(at) + w * 256;
+        at += warps * 1024;
+        fill_positions(pos48);
         __syncthreads();
     }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 
-    if constexpr (PIPE == kAhead) {
-        float4* mytile = tile + w * 256;
-        auto ask = [&](const PackJobDev& j, const UnitPos& up) {
-            if (up.elems == 0 || lane != 0) return;
-            const size_t first = (size_t)up.row * j.in + (size_t)up.chunk * 1024;
-            ptx::bulk_prefetch_l2(j.W + first, (uint32_t)up.elems * 4u);
-            if (j.U) ptx::bulk_prefetch_l2(j.U + first, (uint32_t)up.elems * 4u);
-        };
-        int index = 0;
-        unsigned unit = blockIdx.x;
-        PackJobDev job{};
-        if (unit < nunits) job = find_job(jobs, njobs, inl, unit, index);
-        for (int it = 0; unit < nunits; ++it, unit += gridDim.x) {
-            const UnitPos up = unit_pos(job, unit, w, warps);
-            const unsigned next = unit + gridDim.x;
-            PackJobDev njob = job;
-            int nindex = index;
-            if (next < nunits) {
-                if (next - job.unit_begin >= units_of(job, warps)) njob = find_job(jobs, njobs, inl, next, nindex);
-                ask(njob, unit_pos(njob, next, w, warps));
-            }
-            if constexpr (DENSE_OUT) {
-                if (jobs) { Zout = dense_jobs[index].Z; Unext = dense_jobs[index].U_next; }
-            }
-            float amax = 0.0f, poison = 0.0f;
-            load_chunk_global(job, up, lane, mytile, amax, poison);
-            pack_finish<N, M, BITS, DENSE_OUT>(job, up, lane, w, mytile, red + (it & 1) * warps, pos48, amax, poison,
-                                              status, Zout, Unext, group_mode, group_rows);
-            __syncwarp();  // the tile is rewritten by the next unit
-            job = njob; index = nindex;
-        }
-    } else if constexpr (PIPE == kDirect) {
-        double* red_e = DIST ? reinterpret_cast<double*>(pos48 + 256) : nullptr;  // 32 per warp
+    if constexpr (PIPE == kDirect) {
         int index = 0;
         const PackJobDev job = find_job(jobs, njobs, inl, blockIdx.x, index);
         if constexpr (DENSE_OUT) {
             if (jobs) { Zout = dense_jobs[index].Z; Unext = dense_jobs[index].U_next; }
         }
         const UnitPos up = unit_pos(job, blockIdx.x, w, warps);
-        float4* mytile = tile + w * 256;
-        float amax = 0.0f, poison = 0.0f;
-        load_chunk_global(job, up, lane, mytile, amax, poison);
-        pack_finish<N, M, BITS, DENSE_OUT, DIST>(job, up, lane, w, mytile, red, pos48, amax, poison, status, Zout, Unext,
-                                                group_mode, group_rows, red_e);
+        const bool wide = wide_rows(job, Zout, Unext);
+        float v[32];
+        load_global(job, up, lane, wide, v);
+        pack_finish<N, M, BITS, DENSE_OUT, DIST>(job, up, lane, w, v, red, pos48, scratch, status, Zout, Unext, wide, group_mode,
+                                                group_rows, red_e);
     } else {
-        uint64_t* bars = reinterpret_cast<uint64_t*>(pos48 + 256);       // [warps][2]
+        uint64_t* bars = reinterpret_cast<uint64_t*>(at);                 // [warps][2]
         volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 2 * warps);
-        float4* mybuf = tile + w * 1024;                                  // [buffer][W, U][256]
+        float* mybuf = reinterpret_cast<float*>(tile) + w * 4096;         // [buffer][W, U][1024]
         const uint32_t bar0 = ptx::smem_u32(bars + 2 * w);
         if (lane == 0) {
             ptx::mbar_init(bar0, 1);
@@ -845,10 +886,10 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
             __syncwarp();                   // the buffer's last reader is done
             if (lane == 0) {
                 const uint32_t bytes = (uint32_t)up.elems * 4u, bar = bar0 + 8u * buf;
-                const size_t first = (size_t)up.row * j.in + (size_t)up.chunk * 1024;
+                const size_t first = (size_t)up.row * j.in + up.first;
                 ptx::mbar_expect_tx(bar, j.U ? 2 * bytes : bytes);
-                ptx::bulk_load(ptx::smem_u32(mybuf + buf * 512), j.W + first, bytes, bar);
-                if (j.U) ptx::bulk_load(ptx::smem_u32(mybuf + buf * 512 + 256), j.U + first, bytes, bar);
+                ptx::bulk_load(ptx::smem_u32(mybuf + buf * 2048), j.W + first, bytes, bar);
+                if (j.U) ptx::bulk_load(ptx::smem_u32(mybuf + buf * 2048 + 1024), j.U + first, bytes, bar);
             }
         };
         int index = 0;
@@ -863,7 +904,7 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
         uint32_t phase = 0;  // bit b: parity of buffer b's next completion
         for (int it = 0; unit < nunits; ++it, unit += gridDim.x) {
             const int buf = it & 1;
-            // the next unit's chunk goes into the other buffer while this one is worked on
+            // the next unit's part goes into the other buffer while this one is worked on
             const unsigned next = unit + gridDim.x;
             PackJobDev njob = job;
             int nindex = index;
@@ -884,11 +925,10 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
                 }
                 phase ^= 1u << buf;
             }
-            float4* mytile = mybuf + buf * 512;
-            float amax = 0.0f, poison = 0.0f;
-            load_chunk_staged(job, up, lane, mytile, mytile + 256, amax, poison);
-            pack_finish<N, M, BITS, DENSE_OUT>(job, up, lane, w, mytile, red + (it & 1) * warps, pos48, amax, poison,
-                                              status, Zout, Unext, group_mode, group_rows);
+            float v[32];
+            load_staged(job, up, lane, mybuf + buf * 2048, mybuf + buf * 2048 + 1024, v);
+            pack_finish<N, M, BITS, DENSE_OUT>(job, up, lane, w, v, red + (it & 1) * warps, pos48, scratch, status, Zout, Unext,
+                                              wide_rows(job, Zout, Unext), group_mode, group_rows);
             job = njob; index = nindex; up = nup;
         }
         // after an expired wait a copy may still be on its way into this block's shared memory
@@ -972,32 +1012,22 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1) dist_scale_kernel(c
                                                                               const __grid_constant__ PackJobInline inl,
                                                                               uint32_t* status, int ncand,
                                                                               int32_t* __restrict__ cand_out) {
-    extern __shared__ float4 tile[];  // [warps][256] float4, [warps][32] doubles, [warps] floats
+    extern __shared__ float4 tile[];  // [warps][32] doubles, [warps] floats
     const int warps = blockDim.x >> 5;
-    double* red_e = reinterpret_cast<double*>(tile + warps * 256);
+    double* red_e = reinterpret_cast<double*>(tile);
     float* red = reinterpret_cast<float*>(red_e + warps * 32);
     int index = 0;
     const PackJobDev job = find_job(jobs, njobs, inl, blockIdx.x, index);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const UnitPos up = unit_pos(job, blockIdx.x, w, warps);
     const int wpr = 1 << job.wpr_log2;
-    float4* mytile = tile + w * 256;
-    float amax = 0.0f, poison = 0.0f;
-    load_chunk_global(job, up, lane, mytile, amax, poison);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    const bool bad = __any_sync(0xffffffffu, poison != poison) || !(amax <= 3.402823466e+38f);
-    if (bad && lane == 0 && status) atomicOr(status, NM_STATUS_NONFINITE);
-    if (wpr > 1) {
-        if (lane == 0) red[w] = amax;
-        __syncthreads();
-        for (int c = 0; c < wpr; ++c) amax = fmaxf(amax, red[up.row_in_block * wpr + c]);
-    } else {
-        __syncwarp();
-    }
+    float v[32];
+    load_global(job, up, lane, wide_rows(job, nullptr, nullptr), v);
+    bool bad;
+    const float amax = row_max(v, lane, w, wpr, up.row_in_block, red, status, bad);
     constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
     const float smax = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
-    const int bj = dist_search<N, M, BITS>(mytile, lane, w, wpr, up.row_in_block, up.row_ok, smax, bad, ncand, red_e);
+    const int bj = dist_search<N, M, BITS>(v, up.steps, lane, w, wpr, up.row_in_block, up.row_ok, smax, bad, ncand, red_e);
     if (up.row_ok && up.chunk == 0 && lane == 0) {
         job.scales[up.row] = __fmul_rn(smax, (float)(64 - bj) * 0.015625f);
         if (cand_out) cand_out[up.row] = bj;
@@ -1008,38 +1038,34 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1) dist_scale_kernel(c
 // host side
 // ---------------------------------------------------------------------------------------------
 using PackFnPtr = void (*)(const PackJobDev*, int, const PackJobInline, uint32_t*, float*, float*, const DenseOutDev*, int, int, unsigned);
-struct PackFn { PackFnPtr fn; int form; bool dist = false; };  // kernel, its form (kDirect, kStaged2, kAhead), with the scale search
+struct PackFn { PackFnPtr fn; int form; bool dist = false; };  // kernel, its form (kDirect, kStaged2), with the scale search
 
-// nm_debug_set_option("pack_form"): 0 = automatic, 1 = kDirect, 2 = kStaged2, 3 = kAhead for blocks of four warps.
+// nm_debug_set_option("pack_form"): 0 = automatic, 2 = kStaged2 wherever it exists (2:4, blocks of four warps, no dense
+// outputs), anything else = kDirect.
 int g_pack_form = 0;
 
-
-template <int N, int M, bool DENSE_OUT, int FORM>
-static PackFn pick_form(int bits) {
-    return bits == 8 ? PackFn{(PackFnPtr)pack_kernel<N, M, 8, 128, DENSE_OUT, FORM>, FORM}
-                     : PackFn{(PackFnPtr)pack_kernel<N, M, 4, 128, DENSE_OUT, FORM>, FORM};
+// Whether a launch of `blocks` blocks of four warps takes the staged form.  2:4 with two operands, two to six rounds of the
+// blocks that kDirect keeps resident, in rows that fill the warps' buffers: blocks that start together otherwise alternate
+// between loading and arithmetic (staged / direct: 12.6 M weights in rows of 1024 and 4096 23.2 / 25.4 us, 25 M 39.6 / 44.0; 38 M
+// 61.5 / 62.0).  Everywhere else kDirect is as fast or faster (rows of 768 and 3072, 14 M weights 27.2 / 27.2; of 384 and
+// 1536, 11 M 37.3 / 27.4; one operand, 25 M weights 37.3 / 25.2; dense outputs on the 24-layer sweep 876 / 741; other
+// patterns 3-45 % faster).  `dual`: every matrix of the launch has both operands and rows of a multiple of 1024 weights.
+static bool staged_form(bool dual, unsigned blocks) {
+    const unsigned resident = (unsigned)sm_count() * 8u;
+    return dual && blocks > 2u * resident && blocks <= 6u * resident;
 }
+static bool fills_buffers(const nm_pack_job_t& j) { return j.U != nullptr && j.in % 1024 == 0; }
 
 template <int N, int M, bool DENSE_OUT>
-static PackFn pick_bits(int bits, int warps, unsigned blocks) {
+static PackFn pick_bits(int bits, int warps, unsigned blocks, bool dual) {
     if (warps <= kPackMinWarps) {
-        // Blocks of four warps.  Measured choices (GB/s on the 24-layer sweep, one unit per block / staged / ahead:
-        // 1:4 6231 / 5916 / 6011, 2:4 5520 / 5276 / 5746, 2:8 5643 / 5175 / 5282, 4:8 5090 / 4435 / 5046; one 2:4 layer
-        // alone 26.8 / 24.7 / 25.1 us; 72 matrices in four formats, four launches: 130 / 197 / 156 us; dense outputs on
-        // the sweep 0.83 / 0.95 / 0.60 of the copy rate):
-        //  - dense outputs: staged;
-        //  - 2:4: staged for launches of a few rounds per resident block (blocks that start together otherwise alternate
-        //    between loading and arithmetic), ahead for very long ones, one unit per block between;
-        //  - every other pattern: one unit per block.
-        const unsigned staged_blocks = (unsigned)(sm_count() * pack_blocks_per_sm(kStaged2));
-        const unsigned ahead_blocks = (unsigned)(sm_count() * pack_blocks_per_sm(kAhead));
-        int form = kDirect;
-        if (DENSE_OUT) form = kStaged2;
-        else if (N == 2 && M == 4) form = blocks <= 8u * staged_blocks ? kStaged2 : (blocks >= 32u * ahead_blocks ? kAhead : kDirect);
-        if (g_pack_form >= 1 && g_pack_form <= 3) form = g_pack_form == 1 ? kDirect : g_pack_form == 2 ? kStaged2 : kAhead;
-        if (form == kDirect) return pick_form<N, M, DENSE_OUT, kDirect>(bits);
-        if (form == kStaged2) return pick_form<N, M, DENSE_OUT, kStaged2>(bits);
-        return pick_form<N, M, DENSE_OUT, kAhead>(bits);
+        if constexpr (N == 2 && M == 4 && !DENSE_OUT) {
+            if (g_pack_form == 2 || (g_pack_form == 0 && staged_form(dual, blocks)))
+                return bits == 8 ? PackFn{(PackFnPtr)pack_kernel<2, 4, 8, 128, false, kStaged2>, kStaged2}
+                                 : PackFn{(PackFnPtr)pack_kernel<2, 4, 4, 128, false, kStaged2>, kStaged2};
+        }
+        return bits == 8 ? PackFn{(PackFnPtr)pack_kernel<N, M, 8, 128, DENSE_OUT>, kDirect}
+                         : PackFn{(PackFnPtr)pack_kernel<N, M, 4, 128, DENSE_OUT>, kDirect};
     }
     if constexpr (DENSE_OUT) {  // the dense outputs need ~128 registers: blocks of at most 512 threads get them
         if (warps <= 16)
@@ -1049,12 +1075,12 @@ static PackFn pick_bits(int bits, int warps, unsigned blocks) {
 }
 
 template <bool DENSE_OUT = false>
-static PackFn pick_kernel(int n, int m, int bits, int warps, unsigned blocks) {
-    if (n == m) return pick_bits<4, 4, DENSE_OUT>(bits, warps, blocks);
-    if (m == 4) return n == 1 ? pick_bits<1, 4, DENSE_OUT>(bits, warps, blocks) : pick_bits<2, 4, DENSE_OUT>(bits, warps, blocks);
-    if (n == 1) return pick_bits<1, 8, DENSE_OUT>(bits, warps, blocks);
-    if (n == 2) return pick_bits<2, 8, DENSE_OUT>(bits, warps, blocks);
-    return pick_bits<4, 8, DENSE_OUT>(bits, warps, blocks);
+static PackFn pick_kernel(int n, int m, int bits, int warps, unsigned blocks, bool dual) {
+    if (n == m) return pick_bits<4, 4, DENSE_OUT>(bits, warps, blocks, dual);
+    if (m == 4) return n == 1 ? pick_bits<1, 4, DENSE_OUT>(bits, warps, blocks, dual) : pick_bits<2, 4, DENSE_OUT>(bits, warps, blocks, dual);
+    if (n == 1) return pick_bits<1, 8, DENSE_OUT>(bits, warps, blocks, dual);
+    if (n == 2) return pick_bits<2, 8, DENSE_OUT>(bits, warps, blocks, dual);
+    return pick_bits<4, 8, DENSE_OUT>(bits, warps, blocks, dual);
 }
 
 static int validate_job(const nm_pack_job_t& j) {
@@ -1090,11 +1116,9 @@ static PackJobDev to_dev(const nm_pack_job_t& j) {
 static int launch_table(PackFn k, const PackJobDev* jobs_dev, int njobs, const PackJobInline& inl, unsigned blocks,
                         int warps, uint32_t* status, cudaStream_t stream, float* Z, float* U_next,
                         const DenseOutDev* dense_jobs, int group_mode, int group_rows) {
-    // chunk tile(s), two sets of row-maximum slots, the 4:8 position table; staged form: also two barriers per warp
-    // and the abort flag, and a grid that stays resident
-    const bool staged = k.form == kStaged2, persistent = k.form != kDirect;
-    size_t smem = (size_t)warps * ((staged ? 1024 : 256) * sizeof(float4) + 2 * sizeof(float)) + 512 +
-                  (staged ? (size_t)warps * 16 + 16 : 0) + (k.dist ? (size_t)warps * 32 * sizeof(double) : 0);
+    // buffers and barriers of the staged form, distances of the search, row-maximum slots, the 4:8 tables (see the kernel)
+    const bool staged = k.form == kStaged2;
+    const size_t smem = (size_t)warps * ((staged ? 16384 + 16 : 0) + (k.dist ? 32 * sizeof(double) : 0) + 2 * sizeof(float) + 1024) + 512 + 16;
     const PackFnPtr fn = k.fn;
     if (smem > 48 * 1024) {  // the attribute is set once per kernel and device
         struct Done { const void* fn; int dev; };
@@ -1110,7 +1134,7 @@ static int launch_table(PackFn k, const PackJobDev* jobs_dev, int njobs, const P
             done.push_back(Done{(const void*)fn, dev});
         }
     }
-    const unsigned grid = persistent ? std::min(blocks, (unsigned)(sm_count() * pack_blocks_per_sm(k.form))) : blocks;
+    const unsigned grid = staged ? std::min(blocks, (unsigned)(sm_count() * kStagedBlocksPerSm)) : blocks;
     fn<<<grid, warps * 32, smem, stream>>>(jobs_dev, njobs, inl, status, Z, U_next, dense_jobs, group_mode, group_rows, blocks);
     NM_CUDA_TRY(cudaGetLastError());
     return NM_OK;
@@ -1123,6 +1147,20 @@ static int launch(PackFn fn, const PackJobDev* jobs_dev, int njobs, const PackJo
     PackJobInline inl{};
     inl.j[0] = single;
     return launch_table(fn, jobs_dev, njobs, inl, blocks, warps, status, stream, Z, U_next, dense_jobs, group_mode, group_rows);
+}
+
+// One matrix, group-wise scales: maxima, scales, projection.
+template <bool DENSE_OUT>
+static int launch_grouped_single(const nm_pack_job_t& j, int group_rows, uint32_t* status, cudaStream_t stream,
+                                 float* Z = nullptr, float* U_next = nullptr) {
+    PackJobDev d = to_dev(j);
+    int rc = launch_group_scales(j.W, j.U, j.out, j.in, j.bits, group_rows, j.scales, stream);
+    if (rc != NM_OK) return rc;
+    const int warps = std::max(kPackMinWarps, 1 << d.wpr_log2);
+    const int rows_per_block = warps >> d.wpr_log2;
+    const unsigned blocks = (unsigned)((j.out + rows_per_block - 1) / rows_per_block);
+    return launch(pick_kernel<DENSE_OUT>(j.n, j.m, j.bits, warps, blocks, fills_buffers(j)), nullptr, 0, d, blocks, warps, status, stream,
+                  Z, U_next, nullptr, kGroupScalesGiven, group_rows);
 }
 
 using DistFn = void (*)(const PackJobDev*, int, const PackJobInline, uint32_t*, int, int32_t*);
@@ -1146,9 +1184,7 @@ static DistFn pick_dist(int n, int m, int bits, int warps) {
 
 static int launch_dist(DistFn fn, const PackJobDev* jobs_dev, int njobs, const PackJobDev& single, unsigned blocks,
                        int warps, uint32_t* status, cudaStream_t stream, int ncand, int32_t* cand) {
-    size_t smem = (size_t)warps * (256 * sizeof(float4) + 32 * sizeof(double) + sizeof(float));
-    if (smem > 48 * 1024)
-        NM_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const size_t smem = (size_t)warps * (32 * sizeof(double) + sizeof(float));
     PackJobInline inl{};
     inl.j[0] = single;
     fn<<<blocks, warps * 32, smem, stream>>>(jobs_dev, njobs, inl, status, ncand, cand);
@@ -1195,7 +1231,7 @@ static int launch_dist_project_single(const nm_pack_job_t& j, int ncand, uint32_
                       kGroupNone, ncand);
     int rc = launch_dist_single(j, ncand, nullptr, status, stream);
     if (rc != NM_OK) return rc;
-    return launch(pick_kernel<DENSE_OUT>(j.n, j.m, j.bits, warps, blocks), nullptr, 0, d, blocks, warps, status, stream, Z, U_next,
+    return launch(pick_kernel<DENSE_OUT>(j.n, j.m, j.bits, warps, blocks, fills_buffers(j)), nullptr, 0, d, blocks, warps, status, stream, Z, U_next,
                   nullptr, kGroupScalesGiven, 0);
 }
 
@@ -1206,18 +1242,19 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
                           uint32_t* status, cudaStream_t s, bool grouped = false, int group_rows = 0,
                           int dist_ncand = 0) {
     // Group jobs that can share one launch: same (n == m ? dense : n, m), bits and block size.
-    struct Key { int n, m, bits, warps; };
+    struct Key { int n, m, bits, warps, dual; };
     std::vector<Key> keys;
     std::vector<std::vector<int>> groups;
     for (int i = 0; i < njobs; ++i) {
         const nm_pack_job_t& j = jobs[i];
         if (j.out == 0 || j.in == 0) continue;
-        Key k{j.n == j.m ? 4 : j.n, j.n == j.m ? 4 : j.m, j.bits,
-              std::max(nm::kPackMinWarps, 1 << nm::wpr_log2_of(j.in))};
+        const int wl = nm::wpr_log2_of(j.in);
+        Key k{j.n == j.m ? 4 : j.n, j.n == j.m ? 4 : j.m, j.bits, std::max(nm::kPackMinWarps, 1 << wl), fills_buffers(j) ? 1 : 0};
         size_t g = 0;
         for (; g < keys.size(); ++g)
             if (keys[g].n == k.n && keys[g].m == k.m && keys[g].bits == k.bits && keys[g].warps == k.warps) break;
         if (g == keys.size()) { keys.push_back(k); groups.emplace_back(); }
+        keys[g].dual &= k.dual;
         groups[g].push_back(i);
     }
     std::vector<nm::PackJobDev> table;
@@ -1230,7 +1267,7 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
         group_first[g] = table.size();
         for (int i : groups[g]) {
             nm::PackJobDev d = nm::to_dev(jobs[i]);
-            int rows_per_block = keys[g].warps >> d.wpr_log2;
+            const int rows_per_block = keys[g].warps >> d.wpr_log2;
             d.unit_begin = blocks;
             unsigned long long nb = ((unsigned long long)d.out + rows_per_block - 1) / rows_per_block;
             if (blocks + nb > 0x7fffffffull) return NM_ERR_UNSUPPORTED;
@@ -1248,7 +1285,7 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
             for (size_t g = 0; g < keys.size(); ++g) {
                 PackJobInline inl{};
                 for (size_t i = 0; i < groups[g].size(); ++i) inl.j[i] = table[group_first[g] + i];
-                int rc = nm::launch_table(nm::pick_kernel<DENSE_OUT>(keys[g].n, keys[g].m, keys[g].bits, keys[g].warps, group_blocks[g]), nullptr,
+                int rc = nm::launch_table(nm::pick_kernel<DENSE_OUT>(keys[g].n, keys[g].m, keys[g].bits, keys[g].warps, group_blocks[g], keys[g].dual), nullptr,
                                           (int)groups[g].size(), inl, group_blocks[g], keys[g].warps, status, s, nullptr,
                                           nullptr, nullptr, kGroupNone, 0);
                 if (rc != NM_OK) return rc;
@@ -1276,7 +1313,7 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
             const nm::PackJobDev* dev = reinterpret_cast<const nm::PackJobDev*>(ws) + group_first[g];
             group_prepare_kernel<<<(unsigned)groups[g].size(), 256, 0, s>>>(dev, group_rows, keys[g].bits, 0);
             NM_CUDA_TRY(cudaGetLastError());
-            int rc = nm::launch(nm::pick_kernel<DENSE_OUT>(keys[g].n, keys[g].m, keys[g].bits, keys[g].warps, group_blocks[g]), dev,
+            int rc = nm::launch(nm::pick_kernel<DENSE_OUT>(keys[g].n, keys[g].m, keys[g].bits, keys[g].warps, group_blocks[g], keys[g].dual), dev,
                                 (int)groups[g].size(), nm::PackJobDev{}, group_blocks[g], keys[g].warps, status, s,
                                 nullptr, nullptr, DENSE_OUT ? dense_dev + group_first[g] : nullptr, kGroupMaxPass, group_rows);
             if (rc != NM_OK) return rc;
@@ -1299,7 +1336,7 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
                                      status, s, dist_ncand, nullptr);
                 if (rc != NM_OK) return rc;
             }
-            rc = nm::launch(nm::pick_kernel<DENSE_OUT>(k.n, k.m, k.bits, k.warps, group_blocks[g]), dev, count, nm::PackJobDev{},
+            rc = nm::launch(nm::pick_kernel<DENSE_OUT>(k.n, k.m, k.bits, k.warps, group_blocks[g], k.dual), dev, count, nm::PackJobDev{},
                             group_blocks[g], k.warps, status, s, nullptr, nullptr, dense_g,
                             (grouped || dist_ncand > 0) ? kGroupScalesGiven : kGroupNone, group_rows);
         }
@@ -1335,7 +1372,7 @@ int nm_project_pack(const float* W, const float* U, int out, int in, int n, int 
     int warps = std::max(nm::kPackMinWarps, 1 << d.wpr_log2);
     int rows_per_block = warps >> d.wpr_log2;
     unsigned blocks = (unsigned)((out + rows_per_block - 1) / rows_per_block);
-    return nm::launch(nm::pick_kernel(n, m, bits, warps, blocks), nullptr, 0, d, blocks, warps, status, (cudaStream_t)stream);
+    return nm::launch(nm::pick_kernel(n, m, bits, warps, blocks, nm::fills_buffers(j)), nullptr, 0, d, blocks, warps, status, (cudaStream_t)stream);
 }
 
 int nm_admm_project(const float* W, const float* U, int out, int in, int n, int m, int bits, float* Z,
@@ -1348,7 +1385,7 @@ int nm_admm_project(const float* W, const float* U, int out, int in, int n, int 
     int warps = std::max(nm::kPackMinWarps, 1 << d.wpr_log2);
     int rows_per_block = warps >> d.wpr_log2;
     unsigned blocks = (unsigned)((out + rows_per_block - 1) / rows_per_block);
-    return nm::launch(nm::pick_kernel<true>(n, m, bits, warps, blocks), nullptr, 0, d, blocks, warps, status,
+    return nm::launch(nm::pick_kernel<true>(n, m, bits, warps, blocks, nm::fills_buffers(j)), nullptr, 0, d, blocks, warps, status,
                       (cudaStream_t)stream, Z, U_next);
 }
 
@@ -1359,14 +1396,7 @@ int nm_project_pack_grouped(const float* W, const float* U, int out, int in, int
     int rc = nm::validate_job(j);
     if (rc != NM_OK) return rc;
     if (out == 0 || in == 0) return NM_OK;
-    rc = nm::launch_group_scales(W, U, out, in, bits, group_rows, scales, (cudaStream_t)stream);
-    if (rc != NM_OK) return rc;
-    nm::PackJobDev d = nm::to_dev(j);
-    int warps = std::max(nm::kPackMinWarps, 1 << d.wpr_log2);
-    int rows_per_block = warps >> d.wpr_log2;
-    unsigned blocks = (unsigned)((out + rows_per_block - 1) / rows_per_block);
-    return nm::launch(nm::pick_kernel(n, m, bits, warps, blocks), nullptr, 0, d, blocks, warps, status, (cudaStream_t)stream,
-                      nullptr, nullptr, nullptr, nm::kGroupScalesGiven, group_rows);
+    return nm::launch_grouped_single<false>(j, group_rows, status, (cudaStream_t)stream);
 }
 
 int nm_admm_project_grouped(const float* W, const float* U, int out, int in, int n, int m, int bits,
@@ -1376,15 +1406,8 @@ int nm_admm_project_grouped(const float* W, const float* U, int out, int in, int
     if (rc != NM_OK) return rc;
     if (!scales) return NM_ERR_NULL;  // also the scratch of the group maxima
     if (out == 0 || in == 0) return NM_OK;
-    rc = nm::launch_group_scales(W, U, out, in, bits, group_rows, scales, (cudaStream_t)stream);
-    if (rc != NM_OK) return rc;
     nm_pack_job_t j{W, U, out, in, n, m, bits, values, meta, scales};
-    nm::PackJobDev d = nm::to_dev(j);
-    int warps = std::max(nm::kPackMinWarps, 1 << d.wpr_log2);
-    int rows_per_block = warps >> d.wpr_log2;
-    unsigned blocks = (unsigned)((out + rows_per_block - 1) / rows_per_block);
-    return nm::launch(nm::pick_kernel<true>(n, m, bits, warps, blocks), nullptr, 0, d, blocks, warps, status,
-                      (cudaStream_t)stream, Z, U_next, nullptr, nm::kGroupScalesGiven, group_rows);
+    return nm::launch_grouped_single<true>(j, group_rows, status, (cudaStream_t)stream, Z, U_next);
 }
 
 int nm_dist_scales(const float* W, const float* U, int out, int in, int n, int m, int bits, int ncand,
