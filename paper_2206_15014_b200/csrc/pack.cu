@@ -940,6 +940,67 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
 }
 
 // ---------------------------------------------------------------------------------------------
+// Group-wise scales in one pass: a cluster of blocks holds a whole group of rows in registers, the blocks exchange their
+// maxima through distributed shared memory, and every warp goes on with its row at the group's scale.  W and U are read
+// once; folding the maxima of all groups first and packing in a second launch read them twice.
+// A unit is one group (`group_rows` rows, those past the matrix idle); it fills gridDim / units blocks, the cluster.
+// ---------------------------------------------------------------------------------------------
+template <int N, int M, int BITS, bool DENSE_OUT>
+__global__ void __launch_bounds__(512, DENSE_OUT ? 1 : 2)
+pack_group_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constant__ PackJobInline inl, uint32_t* status,
+                  float* __restrict__ Zout, float* __restrict__ Unext, const DenseOutDev* __restrict__ dense_jobs,
+                  int group_rows, unsigned cluster) {
+    // [warps] maxima, [8] maxima of the cluster's blocks, (4:8) position table and [warps][8][32] floats
+    extern __shared__ float4 tile[];
+    const int warps = blockDim.x >> 5, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    float* red = reinterpret_cast<float*>(tile);
+    uint32_t* peers = reinterpret_cast<uint32_t*>(red + 16);
+    uint16_t* pos48 = reinterpret_cast<uint16_t*>(peers + 8);
+    float* scratch = reinterpret_cast<float*>(pos48 + 256) + w * 256;
+    ptx::cluster_arrive();  // the other blocks' shared memory may be written once all of them run
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if constexpr (N == 4 && M == 8) fill_positions(pos48);  // ordered by the barrier below
+    const unsigned unit = blockIdx.x / cluster, rank = blockIdx.x % cluster;
+    int index = 0;
+    const PackJobDev job = find_job(jobs, njobs, inl, unit, index);
+    if constexpr (DENSE_OUT) {
+        if (jobs) { Zout = dense_jobs[index].Z; Unext = dense_jobs[index].U_next; }
+    }
+    const int wpr = 1 << job.wpr_log2, gw = (int)rank * warps + w;  // warp of the group
+    UnitPos up;
+    up.chunk = gw & (wpr - 1);
+    up.row_in_block = w >> job.wpr_log2;
+    up.row = (long long)(unit - job.unit_begin) * group_rows + (gw >> job.wpr_log2);
+    up.row_ok = up.row < job.out;
+    up.steps = (((job.in + 255) >> 8) + wpr - 1) >> job.wpr_log2;
+    up.first = up.chunk * up.steps * 256;
+    up.elems = up.row_ok ? max(0, min(up.steps * 256, job.in - up.first)) : 0;
+    const bool wide = wide_rows(job, Zout, Unext);
+    float v[32];
+    load_global(job, up, lane, wide, v);
+    bool bad;
+    float amax = row_max(v, lane, w, 1, 0, red, status, bad);  // of this warp's part
+    if (lane == 0) red[w] = amax;
+    __syncthreads();
+    ptx::cluster_wait();
+    if (w == 0) {
+        amax = lane < warps ? red[lane] : 0.0f;
+        const uint32_t block_max = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));
+        if (lane < (int)cluster) ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(peers + rank), (uint32_t)lane), block_max);
+    }
+    __syncwarp();
+    ptx::cluster_arrive();
+    ptx::cluster_wait();
+    amax = 0.0f;
+    for (unsigned c = 0; c < cluster; ++c) amax = fmaxf(amax, __uint_as_float(peers[c]));
+    if (!up.row_ok) return;
+    constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
+    const float s = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
+    if (up.chunk == 0 && lane == 0) job.scales[up.row] = s;
+    pack_row<N, M, BITS, DENSE_OUT, false>(job, up, lane, v, s, bad, pos48, scratch, Zout, Unext, wide);
+}
+
+// ---------------------------------------------------------------------------------------------
 // Group-wise scales: rows r with the same r / group_rows share one ADMM-Max scale.  A first pass folds
 // max |W + U| of every row into the first entry of its group in `scales` (non-negative floats order like
 // their bit patterns, so an unsigned atomicMax does it); a second turns each group's maximum into the
@@ -1160,14 +1221,70 @@ static int launch(PackFn fn, const PackJobDev* jobs_dev, int njobs, const PackJo
     return launch_table(fn, jobs_dev, njobs, inl, blocks, warps, status, stream, Z, U_next, dense_jobs, group_mode, group_rows, chained);
 }
 
-// One matrix, group-wise scales: maxima, scales, projection.
+// Cluster of pack_group_kernel for groups of `group_rows` rows of 1 << wpr_log2 warps: blocks of four to sixteen warps, at most
+// eight (the portable cluster size), rows whole in a block; blocks of at most eight warps where that is possible, so
+// that several clusters share an SM.  False: no such cluster (a group of fewer than four warps or more than 128, or an awkward
+// factor), the two-pass route.
+static bool group_cluster(int group_rows, int wpr_log2, int* warps, int* cluster) {
+    const long long gw = (long long)group_rows << wpr_log2;
+    if (group_rows <= 0 || wpr_log2 > 2 || gw < 4 || gw > 128) return false;
+    for (int limit = 8; limit <= 16; limit += 8)
+        for (int c = 1; c <= 8; ++c) {
+            const int bw = (int)gw / c;
+            if (gw % c || bw > limit || bw < 4 || bw % (1 << wpr_log2)) continue;
+            *warps = bw; *cluster = c;
+            return true;
+        }
+    return false;
+}
+
+using GroupFn = void (*)(const PackJobDev*, int, const PackJobInline, uint32_t*, float*, float*, const DenseOutDev*, int, unsigned);
+
+template <bool DENSE_OUT>
+static GroupFn pick_group(int n, int m, int bits) {
+    const bool b8 = bits == 8;
+    if (n == m) return b8 ? pack_group_kernel<4, 4, 8, DENSE_OUT> : pack_group_kernel<4, 4, 4, DENSE_OUT>;
+    if (m == 4 && n == 1) return b8 ? pack_group_kernel<1, 4, 8, DENSE_OUT> : pack_group_kernel<1, 4, 4, DENSE_OUT>;
+    if (m == 4) return b8 ? pack_group_kernel<2, 4, 8, DENSE_OUT> : pack_group_kernel<2, 4, 4, DENSE_OUT>;
+    if (n == 1) return b8 ? pack_group_kernel<1, 8, 8, DENSE_OUT> : pack_group_kernel<1, 8, 4, DENSE_OUT>;
+    if (n == 2) return b8 ? pack_group_kernel<2, 8, 8, DENSE_OUT> : pack_group_kernel<2, 8, 4, DENSE_OUT>;
+    return b8 ? pack_group_kernel<4, 8, 8, DENSE_OUT> : pack_group_kernel<4, 8, 4, DENSE_OUT>;
+}
+
+// `units` groups; the jobs of a launch have the same n, m, bits and warps per row.
+template <bool DENSE_OUT>
+static int launch_group(int n, int m, int bits, int warps, int cluster, const PackJobDev* jobs_dev, int njobs, const PackJobDev& single,
+                        unsigned units, uint32_t* status, cudaStream_t stream, float* Z, float* U_next,
+                        const DenseOutDev* dense_jobs, int group_rows) {
+    PackJobInline inl{};
+    inl.j[0] = single;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(units * (unsigned)cluster, 1, 1);
+    cfg.blockDim = dim3(warps * 32, 1, 1);
+    cfg.dynamicSmemBytes = 96 + (n == 4 && m == 8 ? 512 + (size_t)warps * 1024 : 0);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    NM_CUDA_TRY(cudaLaunchKernelEx(&cfg, pick_group<DENSE_OUT>(n, m, bits), jobs_dev, njobs, inl, status, Z, U_next, dense_jobs,
+                                   group_rows, (unsigned)cluster));
+    return NM_OK;
+}
+
+// One matrix, group-wise scales: one pass where a cluster holds a group, otherwise maxima, scales, projection.
 template <bool DENSE_OUT>
 static int launch_grouped_single(const nm_pack_job_t& j, int group_rows, uint32_t* status, cudaStream_t stream,
                                  float* Z = nullptr, float* U_next = nullptr) {
     PackJobDev d = to_dev(j);
+    int warps = 0, cluster = 0;
+    if (group_cluster(group_rows, d.wpr_log2, &warps, &cluster)) {
+        const unsigned units = (unsigned)(((long long)j.out + group_rows - 1) / group_rows);
+        return launch_group<DENSE_OUT>(j.n, j.m, j.bits, warps, cluster, nullptr, 0, d, units, status, stream, Z, U_next, nullptr, group_rows);
+    }
     int rc = launch_group_scales(j.W, j.U, j.out, j.in, j.bits, group_rows, j.scales, stream);
     if (rc != NM_OK) return rc;
-    const int warps = std::max(kPackMinWarps, 1 << d.wpr_log2);
+    warps = std::max(kPackMinWarps, 1 << d.wpr_log2);
     const int rows_per_block = warps >> d.wpr_log2;
     const unsigned blocks = (unsigned)((j.out + rows_per_block - 1) / rows_per_block);
     return launch(pick_kernel<DENSE_OUT>(j.n, j.m, j.bits, warps, blocks, fills_buffers(j)), nullptr, 0, d, blocks, warps, status, stream,
@@ -1252,18 +1369,22 @@ template <bool DENSE_OUT>
 static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, int njobs, void* ws,
                           uint32_t* status, cudaStream_t s, bool grouped = false, int group_rows = 0,
                           int dist_ncand = 0) {
-    // Group jobs that can share one launch: same (n == m ? dense : n, m), bits and block size.
-    struct Key { int n, m, bits, warps, dual; };
+    // Group jobs that can share one launch: same (n == m ? dense : n, m), bits and block size.  Where a cluster of blocks holds a
+    // group of rows (group_cluster) the block size follows from the warps per row.
+    struct Key { int n, m, bits, warps, cluster, dual; };
     std::vector<Key> keys;
     std::vector<std::vector<int>> groups;
     for (int i = 0; i < njobs; ++i) {
         const nm_pack_job_t& j = jobs[i];
         if (j.out == 0 || j.in == 0) continue;
         const int wl = nm::wpr_log2_of(j.in);
-        Key k{j.n == j.m ? 4 : j.n, j.n == j.m ? 4 : j.m, j.bits, std::max(nm::kPackMinWarps, 1 << wl), fills_buffers(j) ? 1 : 0};
+        Key k{j.n == j.m ? 4 : j.n, j.n == j.m ? 4 : j.m, j.bits, std::max(nm::kPackMinWarps, 1 << wl), 0, fills_buffers(j) ? 1 : 0};
+        int gw = 0, gc = 0;
+        if (grouped && group_cluster(group_rows, wl, &gw, &gc)) { k.warps = gw; k.cluster = gc; }
         size_t g = 0;
         for (; g < keys.size(); ++g)
-            if (keys[g].n == k.n && keys[g].m == k.m && keys[g].bits == k.bits && keys[g].warps == k.warps) break;
+            if (keys[g].n == k.n && keys[g].m == k.m && keys[g].bits == k.bits && keys[g].warps == k.warps && keys[g].cluster == k.cluster &&
+                (!k.cluster || nm::wpr_log2_of(jobs[groups[g][0]].in) == wl)) break;
         if (g == keys.size()) { keys.push_back(k); groups.emplace_back(); }
         keys[g].dual &= k.dual;
         groups[g].push_back(i);
@@ -1278,10 +1399,10 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
         group_first[g] = table.size();
         for (int i : groups[g]) {
             nm::PackJobDev d = nm::to_dev(jobs[i]);
-            const int rows_per_block = keys[g].warps >> d.wpr_log2;
+            const int rows_per_block = keys[g].cluster ? group_rows : keys[g].warps >> d.wpr_log2;
             d.unit_begin = blocks;
             unsigned long long nb = ((unsigned long long)d.out + rows_per_block - 1) / rows_per_block;
-            if (blocks + nb > 0x7fffffffull) return NM_ERR_UNSUPPORTED;
+            if ((blocks + nb) * (keys[g].cluster ? keys[g].cluster : 1) > 0x7fffffffull) return NM_ERR_UNSUPPORTED;
             blocks += (unsigned)nb;
             table.push_back(d);
             if (DENSE_OUT) dense_table.push_back(dense[i]);
@@ -1321,6 +1442,7 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
     if (grouped) {
         // group-wise scales: clear, fold the row maxima per group (a first pass of the same kernel), finish
         for (size_t g = 0; g < keys.size(); ++g) {
+            if (keys[g].cluster) continue;
             const nm::PackJobDev* dev = reinterpret_cast<const nm::PackJobDev*>(ws) + group_first[g];
             group_prepare_kernel<<<(unsigned)groups[g].size(), 256, 0, s>>>(dev, group_rows, keys[g].bits, 0);
             NM_CUDA_TRY(cudaGetLastError());
@@ -1341,7 +1463,10 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
         // after the one before it (72 matrices in four formats 104 -> 90 us).
         const bool chained = g > 0 && !grouped && (dist_ncand == 0 || (k.warps <= kPackMinWarps && keys[g - 1].warps <= kPackMinWarps));
         int rc;
-        if (dist_ncand > 0 && k.warps <= kPackMinWarps) {  // ADMM-Dist: search and projection in one kernel
+        if (k.cluster) {
+            rc = nm::launch_group<DENSE_OUT>(k.n, k.m, k.bits, k.warps, k.cluster, dev, count, nm::PackJobDev{}, group_blocks[g], status, s,
+                                             nullptr, nullptr, dense_g, group_rows);
+        } else if (dist_ncand > 0 && k.warps <= kPackMinWarps) {  // ADMM-Dist: search and projection in one kernel
             rc = nm::launch(nm::pick_dist_pack<DENSE_OUT>(k.n, k.m, k.bits), dev, count, nm::PackJobDev{}, group_blocks[g], k.warps,
                             status, s, nullptr, nullptr, dense_g, kGroupNone, dist_ncand, chained);
         } else {
