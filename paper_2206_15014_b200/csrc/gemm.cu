@@ -32,6 +32,7 @@
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 
 namespace nm {
 
@@ -1179,10 +1180,11 @@ struct DebugOptions {
     int no_wide;      // never the 512-channel pair kernel
     int wide_any;     // the 512-channel pair kernel whenever the shape allows it, however few tiles there are
     int wide_bn;      // token-tile width of that kernel: 224 or 192 (0 = automatic)
+    int one_bn;       // token-tile width of the one-CTA kernel (0 = automatic)
     int band;         // band size of the streamed pair kernel's tile order (0 = automatic)
     int skip_stage;   // NM_TEST_HOOKS builds: 1 + the pipeline stage CTA 0's producer leaves out (0 = none)
 };
-static DebugOptions g_opt = {0, 0, 0, 0, 0, 0, 0, 0};
+static DebugOptions g_opt = {};
 
 // Trace buffer of NM_TRACE builds (device, kTraceStages + kTraceTiles rows of 8 u64), handed to every GEMM launch.
 static unsigned long long* g_trace_buffer = nullptr;
@@ -1437,14 +1439,39 @@ static int pick_pair(const LinearArgs& a) {
     return launch_gemm_pair<SPARSE, 192, EPI, false>(a);
 }
 
+// Token-tile width of the one-CTA kernel: the one whose slowest CTA has the least to do, a tile costing its width plus `fixed`
+// tokens (what a tile costs however narrow it is: its weights, barriers, start and end); the wider one on equality.
+// The widest that still fills the SMs, the rule before, left half of a last wave idle: 2085 tokens 1024 -> 1002 dense
+// 8.7 -> 7.0 us (64 -> 128), 2000 tokens 3072 -> 768 int8 17.4 -> 13.4 and 2500 tokens 2560 -> 640 15.1 -> 11.2 (64 -> 96),
+// 384 tokens 1024 -> 4096 8.5 -> 6.9 (64 -> 128), 900 tokens 768 -> 3072 dense 8.8 -> 7.9 (128 -> 192), 128 tokens 768 -> 768
+// 5.1 -> 4.7 (64 -> 32).  The choice was the best of the five, or within 2 % of it, on 24 shapes.
+template <bool SPARSE>
+static int one_cta_bn(const LinearArgs& a, std::initializer_list<int> widths, int fixed) {
+    const long long out_tiles = (a.W->out + kBM - 1) / kBM, sms = sm_count();
+    int best = 0;
+    long long best_cost = 0;
+    for (int bn : widths) {
+        if (SPARSE && a.W->in / 32 > kTmemCols - 2 * bn) continue;  // the metadata of the reduction beside two accumulators
+        if (g_opt.one_bn && bn != g_opt.one_bn) continue;
+        const long long tiles = out_tiles * ((a.tokens + bn - 1) / bn);
+        const long long cost = ((tiles + sms - 1) / sms) * (bn + fixed);
+        if (!best || cost < best_cost) { best = bn; best_cost = cost; }
+    }
+    return best;
+}
+
 template <bool SPARSE, int EPI, bool XF>
 static int pick_bn(const LinearArgs& a) {
     const int out_tiles = (a.W->out + kBM - 1) / kBM, sms = sm_count();
     if constexpr (!XF) {
-        const bool fits192 = !SPARSE || a.W->in / 32 <= GemmCfg<SPARSE, 192>::META_COLS;
-        if (fits192 && (long long)out_tiles * ((a.tokens + 191) / 192) >= sms) return launch_gemm<SPARSE, 192, EPI, W_TMA>(a);
-        if ((long long)out_tiles * ((a.tokens + 127) / 128) >= sms) return launch_gemm<SPARSE, 128, EPI, W_TMA>(a);
-        return launch_gemm<SPARSE, 64, EPI, W_TMA>(a);
+        const int best = one_cta_bn<SPARSE>(a, {192, 128, 96, 64, 32}, 64);
+        switch (best) {
+            case 192: return launch_gemm<SPARSE, 192, EPI, W_TMA>(a);
+            case 128: return launch_gemm<SPARSE, 128, EPI, W_TMA>(a);
+            case 96: return launch_gemm<SPARSE, 96, EPI, W_TMA>(a);
+            case 64: return launch_gemm<SPARSE, 64, EPI, W_TMA>(a);
+            default: return launch_gemm<SPARSE, 32, EPI, W_TMA>(a);
+        }
     } else {
         // Sparse-target formats with a short reduction and work for every SM pair: the CTA-pair kernel with the weights
         // rebuilt once per output tile into its resident region (32-bit outputs).
@@ -1457,12 +1484,11 @@ static int pick_bn(const LinearArgs& a) {
         constexpr int BNR = SPARSE ? 192 : 128;
         if (a.W->in / kKB <= kResidentKB && (long long)out_tiles * ((a.tokens + BNR - 1) / BNR) >= sms && !g_opt.no_resident)
             return launch_gemm<SPARSE, BNR, EPI, W_RESIDENT>(a);
-        if constexpr (SPARSE) {  // wider token tiles: each built weight tile serves more columns
-            if (a.W->in / 32 <= GemmCfg<SPARSE, 192>::META_COLS && (long long)out_tiles * ((a.tokens + 191) / 192) >= sms)
-                return launch_gemm<SPARSE, 192, EPI, W_BUILD>(a);
+        switch (one_cta_bn<SPARSE>(a, {192, 128, 64}, 160)) {
+            case 192: return launch_gemm<SPARSE, 192, EPI, W_BUILD>(a);
+            case 128: return launch_gemm<SPARSE, 128, EPI, W_BUILD>(a);
+            default: return launch_gemm<SPARSE, 64, EPI, W_BUILD>(a);
         }
-        if ((long long)out_tiles * ((a.tokens + 127) / 128) >= sms) return launch_gemm<SPARSE, 128, EPI, W_BUILD>(a);
-        return launch_gemm<SPARSE, 64, EPI, W_BUILD>(a);
     }
 }
 
@@ -1537,7 +1563,7 @@ int nm_debug_set_option(const char* name, int value) {
     struct { const char* name; int* slot; } table[] = {
         {"no_pdl", &nm::g_opt.no_pdl}, {"no_pair", &nm::g_opt.no_pair}, {"no_resident", &nm::g_opt.no_resident},
         {"no_wide", &nm::g_opt.no_wide}, {"wide_any", &nm::g_opt.wide_any}, {"wide_bn", &nm::g_opt.wide_bn},
-        {"band", &nm::g_opt.band}, {"pack_form", &nm::g_pack_form}};
+        {"one_bn", &nm::g_opt.one_bn}, {"band", &nm::g_opt.band}, {"pack_form", &nm::g_pack_form}};
     for (auto& e : table)
         if (!strcmp(name, e.name)) { *e.slot = value; return NM_OK; }
 #ifdef NM_TEST_HOOKS
