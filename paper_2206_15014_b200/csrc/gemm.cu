@@ -685,6 +685,27 @@ struct PairCfg {
     static_assert(BN % 32 == 0 && BN <= 256, "token tile");
 };
 
+// Index metadata of one weight row (this lane's) into TMEM columns taddr .. taddr + total_words - 1: `row_words` words from
+// the row, eight pieces of four in flight together, then the valid pattern "positions 0,1": the last stage may span more
+// reduction elements than the row has, and rows past `out` (row_words = 0) must hold valid patterns too; their
+// products are zero or discarded.  A function of its own: inlined into the epilogue's loop the batch cost more through the
+// instruction cache than it saved (16384 tokens 1024 -> 4096 61.4 us before, 62.7 inlined, 60.1 so; 1024 -> 1024 21.8 / 21.8 /
+// 21.3; 49152 tokens 1024 -> 1024 bfloat16 42.0 -> 40.8).  Not with int8 outputs (12288 tokens 768 -> 3072 42.0 / 42.5) and not
+// in the BUILD form.
+__device__ __noinline__ void meta_to_tmem(const uint4* src, int row_words, int total_words, uint32_t taddr) {
+    for (int c0 = 0; c0 < total_words; c0 += 32) {
+        uint4 w[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            w[j] = c0 + 4 * j < row_words ? __ldg(src + (c0 >> 2) + j) : make_uint4(0x44444444u, 0x44444444u, 0x44444444u, 0x44444444u);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (c0 + 4 * j < total_words) ptx::tmem_st_32x4(taddr + c0 + 4 * j, w[j].x, w[j].y, w[j].z, w[j].w);
+    }
+    ptx::tmem_st_wait();
+    ptx::tc_fence_before();
+}
+
 // BUILD (with RES, sparse target): the weights are not stored in the tensor core's form (packed 4-bit codes, 1:4, 2:8,
 // 1:8).  Instead of a TMA copy, eight builder warps rebuild the CTA's 128 weight rows for the whole reduction in the resident
 // region once per output tile (xform.cuh: widening, placement into 2-of-4 slots), and the metadata warps derive the
@@ -932,20 +953,21 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
 
         auto load_meta = [&](int out_tile) {
             const int n = out_tile * (2 * kBM) + (int)rank * kBM + row;
-            const uint4* src = reinterpret_cast<const uint4*>(p.meta + (size_t)n * p.mrow_words);
-            // A stage spans KB reduction elements; when the reduction ends inside the last stage (in % KB != 0)
-            // its remaining MMAs multiply zero-filled weights, but their index fields must still be valid 2:4
-            // patterns: the columns past the row's metadata get "positions 0,1", as rows past `out` do.
-            for (int c = 0; c < p.kblocks * (Cfg::KB / 32); c += 4) {
-                uint4 w = make_uint4(0x44444444u, 0x44444444u, 0x44444444u, 0x44444444u);
-                if (n < p.out && c < p.mrow_words) {
-                    if constexpr (BUILD) w = xf::hw_meta(p.pat, xf::meta_raw(p.pat, reinterpret_cast<const uint8_t*>(p.meta) + (size_t)n * p.mrow_bytes + (size_t)(c >> 2) * xf::meta_bytes(p.pat)), lut);
-                    else w = __ldg(src + (c >> 2));
+            if constexpr (BUILD || EPI == EPI_Q8) {
+                for (int c = 0; c < p.kblocks * (Cfg::KB / 32); c += 4) {
+                    uint4 w = make_uint4(0x44444444u, 0x44444444u, 0x44444444u, 0x44444444u);  // as in meta_to_tmem
+                    if (n < p.out && c < p.mrow_words) {
+                        if constexpr (BUILD) w = xf::hw_meta(p.pat, xf::meta_raw(p.pat, reinterpret_cast<const uint8_t*>(p.meta) + (size_t)n * p.mrow_bytes + (size_t)(c >> 2) * xf::meta_bytes(p.pat)), lut);
+                        else w = __ldg(reinterpret_cast<const uint4*>(p.meta + (size_t)n * p.mrow_words) + (c >> 2));
+                    }
+                    ptx::tmem_st_32x4(lane_taddr + Cfg::META_COL + c, w.x, w.y, w.z, w.w);
                 }
-                ptx::tmem_st_32x4(lane_taddr + Cfg::META_COL + c, w.x, w.y, w.z, w.w);
+                ptx::tmem_st_wait();
+                ptx::tc_fence_before();
+            } else {
+                const uint4* src = reinterpret_cast<const uint4*>(p.meta + (size_t)(n < p.out ? n : 0) * p.mrow_words);
+                meta_to_tmem(src, n < p.out ? p.mrow_words : 0, p.kblocks * (Cfg::KB / 32), lane_taddr + Cfg::META_COL);
             }
-            ptx::tmem_st_wait();
-            ptx::tc_fence_before();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive_cluster(lead_meta);
         };
