@@ -339,8 +339,10 @@ int nm_probe_tma_stream(const void *W, int w_rows, int w_row_bytes, const void *
  * dependent-launch attribute), "no_pair" (one-CTA kernels only), "no_resident" (always stream the weights),
  * "no_wide" (never the 512-channel pair kernel), "wide_any" (the 512-channel pair kernel whenever the shape
  * allows it, however few tiles there are), "wide_bn" (its token-tile width, 224 or 192), "band" (band size of the streamed pair kernel's tile order),
- * "pack_form" (form of the projection kernel in blocks of four warps: 1 = one unit per block, 2 = persistent with
- * chunks staged in shared memory by bulk copies, 3 = persistent with the next chunk asked for ahead into L2).
+ * "one_bn" (token-tile width of the one-CTA kernel: 192, 128, 96, 64 or 32 where it exists), "xres" (the pair kernel with resident
+ * activations: 1 = wherever a pair kernel with a reduction of at most 1024 runs, 2 = never),
+ * "pack_form" (form of the projection kernel in blocks of four warps: 2 = persistent with the next rows staged in shared
+ * memory by bulk copies, where that form exists: 2:4 without dense outputs; 1 or 3 = one unit per block).
  * Results never depend on them.  Returns NM_ERR_UNSUPPORTED for an unknown name.  A library built with
  * -DNM_TEST_HOOKS (build.py --variant shortwait: device-side waits limited to about a millisecond) also takes
  * "skip_stage" = 1 + the pipeline stage that CTA 0's producer leaves unissued (0 = none): the bounded waits then

@@ -155,6 +155,7 @@ constexpr int kTraceStages = 512, kTraceTiles = 64;
 #endif
 
 #ifdef NM_TRACE
+#define NM_TRACE_ONLY(x) x
 #define NM_TRACE_STAGE(it, col) do { if (p.trace && blockIdx.x == 0 && (it) < (uint32_t)kTraceStages) p.trace[8 * (size_t)(it) + (col)] = clock64(); } while (0)
 #define NM_TRACE_TILE(i, col) do { if (p.trace && blockIdx.x == 0 && (i) < kTraceTiles) p.trace[8 * (size_t)(kTraceStages + (i)) + (col)] = clock64(); } while (0)
 // Phases of the first epilogue warp's work on a tile, summed per tile into columns 3..7 of the tile's row: waiting for the
@@ -164,6 +165,7 @@ constexpr int kTraceStages = 512, kTraceTiles = 64;
 #define NM_TRACE_EPI_ADD(k) do { const long long tr_now = clock64(); tr_acc[k] += tr_now - tr_t; tr_t = tr_now; } while (0)
 #define NM_TRACE_EPI_FLUSH(i) do { if (p.trace && blockIdx.x == 0 && (i) < kTraceTiles) { for (int k = 0; k < 5; ++k) { p.trace[8 * (size_t)(kTraceStages + (i)) + 3 + k] = tr_acc[k]; tr_acc[k] = 0; } } } while (0)
 #else
+#define NM_TRACE_ONLY(x)
 #define NM_TRACE_STAGE(it, col) do { } while (0)
 #define NM_TRACE_TILE(i, col) do { } while (0)
 #define NM_TRACE_EPI_DECL do { } while (0)
@@ -1188,6 +1190,7 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
 }  // namespace nm
 
 #include "gemm_wide.cuh"
+#include "gemm_xres.cuh"
 
 namespace nm {
 
@@ -1202,6 +1205,7 @@ struct DebugOptions {
     int no_wide;      // never the 512-channel pair kernel
     int wide_any;     // the 512-channel pair kernel whenever the shape allows it, however few tiles there are
     int wide_bn;      // token-tile width of that kernel: 224 or 192 (0 = automatic)
+    int xres;         // the pair kernel with resident activations: 1 = whenever the shape allows it, 2 = never
     int one_bn;       // token-tile width of the one-CTA kernel (0 = automatic)
     int band;         // band size of the streamed pair kernel's tile order (0 = automatic)
     int skip_stage;   // NM_TEST_HOOKS builds: 1 + the pipeline stage CTA 0's producer leaves out (0 = none)
@@ -1420,6 +1424,72 @@ static int launch_gemm_wide(const LinearArgs& a) {
     return NM_OK;
 }
 
+// Pair kernel with resident activations (gemm_xres.cuh).
+template <bool SPARSE, int EPI>
+static int launch_gemm_xres(const LinearArgs& a) {
+    using Cfg = XresCfg<SPARSE>;
+    const nm_packed_t& W = *a.W;
+    CUtensorMap tw, tx, ty;
+    int rc = make_map(&tw, W.values, (uint64_t)W.out, (uint64_t)(SPARSE ? W.in / 2 : W.in), kBM, 128, CU_TENSOR_MAP_SWIZZLE_128B);
+    if (rc != NM_OK) return rc;
+    rc = make_map_x3(&tx, a.X, (uint64_t)a.tokens, (uint64_t)W.in, Cfg::B_ROWS, Cfg::SLICES);
+    if (rc != NM_OK) return rc;
+    bool tma_store = false;
+    rc = make_store_map<EPI>(&ty, a, &tma_store);
+    if (rc != NM_OK) return rc;
+    GemmParams p{};
+    p.tma_store = tma_store ? 1 : 0;
+    p.tokens = a.tokens; p.out = W.out; p.in = W.in;
+    p.n_tok_tiles = (a.tokens + Cfg::BN - 1) / Cfg::BN;
+    p.n_out_tiles = (W.out + 2 * kBM - 1) / (2 * kBM);
+    p.n_tiles = p.n_tok_tiles * p.n_out_tiles;
+    p.kblocks = (W.in + Cfg::KB - 1) / Cfg::KB;
+    p.meta = (const uint32_t*)W.meta; p.mrow_words = W.in / 32;
+    p.sw = a.sw; p.bias = a.bias; p.sx_dev = a.sx_dev; p.sx_host = a.sx;
+    p.Y = a.Y; p.ACC = a.ACC; p.NARROW = a.NARROW; p.sy = a.sy; p.absmax = a.absmax; p.status = a.status; p.trace = g_trace_buffer; p.skip_stage = g_opt.skip_stage - 1;
+    auto fn = nm_gemm_xres_kernel<SPARSE, EPI>;
+    NM_CUDA_TRY(allow_dynamic_smem((const void*)fn, Cfg::SMEM));
+    const int pairs = p.n_tiles < sm_count() / 2 ? p.n_tiles : sm_count() / 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * pairs, 1, 1);
+    cfg.blockDim = dim3(kXresThreads<EPI>, 1, 1);
+    cfg.dynamicSmemBytes = Cfg::SMEM;
+    cfg.stream = a.stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = g_opt.no_pdl ? 1 : 2;
+    NM_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, tw, tx, ty, p));
+    return NM_OK;
+}
+
+// Where the kernel with resident activations is the faster pair kernel.  At least two output tiles (with one the activations
+// are not read twice), and then by measurement, this kernel / the other one in us:
+//  - dense weights, which the other kernel streams besides the activations: always (6144 tokens 768 -> 768 10.6 / 12.8, 768 -> 3072
+//    21.0 / 23.7, 12288 tokens 1024 -> 4096 bfloat16 47.7 / 51.4), except for narrow outputs whose rows are not 16-byte
+//    aligned (20000 tokens 1024 -> 1500 bfloat16 37.9 / 37.2);
+//  - 2:4 weights: up to 896 reduction elements (6144 tokens 768 -> 768 9.9 / 11.3, 768 -> 2304 15.4 / 16.8, 9000 tokens 512 -> 2048
+//    18.0 / 20.6, 40000 tokens 768 -> 3072 bfloat16 82.9 / 83.9); at 1024 only while a pair has few tiles, then the fill of the
+//    resident weights of the other kernel is what counts (5000 tokens 1024 -> 1024 10.4 / 12.1, 16384 tokens 1024 -> 3072, 14
+//    tiles, 47.2 / 48.7; 1024 -> 4096, 19 tiles, 62.0 / 60.2; bfloat16: 5000 tokens 1024 -> 4096, 6 tiles, 21.2 / 22.5; 49152
+//    tokens 1024 -> 1024, 14 tiles, 44.2 / 40.9);
+//  - int8 outputs of 2:4 weights, whose conversion sets the pace: a few tiles (3977 tokens 768 -> 3072, 3 tiles, 18.6 / 18.9; 12288
+//    tokens 768 -> 3072, 10 tiles, 43.5 / 42.5).
+template <bool SPARSE, int EPI>
+static bool use_xres(const LinearArgs& a) {
+    const nm_packed_t& W = *a.W;
+    if (W.in > 1024 || g_opt.xres == 2 || g_opt.no_resident) return false;
+    if (g_opt.xres == 1) return true;
+    const long long out_tiles = (W.out + 2 * kBM - 1) / (2 * kBM), pairs = sm_count() / 2;
+    const long long per_pair = (out_tiles * ((a.tokens + 191) / 192) + pairs - 1) / pairs;
+    if (out_tiles < 2) return false;
+    if (!SPARSE) return !kNarrow<EPI> || (size_t)W.out * sizeof(typename EpiOut<EPI>::type) % 16 == 0;
+    if (EPI == EPI_Q8) return per_pair <= 4;
+    return W.in <= 896 || per_pair <= (EPI == EPI_BF16 ? 8 : 16);
+}
+
 // Token-tile width of the wide kernel: the one whose slowest pair has the least to do (tiles per pair, rounded
 // up, times the tile width); 0 = the wide kernel does not apply (short reductions keep their weights resident in
 // the 256-channel kernel; a matrix of at most 256 channels would leave one of the two blocks idle; narrow outputs
@@ -1454,6 +1524,7 @@ static bool use_pair(const LinearArgs& a) {
 // Pair kernel with the weights streamed through the ring, or (2:4, reduction up to 1024) kept resident.
 template <bool SPARSE, int EPI>
 static int pick_pair(const LinearArgs& a) {
+    if (use_xres<SPARSE, EPI>(a)) return launch_gemm_xres<SPARSE, EPI>(a);
     if constexpr (SPARSE) {
         if (a.W->in <= kPairResStages * PairCfg<true, 192>::KB && !g_opt.no_resident)
             return launch_gemm_pair<true, 192, EPI, true>(a);
@@ -1585,7 +1656,7 @@ int nm_debug_set_option(const char* name, int value) {
     struct { const char* name; int* slot; } table[] = {
         {"no_pdl", &nm::g_opt.no_pdl}, {"no_pair", &nm::g_opt.no_pair}, {"no_resident", &nm::g_opt.no_resident},
         {"no_wide", &nm::g_opt.no_wide}, {"wide_any", &nm::g_opt.wide_any}, {"wide_bn", &nm::g_opt.wide_bn},
-        {"one_bn", &nm::g_opt.one_bn}, {"band", &nm::g_opt.band}, {"pack_form", &nm::g_pack_form}};
+        {"one_bn", &nm::g_opt.one_bn}, {"xres", &nm::g_opt.xres}, {"band", &nm::g_opt.band}, {"pack_form", &nm::g_pack_form}};
     for (auto& e : table)
         if (!strcmp(name, e.name)) { *e.slot = value; return NM_OK; }
 #ifdef NM_TEST_HOOKS
