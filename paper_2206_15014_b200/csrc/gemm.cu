@@ -1490,6 +1490,17 @@ static bool use_xres(const LinearArgs& a) {
     return W.in <= 896 || per_pair <= (EPI == EPI_BF16 ? 8 : 16);
 }
 
+// Whether the one-CTA kernel has at most one 192-token tile for every SM.  It then beats the pair kernels where their larger
+// tiles leave SMs idle or need a second round: 3977 tokens 3072 -> 768 (126 tiles of 128 x 192; 42 of 512 x 192) 14.9 against 17.9 us, packed 4-bit codes 20.2
+// against 27.6; 4500 tokens (144 tiles) 15.2 / 17.8; 5000 tokens 2560 -> 640 13.8 / 16.2.  With a second wave it loses: 5500 tokens 3072 ->
+// 768 (174 tiles) 22.5 / 18.3.  Against the 256-channel kernels: 5000 tokens 640 -> 640 (135 tiles; 81 of 256 x 192 on 74 pairs) 7.3 / 9.5,
+// dense 2560 -> 640 14.0 / 19.1, 9000 tokens 896 -> 384 8.6 / 10.6,
+// packed 4-bit codes 5000 tokens 640 -> 640 9.3 / 12.3.
+static bool one_wave(const LinearArgs& a) {
+    const long long tiles = (long long)((a.W->out + kBM - 1) / kBM) * ((a.tokens + 191) / 192);
+    return tiles <= sm_count() && a.W->in / 32 <= kTmemCols - 2 * 192;
+}
+
 // Token-tile width of the wide kernel: the one whose slowest pair has the least to do (tiles per pair, rounded
 // up, times the tile width); 0 = the wide kernel does not apply (short reductions keep their weights resident in
 // the 256-channel kernel; a matrix of at most 256 channels would leave one of the two blocks idle; narrow outputs
@@ -1499,6 +1510,7 @@ static int wide_bn(const LinearArgs& a) {
     if (g_opt.no_wide || g_opt.no_pair) return 0;
     const nm_packed_t& W = *a.W;
     if (W.in <= kPairResStages * PairCfg<true, 192>::KB || W.out <= 2 * kBM) return 0;
+    if (one_wave(a) && !g_opt.wide_any) return 0;
     const long long pairs = sm_count() / 2, out_tiles = (W.out + 4 * kBM - 1) / (4 * kBM);
     int best = 0;
     long long best_cost = 0;
@@ -1518,6 +1530,7 @@ static bool use_pair(const LinearArgs& a) {
     if (g_opt.no_pair) return false;
     const long long tiles = (long long)((a.W->out + 2 * kBM - 1) / (2 * kBM)) * ((a.tokens + 191) / 192);
     const bool fits = !SPARSE || a.W->in / 32 <= PairCfg<SPARSE, 192>::META_COLS;
+    if (tiles > sm_count() / 2 && one_wave(a)) return false;  // a second round of pair tiles against one of small tiles
     return fits && tiles >= sm_count() / 2;
 }
 
@@ -1570,7 +1583,8 @@ static int pick_bn(const LinearArgs& a) {
         // rebuilt once per output tile into its resident region (32-bit outputs).
         if constexpr (SPARSE && (EPI == EPI_F32 || EPI == EPI_ACC)) {
             const long long pair_tiles = (long long)((a.W->out + 2 * kBM - 1) / (2 * kBM)) * ((a.tokens + 191) / 192);
-            if (a.W->in <= kPairResStages * PairCfg<true, 192>::KB && pair_tiles >= sms / 2 && !g_opt.no_pair && !g_opt.no_resident)
+            if (a.W->in <= kPairResStages * PairCfg<true, 192>::KB && pair_tiles >= sms / 2 && !(pair_tiles > sms / 2 && one_wave(a)) &&
+                !g_opt.no_pair && !g_opt.no_resident)
                 return launch_gemm_pair<true, 192, EPI, true, true>(a);
         }
         // Short reductions with many token tiles per output tile: build each weight tile once and keep it.

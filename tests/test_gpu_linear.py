@@ -69,6 +69,13 @@ def test_metadata_batches(n, m, bits, K):
     _run(40, 64, K, 200, n, m, bits)
 
 
+@pytest.mark.parametrize("n,m,bits", [(2, 4, 8), (2, 4, 4), (1, 4, 8), (4, 4, 8)])
+@pytest.mark.parametrize("T,K,out", [(29 * 192 - 5, 1152, 640), (29 * 192 + 1, 1152, 640), (29 * 192, 640, 640), (1900, 4096, 384)])
+def test_long_reduction_around_one_wave_of_tiles(n, m, bits, T, K, out):
+    # 145 and 150 tiles of 128 x 192 on 148 SMs: the one-CTA kernel up to one wave, the pair kernels beyond
+    _run(41, T, K, out, n, m, bits)
+
+
 @pytest.mark.parametrize("n,m,bits", ALL_MODES)
 def test_bert_base_attention_projection(n, m, bits):
     # 128 tokens x 768 -> 768 (the small single-GEMM configuration)
