@@ -802,8 +802,8 @@ def pack_sweep(nm, torch, dev, status, reps=5):
             times.append(e0.elapsed_time(e1))
         us = float(np.median(times)) * 1e3
         table[f"{n}:{m}/{bits}b"] = {"us": us, "gbs": nbytes / us / 1e3, "bytes": nbytes}
-    # group-wise scales (32 output channels per scale, the paper's default), one batched call: two passes over
-    # W and U (row maxima per group, then the projection); GB/s on the same algorithmic bytes as the per-channel pack
+    # group-wise scales (32 output channels per scale, the paper's default), one batched call: one launch per row length,
+    # a cluster of blocks per group; GB/s on the same algorithmic bytes as the per-channel pack
     grouped_jobs = nm.make_pack_jobs([(W, U, 2, 4, 8, v, mt, sc) for (W, U, v, mt, sc) in mats])
     def grouped_pass():
         nm.nm_project_pack_grouped_batched(grouped_jobs, len(mats), 32, ws, ws_bytes, status)
@@ -819,10 +819,10 @@ def pack_sweep(nm, torch, dev, status, reps=5):
         times.append(e0.elapsed_time(e1))
     grouped_us = float(np.median(times)) * 1e3
     grouped = {"us": grouped_us, "gbs": table["2:4/8b"]["bytes"] / grouped_us / 1e3, "bytes": table["2:4/8b"]["bytes"],
-               "launches": 4, "group_rows": 32}
-    # ADMM-Dist scale search (32 candidate scales per output channel) followed by the projection at the chosen
-    # scale, 2:4 with 4-bit and 8-bit codes, one batched call (2 launches).  The search is bound by instruction
-    # issue, not by memory: reported as time and as candidate evaluations (kept value x candidate) per second.
+               "launches": 2, "group_rows": 32}
+    # ADMM-Dist scale search (32 candidate scales per output channel) and the projection at the chosen scale in one
+    # kernel, 2:4 with 4-bit and 8-bit codes, one batched call.  It is bound by arithmetic, not by memory: reported as
+    # time and as candidate evaluations (kept value x candidate) per second of what it takes beyond the plain projection.
     dist = {}
     kept = sum(o * k for o, k in shapes) // 2
     for bits in (4, 8):
@@ -840,7 +840,7 @@ def pack_sweep(nm, torch, dev, status, reps=5):
             torch.cuda.synchronize()
             times.append(e0.elapsed_time(e1))
         us = float(np.median(times)) * 1e3
-        dist[f"2:4/{bits}b"] = {"us": us, "search_us": us - table[f"2:4/{bits}b"]["us"], "candidates": 32, "launches": 2,
+        dist[f"2:4/{bits}b"] = {"us": us, "search_us": us - table[f"2:4/{bits}b"]["us"], "candidates": 32, "launches": 1,
                                 "evals_per_s": kept * 32 / (us - table[f"2:4/{bits}b"]["us"]) * 1e6}
     # ADMM step with dense outputs over the same 96 matrices (one batched call): W and U read, Z and
     # U_next (in place over U, so it runs last) written, 16 bytes per parameter; 2:4 / 8-bit, no packed outputs
