@@ -942,14 +942,15 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
 // ---------------------------------------------------------------------------------------------
 // Group-wise scales in one pass: a cluster of blocks holds a whole group of rows in registers, the blocks exchange their
 // maxima through distributed shared memory, and every warp goes on with its row at the group's scale.  W and U are read
-// once; folding the maxima of all groups first and packing in a second launch read them twice.
+// once; folding the maxima of all groups first and packing in a second launch read them twice (75 M weights, 2:4 / 4 bit, groups of 32
+// rows: 232 us, 154 so).  Bound by the loads of a cluster, which wait for the barrier of the one before (DRAM at 45 %).
 // A unit is one group (`group_rows` rows, those past the matrix idle); it fills gridDim / units blocks, the cluster.
 // ---------------------------------------------------------------------------------------------
 template <int N, int M, int BITS, bool DENSE_OUT>
 __global__ void __launch_bounds__(512, DENSE_OUT ? 1 : 2)
 pack_group_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constant__ PackJobInline inl, uint32_t* status,
                   float* __restrict__ Zout, float* __restrict__ Unext, const DenseOutDev* __restrict__ dense_jobs,
-                  int group_rows, unsigned cluster) {
+                  int group_rows, unsigned cluster, bool chained) {
     // [warps] maxima, [8] maxima of the cluster's blocks, (4:8) position table and [warps][8][32] floats
     extern __shared__ float4 tile[];
     const int warps = blockDim.x >> 5, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -993,11 +994,13 @@ pack_group_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_c
     ptx::cluster_wait();
     amax = 0.0f;
     for (unsigned c = 0; c < cluster; ++c) amax = fmaxf(amax, __uint_as_float(peers[c]));
-    if (!up.row_ok) return;
-    constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
-    const float s = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
-    if (up.chunk == 0 && lane == 0) job.scales[up.row] = s;
-    pack_row<N, M, BITS, DENSE_OUT, false>(job, up, lane, v, s, bad, pos48, scratch, Zout, Unext, wide);
+    if (up.row_ok) {
+        constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
+        const float s = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
+        if (up.chunk == 0 && lane == 0) job.scales[up.row] = s;
+        pack_row<N, M, BITS, DENSE_OUT, false>(job, up, lane, v, s, bad, pos48, scratch, Zout, Unext, wide);
+    }
+    if (chained) ptx::grid_dep_wait();  // as in pack_kernel
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1238,7 +1241,7 @@ static bool group_cluster(int group_rows, int wpr_log2, int* warps, int* cluster
     return false;
 }
 
-using GroupFn = void (*)(const PackJobDev*, int, const PackJobInline, uint32_t*, float*, float*, const DenseOutDev*, int, unsigned);
+using GroupFn = void (*)(const PackJobDev*, int, const PackJobInline, uint32_t*, float*, float*, const DenseOutDev*, int, unsigned, bool);
 
 template <bool DENSE_OUT>
 static GroupFn pick_group(int n, int m, int bits) {
@@ -1255,7 +1258,7 @@ static GroupFn pick_group(int n, int m, int bits) {
 template <bool DENSE_OUT>
 static int launch_group(int n, int m, int bits, int warps, int cluster, const PackJobDev* jobs_dev, int njobs, const PackJobDev& single,
                         unsigned units, uint32_t* status, cudaStream_t stream, float* Z, float* U_next,
-                        const DenseOutDev* dense_jobs, int group_rows) {
+                        const DenseOutDev* dense_jobs, int group_rows, bool chained = false) {
     PackJobInline inl{};
     inl.j[0] = single;
     cudaLaunchConfig_t cfg = {};
@@ -1263,12 +1266,14 @@ static int launch_group(int n, int m, int bits, int warps, int cluster, const Pa
     cfg.blockDim = dim3(warps * 32, 1, 1);
     cfg.dynamicSmemBytes = 96 + (n == 4 && m == 8 ? 512 + (size_t)warps * 1024 : 0);
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = chained ? 2 : 1;
     NM_CUDA_TRY(cudaLaunchKernelEx(&cfg, pick_group<DENSE_OUT>(n, m, bits), jobs_dev, njobs, inl, status, Z, U_next, dense_jobs,
-                                   group_rows, (unsigned)cluster));
+                                   group_rows, (unsigned)cluster, chained));
     return NM_OK;
 }
 
@@ -1460,12 +1465,13 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
         const int count = (int)groups[g].size();
         const DenseOutDev* dense_g = DENSE_OUT ? dense_dev + group_first[g] : nullptr;
         // Launches after the first start while the one before them drains: they work on other matrices, and each ends only
-        // after the one before it (72 matrices in four formats 104 -> 90 us).
-        const bool chained = g > 0 && !grouped && (dist_ncand == 0 || (k.warps <= kPackMinWarps && keys[g - 1].warps <= kPackMinWarps));
+        // after the one before it (72 matrices in four formats 104 -> 90 us, with group-wise scales 179 -> 139).
+        const bool chained = g > 0 && (grouped ? k.cluster && keys[g - 1].cluster
+                                               : dist_ncand == 0 || (k.warps <= kPackMinWarps && keys[g - 1].warps <= kPackMinWarps));
         int rc;
         if (k.cluster) {
             rc = nm::launch_group<DENSE_OUT>(k.n, k.m, k.bits, k.warps, k.cluster, dev, count, nm::PackJobDev{}, group_blocks[g], status, s,
-                                             nullptr, nullptr, dense_g, group_rows);
+                                             nullptr, nullptr, dense_g, group_rows, chained);
         } else if (dist_ncand > 0 && k.warps <= kPackMinWarps) {  // ADMM-Dist: search and projection in one kernel
             rc = nm::launch(nm::pick_dist_pack<DENSE_OUT>(k.n, k.m, k.bits), dev, count, nm::PackJobDev{}, group_blocks[g], k.warps,
                             status, s, nullptr, nullptr, dense_g, kGroupNone, dist_ncand, chained);

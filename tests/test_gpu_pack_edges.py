@@ -124,3 +124,30 @@ def test_overlapping_launches_of_a_batch_end_before_what_follows():
     D = oracle.unpack(refs[0][0], refs[0][1], 4096, 1024, 2, 4, 8)
     _, Y_ref = oracle.int_linear(X.cpu().numpy(), D, np.float32(0.01), refs[0][2], None)
     assert np.array_equal(ys[0].cpu().numpy(), Y_ref)
+
+
+def test_overlapping_group_launches_of_a_batch():
+    """The same for group-wise scales: one cluster launch per format and row length, and a two-pass one (rows of 6144) among them."""
+    import paper_2206_15014_b200 as nm
+    from gpu_util import DEV, to_dev
+    fmts = [(2, 4, 8), (4, 4, 8), (2, 4, 8), (2, 4, 4), (4, 8, 8), (2, 4, 8)]
+    shapes = [(2000, 1024), (96, 4096), (100, 4096), (64, 6144), (700, 768), (33, 1536)]
+    jobs, bufs, refs = [], [], []
+    for i, ((n, m, bits), (out, k)) in enumerate(zip(fmts, shapes)):
+        W, U = wl.pack_sweep_matrix(24, i, out, k)
+        b = _buffers(out, k, n, m, bits)
+        jobs.append((to_dev(W), to_dev(U), n, m, bits, b[0], b[1] if n != m else None, b[2]))
+        bufs.append(b)
+        refs.append(oracle.project_pack_grouped(W, U, n, m, bits, 32))
+    ws_bytes = nm.nm_pack_workspace_bytes(len(jobs))
+    ws = torch.empty(ws_bytes, dtype=torch.uint8, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    for _ in range(3):
+        for b in bufs:
+            b[0][: b[3]].fill_(0x11)
+            b[2].fill_(-1.0)
+        nm.nm_project_pack_grouped_batched(nm.make_pack_jobs(jobs), len(jobs), 32, ws, ws_bytes, status)
+        copies = [(b[0].clone(), b[1].clone(), b[2].clone(), b[3], b[4]) for b in bufs]
+        assert nm.nm_poll_status(status) == nm.NM_OK
+        for c, r in zip(copies, refs):
+            _same(c, r)
