@@ -943,7 +943,8 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
 // Group-wise scales in one pass: a cluster of blocks holds a whole group of rows in registers, the blocks exchange their
 // maxima through distributed shared memory, and every warp goes on with its row at the group's scale.  W and U are read
 // once; folding the maxima of all groups first and packing in a second launch read them twice (75 M weights, 2:4 / 4 bit, groups of 32
-// rows: 232 us, 154 so).  Bound by the loads of a cluster, which wait for the barrier of the one before (DRAM at 45 %).
+// rows: 232 us, 154 so).  What bounds it: a cluster loads, meets
+// at its barrier and packs in turn, with two to four blocks an SM to overlap that (DRAM at 45 %).
 // A unit is one group (`group_rows` rows, those past the matrix idle); it fills gridDim / units blocks, the cluster.
 // ---------------------------------------------------------------------------------------------
 template <int N, int M, int BITS, bool DENSE_OUT>
