@@ -4,8 +4,8 @@ A second build of the library (short wait limits, plus a test hook that makes CT
 stage unissued: nothing armed, nothing in flight, no address touched) runs in a child process; the stage's barrier
 never completes, the gate's wait expires after about a millisecond, the kernel raises NM_STATUS_TIMEOUT, drains and
 returns, and the next call on the same stream matches the oracle.  One case per kernel family that this form has been
-shown to be safe for (the 512-channel pair kernel's case is not run: see timeout_case.py), and one for the staged projection
-kernel, where a warp leaves the bulk copies of one chunk unissued and its wait for the chunk expires."""
+shown to be safe for (the 512-channel pair kernel is not among them), and one for the staged projection kernel, where a
+warp leaves the bulk copies of one chunk unissued and its wait for the chunk expires."""
 import os
 import subprocess
 import sys
