@@ -902,6 +902,10 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
             issue(job, up, 0, 0);
         }
         uint32_t phase = 0;  // bit b: parity of buffer b's next completion
+        // The slots of the row maximum alternate over the units whose rows span warps: only those pass the block's barrier, so
+        // the one before the last has been read by every warp when its slots are written again.  (Alternating over all units
+        // would reuse them after an odd number of one-warp units, which no barrier separates.)
+        unsigned spanning = 0;
         for (int it = 0; unit < nunits; ++it, unit += gridDim.x) {
             const int buf = it & 1;
             // the next unit's part goes into the other buffer while this one is worked on
@@ -927,8 +931,9 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
             }
             float v[32];
             load_staged(job, up, lane, mybuf + buf * 2048, mybuf + buf * 2048 + 1024, v);
-            pack_finish<N, M, BITS, DENSE_OUT>(job, up, lane, w, v, red + (it & 1) * warps, pos48, scratch, status, Zout, Unext,
+            pack_finish<N, M, BITS, DENSE_OUT>(job, up, lane, w, v, red + (spanning & 1u) * warps, pos48, scratch, status, Zout, Unext,
                                               wide_rows(job, Zout, Unext), group_mode, group_rows);
+            spanning += job.wpr_log2 != 0 ? 1u : 0u;
             job = njob; index = nindex; up = nup;
         }
         // after an expired wait a copy may still be on its way into this block's shared memory

@@ -89,6 +89,37 @@ def test_forms_batched_through_the_job_table(form):
         assert np.array_equal(job[7].cpu().numpy(), s_ref)
 
 
+def test_staged_units_of_several_warps_and_of_one_in_turn():
+    """Rows of four warps, of one and of four again in the consecutive units of every resident block (444 of them): the slots
+    of the row maximum are shared by the rows of several warps alone."""
+    import paper_2206_15014_b200 as nm
+    from gpu_util import DEV, to_dev
+    blocks = 3 * torch.cuda.get_device_properties(DEV).multi_processor_count
+    jobs, refs = [], []
+    for i, k in enumerate([4096, 1024, 4096, 1024, 2048, 4096]):
+        out = blocks * 4096 // k  # one unit per block
+        W, U = wl.pack_sweep_matrix(31, i, out, k)
+        W *= (1.0 + np.arange(out, dtype=np.float32) % 7)[:, None]  # neighbouring rows differ in scale
+        vb, mb = nm.nm_packed_sizes(out, k, 2, 4, 8)
+        jobs.append((to_dev(W), to_dev(U), 2, 4, 8, torch.zeros(vb, dtype=torch.uint8, device=DEV),
+                     torch.zeros(mb // 4, dtype=torch.int32, device=DEV), torch.zeros(out, dtype=torch.float32, device=DEV)))
+        refs.append(oracle.project_pack(W, U, 2, 4, 8))
+    ws_bytes = nm.nm_pack_workspace_bytes(len(jobs))
+    ws = torch.empty(ws_bytes, dtype=torch.uint8, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    nm.nm_debug_set_option("pack_form", 2)
+    try:
+        for _ in range(5):
+            nm.nm_project_pack_batched(nm.make_pack_jobs(jobs), len(jobs), ws, ws_bytes, status)
+        assert nm.nm_poll_status(status) == 0
+    finally:
+        nm.nm_debug_set_option("pack_form", 0)
+    for job, (v_ref, m_ref, s_ref) in zip(jobs, refs):
+        assert np.array_equal(job[7].cpu().numpy(), s_ref)
+        assert np.array_equal(job[5].cpu().numpy().reshape(v_ref.shape), v_ref)
+        assert np.array_equal(job[6].cpu().numpy().view(np.uint32).reshape(m_ref.shape), m_ref)
+
+
 @pytest.mark.parametrize("n,m,bits", [(2, 4, 8), (4, 8, 8), (1, 4, 4), (4, 4, 4)])
 def test_forms_admm_step(form, n, m, bits):
     """Dense outputs (Z, U_next) besides the packed ones, 3000 rows: several rounds per resident block."""
