@@ -52,6 +52,9 @@ constexpr int kMaxStages = 7;       // the relay cycles through 8 named barriers
 #define NM_WAIT_LIMIT (1ll << 31)
 #endif
 constexpr long long kAbortDrain = 1ll << 17;  // SM clocks a producer of a CTA pair waits after an expired wait so that its copies in flight land
+// ... and its gate waits after one before it lets the MMA warp run on (see relay_step): a role in a wait looks at the abort flag
+// at every 64th poll, a poll that fails takes about 7800 clocks (measured), so all of them have left after half a million.
+constexpr long long kGateDrain = 1ll << 21;
 constexpr long long kWaitLimit = NM_WAIT_LIMIT;  // SM clocks per device-side wait (about a second; test builds shorten it)
 
 // What the epilogue writes: y = fma(acc, sx * sw[o], b[o]) as fp32; the raw int32 accumulators; y re-quantised
@@ -379,6 +382,7 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         auto wait = [&](uint32_t bar, uint32_t parity) {
             if (lane == 0 && ok && !ptx::mbar_wait_bounded(bar, parity, abort_flag, kWaitLimit)) {
                 raise_timeout();
+                ptx::wait_clocks(kGateDrain);
                 ok = false;
             }
         };
@@ -824,9 +828,8 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                     NM_TRACE_STAGE(it, 1);
                 }
             }
-            // After an expired wait (here or anywhere in the pair) the MMA thread runs through its remaining steps without
-            // waiting for data, so the stages' barriers no longer say whether this producer's last copies have landed:
-            // give them time before the CTA and its shared memory go away.
+            // After an expired wait (here or anywhere in the pair) nobody waits for this producer's last copies, and the stages'
+            // barriers count the bytes of both CTAs: give the copies time before the CTA and its shared memory go away.
             if (!ok || *abort_flag) ptx::wait_clocks(kAbortDrain);
         }
     } else if (BUILD && warp > kGateWarp) {
@@ -874,6 +877,7 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
             auto wait = [&](uint32_t bar, uint32_t parity) {
                 if (lane == 0 && ok && !ptx::mbar_wait_bounded(bar, parity, abort_flag, kWaitLimit)) {
                     raise_timeout();
+                    ptx::wait_clocks(kGateDrain);
                     ok = false;
                 }
             };

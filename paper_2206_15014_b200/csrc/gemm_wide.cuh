@@ -160,9 +160,8 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                     if (++s == S) { s = 0; parity ^= 1u; }
                 }
             }
-            // After an expired wait (here or anywhere in the pair) the MMA thread runs through its remaining steps without
-            // waiting for data, so the stages' barriers no longer say whether this producer's last copies have landed:
-            // give them time before the CTA and its shared memory go away.
+            // After an expired wait (here or anywhere in the pair) nobody waits for this producer's last copies, and the stages'
+            // barriers count the bytes of both CTAs: give the copies time before the CTA and its shared memory go away.
             if (!ok || *abort_flag) ptx::wait_clocks(kAbortDrain);
         }
     } else if (W4 && warp >= kWideMetaWarp0 + 4) {
@@ -280,6 +279,7 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
             auto wait = [&](uint32_t bar, uint32_t parity) {
                 if (lane == 0 && ok && !ptx::mbar_wait_bounded(bar, parity, abort_flag, kWaitLimit)) {
                     raise_timeout();
+                    ptx::wait_clocks(kGateDrain);
                     ok = false;
                 }
             };

@@ -103,6 +103,10 @@ __device__ __forceinline__ void named_bar_arrive(uint32_t id, uint32_t threads) 
 // ahead of the MMA warp by as many steps as it has found ready.  Once a bounded wait has expired anywhere in the CTA the gate
 // no longer waits for data; it would then lap the MMA warp on the ring of named barriers (arriving twice on an id the
 // MMA warp has not reached), so from then on it meets the MMA warp at every step.
+// Before the gate goes on it gives every other role time to see the flag and to leave (kGateDrain).  The MMA warp's commits, which
+// then hand back stages that were never full, would otherwise let producers, builders and metadata warps go round the ring
+// once more (their waits succeed at once, without a look at the flag) and arrive on a "full" barrier whose phase a missing
+// arrival or missing bytes still hold open, beyond the count it was set up for.
 __device__ __forceinline__ void relay_step(uint32_t id, volatile uint32_t* abort_flag) {
     if (__any_sync(0xffffffffu, *abort_flag != 0u)) named_bar_sync(id, 64);
     else named_bar_arrive(id, 64);
