@@ -206,6 +206,10 @@ int nm_admm_project_dist(const float *W, const float *U, int out, int in, int n,
  * library owns only until the call returns, so it must not be captured into a CUDA graph: on a capturing
  * stream such a call returns NM_ERR_UNSUPPORTED and enqueues nothing.  The same holds for
  * nm_project_pack_batched_noalloc.
+ * Jobs of one call that share (n, m, bits) and block size run in one launch, in no order among each other: no output of
+ * one may overlap a buffer of another.  The launches of a call stand in the order of their first jobs; those whose
+ * outputs overlap another's buffers run one after the other, the others may overlap in time.  The same holds for every
+ * *_batched call.
  */
 int nm_project_pack_batched(const nm_pack_job_t *jobs, int njobs, void *ws, size_t ws_bytes,
                             uint32_t *status, void *stream);

@@ -1374,6 +1374,50 @@ static int launch_dist_project_single(const nm_pack_job_t& j, int ncand, uint32_
                   nullptr, kGroupScalesGiven, 0);
 }
 
+// Whether the launches of a call work on separate buffers: no output of a job of one launch overlaps a buffer of a job of
+// another.  `table` holds the jobs launch by launch, `first` the number of each launch's first one; `dense` is parallel to
+// `table` or NULL.  One pass over the buffers by address; of those before a buffer it remembers, among the outputs and among all, the
+// one that reaches furthest and the furthest of another launch.
+static bool separate_launches(const std::vector<PackJobDev>& table, const DenseOutDev* dense, const std::vector<size_t>& first) {
+    struct Span { uintptr_t begin, end; size_t launch; bool out; };
+    std::vector<Span> spans;
+    spans.reserve(table.size() * (dense ? 7 : 5));
+    size_t launch = 0;
+    for (size_t i = 0; i < table.size(); ++i) {
+        while (launch + 1 < first.size() && i >= first[launch + 1]) ++launch;
+        const PackJobDev& j = table[i];
+        auto add = [&](const void* p, size_t row_bytes, bool out) {
+            if (p && row_bytes) spans.push_back(Span{(uintptr_t)p, (uintptr_t)p + row_bytes * (size_t)j.out, launch, out});
+        };
+        add(j.W, (size_t)j.in * 4, false);
+        add(j.U, (size_t)j.in * 4, false);
+        add(j.values, j.vrow_bytes, true);
+        add(j.meta, (size_t)j.mrow_words * 4, true);
+        add(j.scales, 4, true);
+        if (dense) {
+            add(dense[i].Z, (size_t)j.in * 4, true);
+            add(dense[i].U_next, (size_t)j.in * 4, true);
+        }
+    }
+    std::sort(spans.begin(), spans.end(), [](const Span& x, const Span& y) { return x.begin < y.begin; });
+    struct Reach {
+        uintptr_t end[2] = {0, 0};  // the furthest, and the furthest of a launch other than that one's
+        size_t launch = 0;          // launch of end[0]
+        uintptr_t of_others(size_t l) const { return l == launch ? end[1] : end[0]; }
+        void take(const Span& s) {
+            if (s.launch == launch) { end[0] = std::max(end[0], s.end); return; }
+            if (s.end > end[0]) { end[1] = end[0]; end[0] = s.end; launch = s.launch; }
+            else end[1] = std::max(end[1], s.end);
+        }
+    } outs, all;
+    for (const Span& s : spans) {
+        if ((s.out ? all : outs).of_others(s.launch) > s.begin) return false;
+        all.take(s);
+        if (s.out) outs.take(s);
+    }
+    return true;
+}
+
 // Shared by the batched entry points: groups the jobs that can share one launch (same pattern, code width
 // and block size), writes the device job table(s) into `ws` and launches one kernel per group.
 template <bool DENSE_OUT>
@@ -1420,17 +1464,23 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
         }
         group_blocks[g] = blocks;
     }
+    // Launches after the first start while the one before them drains, and each ends only after the one before it (72 matrices in
+    // four formats 104 -> 90 us, with group-wise scales 179 -> 139), unless one's outputs overlap another's buffers (two jobs of
+    // different formats on the same U, one of them in place): those run one after the other, in the order of the launches.
+    // Looked at when the first launch is under way.
+    bool separate = false;
     // Small plain batches: every group's table fits in the kernel's parameters, nothing is copied to `ws`.
     if (!DENSE_OUT && !grouped && dist_ncand == 0) {
         bool fits = true;
         for (size_t g = 0; g < keys.size(); ++g) fits = fits && groups[g].size() <= (size_t)kInlineJobs;
         if (fits) {
             for (size_t g = 0; g < keys.size(); ++g) {
+                if (g == 1) separate = separate_launches(table, nullptr, group_first);
                 PackJobInline inl{};
                 for (size_t i = 0; i < groups[g].size(); ++i) inl.j[i] = table[group_first[g] + i];
                 int rc = nm::launch_table(nm::pick_kernel<DENSE_OUT>(keys[g].n, keys[g].m, keys[g].bits, keys[g].warps, group_blocks[g], keys[g].dual), nullptr,
                                           (int)groups[g].size(), inl, group_blocks[g], keys[g].warps, status, s, nullptr,
-                                          nullptr, nullptr, kGroupNone, 0, g > 0);
+                                          nullptr, nullptr, kGroupNone, 0, g > 0 && separate);
                 if (rc != NM_OK) return rc;
             }
             return NM_OK;
@@ -1470,10 +1520,9 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
         const Key& k = keys[g];
         const int count = (int)groups[g].size();
         const DenseOutDev* dense_g = DENSE_OUT ? dense_dev + group_first[g] : nullptr;
-        // Launches after the first start while the one before them drains: they work on other matrices, and each ends only
-        // after the one before it (72 matrices in four formats 104 -> 90 us, with group-wise scales 179 -> 139).
-        const bool chained = g > 0 && (grouped ? k.cluster && keys[g - 1].cluster
-                                               : dist_ncand == 0 || (k.warps <= kPackMinWarps && keys[g - 1].warps <= kPackMinWarps));
+        if (g == 1) separate = separate_launches(table, DENSE_OUT ? dense_table.data() : nullptr, group_first);
+        const bool chained = g > 0 && separate && (grouped ? k.cluster && keys[g - 1].cluster
+                                                             : dist_ncand == 0 || (k.warps <= kPackMinWarps && keys[g - 1].warps <= kPackMinWarps));
         int rc;
         if (k.cluster) {
             rc = nm::launch_group<DENSE_OUT>(k.n, k.m, k.bits, k.warps, k.cluster, dev, count, nm::PackJobDev{}, group_blocks[g], status, s,

@@ -151,3 +151,38 @@ def test_overlapping_group_launches_of_a_batch():
         assert nm.nm_poll_status(status) == nm.NM_OK
         for c, r in zip(copies, refs):
             _same(c, r)
+
+
+@pytest.mark.parametrize("kind", ["row", "group", "dist"])
+def test_jobs_of_different_formats_on_one_dual_in_place_run_in_order(kind):
+    """Three formats on the same W and U, the second one updating U in place: its launch must wait for the first, and the third
+    reads what it wrote, as three calls of the one-matrix entry point do."""
+    import paper_2206_15014_b200 as nm
+    from gpu_util import DEV, to_dev
+    out, k, G, ncand = 4096, 1024, 32, 4
+    fmts = [(2, 4, 8), (4, 4, 4), (1, 4, 8)]
+    single, batched, extra = {"row": (nm.nm_admm_project, nm.nm_admm_project_batched, ()),
+                              "group": (nm.nm_admm_project_grouped, nm.nm_admm_project_grouped_batched, (G,)),
+                              "dist": (nm.nm_admm_project_dist, nm.nm_admm_project_dist_batched, (ncand,))}[kind]
+    W, U = wl.pack_sweep_matrix(25, 0, out, k)
+    Wd, U0 = to_dev(W), to_dev(U * 8.0)
+    ws_bytes = nm.nm_admm_workspace_bytes(len(fmts))
+    ws = torch.empty(ws_bytes, dtype=torch.uint8, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+
+    def buffers():
+        Ud = U0.clone()
+        return (Ud, [torch.zeros_like(Wd) for _ in fmts], [torch.zeros_like(Wd), Ud, torch.zeros_like(Wd)],
+                [torch.zeros(out, dtype=torch.float32, device=DEV) for _ in fmts])
+
+    Ud, Z_ref, Un_ref, s_ref = buffers()
+    for i, f in enumerate(fmts):
+        single(Wd, Ud, out, k, *f, *extra, Z_ref[i], Un_ref[i], None, None, s_ref[i], status)
+        assert nm.nm_poll_status(status) == nm.NM_OK
+    for _ in range(3):
+        Ud, Z, Un, sc = buffers()
+        jobs = nm.make_admm_jobs([(Wd, Ud, *f, Z[i], Un[i], None, None, sc[i]) for i, f in enumerate(fmts)])
+        batched(jobs, len(fmts), *extra, ws, ws_bytes, status)
+        assert nm.nm_poll_status(status) == nm.NM_OK
+        for i in range(len(fmts)):
+            assert torch.equal(sc[i], s_ref[i]) and torch.equal(Z[i], Z_ref[i]) and torch.equal(Un[i], Un_ref[i]), f"job {i}"
