@@ -113,8 +113,14 @@ __device__ __forceinline__ typename EpiOut<EPI>::type epi_convert(uint32_t acc, 
 // Pieces of metadata (16 bytes: one row, one 128-wide k-block) that a metadata warp of the one-CTA kernel has in flight (four
 // in the forms with weight-building warps, which are short of registers).  One at a time, each load waited for before its
 // store to TMEM, they held up the first MMA: 384 tokens 1024 -> 3072 7.6 -> 6.6 us, 4096 -> 1024 16.8 -> 14.7, 64 tokens
-// 4096 -> 4096 18.1 -> 14.9.  In the pair kernels the same made larger problems 1-3 % slower.
+// 4096 -> 4096 18.1 -> 14.9.
 template <bool XF> constexpr int kMetaBatchOf = XF ? 4 : 8;
+// Metadata that has to be converted goes piece by piece all the same where the four copies of the conversion cost more (fetching
+// their code) than the loads' latency: rows of at most this many words (reductions of at most 768), and the metadata of an output
+// tile that is not the CTA's first.  Over the shapes with 256, 640 and 768 reduction elements 4, 3 and 2 % less than in batches (3000
+// tokens 256 -> 256 1:4 / 8 bit 6.5 -> 5.9 us); from 1024 on batches are the faster ones, by up to 9 %.  32768 tokens 1152 -> 640 1:4 / 8
+// bit, where a few CTAs change their output tile, 44.2 -> 41.6.
+constexpr int kMetaShort = 24;
 
 // Where the weight operand comes from: TMA (already in tensor-core form), built per k-block into the
 // stage ring, or built once per output tile into a resident region (reduction length <= kResidentKB k-blocks).
@@ -461,43 +467,44 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         uint32_t n_stores = 0;
         bool ok = true;
 
-        constexpr int kMetaBatch = kMetaBatchOf<XF>;
-        // Metadata of this lane's weight row, kMetaBatch 16-byte pieces (one 128-wide k-block each) at a time: all loads of
-        // a batch are in flight together.
-        uint4 mw[kMetaBatch];
-        auto fetch_meta = [&](int out_tile, int c0) {
+        // Index metadata of this lane's weight row for the whole reduction; rows past the end get a valid "positions 0,1" pattern,
+        // their products are discarded.  The form with resident built weights always goes piece by piece, and fetches the channel
+        // constants behind the wait for the accumulator: with batches, and the constants in front of it, int8 and bfloat16 outputs took
+        // 2 % more over all shapes and up to 11 % (32768 tokens 256 -> 256 1:4 / 8 bit bfloat16 13.5 us against 12.1, 12000 tokens
+        // 512 -> 2048 2:4 / 4 bit 26.1 against 24.2).
+        auto load_meta = [&](int out_tile, bool first) {
             const int n = out_tile * kBM + row;
-            const uint8_t* src = reinterpret_cast<const uint8_t*>(p.meta) + (size_t)(n < p.out ? n : 0) * (XF ? p.mrow_bytes : 4 * p.mrow_words);
-#pragma unroll
-            for (int j = 0; j < kMetaBatch; ++j) {
-                const int c = c0 + 4 * j;
-                mw[j] = make_uint4(0u, 0u, 0u, 0u);
-                if (n < p.out && c < p.mrow_words) {
-                    if constexpr (XF) mw[j] = xf::meta_raw(p.pat, src + (size_t)(c >> 2) * xf::meta_bytes(p.pat));
-                    else mw[j] = xf::ldg16(src + (size_t)c * 4);
-                }
-            }
-        };
-        auto put_meta = [&](int out_tile, int c0) {
-            const bool row_ok = out_tile * kBM + row < p.out;
-#pragma unroll
-            for (int j = 0; j < kMetaBatch; ++j) {
-                const int c = c0 + 4 * j;
-                if (c < p.mrow_words) {
-                    // rows past the end get a valid "positions 0,1" pattern; their products are discarded
-                    uint4 w = make_uint4(0x44444444u, 0x44444444u, 0x44444444u, 0x44444444u);
-                    if (row_ok) {
-                        if constexpr (XF) w = xf::hw_meta(p.pat, mw[j], lut);
-                        else w = mw[j];
-                    }
+            const bool row_ok = n < p.out;
+            const uint4 idle = make_uint4(0x44444444u, 0x44444444u, 0x44444444u, 0x44444444u);
+            const uint8_t* src = reinterpret_cast<const uint8_t*>(p.meta) + (size_t)(row_ok ? n : 0) * (XF ? p.mrow_bytes : 4 * p.mrow_words);
+            const int piece = XF ? xf::meta_bytes(p.pat) : 16;  // stored bytes of a k-block
+            if (RES || (XF && (!first || p.mrow_words <= kMetaShort))) {
+                for (int c = 0; c < p.mrow_words; c += 4) {
+                    uint4 w = idle;
+                    if (row_ok) w = xf::hw_meta(p.pat, xf::meta_raw(p.pat, src + (size_t)(c >> 2) * piece), lut);
                     ptx::tmem_st_32x4(lane_taddr + Cfg::META_COL + c, w.x, w.y, w.z, w.w);
                 }
-            }
-        };
-        auto load_meta = [&](int out_tile, bool first_batch_fetched) {
-            for (int c0 = 0; c0 < p.mrow_words; c0 += 4 * kMetaBatch) {
-                if (c0 > 0 || !first_batch_fetched) fetch_meta(out_tile, c0);
-                put_meta(out_tile, c0);
+            } else {
+                constexpr int kMetaBatch = kMetaBatchOf<XF>;
+                for (int c0 = 0; c0 < p.mrow_words; c0 += 4 * kMetaBatch) {  // all loads of a batch are in flight together
+                    uint4 mw[kMetaBatch];
+#pragma unroll
+                    for (int j = 0; j < kMetaBatch; ++j) {
+                        mw[j] = idle;
+                        if (row_ok && c0 + 4 * j < p.mrow_words) {
+                            if constexpr (XF) mw[j] = xf::meta_raw(p.pat, src + (size_t)((c0 >> 2) + j) * piece);
+                            else mw[j] = xf::ldg16(src + (size_t)((c0 >> 2) + j) * 16);
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < kMetaBatch; ++j) {
+                        if (c0 + 4 * j < p.mrow_words) {
+                            uint4 w = mw[j];
+                            if constexpr (XF) w = row_ok ? xf::hw_meta(p.pat, mw[j], lut) : idle;
+                            ptx::tmem_st_32x4(lane_taddr + Cfg::META_COL + c0 + 4 * j, w.x, w.y, w.z, w.w);
+                        }
+                    }
+                }
             }
             ptx::tmem_st_wait();
             ptx::tc_fence_before();
@@ -513,23 +520,28 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         for (int i = 0; i < tile_count && ok; ++i) {
             const int tile = tile_begin + i, out_tile = tile / p.n_tok_tiles, buf = i & 1;
             const int n0 = out_tile * kBM, n = n0 + row, t0 = (tile % p.n_tok_tiles) * BN;
-            if (SPARSE && i == 0 && half == 0) load_meta(out_tile, false);
-            // what the tile needs from global memory is fetched before the wait for its accumulator
-            const bool n_ok = n < p.out;
-            if (EPI != EPI_ACC && out_tile != scaled_out_tile) {  // channel constants: fetched once per output tile
+            if (SPARSE && i == 0 && half == 0) load_meta(out_tile, true);
+            if (!(RES && SPARSE) && EPI != EPI_ACC && out_tile != scaled_out_tile) {  // channel constants: once per output tile
                 scaled_out_tile = out_tile;
-                c_n = n_ok ? __fmul_rn(sx, p.sw[n]) : 0.0f;
-                b_n = n_ok && p.bias ? p.bias[n] : 0.0f;
+                c_n = n < p.out ? __fmul_rn(sx, p.sw[n]) : 0.0f;
+                b_n = n < p.out && p.bias ? p.bias[n] : 0.0f;
             }
-            const int next_out_tile = i + 1 < tile_count ? (tile + 1) / p.n_tok_tiles : out_tile;
-            const bool new_meta = SPARSE && half == 0 && next_out_tile != out_tile;
             bool got = ptx::mbar_wait_bounded(acc_full_bar(buf), (i >> 1) & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
             if (!ok && lane == 0) raise_timeout();
             if constexpr (kNarrow<EPI>) ok = ptx::named_bar_and(kNarrowAgree + half, 128, ok);  // the group stops together
             if (!ok) break;
             ptx::tc_fence_after();
-            if (new_meta) load_meta(next_out_tile, false);  // MMAs of this output tile are done
+            if (SPARSE && half == 0 && i + 1 < tile_count) {
+                const int next_out_tile = (tile + 1) / p.n_tok_tiles;
+                if (next_out_tile != out_tile) load_meta(next_out_tile, false);  // MMAs of this output tile are done
+            }
+            const bool n_ok = n < p.out;
+            if (RES && SPARSE && EPI != EPI_ACC && out_tile != scaled_out_tile) {  // (see load_meta)
+                scaled_out_tile = out_tile;
+                c_n = n_ok ? __fmul_rn(sx, p.sw[n]) : 0.0f;
+                b_n = n_ok && p.bias ? p.bias[n] : 0.0f;
+            }
             const int nact = min(CH, (p.tokens - t0 + 31) >> 5);  // chunks that hold tokens (warp-uniform)
             // Accumulator chunks are read one ahead of their conversion (two register buffers); the
             // transform kernels, short of registers with their extra warps, read each chunk when it is due.

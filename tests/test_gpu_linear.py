@@ -69,6 +69,21 @@ def test_metadata_batches(n, m, bits, K):
     _run(40, 64, K, 200, n, m, bits)
 
 
+@pytest.mark.parametrize("n,m,bits", [(2, 4, 4), (1, 4, 8), (2, 8, 4)])
+@pytest.mark.parametrize("K", [768, 1152])
+@pytest.mark.parametrize("resident", [True, False])
+def test_metadata_of_later_output_tiles(n, m, bits, K, resident):
+    # 189 tiles of 128 x 192 on 148 SMs: some CTAs change their output tile; rebuilt weights, per stage or kept resident
+    import paper_2206_15014_b200 as nm
+    nm.nm_debug_set_option("no_pair", 1)
+    nm.nm_debug_set_option("no_resident", 0 if resident else 1)
+    try:
+        _run(42, 12000, K, 384, n, m, bits)
+    finally:
+        nm.nm_debug_set_option("no_pair", 0)
+        nm.nm_debug_set_option("no_resident", 0)
+
+
 @pytest.mark.parametrize("n,m,bits", [(2, 4, 8), (2, 4, 4), (1, 4, 8), (4, 4, 8)])
 @pytest.mark.parametrize("T,K,out", [(29 * 192 - 5, 1152, 640), (29 * 192 + 1, 1152, 640), (29 * 192, 640, 640), (1900, 4096, 384)])
 def test_long_reduction_around_one_wave_of_tiles(n, m, bits, T, K, out):
