@@ -338,8 +338,8 @@ int nm_probe_tma_stream(const void *W, int w_rows, int w_row_bytes, const void *
 
 /*
  * Measurement and test aid (the paper has no counterpart): overrides the kernel nm_int_linear and its variants
- * (and, with "pack_form", the projection entry points) pick, process-wide, for every later call (not thread-safe against calls in flight on other host threads).
- * All options are 0 by default = the library's own choice.  Names: "no_pdl" (launch without the programmatic-
+ * (and, with "pack_form" and "no_pdl", the other entry points) pick, process-wide, for every later call (not thread-safe against calls in flight on other host threads).
+ * All options are 0 by default = the library's own choice.  Names: "no_pdl" (no launch, of any entry point, with the programmatic-
  * dependent-launch attribute), "no_pair" (one-CTA kernels only), "no_resident" (always stream the weights),
  * "no_wide" (never the 512-channel pair kernel), "wide_any" (the 512-channel pair kernel whenever the shape
  * allows it, however few tiles there are), "wide_bn" (its token-tile width, 224 or 192), "band" (band size of the streamed pair kernel's tile order),

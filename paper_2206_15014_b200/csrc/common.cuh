@@ -32,6 +32,8 @@ inline size_t meta_row_words(int in, int n, int m) {
 
 // Form of the projection kernel forced by nm_debug_set_option("pack_form") (0 = automatic).
 extern int g_pack_form;
+// nm_debug_set_option("no_pdl"): no launch of the library carries the programmatic-dependent-launch attribute.
+extern int g_no_pdl;
 
 #ifdef NM_TEST_HOOKS
 // Timeout test only: the unit (per block) whose copies warp 0 of block 0 of the staged projection kernel leaves unissued.

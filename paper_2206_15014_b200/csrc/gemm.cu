@@ -1215,7 +1215,6 @@ namespace nm {
 // ---------------------------------------------------------------------------------------------
 // Kernel-choice overrides for measurements and tests (nm_debug_set_option); all zero = the library's own choice.
 struct DebugOptions {
-    int no_pdl;       // launch without the programmatic-dependent-launch attribute
     int no_pair;      // one-CTA kernels only
     int no_resident;  // always stream the weights through the stage ring
     int no_wide;      // never the 512-channel pair kernel
@@ -1227,6 +1226,7 @@ struct DebugOptions {
     int skip_stage;   // NM_TEST_HOOKS builds: 1 + the pipeline stage CTA 0's producer leaves out (0 = none)
 };
 static DebugOptions g_opt = {};
+int g_no_pdl = 0;
 
 // Trace buffer of NM_TRACE builds (device, kTraceStages + kTraceTiles rows of 8 u64), handed to every GEMM launch.
 static unsigned long long* g_trace_buffer = nullptr;
@@ -1312,7 +1312,7 @@ static int launch_gemm(const LinearArgs& a) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = g_opt.no_pdl ? 0 : 1;
+    cfg.attrs = attr; cfg.numAttrs = g_no_pdl ? 0 : 1;
     NM_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, tw, tx, ty, p));
     return NM_OK;
 }
@@ -1387,7 +1387,7 @@ static int launch_gemm_pair(const LinearArgs& a) {
     // (griddepcontrol.wait) before its first access to global memory
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = g_opt.no_pdl ? 1 : 2;
+    cfg.attrs = attr; cfg.numAttrs = g_no_pdl ? 1 : 2;
     NM_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, tw, tx, ty, p, sched));
     return NM_OK;
 }
@@ -1435,7 +1435,7 @@ static int launch_gemm_wide(const LinearArgs& a) {
     attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = g_opt.no_pdl ? 1 : 2;
+    cfg.attrs = attr; cfg.numAttrs = g_no_pdl ? 1 : 2;
     NM_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, tw, tx, ty, p, sched));
     return NM_OK;
 }
@@ -1476,7 +1476,7 @@ static int launch_gemm_xres(const LinearArgs& a) {
     attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = g_opt.no_pdl ? 1 : 2;
+    cfg.attrs = attr; cfg.numAttrs = g_no_pdl ? 1 : 2;
     NM_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, tw, tx, ty, p));
     return NM_OK;
 }
@@ -1684,7 +1684,7 @@ int nm_pair_tile_plan(int n_tok_tiles, int n_out_tiles, int pairs, int resident,
 int nm_debug_set_option(const char* name, int value) {
     if (!name) return NM_ERR_NULL;
     struct { const char* name; int* slot; } table[] = {
-        {"no_pdl", &nm::g_opt.no_pdl}, {"no_pair", &nm::g_opt.no_pair}, {"no_resident", &nm::g_opt.no_resident},
+        {"no_pdl", &nm::g_no_pdl}, {"no_pair", &nm::g_opt.no_pair}, {"no_resident", &nm::g_opt.no_resident},
         {"no_wide", &nm::g_opt.no_wide}, {"wide_any", &nm::g_opt.wide_any}, {"wide_bn", &nm::g_opt.wide_bn},
         {"one_bn", &nm::g_opt.one_bn}, {"xres", &nm::g_opt.xres}, {"band", &nm::g_opt.band}, {"pack_form", &nm::g_pack_form}};
     for (auto& e : table)

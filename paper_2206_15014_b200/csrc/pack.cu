@@ -1475,7 +1475,7 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
         for (size_t g = 0; g < keys.size(); ++g) fits = fits && groups[g].size() <= (size_t)kInlineJobs;
         if (fits) {
             for (size_t g = 0; g < keys.size(); ++g) {
-                if (g == 1) separate = separate_launches(table, nullptr, group_first);
+                if (g == 1) separate = !g_no_pdl && separate_launches(table, nullptr, group_first);
                 PackJobInline inl{};
                 for (size_t i = 0; i < groups[g].size(); ++i) inl.j[i] = table[group_first[g] + i];
                 int rc = nm::launch_table(nm::pick_kernel<DENSE_OUT>(keys[g].n, keys[g].m, keys[g].bits, keys[g].warps, group_blocks[g], keys[g].dual), nullptr,
@@ -1520,7 +1520,7 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
         const Key& k = keys[g];
         const int count = (int)groups[g].size();
         const DenseOutDev* dense_g = DENSE_OUT ? dense_dev + group_first[g] : nullptr;
-        if (g == 1) separate = separate_launches(table, DENSE_OUT ? dense_table.data() : nullptr, group_first);
+        if (g == 1) separate = !g_no_pdl && separate_launches(table, DENSE_OUT ? dense_table.data() : nullptr, group_first);
         const bool chained = g > 0 && separate && (grouped ? k.cluster && keys[g - 1].cluster
                                                              : dist_ncand == 0 || (k.warps <= kPackMinWarps && keys[g - 1].warps <= kPackMinWarps));
         int rc;

@@ -127,7 +127,7 @@ static cudaError_t launch_dependent(void (*kernel)(P...), int grid, cudaStream_t
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    cfg.attrs = attr; cfg.numAttrs = g_no_pdl ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 

@@ -108,7 +108,8 @@ def test_overlapping_launches_of_a_batch_end_before_what_follows():
     X = torch.randint(-127, 128, (64, 1024), dtype=torch.int8, device=DEV)
     desc = nm.make_packed(4096, 1024, 2, 4, 8, bufs[0][0], bufs[0][1])
     ys = []
-    for _ in range(3):
+    for no_pdl in (0, 0, 1):
+        nm.nm_debug_set_option("no_pdl", no_pdl)
         for b in bufs:
             b[0][: b[3]].fill_(0x11)
             b[2].fill_(-1.0)
@@ -120,6 +121,7 @@ def test_overlapping_launches_of_a_batch_end_before_what_follows():
         for c, r in zip(copies, refs):
             _same(c, r)
         ys.append(Y)
+        nm.nm_debug_set_option("no_pdl", 0)
     assert torch.equal(ys[0], ys[1]) and torch.equal(ys[0], ys[2]) and ys[0].any()
     D = oracle.unpack(refs[0][0], refs[0][1], 4096, 1024, 2, 4, 8)
     _, Y_ref = oracle.int_linear(X.cpu().numpy(), D, np.float32(0.01), refs[0][2], None)

@@ -91,3 +91,9 @@ def test_back_to_back_with_the_linear_layer():
     for _ in range(5):
         y, sx = chain(False)
         assert torch.equal(y, y_ref) and torch.equal(sx, sx_ref)
+    nm.nm_debug_set_option("no_pdl", 1)  # every launch an ordinary one
+    try:
+        y, sx = chain(False)
+    finally:
+        nm.nm_debug_set_option("no_pdl", 0)
+    assert torch.equal(y, y_ref) and torch.equal(sx, sx_ref)
