@@ -15,8 +15,9 @@ pytestmark = pytest.mark.gpu
 # int8 2:4 and dense (TMA weights, CTA pairs when large), and weights rebuilt in shared memory
 MODES = [(2, 4, 8), (4, 4, 8), (2, 4, 4), (1, 4, 8), (2, 8, 8), (4, 8, 8)]
 # (tokens, K, out): one tile; ragged, out % 16 != 0 (plain stores) ; out % 16 == 0 but ragged tokens;
-# many tiles with resident weights and output-tile changes; long reduction with streamed weights
-# the last one: resident weights on CTA pairs with rows that no TMA store can address (plain stores from sixteen warps)
+# many tiles of a short reduction (CTA pairs) with output-tile changes; long reduction with streamed weights
+# the last one: CTA pairs with rows that no TMA store can address (plain stores from sixteen warps)
+# (the pair kernels for short reductions one by one: test_gpu_xres.py)
 SHAPES = [(64, 128, 128), (100, 384, 200), (77, 256, 208), (4096 + 37, 512, 1280), (6000 + 3, 2048, 640), (7680 + 5, 512, 516)]
 
 
@@ -82,7 +83,7 @@ def test_int8_chain_of_two_layers():
 def test_accumulators_from_zero_to_the_largest(n, m, bits, T, K, out):
     """Constant rows of X against all-ones weights give every token its own accumulator value, from 0 up to the
     largest the operands allow (beyond 2^22 and 2^24 in magnitude for 8-bit codes, where int -> float rounds): fp32,
-    int8 and bfloat16 outputs bit for bit on the one-CTA, resident-weight pair and 512-channel pair kernels."""
+    int8 and bfloat16 outputs bit for bit on the one-CTA kernel, the pair kernels for short reductions and the 512-channel one."""
     from gpu_util import PackedOnDevice, gpu_int_linear, gpu_int_linear_q8, gpu_int_linear_bf16
     oracle.set_threads(oracle.max_threads())
     W = np.ones((out, K), np.float32)

@@ -1,10 +1,11 @@
-"""GPU parity of the projection kernel's three forms in blocks of four warps, each forced in turn.
+"""GPU parity of the projection kernel's two forms in blocks of four warps, each forced in turn, and at the sizes where
+the library changes from one to the other.
 
-The library picks the form from the launch (dense outputs and short launches: chunks staged in shared memory
-by bulk copies; long launches: chunks asked for ahead into L2; the one-unit-per-block form stays for
-measurements), so the other parity tests meet mostly one of them.  Here every form runs every pattern and
-code width on rows of one and four warps, ragged tails, a launch of many rounds per resident block, a batch
-through the device job table, and the ADMM step with dense outputs, bit for bit against the oracle.
+"direct" (one unit per block, loads straight into registers) exists for every pattern, code width and output.  "staged"
+(persistent, the next rows brought into shared memory by bulk copies) exists for 2:4 without dense outputs; the library takes it
+for launches with two operands and rows of a multiple of 1024 weights, of two to six rounds of the direct form's resident
+blocks.  Rows of one and four warps, ragged tails, a launch of many rounds per resident block, a batch through the device job
+table, and (direct) the ADMM step with dense outputs, bit for bit against the oracle.
 """
 import numpy as np
 import pytest
@@ -16,10 +17,10 @@ import workloads as wl
 pytestmark = pytest.mark.gpu
 
 PATTERNS = [(1, 4), (2, 4), (1, 8), (2, 8), (4, 8), (4, 4)]
-FORMS = {"direct": 1, "staged": 2, "ahead": 3}
+FORMS = {"direct": 1, "staged": 2}
 
 
-@pytest.fixture(params=sorted(FORMS))
+@pytest.fixture
 def form(request):
     import paper_2206_15014_b200 as nm
     nm.nm_debug_set_option("pack_form", FORMS[request.param])
@@ -38,7 +39,7 @@ def _check_pack(W, U, n, m, bits):
         assert np.array_equal(meta, meta_ref), "metadata differs"
 
 
-@pytest.mark.parametrize("n,m", PATTERNS)
+@pytest.mark.parametrize("form,n,m", [("direct", *p) for p in PATTERNS] + [("staged", 2, 4)], indirect=["form"])
 @pytest.mark.parametrize("bits", [8, 4])
 def test_forms_rows_and_ragged(form, n, m, bits):
     oracle.set_threads(oracle.max_threads())
@@ -52,7 +53,8 @@ def test_forms_rows_and_ragged(form, n, m, bits):
         _check_pack(wl.with_outliers(110 + seed, out, k), wl.tie_heavy(120 + seed, out, k, levels=1), n, m, bits)
 
 
-@pytest.mark.parametrize("n,m,bits", [(2, 4, 8), (4, 8, 4), (1, 8, 8)])
+@pytest.mark.parametrize("form,n,m,bits", [("staged", 2, 4, 8), ("direct", 2, 4, 8), ("direct", 4, 8, 4), ("direct", 1, 8, 8)],
+                         indirect=["form"])
 def test_forms_many_rounds(form, n, m, bits):
     """More units than resident blocks, several times over (9001 rows of 1024: 2251 units; 1500 rows of 3072: a row
     spans four warps, one of them past the row's end), with the last block's rows running out."""
@@ -62,6 +64,7 @@ def test_forms_many_rounds(form, n, m, bits):
         _check_pack(W, U, n, m, bits)
 
 
+@pytest.mark.parametrize("form", sorted(FORMS), indirect=True)
 def test_forms_batched_through_the_job_table(form):
     """Twelve matrices of mixed shapes in one launch (device job table): a block's consecutive units cross from one
     job into the next."""
@@ -121,8 +124,8 @@ def test_staged_units_of_several_warps_and_of_one_in_turn():
 
 
 @pytest.mark.parametrize("n,m,bits", [(2, 4, 8), (4, 8, 8), (1, 4, 4), (4, 4, 4)])
-def test_forms_admm_step(form, n, m, bits):
-    """Dense outputs (Z, U_next) besides the packed ones, 3000 rows: several rounds per resident block."""
+def test_forms_admm_step(n, m, bits):
+    """Dense outputs (Z, U_next) besides the packed ones (the direct form only)."""
     import paper_2206_15014_b200 as nm
     from gpu_util import DEV, to_dev
     oracle.set_threads(oracle.max_threads())
@@ -147,3 +150,41 @@ def test_forms_admm_step(form, n, m, bits):
         assert np.array_equal(values.cpu().numpy(), np.asarray(v_ref).reshape(-1))
         if n != m:
             assert np.array_equal(meta.cpu().numpy().view(np.uint32)[: mb // 4], np.asarray(meta_ref).reshape(-1))
+
+
+def _automatic(outs, k, with_u, bits=8):
+    """The jobs in one call with the library's own choice of form, every output against the oracle."""
+    import paper_2206_15014_b200 as nm
+    from gpu_util import DEV, to_dev
+    oracle.set_threads(oracle.max_threads())
+    jobs, refs = [], []
+    for i, (out, has_u) in enumerate(zip(outs, with_u)):
+        W, U = wl.pack_sweep_matrix(41, i, out, k)
+        U = U if has_u else None
+        vb, mb = nm.nm_packed_sizes(out, k, 2, 4, bits)
+        jobs.append((to_dev(W), None if U is None else to_dev(U), 2, 4, bits, torch.zeros(vb, dtype=torch.uint8, device=DEV),
+                     torch.zeros(mb // 4, dtype=torch.int32, device=DEV), torch.zeros(out, dtype=torch.float32, device=DEV)))
+        refs.append(oracle.project_pack(W, U, 2, 4, bits))
+    ws_bytes = nm.nm_pack_workspace_bytes(len(jobs))
+    ws = torch.empty(ws_bytes, dtype=torch.uint8, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    nm.nm_project_pack_batched(nm.make_pack_jobs(jobs), len(jobs), ws, ws_bytes, status)
+    assert nm.nm_poll_status(status) == 0
+    for job, (v_ref, m_ref, s_ref) in zip(jobs, refs):
+        assert np.array_equal(job[7].cpu().numpy(), s_ref)
+        assert np.array_equal(job[5].cpu().numpy().reshape(v_ref.shape), v_ref)
+        assert np.array_equal(job[6].cpu().numpy().view(np.uint32).reshape(m_ref.shape), m_ref)
+
+
+@pytest.mark.parametrize("rounds,beyond", [(2, 0), (2, 1), (6, 0), (6, 1)])
+def test_both_sides_of_the_librarys_choice(rounds, beyond):
+    """Up to two rounds of eight resident blocks a multiprocessor direct, beyond staged; up to six staged, beyond direct."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    _automatic([4 * (rounds * 8 * sms + beyond)], 1024, [True])  # four rows a block
+
+
+@pytest.mark.parametrize("with_u", [[True, True, True], [True, False, True]])
+def test_one_operand_in_a_batch_of_two_operand_jobs(with_u):
+    """Three rounds of blocks: staged when every job has a U, direct when one has none."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    _automatic([4 * 8 * sms] * 3, 1024, with_u, bits=4)

@@ -1,7 +1,8 @@
-"""GPU parity of the CTA-pair kernel with resident activations (2:4 and dense int8 weights, reductions of at most 1024) against the
-CPU oracle: accumulators, fp32, int8 and bfloat16 outputs, bit for bit.  The option "xres" sends every shape that the
-kernel takes to it, however few tiles there are: reductions that end inside a stage, one token, ragged token and output
-tiles, output rows that TMA cannot store, and runs of tiles that cross token tiles inside a pair."""
+"""GPU parity of the CTA-pair kernels for reductions of at most 1024 (2:4 and dense int8 weights) against the CPU oracle:
+accumulators, fp32, int8 and bfloat16 outputs, bit for bit.  The option "xres" sends every shape to the kernel with resident
+activations (1) or to the other pair kernel (2: resident 2:4 weights, streamed dense ones), however few tiles there are:
+reductions that end inside a stage, one token, ragged token and output tiles, output rows that TMA cannot store, and runs of
+tiles that cross token or output tiles inside a pair."""
 import numpy as np
 import pytest
 
@@ -11,10 +12,10 @@ import workloads as wl
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(autouse=True)
-def resident_activations():
+@pytest.fixture(autouse=True, params=[1, 2], ids=["resident_activations", "other_pair_kernel"])
+def kernel_choice(request):
     import paper_2206_15014_b200 as nm
-    nm.nm_debug_set_option("xres", 1)
+    nm.nm_debug_set_option("xres", request.param)
     yield
     nm.nm_debug_set_option("xres", 0)
 
