@@ -84,8 +84,6 @@ __device__ __forceinline__ float max_abs_nan(float a, float b, float m) {
     return r;
 }
 
-// Bit mask of the positions kept in one group: position i is kept iff fewer than N others beat it,
-// where j beats i when |v_j| > |v_i|, or |v_j| == |v_i| and j < i.
 // n = 1, and 2 of 8: the kept values and their positions straight from one or two passes of
 // "largest magnitude, first one on equality" (strict >), positions ascending.
 template <int N, int M>
@@ -133,33 +131,10 @@ __device__ __forceinline__ unsigned select_2_of_4(const float* v, float* sel) {
     return both01 ? 0x4u : (both23 ? 0xEu : mixed);
 }
 
+// Bit mask of the positions kept in one group (2 of 4 in the search, 4 of 8): position i is kept iff fewer than N others beat it,
+// where j beats i when |v_j| > |v_i|, or |v_j| == |v_i| and j < i.
 template <int N, int M>
 __device__ __forceinline__ unsigned keep_mask(const float* a) {
-    if constexpr (N == 1 || (N == 2 && M == 8)) {  // (the pack kernel's 2:4 has its own tournament, select_2_of_4)
-        // One or two passes of "largest magnitude, first one on equality" (a strict > keeps the lower
-        // index): the same support as the rank rule, with 7 + 7 compares instead of 28 for m = 8.
-        float best = a[0];
-        unsigned bi = 0;
-#pragma unroll
-        for (int j = 1; j < M; ++j) {
-            const bool gt = a[j] > best;
-            best = gt ? a[j] : best;
-            bi = gt ? (unsigned)j : bi;
-        }
-        unsigned mask = 1u << bi;
-        if constexpr (N == 2) {
-            float best2 = -1.0f;  // magnitudes are >= 0
-            unsigned bj = 0;
-#pragma unroll
-            for (int j = 0; j < M; ++j) {
-                const bool gt = (a[j] > best2) && ((unsigned)j != bi);
-                best2 = gt ? a[j] : best2;
-                bj = gt ? (unsigned)j : bj;
-            }
-            mask |= 1u << bj;
-        }
-        return mask;
-    }
     if constexpr (N == 4 && M == 8) {
         // Four of eight: the fourth largest magnitude T from a selection network (both halves sorted with five
         // compare-exchanges each, then the four maxima of a bitonic half-cleaner hold the four largest and their
@@ -911,15 +886,11 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
             // the next unit's part goes into the other buffer while this one is worked on
             const unsigned next = unit + gridDim.x;
             PackJobDev njob = job;
-            int nindex = index;
             UnitPos nup{};
             if (next < nunits) {
-                if (next - job.unit_begin >= units_of(job, warps)) njob = find_job(jobs, njobs, inl, next, nindex);
+                if (next - job.unit_begin >= units_of(job, warps)) njob = find_job(jobs, njobs, inl, next, index);
                 nup = unit_pos(njob, next, w, warps);
                 issue(njob, nup, buf ^ 1, it + 1);
-            }
-            if constexpr (DENSE_OUT) {
-                if (jobs) { Zout = dense_jobs[index].Z; Unext = dense_jobs[index].U_next; }
             }
             if (up.elems != 0) {
                 if (!ptx::mbar_wait_bounded(bar0 + 8u * buf, (phase >> buf) & 1u, abort_flag, kPackWaitLimit)) {
@@ -934,7 +905,7 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
             pack_finish<N, M, BITS, DENSE_OUT>(job, up, lane, w, v, red + (spanning & 1u) * warps, pos48, scratch, status, Zout, Unext,
                                               wide_rows(job, Zout, Unext), group_mode, group_rows);
             spanning += job.wpr_log2 != 0 ? 1u : 0u;
-            job = njob; index = nindex; up = nup;
+            job = njob; up = nup;
         }
         // after an expired wait a copy may still be on its way into this block's shared memory
         if (*abort_flag) ptx::wait_clocks(1 << 17);
@@ -1308,7 +1279,7 @@ template <int N, int M>
 static DistFn pick_dist_bits(int bits, int warps) {
     if (warps <= kPackMinWarps)
         return bits == 8 ? (DistFn)dist_scale_kernel<N, M, 8, 128> : (DistFn)dist_scale_kernel<N, M, 4, 128>;
-    if (warps <= 16)  // the kept values as fp32 and fp64 need up to ~128 registers
+    if (warps <= 16)  // the row's values and the kept ones beside them need up to ~128 registers
         return bits == 8 ? (DistFn)dist_scale_kernel<N, M, 8, 512> : (DistFn)dist_scale_kernel<N, M, 4, 512>;
     return bits == 8 ? (DistFn)dist_scale_kernel<N, M, 8, 1024> : (DistFn)dist_scale_kernel<N, M, 4, 1024>;
 }
@@ -1331,8 +1302,8 @@ static int launch_dist(DistFn fn, const PackJobDev* jobs_dev, int njobs, const P
     return NM_OK;
 }
 
-// Search and projection in one kernel (blocks of four warps): the search keeps the row in shared memory, so W and U are read
-// once: 85 M weights at 2:4 / 4 bit 533 us against 405 + 156 us for the search followed by the projection.
+// Search and projection in one kernel (blocks of four warps): the row stays in registers from the one to the other, so W and U are
+// read once: 85 M weights at 2:4 / 4 bit 533 us against 405 + 156 us for the search followed by the projection.
 template <int N, int M, bool DENSE_OUT>
 static PackFn pick_dist_pack_bits(int bits) {
     return bits == 8 ? PackFn{(PackFnPtr)pack_kernel<N, M, 8, 128, DENSE_OUT, kDirect, true>, kDirect, true}
