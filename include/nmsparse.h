@@ -90,10 +90,10 @@ int nm_packed_sizes(int out, int in, int n, int m, int bits, size_t *values_byte
  * Accepted: (n, m) in {1:4, 2:4, 1:8, 2:8, 4:8} or n == m; bits in {4, 8}; in <= 32768.
  * W, U, values 16-byte aligned, meta and scales 4-byte aligned.
  * Sets NM_STATUS_NONFINITE in *status (nullable) when W + U holds NaN/Inf; outputs of such rows are
- * unspecified.  One pass over W and U; outputs are written once.  Rows of at most 4096 values reach the
- * kernel through bulk copies whose arrival a warp awaits for about a second at most: NM_STATUS_TIMEOUT in
- * *status when such a wait expired (the outputs are then void); the same holds for every entry point below
- * that projects.
+ * unspecified.  One pass over W and U; outputs are written once.  2:4 with both operands and rows of 1024,
+ * 2048, 3072 or 4096 values may reach the kernel through bulk copies whose arrival a warp awaits for about a
+ * second at most: NM_STATUS_TIMEOUT in *status when such a wait expired (the outputs are then void); the same
+ * holds for every entry point below that projects without dense outputs.
  */
 int nm_project_pack(const float *W, const float *U, int out, int in, int n, int m, int bits,
                     void *values, void *meta, float *scales, uint32_t *status, void *stream);
@@ -121,9 +121,11 @@ int nm_admm_project(const float *W, const float *U, int out, int in, int n, int 
  * r / group_rows share the ADMM-Max scale max |W + U| over those rows / (2^(bits-1) - 1); group_rows
  * <= 0 means one scale for the whole matrix; the last group may be short.  scales[r] (required: it
  * is also the scratch of the group maxima) receives the scale of row r's group, so that it can be
- * handed to nm_int_linear unchanged.  Otherwise as nm_project_pack / nm_admm_project.  Two passes
- * over W and U (the maxima, then the projection); for matrices that fit in L2 the second pass is
- * served from there.
+ * handed to nm_int_linear unchanged.  Otherwise as nm_project_pack / nm_admm_project.  One pass over W
+ * and U where a cluster of at most eight blocks holds a group: rows of at most 4096 values, the warps of a group
+ * (one per row, two beyond 1024 values, four beyond 2048) 4 to 128 and divisible into blocks of four to sixteen.
+ * Otherwise two passes (the maxima, then the projection), for matrices that fit in L2 the second served from
+ * there.
  */
 int nm_project_pack_grouped(const float *W, const float *U, int out, int in, int n, int m, int bits,
                             int group_rows, void *values, void *meta, float *scales,
@@ -132,8 +134,8 @@ int nm_admm_project_grouped(const float *W, const float *U, int out, int in, int
                             int group_rows, float *Z, float *U_next, void *values, void *meta,
                             float *scales, uint32_t *status, void *stream);
 /* nm_project_pack_grouped for many matrices (jobs, ws as for nm_project_pack_batched; one group_rows for all):
- * per group of jobs that share (n, m, bits) and block size one launch folds the row maxima, one
- * finishes the scales and one projects and packs. */
+ * one launch for the jobs that share (n, m, bits) and warps per row where a cluster holds a group, otherwise four for
+ * those that share (n, m, bits) and block size (clear, fold the row maxima, finish the scales, project and pack). */
 int nm_project_pack_grouped_batched(const nm_pack_job_t *jobs, int njobs, int group_rows, void *ws,
                                     size_t ws_bytes, uint32_t *status, void *stream);
 
@@ -176,11 +178,13 @@ int nm_admm_project_grouped_batched(const nm_admm_job_t *jobs, int njobs, int gr
  *   nm_project_pack_dist  the search, then nm_project_pack with that scale (codes beyond the
  *                         shrunken range clamp to -2^(bits-1) / 2^(bits-1)-1 as Eq. 5 says).
  *   nm_admm_project_dist  the search, then nm_admm_project with that scale; `scales` is required.
- *   nm_project_pack_dist_batched  many matrices (jobs, ws as for nm_project_pack_batched): per
- *                         group of jobs that share (n, m, bits) and block size one launch searches
- *                         and one projects and packs.
- * Two passes over W and U (the second is served from L2 for matrices that fit there).  The search
- * is bound by arithmetic, not by memory.  Pointers, shapes, errors and the NM_STATUS_NONFINITE bit
+ *   nm_project_pack_dist_batched  many matrices (jobs, ws as for nm_project_pack_batched): one
+ *                         launch (rows of more than 4096 values: two) per group of jobs that share
+ *                         (n, m, bits) and block size.
+ * Rows of at most 4096 values are searched and projected in one kernel and one pass over W and U; longer
+ * ones in two (the second is served from L2 for matrices that fit there).  The search is bound by
+ * arithmetic, not by memory: all candidates in single precision first, those that its error bound leaves
+ * in double.  Pointers, shapes, errors and the NM_STATUS_NONFINITE bit
  * as for nm_project_pack; ncand out of range returns NM_ERR_SHAPE.  Which of two candidates whose
  * distances agree to the last few bits of a double wins depends on the order of the summation.
  */

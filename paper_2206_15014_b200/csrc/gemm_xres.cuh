@@ -9,11 +9,12 @@
 // The index metadata changes with every tile: four metadata warps (one per TMEM lane quarter, both CTAs) keep a ring of
 // four buffers of 32 TMEM columns filled, one tile's reduction each.  A token tile's slices are replaced one by one as the
 // last output tile's MMAs are done with them.
-// What bounds it: with fp32 outputs the stores (as in nm_gemm_pair_kernel); with narrow ones operand reads from shared memory
-// together with the epilogue's accesses to it.  Without any epilogue a 2:4 stage (four MMAs, 384 clocks at the tensor
-// rate) takes 870 clocks here and in nm_gemm_pair_kernel; two MMAs of half the width instead, which read the weights
-// twice, add 230 clocks per 16 KB, alternating accumulators change nothing, and weights in 64-byte rows are slower (16384 tokens
-// 1024 -> 4096 64.6 / 62.0 us).
+// What bounds it: with fp32 and int8 outputs the epilogue (stores; conversion): 2-3 k of a tile's 5.5-7 k clocks go by waiting for
+// an accumulator.  With bfloat16 the stages: about 1.1 k clocks each, 800 inside a tile with the other outputs, evenly over the
+// k-blocks, for 384 of MMAs at the tensor rate and 448 of shared memory (16 KB written, 40 KB read, counted, at 128 B/clk); 870 without any
+// epilogue, here and in nm_gemm_pair_kernel alike.  What makes the difference is not known: two MMAs of half the width instead, which
+// read the weights twice, add 230 clocks per 16 KB, alternating accumulators change nothing, and weights in 64-byte rows are
+// slower (16384 tokens 1024 -> 4096 64.6 / 62.0 us).
 #pragma once
 
 namespace nm {
