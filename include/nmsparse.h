@@ -90,9 +90,9 @@ int nm_packed_sizes(int out, int in, int n, int m, int bits, size_t *values_byte
  * Accepted: (n, m) in {1:4, 2:4, 1:8, 2:8, 4:8} or n == m; bits in {4, 8}; in <= 32768.
  * W, U, values 16-byte aligned, meta and scales 4-byte aligned.
  * Sets NM_STATUS_NONFINITE in *status (nullable) when W + U holds NaN/Inf; outputs of such rows are
- * unspecified.  One pass over W and U; outputs are written once.  2:4 with both operands and rows of 1024,
- * 2048, 3072 or 4096 values may reach the kernel through bulk copies whose arrival a warp awaits for about a
- * second at most: NM_STATUS_TIMEOUT in *status when such a wait expired (the outputs are then void); the same
+ * unspecified.  One pass over W and U; outputs are written once.  With both operands, n <= 2 and rows of
+ * 1024, 2048, 3072 or 4096 values they may reach the kernel through bulk copies whose arrival a warp awaits for
+ * about a second at most: NM_STATUS_TIMEOUT in *status when such a wait expired (the outputs are then void); the same
  * holds for every entry point below that projects without dense outputs.
  */
 int nm_project_pack(const float *W, const float *U, int out, int in, int n, int m, int bits,
@@ -350,7 +350,7 @@ int nm_probe_tma_stream(const void *W, int w_rows, int w_row_bytes, const void *
  * "one_bn" (token-tile width of the one-CTA kernel: 192, 128, 96, 64 or 32 where it exists), "xres" (the pair kernel with resident
  * activations: 1 = wherever a pair kernel with a reduction of at most 1024 runs, 2 = never),
  * "pack_form" (form of the projection kernel in blocks of four warps: 2 = persistent with the next rows staged in shared
- * memory by bulk copies, where that form exists: 2:4 without dense outputs; 1 or 3 = one unit per block).
+ * memory by bulk copies, where that form exists: 1:4, 2:4, 1:8 and 2:8 without dense outputs; 1 or 3 = one unit per block).
  * Results never depend on them.  Returns NM_ERR_UNSUPPORTED for an unknown name.  A library built with
  * -DNM_TEST_HOOKS (build.py --variant shortwait: device-side waits limited to about a millisecond) also takes
  * "skip_stage" = 1 + the pipeline stage that CTA 0's producer leaves unissued (0 = none): the bounded waits then

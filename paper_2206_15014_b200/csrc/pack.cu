@@ -800,12 +800,15 @@ constexpr int kStagedBlocksPerSm = 3;
 template <int N, int M, bool DENSE_OUT, bool DIST>
 constexpr int kDirectBlocksPerSm = DIST ? (32 / M * N <= 8 ? 6 : 4) : DENSE_OUT ? 6 : 8;
 
-template <int N, int M, int BITS, int MAXT, bool DENSE_OUT = false, int PIPE = kDirect, bool DIST = false>
-__global__ void __launch_bounds__(MAXT, PIPE != kDirect ? kStagedBlocksPerSm : (MAXT == 128 ? kDirectBlocksPerSm<N, M, DENSE_OUT, DIST> : 1))
+constexpr int kFewBlocksPerSm = 5;  // the plain projection of two operands where no SM gets more blocks (see pick_bits)
+
+template <int N, int M, int BITS, int MAXT, bool DENSE_OUT = false, int PIPE = kDirect, bool DIST = false,
+          int PER_SM = kDirectBlocksPerSm<N, M, DENSE_OUT, DIST>>
+__global__ void __launch_bounds__(MAXT, PIPE != kDirect ? kStagedBlocksPerSm : (MAXT == 128 ? PER_SM : 1))
 pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constant__ PackJobInline inl, uint32_t* status,
             float* __restrict__ Zout, float* __restrict__ Unext, const DenseOutDev* __restrict__ dense_jobs,
             int group_mode, int group_rows, unsigned nunits, bool chained) {
-    static_assert(PIPE == kDirect || (MAXT == 128 && N == 2 && M == 4 && !DENSE_OUT && !DIST), "see staged_form");
+    static_assert(PIPE == kDirect || (MAXT == 128 && N <= 2 && !DENSE_OUT && !DIST), "see staged_form");
     // staged: [warps][2 buffers][W, U][1024] floats.  Then (DIST) [warps][32] doubles, [2][warps] floats for the row maximum, (4:8) the
     // position table and [warps][8][32] floats, (staged) [warps][2] mbarriers and the abort flag.
     extern __shared__ float4 tile[];
@@ -1084,29 +1087,50 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1) dist_scale_kernel(c
 using PackFnPtr = void (*)(const PackJobDev*, int, const PackJobInline, uint32_t*, float*, float*, const DenseOutDev*, int, int, unsigned, bool);
 struct PackFn { PackFnPtr fn; int form; bool dist = false; };  // kernel, its form (kDirect, kStaged2), with the scale search
 
-// nm_debug_set_option("pack_form"): 0 = automatic, 2 = kStaged2 wherever it exists (2:4, blocks of four warps, no dense
-// outputs), anything else = kDirect.
+// nm_debug_set_option("pack_form"): 0 = automatic, 2 = kStaged2 wherever it exists (blocks of four warps, 1:4, 2:4, 1:8 and 2:8, no
+// dense outputs), anything else = kDirect.
 int g_pack_form = 0;
 
-// Whether a launch of `blocks` blocks of four warps takes the staged form.  2:4 with two operands, two to six rounds of the
-// blocks that kDirect keeps resident, in rows that fill the warps' buffers: blocks that start together otherwise alternate
-// between loading and arithmetic (staged / direct: 12.6 M weights in rows of 1024 and 4096 23.2 / 25.4 us, 25 M 39.6 / 44.0; 38 M
-// 61.5 / 62.0).  Everywhere else kDirect is as fast or faster (rows of 768 and 3072, 14 M weights 27.2 / 27.2; of 384 and
-// 1536, 11 M 37.3 / 27.4; one operand, 25 M weights 37.3 / 25.2; dense outputs on the 24-layer sweep 876 / 741; other
-// patterns 3-45 % faster).  `dual`: every matrix of the launch has both operands and rows of a multiple of 1024 weights.
-static bool staged_form(bool dual, unsigned blocks) {
-    const unsigned resident = (unsigned)sm_count() * 8u;
-    return dual && blocks > 2u * resident && blocks <= 6u * resident;
+// What the matrices of a launch have in common: some have no U; all have one; ... and rows of a multiple of 1024 weights; ... and rows of
+// 1024, 2048 or 4096, which fill the staged form's buffers.
+enum { kOneOperand = 0, kTwoOperands = 1, kThousands = 2, kFullBuffers = 3 };
+static int operands_of(const nm_pack_job_t& j) {
+    if (!j.U) return kOneOperand;
+    if (j.in % 1024) return kTwoOperands;
+    return (j.in & (j.in - 1)) == 0 && j.in <= 4096 ? kFullBuffers : kThousands;
 }
-static bool fills_buffers(const nm_pack_job_t& j) { return j.U != nullptr && j.in % 1024 == 0; }
+
+// Whether a launch of `blocks` blocks of four warps takes the staged form: two operands, more blocks than kDirect keeps resident, which
+// otherwise start together and alternate between loading and arithmetic.  Staged / direct in us, one matrix, W and U:
+//   rows of 1024, 2048, 4096, whatever their number: 6.3 M weights of 1:4 / 4 bit in rows of 4096 12.5 / 14.3, 2:8 / 8 bit 14.2 / 15.9, 2:4 / 8
+//   bit 13.4 / 15.2; 50 M 67 / 75, 79 / 84, 71 / 82; 50 M in rows of 1024 71 / 72, 75 / 82, 75 / 79;
+//   several matrices only up to six rounds, beyond them the direct form's blocks are out of step by themselves (24 layers of BERT-large
+//   457 / 414, 4 layers 92 / 86);
+//   2:4 in rows of 3072 up to six rounds (17 M 30.5 / 31.6); 2:8 there and more rounds lose (17 M 33.2 / 32.1, 2:4 50 M 81 / 78).
+// Up to one round the direct form is the faster one (4.2 M of 1:4 / 4 bit 10.3 / 9.8), as with one operand (25 M 37.3 / 25.2) and in rows
+// of other lengths (of 384 and 1536, 11 M 37.3 / 27.4).
+template <int N, int M>
+static bool staged_form(int operands, unsigned blocks, int njobs) {
+    const unsigned resident = (unsigned)sm_count() * 8u;
+    if (operands < kThousands || blocks <= resident) return false;
+    if (operands == kFullBuffers && njobs <= 1) return true;
+    return blocks <= 6u * resident && (operands == kFullBuffers || (N == 2 && M == 4));
+}
 
 template <int N, int M, bool DENSE_OUT>
-static PackFn pick_bits(int bits, int warps, unsigned blocks, bool dual) {
+static PackFn pick_bits(int bits, int warps, unsigned blocks, int operands, int njobs) {
     if (warps <= kPackMinWarps) {
-        if constexpr (N == 2 && M == 4 && !DENSE_OUT) {
-            if (g_pack_form == 2 || (g_pack_form == 0 && staged_form(dual, blocks)))
-                return bits == 8 ? PackFn{(PackFnPtr)pack_kernel<2, 4, 8, 128, false, kStaged2>, kStaged2}
-                                 : PackFn{(PackFnPtr)pack_kernel<2, 4, 4, 128, false, kStaged2>, kStaged2};
+        if constexpr (N <= 2 && !DENSE_OUT) {
+            if (g_pack_form == 2 || (g_pack_form == 0 && staged_form<N, M>(operands, blocks, njobs)))
+                return bits == 8 ? PackFn{(PackFnPtr)pack_kernel<N, M, 8, 128, false, kStaged2>, kStaged2}
+                                 : PackFn{(PackFnPtr)pack_kernel<N, M, 4, 128, false, kStaged2>, kStaged2};
+        }
+        // Two operands and at most kFewBlocksPerSm blocks an SM: the instance with the registers to have both operands' loads in flight
+        // together (1.0 M weights of 1:4 / 4 bit in rows of 4096 5.6 -> 5.1 us, 2.1 M of 2:4 / 8 bit in rows of 3072 6.9 -> 6.4).
+        if constexpr (!DENSE_OUT) {
+            if (operands != kOneOperand && blocks <= (unsigned)(sm_count() * kFewBlocksPerSm))
+                return bits == 8 ? PackFn{(PackFnPtr)pack_kernel<N, M, 8, 128, false, kDirect, false, kFewBlocksPerSm>, kDirect}
+                                 : PackFn{(PackFnPtr)pack_kernel<N, M, 4, 128, false, kDirect, false, kFewBlocksPerSm>, kDirect};
         }
         return bits == 8 ? PackFn{(PackFnPtr)pack_kernel<N, M, 8, 128, DENSE_OUT>, kDirect}
                          : PackFn{(PackFnPtr)pack_kernel<N, M, 4, 128, DENSE_OUT>, kDirect};
@@ -1119,12 +1143,12 @@ static PackFn pick_bits(int bits, int warps, unsigned blocks, bool dual) {
 }
 
 template <bool DENSE_OUT = false>
-static PackFn pick_kernel(int n, int m, int bits, int warps, unsigned blocks, bool dual) {
-    if (n == m) return pick_bits<4, 4, DENSE_OUT>(bits, warps, blocks, dual);
-    if (m == 4) return n == 1 ? pick_bits<1, 4, DENSE_OUT>(bits, warps, blocks, dual) : pick_bits<2, 4, DENSE_OUT>(bits, warps, blocks, dual);
-    if (n == 1) return pick_bits<1, 8, DENSE_OUT>(bits, warps, blocks, dual);
-    if (n == 2) return pick_bits<2, 8, DENSE_OUT>(bits, warps, blocks, dual);
-    return pick_bits<4, 8, DENSE_OUT>(bits, warps, blocks, dual);
+static PackFn pick_kernel(int n, int m, int bits, int warps, unsigned blocks, int operands, int njobs = 1) {
+    if (n == m) return pick_bits<4, 4, DENSE_OUT>(bits, warps, blocks, operands, njobs);
+    if (m == 4) return n == 1 ? pick_bits<1, 4, DENSE_OUT>(bits, warps, blocks, operands, njobs) : pick_bits<2, 4, DENSE_OUT>(bits, warps, blocks, operands, njobs);
+    if (n == 1) return pick_bits<1, 8, DENSE_OUT>(bits, warps, blocks, operands, njobs);
+    if (n == 2) return pick_bits<2, 8, DENSE_OUT>(bits, warps, blocks, operands, njobs);
+    return pick_bits<4, 8, DENSE_OUT>(bits, warps, blocks, operands, njobs);
 }
 
 static int validate_job(const nm_pack_job_t& j) {
@@ -1269,7 +1293,7 @@ static int launch_grouped_single(const nm_pack_job_t& j, int group_rows, uint32_
     warps = std::max(kPackMinWarps, 1 << d.wpr_log2);
     const int rows_per_block = warps >> d.wpr_log2;
     const unsigned blocks = (unsigned)((j.out + rows_per_block - 1) / rows_per_block);
-    return launch(pick_kernel<DENSE_OUT>(j.n, j.m, j.bits, warps, blocks, fills_buffers(j)), nullptr, 0, d, blocks, warps, status, stream,
+    return launch(pick_kernel<DENSE_OUT>(j.n, j.m, j.bits, warps, blocks, operands_of(j)), nullptr, 0, d, blocks, warps, status, stream,
                   Z, U_next, nullptr, kGroupScalesGiven, group_rows);
 }
 
@@ -1341,7 +1365,7 @@ static int launch_dist_project_single(const nm_pack_job_t& j, int ncand, uint32_
                       kGroupNone, ncand);
     int rc = launch_dist_single(j, ncand, nullptr, status, stream);
     if (rc != NM_OK) return rc;
-    return launch(pick_kernel<DENSE_OUT>(j.n, j.m, j.bits, warps, blocks, fills_buffers(j)), nullptr, 0, d, blocks, warps, status, stream, Z, U_next,
+    return launch(pick_kernel<DENSE_OUT>(j.n, j.m, j.bits, warps, blocks, operands_of(j)), nullptr, 0, d, blocks, warps, status, stream, Z, U_next,
                   nullptr, kGroupScalesGiven, 0);
 }
 
@@ -1397,14 +1421,14 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
                           int dist_ncand = 0) {
     // Group jobs that can share one launch: same (n == m ? dense : n, m), bits and block size.  Where a cluster of blocks holds a
     // group of rows (group_cluster) the block size follows from the warps per row.
-    struct Key { int n, m, bits, warps, cluster, dual; };
+    struct Key { int n, m, bits, warps, cluster, operands; };
     std::vector<Key> keys;
     std::vector<std::vector<int>> groups;
     for (int i = 0; i < njobs; ++i) {
         const nm_pack_job_t& j = jobs[i];
         if (j.out == 0 || j.in == 0) continue;
         const int wl = nm::wpr_log2_of(j.in);
-        Key k{j.n == j.m ? 4 : j.n, j.n == j.m ? 4 : j.m, j.bits, std::max(nm::kPackMinWarps, 1 << wl), 0, fills_buffers(j) ? 1 : 0};
+        Key k{j.n == j.m ? 4 : j.n, j.n == j.m ? 4 : j.m, j.bits, std::max(nm::kPackMinWarps, 1 << wl), 0, operands_of(j)};
         int gw = 0, gc = 0;
         if (grouped && group_cluster(group_rows, wl, &gw, &gc)) { k.warps = gw; k.cluster = gc; }
         size_t g = 0;
@@ -1412,7 +1436,7 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
             if (keys[g].n == k.n && keys[g].m == k.m && keys[g].bits == k.bits && keys[g].warps == k.warps && keys[g].cluster == k.cluster &&
                 (!k.cluster || nm::wpr_log2_of(jobs[groups[g][0]].in) == wl)) break;
         if (g == keys.size()) { keys.push_back(k); groups.emplace_back(); }
-        keys[g].dual &= k.dual;
+        keys[g].operands = std::min(keys[g].operands, k.operands);
         groups[g].push_back(i);
     }
     std::vector<nm::PackJobDev> table;
@@ -1449,7 +1473,7 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
                 if (g == 1) separate = !g_no_pdl && separate_launches(table, nullptr, group_first);
                 PackJobInline inl{};
                 for (size_t i = 0; i < groups[g].size(); ++i) inl.j[i] = table[group_first[g] + i];
-                int rc = nm::launch_table(nm::pick_kernel<DENSE_OUT>(keys[g].n, keys[g].m, keys[g].bits, keys[g].warps, group_blocks[g], keys[g].dual), nullptr,
+                int rc = nm::launch_table(nm::pick_kernel<DENSE_OUT>(keys[g].n, keys[g].m, keys[g].bits, keys[g].warps, group_blocks[g], keys[g].operands, (int)groups[g].size()), nullptr,
                                           (int)groups[g].size(), inl, group_blocks[g], keys[g].warps, status, s, nullptr,
                                           nullptr, nullptr, kGroupNone, 0, g > 0 && separate);
                 if (rc != NM_OK) return rc;
@@ -1478,7 +1502,7 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
             const nm::PackJobDev* dev = reinterpret_cast<const nm::PackJobDev*>(ws) + group_first[g];
             group_prepare_kernel<<<(unsigned)groups[g].size(), 256, 0, s>>>(dev, group_rows, keys[g].bits, 0);
             NM_CUDA_TRY(cudaGetLastError());
-            int rc = nm::launch(nm::pick_kernel<DENSE_OUT>(keys[g].n, keys[g].m, keys[g].bits, keys[g].warps, group_blocks[g], keys[g].dual), dev,
+            int rc = nm::launch(nm::pick_kernel<DENSE_OUT>(keys[g].n, keys[g].m, keys[g].bits, keys[g].warps, group_blocks[g], keys[g].operands, (int)groups[g].size()), dev,
                                 (int)groups[g].size(), nm::PackJobDev{}, group_blocks[g], keys[g].warps, status, s,
                                 nullptr, nullptr, DENSE_OUT ? dense_dev + group_first[g] : nullptr, kGroupMaxPass, group_rows);
             if (rc != NM_OK) return rc;
@@ -1507,7 +1531,7 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
                                      status, s, dist_ncand, nullptr);
                 if (rc != NM_OK) return rc;
             }
-            rc = nm::launch(nm::pick_kernel<DENSE_OUT>(k.n, k.m, k.bits, k.warps, group_blocks[g], k.dual), dev, count, nm::PackJobDev{},
+            rc = nm::launch(nm::pick_kernel<DENSE_OUT>(k.n, k.m, k.bits, k.warps, group_blocks[g], k.operands, count), dev, count, nm::PackJobDev{},
                             group_blocks[g], k.warps, status, s, nullptr, nullptr, dense_g,
                             (grouped || dist_ncand > 0) ? kGroupScalesGiven : kGroupNone, group_rows, chained);
         }
@@ -1543,7 +1567,7 @@ int nm_project_pack(const float* W, const float* U, int out, int in, int n, int 
     int warps = std::max(nm::kPackMinWarps, 1 << d.wpr_log2);
     int rows_per_block = warps >> d.wpr_log2;
     unsigned blocks = (unsigned)((out + rows_per_block - 1) / rows_per_block);
-    return nm::launch(nm::pick_kernel(n, m, bits, warps, blocks, nm::fills_buffers(j)), nullptr, 0, d, blocks, warps, status, (cudaStream_t)stream);
+    return nm::launch(nm::pick_kernel(n, m, bits, warps, blocks, nm::operands_of(j)), nullptr, 0, d, blocks, warps, status, (cudaStream_t)stream);
 }
 
 int nm_admm_project(const float* W, const float* U, int out, int in, int n, int m, int bits, float* Z,
@@ -1556,7 +1580,7 @@ int nm_admm_project(const float* W, const float* U, int out, int in, int n, int 
     int warps = std::max(nm::kPackMinWarps, 1 << d.wpr_log2);
     int rows_per_block = warps >> d.wpr_log2;
     unsigned blocks = (unsigned)((out + rows_per_block - 1) / rows_per_block);
-    return nm::launch(nm::pick_kernel<true>(n, m, bits, warps, blocks, nm::fills_buffers(j)), nullptr, 0, d, blocks, warps, status,
+    return nm::launch(nm::pick_kernel<true>(n, m, bits, warps, blocks, nm::operands_of(j)), nullptr, 0, d, blocks, warps, status,
                       (cudaStream_t)stream, Z, U_next);
 }
 

@@ -1,10 +1,11 @@
 """GPU parity of the projection kernel's two forms in blocks of four warps, each forced in turn, and at the sizes where
 the library changes from one to the other.
 
-"direct" (one unit per block, loads straight into registers) exists for every pattern, code width and output.  "staged"
-(persistent, the next rows brought into shared memory by bulk copies) exists for 2:4 without dense outputs; the library takes it
-for launches with two operands and rows of a multiple of 1024 weights, of two to six rounds of the direct form's resident
-blocks.  Rows of one and four warps, ragged tails, a launch of many rounds per resident block, a batch through the device job
+"direct" (one unit per block, loads straight into registers) exists for every pattern, code width and output, with two register
+budgets.  "staged" (persistent, the next rows brought into shared memory by bulk copies) exists for 1:4, 2:4, 1:8 and 2:8 without
+dense outputs; the library takes it for launches with two operands and rows of 1024, 2048 or 4096 weights (2:4: of a multiple of
+1024) of more than one round of the direct form's resident blocks, several matrices up to six.
+Rows of one and four warps, ragged tails, a launch of many rounds per resident block, a batch through the device job
 table, and (direct) the ADMM step with dense outputs, bit for bit against the oracle.
 """
 import numpy as np
@@ -17,6 +18,7 @@ import workloads as wl
 pytestmark = pytest.mark.gpu
 
 PATTERNS = [(1, 4), (2, 4), (1, 8), (2, 8), (4, 8), (4, 4)]
+STAGED = [(1, 4), (2, 4), (1, 8), (2, 8)]
 FORMS = {"direct": 1, "staged": 2}
 
 
@@ -39,7 +41,7 @@ def _check_pack(W, U, n, m, bits):
         assert np.array_equal(meta, meta_ref), "metadata differs"
 
 
-@pytest.mark.parametrize("form,n,m", [("direct", *p) for p in PATTERNS] + [("staged", 2, 4)], indirect=["form"])
+@pytest.mark.parametrize("form,n,m", [("direct", *p) for p in PATTERNS] + [("staged", *p) for p in STAGED], indirect=["form"])
 @pytest.mark.parametrize("bits", [8, 4])
 def test_forms_rows_and_ragged(form, n, m, bits):
     oracle.set_threads(oracle.max_threads())
@@ -53,7 +55,7 @@ def test_forms_rows_and_ragged(form, n, m, bits):
         _check_pack(wl.with_outliers(110 + seed, out, k), wl.tie_heavy(120 + seed, out, k, levels=1), n, m, bits)
 
 
-@pytest.mark.parametrize("form,n,m,bits", [("staged", 2, 4, 8), ("direct", 2, 4, 8), ("direct", 4, 8, 4), ("direct", 1, 8, 8)],
+@pytest.mark.parametrize("form,n,m,bits", [("staged", 2, 4, 8), ("staged", 1, 4, 4), ("staged", 2, 8, 8), ("staged", 1, 8, 4), ("direct", 2, 4, 8), ("direct", 4, 8, 4), ("direct", 1, 8, 8)],
                          indirect=["form"])
 def test_forms_many_rounds(form, n, m, bits):
     """More units than resident blocks, several times over (9001 rows of 1024: 2251 units; 1500 rows of 3072: a row
@@ -152,7 +154,7 @@ def test_forms_admm_step(n, m, bits):
             assert np.array_equal(meta.cpu().numpy().view(np.uint32)[: mb // 4], np.asarray(meta_ref).reshape(-1))
 
 
-def _automatic(outs, k, with_u, bits=8):
+def _automatic(outs, k, with_u, n=2, m=4, bits=8):
     """The jobs in one call with the library's own choice of form, every output against the oracle."""
     import paper_2206_15014_b200 as nm
     from gpu_util import DEV, to_dev
@@ -161,10 +163,10 @@ def _automatic(outs, k, with_u, bits=8):
     for i, (out, has_u) in enumerate(zip(outs, with_u)):
         W, U = wl.pack_sweep_matrix(41, i, out, k)
         U = U if has_u else None
-        vb, mb = nm.nm_packed_sizes(out, k, 2, 4, bits)
-        jobs.append((to_dev(W), None if U is None else to_dev(U), 2, 4, bits, torch.zeros(vb, dtype=torch.uint8, device=DEV),
+        vb, mb = nm.nm_packed_sizes(out, k, n, m, bits)
+        jobs.append((to_dev(W), None if U is None else to_dev(U), n, m, bits, torch.zeros(vb, dtype=torch.uint8, device=DEV),
                      torch.zeros(mb // 4, dtype=torch.int32, device=DEV), torch.zeros(out, dtype=torch.float32, device=DEV)))
-        refs.append(oracle.project_pack(W, U, 2, 4, bits))
+        refs.append(oracle.project_pack(W, U, n, m, bits))
     ws_bytes = nm.nm_pack_workspace_bytes(len(jobs))
     ws = torch.empty(ws_bytes, dtype=torch.uint8, device=DEV)
     status = torch.zeros(1, dtype=torch.int32, device=DEV)
@@ -176,11 +178,23 @@ def _automatic(outs, k, with_u, bits=8):
         assert np.array_equal(job[6].cpu().numpy().view(np.uint32).reshape(m_ref.shape), m_ref)
 
 
-@pytest.mark.parametrize("rounds,beyond", [(2, 0), (2, 1), (6, 0), (6, 1)])
-def test_both_sides_of_the_librarys_choice(rounds, beyond):
-    """Up to two rounds of eight resident blocks a multiprocessor direct, beyond staged; up to six staged, beyond direct."""
+@pytest.mark.parametrize("n,m,bits", [(1, 4, 4), (2, 4, 8), (1, 8, 8), (2, 8, 4)])
+@pytest.mark.parametrize("blocks_per_sm,beyond", [(5, 0), (5, 1), (8, 0), (8, 1)])
+@pytest.mark.parametrize("k", [1024, 3072])
+def test_both_sides_of_the_librarys_choice(n, m, bits, blocks_per_sm, beyond, k):
+    """One matrix with two operands: up to five blocks a multiprocessor direct with more registers, up to eight direct, beyond
+    staged (rows of 3072: 2:4 only)."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    _automatic([4 * (rounds * 8 * sms + beyond)], 1024, [True])  # four rows a block
+    rows = 4 if k == 1024 else 1  # a block's
+    _automatic([rows * (blocks_per_sm * sms + beyond)], k, [True], n, m, bits)
+
+
+@pytest.mark.parametrize("beyond", [0, 1])
+@pytest.mark.parametrize("n,m", [(2, 4), (1, 8)])
+def test_six_rounds_of_several_matrices(n, m, beyond):
+    """Two matrices: up to six rounds of eight blocks a multiprocessor staged, beyond direct."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    _automatic([4 * (3 * 8 * sms), 4 * (3 * 8 * sms + beyond)], 1024, [True, True], n, m)
 
 
 @pytest.mark.parametrize("with_u", [[True, True, True], [True, False, True]])
@@ -188,3 +202,14 @@ def test_one_operand_in_a_batch_of_two_operand_jobs(with_u):
     """Three rounds of blocks: staged when every job has a U, direct when one has none."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     _automatic([4 * 8 * sms] * 3, 1024, with_u, bits=4)
+
+
+def test_few_blocks_of_every_pattern():
+    """Launches of a few blocks with two operands, rows of every kind: the direct form with more registers."""
+    for n, m in PATTERNS:
+        for out, k in ((7, 768), (9, 1032 if m == 4 else 1040), (130, 1024), (3, 4096)):
+            if n == m:
+                W, U = wl.pack_sweep_matrix(43, out, out, k)
+                _check_pack(W, U, n, m, 8)
+            else:
+                _automatic([out], k, [True], n, m, 8)
