@@ -8,6 +8,7 @@ library has not been built (run ``python paper_2206_15014_b200/build.py``).
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -356,3 +357,17 @@ def nm_quantize_act(Y, count, absmax, Xq, sx_out=None, stream=None):
 def nm_poll_status(status=None, stream=None):
     """Synchronises the stream and returns the NM_* code held in the device status word."""
     return int(_lib.nm_poll_status(_ptr(status), _stream(stream)))
+
+
+# The calls that a program makes once per layer go through a small extension module (csrc/marshal.c), which converts plain
+# arguments itself and hands anything else to the functions above.
+def _fast_entries():
+    spec = importlib.util.spec_from_file_location("_marshal", os.path.join(_HERE, "_marshal.so"))
+    marshal = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(marshal)
+    for name in ("nm_int_linear", "nm_int_linear_dsx", "nm_int_linear_q8", "nm_int_linear_bf16", "nm_absmax", "nm_quantize_act"):
+        address = ctypes.cast(getattr(_lib, name), ctypes.c_void_p).value
+        globals()[name] = marshal.entry(name, address, globals()[name], nm_packed_t, _chk)
+
+
+_fast_entries()

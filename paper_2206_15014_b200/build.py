@@ -4,6 +4,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -17,6 +18,21 @@ FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std
 # Other builds of the same sources: "trace" compiles time stamps into the GEMM kernels (nm_debug_set_trace),
 # "shortwait" gives every device-side wait a limit of about a millisecond (the timeout test runs against it).
 VARIANTS = {"": [], "trace": ["-DNM_TRACE"], "shortwait": ["-DNM_WAIT_LIMIT=(1ll<<21)", "-DNM_TEST_HOOKS"]}
+
+
+# Extension module of the Python binding (csrc/marshal.c): plain C against the interpreter's headers.
+MARSHAL = os.path.join(HERE, "_marshal.so")
+
+
+def build_marshal(force: bool = False) -> str:
+    src, header = os.path.join(CSRC, "marshal.c"), os.path.join(os.path.dirname(HERE), "include", "nmsparse.h")
+    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= max(os.path.getmtime(src), os.path.getmtime(header)):
+        return MARSHAL
+    tmp = MARSHAL + f".tmp{os.getpid()}"
+    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"],
+                           src, "-o", tmp])
+    os.replace(tmp, MARSHAL)
+    return MARSHAL
 
 
 def lib_path(variant: str = "") -> str:
@@ -34,6 +50,7 @@ def _stale(lib: str = LIB) -> bool:
 
 def build(force: bool = False, verbose: bool = False, variant: str = "") -> str:
     LIB = lib_path(variant)
+    build_marshal(force)
     if not force and not _stale(LIB):
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

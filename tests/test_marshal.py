@@ -1,0 +1,60 @@
+"""The extension module of the binding takes every call form that its Python twins take, with the same results and errors
+(no GPU needed: calls that return before a launch)."""
+import ctypes
+import inspect
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2206_15014_b200 as nm
+
+NAMES = ("nm_int_linear", "nm_int_linear_dsx", "nm_int_linear_q8", "nm_int_linear_bf16", "nm_absmax", "nm_quantize_act")
+
+
+def _args(name):
+    t = torch.zeros(64, dtype=torch.float32)
+    w = nm.make_packed(128, 128, 2, 4, 8, t, t)
+    return {"nm_int_linear": (t, 0, w, 0.5, t, t, t), "nm_int_linear_dsx": (t, 0, w, t, t, t, t),
+            "nm_int_linear_q8": (t, 0, w, 0.5, t, t, 1.0, t), "nm_int_linear_bf16": (t, 0, w, 0.5, t, t, t),
+            "nm_absmax": (t, 0, t), "nm_quantize_act": (None, 0, t, None)}[name]
+
+
+def _outcome(fn, *args, **kw):
+    try:
+        return ("value", fn(*args, **kw))
+    except Exception as e:
+        return (type(e), getattr(e, "code", None), str(e))
+
+
+@pytest.mark.parametrize("name", NAMES)
+def test_same_outcome_as_the_twin(name):
+    fast, twin = getattr(nm, name), inspect.unwrap(getattr(nm, name))
+    assert fast is not twin and inspect.signature(fast) == inspect.signature(twin) and fast.__name__ == name
+    args, names = _args(name), list(inspect.signature(twin).parameters)
+    forms = [(args, {"stream": 0}), ((), dict(zip(names, args), stream=0)), (args[:2], dict(zip(names[2:], args[2:]), stream=0)),
+             (args, {"stream": 0, "nope": 1}), (args + args[-1:], {names[0]: args[0], "stream": 0}), (args[:-1], {"stream": 0}),
+             (args, {"stream": "x"})]
+    for i in range(len(args)):  # every argument of every wrong kind, and of kinds that only the twin converts
+        other = [1.5, "a", None, 2 ** 70, np.int64(0)]
+        if names[i] not in ("tokens", "count", "absmax"):  # (nothing that would launch)
+            other += [True, -1, torch.zeros(3)]
+        forms += [(args[:i] + (v,) + args[i + 1:], {"stream": 0}) for v in other]
+    for a, kw in forms:
+        if name == "nm_quantize_act":
+            kw = dict(kw, sx_out=args[2])  # the maximum's own buffer: refused before a launch
+        assert _outcome(fast, *a, **kw) == _outcome(twin, *a, **kw), (a, kw)
+
+
+def test_error_codes_and_descriptor_checks():
+    t = torch.zeros(64)
+    w = nm.make_packed(128, 100, 2, 4, 8, t, t)  # not whole k-blocks
+    with pytest.raises(nm.NmError) as e:
+        nm.nm_int_linear(t, 4, w, 0.5, t, None, t, stream=0)
+    assert e.value.code == nm.NM_ERR_SHAPE and "nm_int_linear" in str(e.value)
+
+    class Other(ctypes.Structure):
+        _fields_ = nm.nm_packed_t._fields_
+
+    with pytest.raises(ctypes.ArgumentError):
+        nm.nm_int_linear(t, 0, Other(), 0.5, t, None, t, stream=0)
