@@ -347,7 +347,8 @@ int nm_probe_tma_stream(const void *W, int w_rows, int w_row_bytes, const void *
  * dependent-launch attribute), "no_pair" (one-CTA kernels only), "no_resident" (always stream the weights),
  * "no_wide" (never the 512-channel pair kernel), "wide_any" (the 512-channel pair kernel whenever the shape
  * allows it, however few tiles there are), "wide_bn" (its token-tile width, 224 or 192), "band" (band size of the streamed pair kernel's tile order),
- * "one_bn" (token-tile width of the one-CTA kernel: 192, 128, 96, 64 or 32 where it exists), "xres" (the pair kernel with resident
+ * "split" (one-CTA tiles with the reduction split over a cluster: 1000 * CTAs + token-tile width, for instance 4096, where that
+ * fits, 1 = never), "one_bn" (token-tile width of the one-CTA kernel: 192, 128, 96, 64 or 32 where it exists), "xres" (the pair kernel with resident
  * activations: 1 = wherever a pair kernel with a reduction of at most 1024 runs, 2 = never),
  * "pack_form" (form of the projection kernel in blocks of four warps: 2 = persistent with the next rows staged in shared
  * memory by bulk copies, where that form exists: 1:4, 2:4, 1:8 and 2:8 without dense outputs; 1 or 3 = one unit per block).

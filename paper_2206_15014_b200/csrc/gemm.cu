@@ -1207,6 +1207,7 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
 
 #include "gemm_wide.cuh"
 #include "gemm_xres.cuh"
+#include "gemm_split.cuh"
 
 namespace nm {
 
@@ -1221,6 +1222,7 @@ struct DebugOptions {
     int wide_any;     // the 512-channel pair kernel whenever the shape allows it, however few tiles there are
     int wide_bn;      // token-tile width of that kernel: 224 or 192 (0 = automatic)
     int xres;         // the pair kernel with resident activations: 1 = whenever the shape allows it, 2 = never
+    int split;        // reduction split over a cluster: 1000 * CTAs + token-tile width, 1 = never (0 = automatic)
     int one_bn;       // token-tile width of the one-CTA kernel (0 = automatic)
     int band;         // band size of the streamed pair kernel's tile order (0 = automatic)
     int skip_stage;   // NM_TEST_HOOKS builds: 1 + the pipeline stage CTA 0's producer leaves out (0 = none)
@@ -1234,7 +1236,7 @@ static unsigned long long* g_trace_buffer = nullptr;
 // cudaFuncSetAttribute(max dynamic shared memory) once per kernel and device instead of on every launch.
 static cudaError_t allow_dynamic_smem(const void* fn, int bytes) {
     struct Done { const void* fn; int dev; };
-    static Done done[64];
+    static Done done[256];
     static int n_done = 0;
     static std::mutex mu;
     int dev = 0;
@@ -1244,7 +1246,7 @@ static cudaError_t allow_dynamic_smem(const void* fn, int bytes) {
     for (int i = 0; i < n_done; ++i)
         if (done[i].fn == fn && done[i].dev == dev) return cudaSuccess;
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess && n_done < 64) done[n_done++] = Done{fn, dev};
+    if (e == cudaSuccess && n_done < 256) done[n_done++] = Done{fn, dev};
     return e;
 }
 
@@ -1481,6 +1483,42 @@ static int launch_gemm_xres(const LinearArgs& a) {
     return NM_OK;
 }
 
+// One-CTA tiles with the reduction split over clusters of `splits` CTAs (gemm_split.cuh).
+template <bool SPARSE, int BN, int EPI>
+static int launch_gemm_split(const LinearArgs& a, int splits) {
+    using Cfg = SplitCfg<SPARSE, BN>;
+    const nm_packed_t& W = *a.W;
+    CUtensorMap tw, tx;
+    int rc = make_map(&tw, W.values, (uint64_t)W.out, (uint64_t)(SPARSE ? W.in / 2 : W.in), kBM, Cfg::A_ROW,
+                      SPARSE ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B);
+    if (rc != NM_OK) return rc;
+    rc = make_map(&tx, a.X, (uint64_t)a.tokens, (uint64_t)W.in, BN, 128, CU_TENSOR_MAP_SWIZZLE_128B);
+    if (rc != NM_OK) return rc;
+    GemmParams p{};
+    p.tokens = a.tokens; p.out = W.out; p.in = W.in;
+    p.n_tok_tiles = (a.tokens + BN - 1) / BN;
+    p.n_tiles = p.n_tok_tiles * ((W.out + kBM - 1) / kBM);
+    p.kblocks = W.in / kKB;
+    p.meta = (const uint32_t*)W.meta; p.mrow_words = W.in / 32;
+    p.sw = a.sw; p.bias = a.bias; p.sx_dev = a.sx_dev; p.sx_host = a.sx;
+    p.Y = a.Y; p.ACC = a.ACC; p.NARROW = a.NARROW; p.sy = a.sy; p.absmax = a.absmax; p.status = a.status;
+    auto fn = nm_gemm_split_kernel<SPARSE, BN, EPI>;
+    NM_CUDA_TRY(allow_dynamic_smem((const void*)fn, Cfg::SMEM));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(p.n_tiles * splits), 1, 1);
+    cfg.blockDim = dim3(kSplitThreads, 1, 1);
+    cfg.dynamicSmemBytes = Cfg::SMEM;
+    cfg.stream = a.stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)splits; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = g_no_pdl ? 1 : 2;
+    NM_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, tw, tx, p, splits));
+    return NM_OK;
+}
+
 // Where the kernel with resident activations is the faster pair kernel.  At least two output tiles (with one the activations
 // are not read twice), and then by measurement, this kernel / the other one in us:
 //  - dense weights, which the other kernel streams besides the activations: always (6144 tokens 768 -> 768 10.6 / 12.8, 768 -> 3072
@@ -1582,11 +1620,79 @@ static int one_cta_bn(const LinearArgs& a, std::initializer_list<int> widths, in
     return best;
 }
 
+// Clusters of `splits` one-CTA tiles that the current device runs at a time (asked once per device; 74, 33 and 14 for 2, 4 and 8 CTAs where
+// the query fails): one more goes into a second round, which costs what the split gains.
+static int resident_clusters(int splits) {
+    static std::mutex mu;
+    static int known[64][3] = {};
+    const int at = splits == 2 ? 0 : splits == 4 ? 1 : 2;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    std::lock_guard<std::mutex> lock(mu);
+    int& n = known[dev][at];
+    if (n == 0) {
+        using Cfg = SplitCfg<true, 64>;
+        auto fn = nm_gemm_split_kernel<true, 64, EPI_F32>;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)splits, 1, 1);
+        cfg.blockDim = dim3(kSplitThreads, 1, 1);
+        cfg.dynamicSmemBytes = Cfg::SMEM;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)splits; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        if (allow_dynamic_smem((const void*)fn, Cfg::SMEM) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, (const void*)fn, &cfg) != cudaSuccess || n < 1) {
+            (void)cudaGetLastError();
+            n = splits == 2 ? 74 : splits == 4 ? 33 : 14;
+        }
+    }
+    return n;
+}
+
+// Where the reduction is split, and how: 1000 * CTAs + token-tile width, or 0.  A split costs its k-blocks, each the tile's width
+// plus 256 tokens, and an exchange of 12 times the width; it is taken where that is at most 0.9 of the unsplit kernel's k-blocks
+// at the same rate.  Over 299 shapes (1 to 1000 tokens, reductions of 384 to 8192) 0.70 of the unsplit time in the geometric mean, 1.03 at the
+// worst, the best of all splits 0.697: 384 tokens 4096 -> 1024 11.9 -> 7.3 us, 64 tokens 768 -> 768 4.5 -> 3.6, 1 token 8192 -> 1024 19.7 -> 5.6;
+// not taken: 384 tokens 1024 -> 3072 5.9 / 6.6.
+template <bool SPARSE>
+static int split_plan(const LinearArgs& a, int unsplit_bn) {
+    if (g_opt.split == 1 || g_opt.one_bn || g_opt.skip_stage) return 0;  // the test hook counts the stages of an unsplit tile
+    const int kblocks = a.W->in / kKB, out_tiles = (a.W->out + kBM - 1) / kBM;
+    const long long unsplit = (long long)kblocks * (unsplit_bn + 256);
+    long long best_cost = 0;
+    int best = 0;
+    for (int splits : {2, 4, 8})
+        for (int bn : {32, 64, 96, 128}) {
+            const int plan = 1000 * splits + bn, per = (kblocks + splits - 1) / splits;
+            if ((bn / splits) % 8 || kblocks < splits || per > kSplitMaxKb) continue;
+            if (g_opt.split && plan != g_opt.split) continue;
+            const long long clusters = (long long)out_tiles * ((a.tokens + bn - 1) / bn);
+            if (clusters * splits > sm_count()) continue;
+            const long long cost = (long long)per * (bn + 256) + 12 * bn;
+            if (!g_opt.split && (10 * cost > 9 * unsplit || clusters > resident_clusters(splits))) continue;
+            if (!best || cost < best_cost) { best = plan; best_cost = cost; }
+        }
+    return best;
+}
+
+template <bool SPARSE, int EPI>
+static int pick_split(const LinearArgs& a, int plan) {
+    const int splits = plan / 1000;
+    switch (plan % 1000) {
+        case 128: return launch_gemm_split<SPARSE, 128, EPI>(a, splits);
+        case 96: return launch_gemm_split<SPARSE, 96, EPI>(a, splits);
+        case 64: return launch_gemm_split<SPARSE, 64, EPI>(a, splits);
+        default: return launch_gemm_split<SPARSE, 32, EPI>(a, splits);
+    }
+}
+
 template <bool SPARSE, int EPI, bool XF>
 static int pick_bn(const LinearArgs& a) {
     const int out_tiles = (a.W->out + kBM - 1) / kBM, sms = sm_count();
     if constexpr (!XF) {
         const int best = one_cta_bn<SPARSE>(a, {192, 128, 96, 64, 32}, 64);
+        if (const int plan = split_plan<SPARSE>(a, best)) return pick_split<SPARSE, EPI>(a, plan);
         switch (best) {
             case 192: return launch_gemm<SPARSE, 192, EPI, W_TMA>(a);
             case 128: return launch_gemm<SPARSE, 128, EPI, W_TMA>(a);
@@ -1686,7 +1792,7 @@ int nm_debug_set_option(const char* name, int value) {
     struct { const char* name; int* slot; } table[] = {
         {"no_pdl", &nm::g_no_pdl}, {"no_pair", &nm::g_opt.no_pair}, {"no_resident", &nm::g_opt.no_resident},
         {"no_wide", &nm::g_opt.no_wide}, {"wide_any", &nm::g_opt.wide_any}, {"wide_bn", &nm::g_opt.wide_bn},
-        {"one_bn", &nm::g_opt.one_bn}, {"xres", &nm::g_opt.xres}, {"band", &nm::g_opt.band}, {"pack_form", &nm::g_pack_form}};
+        {"one_bn", &nm::g_opt.one_bn}, {"split", &nm::g_opt.split}, {"xres", &nm::g_opt.xres}, {"band", &nm::g_opt.band}, {"pack_form", &nm::g_pack_form}};
     for (auto& e : table)
         if (!strcmp(name, e.name)) { *e.slot = value; return NM_OK; }
 #ifdef NM_TEST_HOOKS
