@@ -228,7 +228,7 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     uint32_t* lut = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(bars) + 512);
 
     constexpr int EW = XF ? kEpiWarpsXf : kEpiWarps, kGateWarp = 2 + EW;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)ptx::warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int per = p.n_tiles / gridDim.x, rem = p.n_tiles % gridDim.x;
     const int tile_begin = blockIdx.x * per + min((int)blockIdx.x, rem);
     const int tile_count = per + ((int)blockIdx.x < rem ? 1 : 0);
@@ -256,7 +256,7 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = ptx::warp_uniform(*tmem_slot);
     // Set-up above overlaps the tail of the kernel before this one in the stream (when launched as its
     // programmatic dependent); nothing in global memory is read or written before this point.
     ptx::grid_dep_wait();
@@ -409,47 +409,48 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ---------------------------------------------
         constexpr uint32_t idesc = ptx::idesc_i8(kBM, BN, SPARSE);
-        uint32_t it = 0;
+        const uint64_t a_desc0 = ptx::smem_desc_kmajor(ptx::smem_u32(RES ? a_res : smem), SPARSE ? 64 : 128, SPARSE ? ptx::kSwizzle64 : ptx::kSwizzle128);
+        const uint64_t b_desc0 = ptx::smem_desc_kmajor(ptx::smem_u32(smem) + Cfg::B_OFF, 128, ptx::kSwizzle128);
+        uint32_t s = 0, relay = 1;
+        int tok = tile_begin % p.n_tok_tiles;
         for (int i = 0; i < tile_count; ++i) {
-            const int buf = i & 1;
-            const uint32_t d_tmem = tmem_base + buf * BN;
-            const bool last_of_out_tile = RES && (tile_begin + i + 1) / p.n_tok_tiles != (tile_begin + i) / p.n_tok_tiles;
-            for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
-                const int s = it % S;
-                ptx::named_bar_sync(1 + (it & 7u), 64);  // stage s holds k-block kb (and, for kb = 0, the
-                                                         // accumulator is free and the metadata in place)
+            const uint32_t buf = i & 1, d_tmem = tmem_base + buf * BN;
+            const bool last_of_out_tile = RES && ++tok == p.n_tok_tiles;  // the next tile is another output tile's
+            if (last_of_out_tile) tok = 0;
+            for (int kb = 0; kb < p.kblocks; ++kb) {
+                ptx::named_bar_sync(relay, 64);  // stage s holds k-block kb (and, for kb = 0, the
+                relay = (relay & 7u) + 1u;       // accumulator is free and the metadata in place)
                 // The tcgen05 fence orders the MMAs after other threads' TMEM accesses (accumulator read
                 // back, metadata stores): needed once per tile.  Executed every stage it drains the MMA
                 // pipe (measured ~585 clk per stage); the staged operands are ordered by the mbarrier.
                 if (kb == 0) ptx::tc_fence_after();
-                if (lane == 0) {
-                    const uint32_t st_addr = ptx::smem_u32(smem + s * Cfg::STAGE), b_addr = st_addr + Cfg::B_OFF;
-                    const uint32_t a_addr = RES ? ptx::smem_u32(a_res + kb * Cfg::A_BYTES) : st_addr;
+                if (ptx::elect_one()) {
+                    const uint64_t a = ptx::desc_advance(a_desc0, RES ? kb * Cfg::A_BYTES : s * Cfg::STAGE), b = ptx::desc_advance(b_desc0, s * Cfg::STAGE);
                     if constexpr (SPARSE) {
 #pragma unroll
                         for (int j = 0; j < 2; ++j)  // 64 logical k each: 32 stored bytes of A, 64 of B
-                            ptx::mma_sp_i8(d_tmem, ptx::smem_desc_kmajor(a_addr + 32 * j, 64, ptx::kSwizzle64),
-                                           ptx::smem_desc_kmajor(b_addr + 64 * j, 128, ptx::kSwizzle128),
+                            ptx::mma_sp_i8(d_tmem, ptx::desc_advance(a, 32 * j), ptx::desc_advance(b, 64 * j),
                                            tmem_base + Cfg::META_COL + kb * 4 + 2 * j, idesc, (kb | j) != 0);
                     } else {
 #pragma unroll
                         for (int j = 0; j < 4; ++j)  // 32 k each
-                            ptx::mma_i8(d_tmem, ptx::smem_desc_kmajor(a_addr + 32 * j, 128, ptx::kSwizzle128),
-                                        ptx::smem_desc_kmajor(b_addr + 32 * j, 128, ptx::kSwizzle128), idesc, (kb | j) != 0);
+                            ptx::mma_i8(d_tmem, ptx::desc_advance(a, 32 * j), ptx::desc_advance(b, 32 * j), idesc, (kb | j) != 0);
                     }
                     ptx::tc_commit(empty_bar(s));  // stage reusable once these MMAs have read it
                     if (kb == p.kblocks - 1) {
                         ptx::tc_commit(acc_full_bar(buf));
-                        if (RES && last_of_out_tile) ptx::tc_commit(a_free_bar);  // the builders may overwrite the weight tile
+                        if (last_of_out_tile) ptx::tc_commit(a_free_bar);  // the builders may overwrite the weight tile
                     }
                 }
                 __syncwarp();
+                if (++s == S) s = 0;
             }
         }
-        if (lane == 0) {  // everything issued has retired before TMEM is released
+        if (ptx::elect_one()) {  // everything issued has retired before TMEM is released
             ptx::tc_commit(drained_bar);
             ptx::mbar_wait_bounded(drained_bar, 0, never_flag, kWaitLimit);
         }
+        __syncwarp();
     } else {
         // ------------------------------ metadata + epilogue warps ------------------------------
         // Warp w may touch TMEM lanes 32 * (w % 4) ... + 31.  With eight warps two share a lane quarter
@@ -756,7 +757,7 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
     uint32_t* lut = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(bars) + 512);  // BUILD: slot tables (xform.cuh)
     static_assert(!BUILD || (RES && SPARSE), "weights are rebuilt only in the resident-weight, sparse-target form");
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)ptx::warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const uint32_t rank = ptx::cluster_ctarank();
     const bool leader = rank == 0;
     const int pair = blockIdx.x >> 1;
@@ -788,7 +789,7 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = ptx::warp_uniform(*tmem_slot);
     // Set-up above overlaps the tail of the kernel before this one in the stream (when launched as its
     // programmatic dependent); nothing in global memory is read or written before this point.
     ptx::grid_dep_wait();
@@ -913,31 +914,30 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
         // ------------------------------ MMA issuer (leader) --------------------------------------
         if (leader) {
             constexpr uint32_t idesc = ptx::idesc_i8(2 * kBM, BN, SPARSE);
-            uint32_t it = 0;
+            const uint64_t a_desc0 = ptx::smem_desc_kmajor(ptx::smem_u32(RES ? a_res : smem), 128, ptx::kSwizzle128);
+            const uint64_t b_desc0 = ptx::smem_desc_kmajor(ptx::smem_u32(smem) + Cfg::B_OFF, 128, ptx::kSwizzle128);
+            uint32_t s = 0, relay = 1;
+            NM_TRACE_ONLY(uint32_t it = 0;)
             for (int i = 0; i < tile_count; ++i) {
-                const int buf = i & 1;
-                const uint32_t d_tmem = tmem_base + buf * BN;
+                const uint32_t buf = i & 1, d_tmem = tmem_base + buf * BN;
                 const bool last_of_out_tile = RES && (tile_begin + i + 1 >= p.n_tiles ||
                     tile_coord(tile_begin + i + 1, p.n_tok_tiles, p.n_out_tiles, p.band).o != tile_coord(tile_begin + i, p.n_tok_tiles, p.n_out_tiles, p.band).o);
-                for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
-                    const int s = it % S;
-                    ptx::named_bar_sync(1 + (it & 7u), 64);
+                for (int kb = 0; kb < p.kblocks; ++kb) {
+                    ptx::named_bar_sync(relay, 64);
+                    relay = (relay & 7u) + 1u;
                     if (kb == 0) ptx::tc_fence_after();  // once per tile (see the one-CTA kernel)
-                    if (lane == 0) {
+                    if (ptx::elect_one()) {
                         NM_TRACE_STAGE(it, 3);
-                        const uint32_t st_addr = ptx::smem_u32(smem + s * Cfg::STAGE), b_addr = st_addr + Cfg::B_OFF;
-                        const uint32_t a_addr = RES ? ptx::smem_u32(a_res + kb * Cfg::A_BYTES) : st_addr;
+                        const uint64_t a = ptx::desc_advance(a_desc0, RES ? kb * Cfg::A_BYTES : s * Cfg::STAGE), b = ptx::desc_advance(b_desc0, s * Cfg::STAGE);
                         if constexpr (SPARSE) {
 #pragma unroll
                             for (int j = 0; j < 4; ++j)  // 64 reduction elements each: 32 stored bytes of A, 64 of X
-                                ptx::mma_sp_i8_pair(d_tmem, ptx::smem_desc_kmajor(a_addr + 32 * j, 128, ptx::kSwizzle128),
-                                                    ptx::smem_desc_kmajor(b_addr + (j >> 1) * Cfg::B_SUB + 64 * (j & 1), 128, ptx::kSwizzle128),
+                                ptx::mma_sp_i8_pair(d_tmem, ptx::desc_advance(a, 32 * j), ptx::desc_advance(b, (j >> 1) * Cfg::B_SUB + 64 * (j & 1)),
                                                     tmem_base + Cfg::META_COL + kb * 8 + 2 * j, idesc, (kb | j) != 0);
                         } else {
 #pragma unroll
                             for (int j = 0; j < 4; ++j)
-                                ptx::mma_i8_pair(d_tmem, ptx::smem_desc_kmajor(a_addr + 32 * j, 128, ptx::kSwizzle128),
-                                                 ptx::smem_desc_kmajor(b_addr + 32 * j, 128, ptx::kSwizzle128), idesc, (kb | j) != 0);
+                                ptx::mma_i8_pair(d_tmem, ptx::desc_advance(a, 32 * j), ptx::desc_advance(b, 32 * j), idesc, (kb | j) != 0);
                         }
                         ptx::tc_commit_pair(empty_bar(s), 3);   // both producers may refill the stage
                         if (kb == p.kblocks - 1) {
@@ -947,12 +947,15 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                         NM_TRACE_STAGE(it, 4);
                     }
                     __syncwarp();
+                    if (++s == S) s = 0;
+                    NM_TRACE_ONLY(++it;)
                 }
             }
-            if (lane == 0) {
+            if (ptx::elect_one()) {
                 ptx::tc_commit_pair(drained_bar, 1);
                 ptx::mbar_wait_bounded(drained_bar, 0, never_flag, kWaitLimit);
             }
+            __syncwarp();
         }
     } else {
         // ------------------------------ metadata + epilogue warps (both CTAs) ----------------------

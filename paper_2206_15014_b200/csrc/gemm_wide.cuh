@@ -92,7 +92,7 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
     volatile uint32_t* abort_flag = tmem_slot + 1;
     volatile uint32_t* never_flag = tmem_slot + 2;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)ptx::warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const uint32_t rank = ptx::cluster_ctarank();
     const bool leader = rank == 0;
     const int pair = blockIdx.x >> 1;
@@ -121,7 +121,7 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = ptx::warp_uniform(*tmem_slot);
     // Set-up above may overlap the tail of the kernel before this one in the stream; global memory is first
     // touched below.
     ptx::grid_dep_wait();
@@ -317,7 +317,7 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                 ptx::named_bar_sync(relay, 64);
                 relay = relay == kWideRelayIds ? 1 : relay + 1;
                 ptx::tc_fence_after();  // orders the MMAs after the metadata stores and accumulator reads of other threads
-                if (lane == 0) {
+                if (ptx::elect_one()) {
                     NM_TRACE_STAGE(g, 3);
                     if (g < total) {
                         const uint64_t a = ptx::desc_advance(a_desc0, off_l), b = ptx::desc_advance(b_desc0, off_l);
@@ -351,10 +351,11 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                 }
                 __syncwarp();
             }
-            if (lane == 0) {  // everything issued has retired before TMEM is released
+            if (ptx::elect_one()) {  // everything issued has retired before TMEM is released
                 ptx::tc_commit_pair(drained_bar, 1);
                 ptx::mbar_wait_bounded(drained_bar, 0, never_flag, kWaitLimit);
             }
+            __syncwarp();
         }
     } else {
         // ------------------------------ epilogue warps (both CTAs) --------------------------------

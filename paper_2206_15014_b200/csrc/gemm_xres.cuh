@@ -68,7 +68,7 @@ nm_gemm_xres_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
     volatile uint32_t* abort_flag = tmem_slot + 1;
     volatile uint32_t* never_flag = tmem_slot + 2;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)ptx::warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const uint32_t rank = ptx::cluster_ctarank();
     const bool leader = rank == 0;
     const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
@@ -98,7 +98,7 @@ nm_gemm_xres_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = ptx::warp_uniform(*tmem_slot);
     // Set-up above overlaps the tail of the kernel before this one in the stream (when launched as its
     // programmatic dependent); nothing in global memory is read or written before this point.
     ptx::grid_dep_wait();
@@ -226,7 +226,7 @@ nm_gemm_xres_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                     ptx::named_bar_sync(relay, 64);
                     relay = (relay & 7u) + 1u;
                     if (kb == 0) ptx::tc_fence_after();  // once per tile (see the one-CTA kernel)
-                    if (lane == 0) {
+                    if (ptx::elect_one()) {
                         NM_TRACE_STAGE(it, 3);
                         const uint64_t a = ptx::desc_advance(a_desc0, s * Cfg::A_BYTES);
                         if constexpr (SPARSE) {
@@ -245,18 +245,19 @@ nm_gemm_xres_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                             if (SPARSE) ptx::tc_commit_pair(meta_empty_bar(i % MB), 3);
                         }
                         NM_TRACE_STAGE(it, 4);
-                        NM_TRACE_ONLY(++it;)
                     }
                     __syncwarp();
+                    NM_TRACE_ONLY(++it;)
                     b = ptx::desc_advance(b, Cfg::SLICES * Cfg::B_SUB);
                     e += 8;
                     if (++s == S) s = 0;
                 }
             }
-            if (lane == 0) {
+            if (ptx::elect_one()) {
                 ptx::tc_commit_pair(drained_bar, 1);
                 ptx::mbar_wait_bounded(drained_bar, 0, never_flag, kWaitLimit);
             }
+            __syncwarp();
         }
     } else {
         // ------------------------------ epilogue warps (both CTAs) --------------------------------

@@ -183,6 +183,17 @@ __device__ __forceinline__ void tmem_st_wait() {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
+// True in one lane of the (converged) warp, always the same one.  A branch on it, in code whose values are the same in all lanes (loop
+// counters, kernel parameters, warp_uniform), lets the compiler keep an MMA's operands in uniform registers, where the instruction
+// takes them from; behind `lane == 0` every operand is first moved there: four MMAs and a commit then take 311 clocks of
+// the issuing warp instead of 204.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+    return r != 0;
+}
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 // ---- tcgen05: matrix multiply ---------------------------------------------------------------------
 // D[tmem] (+)= A[smem] * B[smem]^T, int8 x int8 -> int32, one CTA.
 __device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
@@ -319,10 +330,7 @@ __device__ __forceinline__ uint64_t smem_desc_kmajor(uint32_t smem_addr, uint32_
 // The same descriptor with its start-address field moved by `byte_offset` (a multiple of 16 that does not
 // carry out of the 14-bit field): one 32-bit add on the low word.
 __device__ __forceinline__ uint64_t desc_advance(uint64_t desc, uint32_t byte_offset) {
-    uint32_t lo = (uint32_t)desc + (byte_offset >> 4), hi = (uint32_t)(desc >> 32);
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
-    return r;
+    return (desc & 0xFFFFFFFF00000000ull) | ((uint32_t)desc + (byte_offset >> 4));
 }
 
 // Instruction descriptor for kind::i8: signed 8-bit A and B (both K-major), int32 accumulator.
