@@ -77,13 +77,6 @@ __device__ __forceinline__ void st8(float* p, const float* x) {
                  "f"(x[5]), "f"(x[6]), "f"(x[7]), "l"(p) : "memory");
 }
 __device__ __forceinline__ void st4(float* p, const float* x) { __stcs(reinterpret_cast<float4*>(p), make_float4(x[0], x[1], x[2], x[3])); }
-// max(|a|, |b|, m), NaN if any is NaN
-__device__ __forceinline__ float max_abs_nan(float a, float b, float m) {
-    float r;
-    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(fabsf(a)), "f"(fabsf(b)), "f"(m));
-    return r;
-}
-
 // n = 1, and 2 of 8: the kept values and their positions straight from one or two passes of
 // "largest magnitude, first one on equality" (strict >), positions ascending.
 template <int N, int M>
@@ -173,23 +166,31 @@ __device__ __forceinline__ unsigned keep_mask(const float* a) {
 // over the candidates s_j = fl32(s_max * (64 - j) / 64), j = 0 .. ncand-1 (s_max = the ADMM-Max scale;
 // lowest j on equal distance).  The decision is taken on distances held in double, in two steps:
 //
-// 1. All candidates in single precision, in units of s_max: y = |v| / s_max, code magnitude k =
-//    min(rne(y * 64 / (64 - j)), end code of v's sign), d = y - k * (64 - j) / 64, sum of d * d: five
-//    operations per candidate and kept value, four of them as packed pairs.  Per value |d| is within
-//    eps = 2^(b - 1) * 2^-19 of the exact distance: y and 64 / (64 - j) carry relative errors of 1.5 * 2^-23 and 2^-24 and
-//    the real scale s_j one of 2^-24, which move d by less than 2^(b - 1) * 2^-21 when the code is the true one; the
-//    code differs only where the quotient is within 2^(b - 1) * 3 * 2^-23 of a tie, and there the two
-//    distances differ by twice that.  By the triangle inequality the root of the exact E_j is within
-//    eps * sqrt(values) of the root of the computed one, whose sums (at most 80 roundings of non-negative terms) are
+// 1. Bounds of every candidate's distance, in units of s_max: y = |v| / s_max.
+//    4 bits (dist_bounds4): with the nearest codes E_j = sum y^2 - 2 s_j * sum over the thresholds (k - 1/2) s_j of what lies above
+//    them, sum of (y - threshold)+.  The values go, rounded to 2^-16, into bins of 1/32, each with its count and the sum of its
+//    remainders, and sums over the higher bins give all (value - threshold)+ but those of the bin that holds the threshold; these lie
+//    between max(0, f - c t) and f (1 - t / width) (c values of remainders f in sum, the threshold at t; both bounds of a
+//    convex function with given mean), exact for one value.  All thresholds are multiples of 1/128, so everything is whole
+//    numbers.  That is a pass over the values and 8 lookups per candidate in place of 32 evaluations of every value.  1.2 to 1.5
+//    of 32 candidates are left on rows of Gaussian weights; bins of 1/16 left 2 to 3.
+//    8 bits: the row's largest value alone rules out all candidates but the first few (3 to 16; see there); those are evaluated in single
+//    precision: code magnitude k = min(rne(y * 64 / (64 - j)), end code of v's sign), d = y - k * (64 - j) / 64, sum of d * d: five
+//    operations per candidate and kept value, four of them as packed pairs, sums (at most 80 roundings of non-negative terms)
 //    good to 2^-17 relative.
-// 2. A candidate whose lower bound exceeds another's upper bound cannot win.  Usually one is left (about 96 of
-//    100 rows of 768 weights at 4 bits); otherwise those that are left are evaluated in double from the fp32
-//    weights (code from the IEEE quotient, d = v - s_j * code and E += d * d as two FMAs, s_j * code being exact in double) and
-//    compared.  Scales outside [2^-126, 2^125] and non-finite rows skip step 1.
+//    Per value |d| is within eps = 2^(b - 1) * 2^-19 of the exact distance: y and 64 / (64 - j) carry relative errors of 1.5 * 2^-23
+//    and 2^-24 and the real scale s_j one of 2^-24, which move d by less than 2^(b - 1) * 2^-21 when the code is the true one; the
+//    code differs only where the quotient is within 2^(b - 1) * 3 * 2^-23 of a tie, and there the two
+//    distances differ by twice that; the rounding to 2^-16 adds 2^-17, half of eps.  By the triangle inequality the root of the exact E_j
+//    is within eps * sqrt(values) of the root of the computed one.
+// 2. A candidate whose lower bound exceeds another's upper bound cannot win.  Usually one is left; otherwise those that are left are
+//    evaluated in double from the fp32 weights (code from the IEEE quotient, d = v - s_j * code and E += d * d as two FMAs, s_j * code
+//    being exact in double) and compared.  Scales outside [2^-126, 2^125] and non-finite rows skip step 1.
 //
 // A row spans `wpr` warps; the partial sums of its warps are added in a fixed order, so the result is
-// deterministic.  Evaluating every candidate in double took 14.8 instructions per candidate and value, among them
-// a quarter-rate conversion: 85 M weights at 2:4 / 4 bit and 32 candidates, search alone 1050 us before, 405 us now.
+// deterministic.  85 M weights at 2:4 / 4 bit and 32 candidates, search and projection: 461 us with all candidates in single precision,
+// 297 so (12.6 M of 2:4 / 8 bit in rows of 1024 0.63 of the time; 398 shapes and formats 0.71 in the geometric mean, 1.05 at the worst, a
+// matrix of 1 M weights of dense 4 bit).  What bounds it now: instructions (61 % of the issue slots), their fetching among the stalls.
 // ---------------------------------------------------------------------------------------------
 template <int N, int M>
 __device__ __forceinline__ void kept_values(const float* v, float* sel) {
@@ -199,16 +200,14 @@ __device__ __forceinline__ void kept_values(const float* v, float* sel) {
     } else if constexpr ((N == 1) || (N == 2 && M == 8)) {
         unsigned selp[N];
         select_passes<N, M>(v, sel, selp);
+    } else if constexpr (N == 2) {
+        (void)select_2_of_4(v, sel);
     } else {
         float a[M];
 #pragma unroll
         for (int p = 0; p < M; ++p) a[p] = fabsf(v[p]);
         const unsigned mask = keep_mask<N, M>(a);
-        if constexpr (N == 2 && M == 4) {
-            const bool b0 = mask & 1u, b1 = mask & 2u, b2 = mask & 4u, b3 = mask & 8u;
-            sel[0] = b0 ? v[0] : (b1 ? v[1] : v[2]);
-            sel[1] = b3 ? v[3] : (b2 ? v[2] : v[1]);
-        } else {
+        {
 #pragma unroll
             for (int c = 0; c < N; ++c) sel[c] = 0.0f;
 #pragma unroll
@@ -224,144 +223,275 @@ __device__ __forceinline__ void kept_values(const float* v, float* sel) {
 }
 
 
-__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-// Distance of candidate j in double over the warp's part of the row (every lane returns the sum over the lanes).
-template <int N, int M, int BITS>
-__device__ __forceinline__ double dist_exact(const float* v, float smax, int j) {
+// Distance of candidate j in double over the warp's part of the row (every lane returns the sum over the lanes), from the lane's `count` kept
+// values, value i at x[32 i].  A short loop over shared memory: few rows come here, and unrolled over registers its code kept the
+// rest of the kernel out of the instruction cache.  Codes from RN(1 / s_j) as in pack_row, the IEEE division only next to a tie.
+template <int BITS>
+__device__ __noinline__ double dist_exact(const float* x, int count, float smax, int j) {
     constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
     constexpr float kLo = -(float)(1 << (BITS - 1)) - 0.49f, kHi = qmax + 0.49f;
     constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
-    const float sj = __fmul_rn(smax, (float)(64 - j) * 0.015625f);
+    const float sj = __fmul_rn(smax, (float)(64 - j) * 0.015625f), rs = __frcp_rn(sj);
+    const bool fast_ok = sj >= 1.17549435e-38f && sj <= 4.25e37f;
     const double nsd = -(double)sj;
-    double e0 = 0.0, e1 = 0.0;
+    double e[2] = {0.0, 0.0};
+    for (int i = 0; i < count; i += 2) {
 #pragma unroll
-    for (int g = 0; g < 32 / M; ++g) {
-        float x[N];
-        kept_values<N, M>(v + g * M, x);
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-            const float qc = fminf(fmaxf(__fdiv_rn(x[i], sj), kLo), kHi);
-            const float r = __fsub_rn(__fadd_rn(qc, kMagic), kMagic);  // nearest-even integer of qc
-            const double d = fma(nsd, (double)r, (double)x[i]);
-            if ((g * N + i) & 1) e1 = fma(d, d, e1); else e0 = fma(d, d, e0);
+        for (int k = 0; k < 2; ++k) {
+            const float xi = x[32 * (i + k)];
+            float t = __fmaf_rn(xi, rs, kMagic);
+            const float f = fabsf(__fmaf_rn(xi, rs, -__fsub_rn(t, kMagic)));
+            t = fminf(fmaxf(t, kMagic - qmax - 1.0f), kMagic + qmax);
+            if (!(f <= 0.49996948f) || !fast_ok) t = __fadd_rn(fminf(fmaxf(__fdiv_rn(xi, sj), kLo), kHi), kMagic);
+            // the code as a double: 2^52 + 2^31 + code is whole
+            const double r = __dsub_rn(__hiloint2double(0x43300000, (__float_as_int(t) - 0x4B400000) ^ (int)0x80000000), 4503601774854144.0);
+            const double d = fma(nsd, r, (double)xi);
+            e[k] = fma(d, d, e[k]);
         }
     }
-    double e = e0 + e1;
+    double sum = e[0] + e[1];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-    return e;
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    return sum;
 }
 
-// Winning candidate of this warp's row.  `red_e` holds 32 doubles per warp of the block.  Every warp of the block calls it
-// (block-wide barriers when a row spans warps).
-template <int N, int M, int BITS>
+// Bins of dist_bounds4, per warp: 128 of the tail of the negative values, 256 of all; each counts its values and sums their remainders.
+constexpr int kTailBins = 128, kAllBins = 256, kTailFirst = 123;
+struct DistBins {
+    uint32_t bin[kTailBins + kAllBins];  // count << 21 | sum of remainders
+    uint2 above[kTailBins + kAllBins];   // count and sum of the values in higher bins, permuted so that lanes store side by side
+};
+
+// Step 1 of the search at 4 bits: bounds of every candidate's distance (lane j: candidate j), less the sum of squares `q` of the warp's
+// values that all candidates share, in units of s_max^2.  See above.
+template <int N, int M>
+__device__ __forceinline__ void dist_bounds4(const float* x, int steps, int lane, float smax, DistBins& h, double& lo, double& hi, float& q) {
+    constexpr int KS = 8 / M * N;
+    constexpr float kMagic = 12582912.0f;
+    uint4* zero = reinterpret_cast<uint4*>(h.bin);
+#pragma unroll
+    for (int i = 0; i < (kTailBins + kAllBins) / 128; ++i) zero[i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    const float r0 = __frcp_rn(smax);
+    q = 0.0f;
+#pragma unroll
+    for (int st = 0; st < 4; ++st)
+        if (st < steps) {  // steps beyond the warp's columns hold zeros
+#pragma unroll
+            for (int i = 0; i < KS; ++i) {
+                const float t = __fmaf_rn(fabsf(__fmul_rn(x[st * KS + i], r0)), 65536.0f, kMagic);
+                const int y = __float_as_int(t) - 0x4B400000;  // magnitude in units of s_max / 65536, at most 7 * 65536
+                const float yf = __fsub_rn(t, kMagic);
+                q = __fmaf_rn(yf, yf, q);
+                if (y >= 16384) {  // the lowest threshold of all candidates is 33 * 512
+                    const uint32_t w = (uint32_t)(y & 2047) | (1u << 21);
+                    atomicAdd(&h.bin[kTailBins + (y >> 11)], w);
+                    if (x[st * KS + i] < 0.0f && y >= kTailFirst * 2048) atomicAdd(&h.bin[(y >> 11) - kTailFirst], w);
+                }
+            }
+        }
+    __syncwarp();
+    // sums over the higher bins: lane l has bins 8 l .. 8 l + 7 of all values and 4 l .. 4 l + 3 of the tail
+    {
+        uint32_t wa[8], wt[4];
+        *reinterpret_cast<uint4*>(wa) = *reinterpret_cast<const uint4*>(h.bin + kTailBins + 8 * lane);
+        *reinterpret_cast<uint4*>(wa + 4) = *reinterpret_cast<const uint4*>(h.bin + kTailBins + 8 * lane + 4);
+        *reinterpret_cast<uint4*>(wt) = *reinterpret_cast<const uint4*>(h.bin + 4 * lane);
+        uint32_t sa[8], st[4], sum_a = 0, sum_t = 0, cnt = 0;  // cnt: tail << 16 | all (at most 1024 each)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            sa[i] = (wa[i] >> 21) * (uint32_t)((8 * lane + i) << 11) + (wa[i] & 0x1FFFFFu);
+            sum_a += sa[i]; cnt += wa[i] >> 21;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            st[i] = (wt[i] >> 21) * (uint32_t)((4 * lane + i + kTailFirst) << 11) + (wt[i] & 0x1FFFFFu);
+            sum_t += st[i]; cnt += (wt[i] >> 21) << 16;
+        }
+        uint32_t xa = sum_a, xt = sum_t, xc = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t ua = __shfl_down_sync(0xffffffffu, xa, o), ut = __shfl_down_sync(0xffffffffu, xt, o), uc = __shfl_down_sync(0xffffffffu, xc, o);
+            if (lane + o < 32) { xa += ua; xt += ut; xc += uc; }
+        }
+        xa -= sum_a; xt -= sum_t; xc -= cnt;
+        uint32_t ca = xc & 0xFFFFu, ct = xc >> 16;
+#pragma unroll
+        for (int i = 7; i >= 0; --i) {
+            h.above[kTailBins + i * 32 + lane] = make_uint2(ca, xa);
+            ca += wa[i] >> 21; xa += sa[i];
+        }
+#pragma unroll
+        for (int i = 3; i >= 0; --i) {
+            h.above[i * 32 + lane] = make_uint2(ct, xt);
+            ct += wt[i] >> 21; xt += st[i];
+        }
+    }
+    __syncwarp();
+    // sum of (value - threshold) over the values above each of the candidate's thresholds
+    const uint32_t m = 64u - (uint32_t)lane;
+    uint32_t g_lo = 0, g_hi = 0;
+    auto threshold = [&](uint32_t u, uint32_t word, uint2 above) {  // u: the threshold in units of s_max / 128
+        const uint32_t part = u & 3u, c = word >> 21, f = word & 0x1FFFFFu;  // where it stands in its bin; the bin's values
+        const uint32_t full = above.y - u * 512u * above.x;
+        const uint32_t l = (uint32_t)max(0, (int)(f - c * part * 512u)), up = (f * (4u - part) + 3u) >> 2;
+        g_lo += full + l;
+        g_hi += full + (c == 1u ? l : up);
+    };
+#pragma unroll
+    for (uint32_t k = 1; k <= 7; ++k) {
+        const uint32_t u = (2u * k - 1u) * m, b = u >> 2;
+        threshold(u, h.bin[kTailBins + b], h.above[kTailBins + ((b & 7u) << 5) + (b >> 3)]);
+    }
+    const uint32_t u8 = 15u * m, b8 = (u8 >> 2) - kTailFirst;
+    threshold(u8, h.bin[b8], h.above[((b8 & 3u) << 5) + (b8 >> 2)]);
+    lo = -4.76837158203125e-7 * (double)m * (double)g_hi;  // 2 s_j / 65536 = m * 2^-21
+    hi = -4.76837158203125e-7 * (double)m * (double)g_lo;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    q *= 2.3283064365386963e-10f;  // 2^-32
+}
+
+template <int N, int M> constexpr int kKeptBytes = 32 / M * N * 128;  // kept values of a warp
+
+// Winning candidate of this warp's row.  `red_e` holds 32 doubles per warp of the block, `bins` (4 bits) one DistBins, `kept` this warp's
+// kept values (ALIAS: in the place of the bins, once nobody reads them).  Every warp of the block calls it (block-wide barriers when a
+// row spans warps).
+template <int N, int M, int BITS, bool ALIAS>
 __device__ __forceinline__ int dist_search(const float* v, int steps, int lane, int w, int wpr, int row_in_block, bool row_ok,
-                                           float smax, bool bad, int ncand, double* red_e) {
+                                           float smax, bool bad, int ncand, double* red_e, DistBins* bins, float* kept) {
     constexpr int KN = 32 / M * N, KS = KN / 4;       // kept values per lane, and per step
     constexpr float qend = (float)(1 << (BITS - 1));  // magnitude of the negative end code
     constexpr float kMagic = 12582912.0f;             // 1.5 * 2^23: adding it rounds to the nearest-even integer
     constexpr float kEps = qend * 1.9073486328125e-6f;  // 2^(b - 1) * 2^-19
     const float inf = __int_as_float(0x7f800000);
     const bool usable = !bad && smax >= 1.17549435e-38f && smax <= 4.25e37f;  // 1 / s_max is a normal number
-    float mine = inf;  // lane j: candidate j's distance in units of s_max^2
-    if (usable && row_ok) {
-        uint64_t y[KN / 2];
-        float lim[KN];
-        {
-            float x[KN];
-#pragma unroll
-            for (int g = 0; g < 32 / M; ++g) kept_values<N, M>(v + g * M, x + g * N);
-            const float r0 = __frcp_rn(smax);
-#pragma unroll
-            for (int i = 0; i < KN; ++i) lim[i] = kMagic + (x[i] < 0.0f ? qend : qend - 1.0f);
-#pragma unroll
-            for (int i = 0; i < KN / 2; ++i) y[i] = pack_f32x2(fabsf(__fmul_rn(x[2 * i], r0)), fabsf(__fmul_rn(x[2 * i + 1], r0)));
-        }
-        const float my_inv = __frcp_rn((float)(64 - lane) * 0.015625f);  // 64 / (64 - j) of candidate j = lane
-        const uint64_t magic2 = pack_f32x2(kMagic, kMagic), nmagic2 = pack_f32x2(-kMagic, -kMagic);
-        // kTrip candidates a trip, their sums over the lanes by a transposing butterfly: lane l ends up with candidate
-        // kTrip * g + l / (32 / kTrip) of trip g and keeps trip l % (32 / kTrip)'s.  Eight a trip where a lane keeps 16 values (85 M
-        // weights at 2:4 / 4 bit 457 us, with two 504); two where it keeps more or fewer: the body of eight no longer fits
-        // the instruction cache (4:4 / 8 bit 276 -> 260 us), or its registers cost occupancy (1:4 144 -> 126).
-        constexpr int kTrip = KN == 16 ? 8 : 2, kLanes = 32 / kTrip;
-        float kept = inf;
-#pragma unroll 1
-        for (int g = 0; kTrip * g < ncand; ++g) {
-            float e[kTrip];
-#pragma unroll
-            for (int k = 0; k < kTrip; ++k) {
-                const float inv = __shfl_sync(0xffffffffu, my_inv, kTrip * g + k);
-                const float na = (float)(kTrip * g + k - 64) * 0.015625f;  // -(64 - j) / 64
-                const uint64_t inv2 = pack_f32x2(inv, inv), na2 = pack_f32x2(na, na);
-                uint64_t acc = 0;
-                auto add = [&](int i) {
-                    float t0, t1;
-                    unpack_f32x2(fma_f32x2(y[i], inv2, magic2), t0, t1);
-                    const uint64_t code = add_f32x2(pack_f32x2(fminf(t0, lim[2 * i]), fminf(t1, lim[2 * i + 1])), nmagic2);
-                    const uint64_t d = fma_f32x2(na2, code, y[i]);
-                    acc = fma_f32x2(d, d, acc);
-                };
-                if constexpr (KS >= 4) {
-#pragma unroll
-                    for (int st = 0; st < 4; ++st)
-                        if (st < steps) {  // steps beyond the warp's columns hold zeros
-#pragma unroll
-                            for (int i = st * KS / 2; i < (st + 1) * KS / 2; ++i) add(i);
-                        }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < KN / 2; ++i) add(i);
-                }
-                float a0, a1;
-                unpack_f32x2(acc, a0, a1);
-                e[k] = a0 + a1;
-            }
-#pragma unroll
-            for (int h = kTrip / 2; h >= 1; h >>= 1) {
-                const bool up = lane & (kLanes * h);
-#pragma unroll
-                for (int k = 0; k < h; ++k) {
-                    const float keep = up ? e[k + h] : e[k], give = up ? e[k] : e[k + h];
-                    e[k] = keep + __shfl_xor_sync(0xffffffffu, give, kLanes * h);
-                }
-            }
-#pragma unroll
-            for (int o = kLanes / 2; o > 0; o >>= 1) e[0] += __shfl_xor_sync(0xffffffffu, e[0], o);
-            if (lane % kLanes == g) kept = e[0];
-        }
-        mine = __shfl_sync(0xffffffffu, kept, (lane % kTrip) * kLanes + lane / kTrip);  // candidate j to lane j
-    }
-    if (wpr > 1) {
-        float* red_f = reinterpret_cast<float*>(red_e);
-        red_f[w * 32 + lane] = mine;
-        __syncthreads();
-        mine = 0.0f;
-        for (int c = 0; c < wpr; ++c) mine += red_f[(row_in_block * wpr + c) * 32 + lane];
-        __syncthreads();  // the array is used again below
-    }
-    // candidates that the bounds leave
     const float slack = kEps * sqrtf((float)(KN * 32 * wpr));
-    const float root = sqrtf(mine), lo = fmaxf(root - slack, 0.0f);
-    float best = lane < ncand ? (root + slack) * (root + slack) * 1.0000153f : inf;
+    bool left = lane < ncand;
+    float x[KN];  // the lane's kept values, for step 2 in shared memory
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
-    const bool left = lane < ncand && (!usable || lo * lo * 0.9999847f <= best);
+    for (int g = 0; g < 32 / M; ++g) {
+        float group[M];  // opaque copies: the selection of pack_row is otherwise shared with this one and kept over the search, in spilled registers
+#pragma unroll
+        for (int i = 0; i < M; ++i) { group[i] = v[g * M + i]; asm volatile("" : "+f"(group[i])); }
+        kept_values<N, M>(group, x + g * N);
+    }
+    if constexpr (!ALIAS) {
+#pragma unroll
+        for (int i = 0; i < KN; ++i) kept[i * 32 + lane] = x[i];
+    }
+    if constexpr (BITS == 4) {
+        double lo = 0.0, hi = 0.0;
+        float q = 0.0f;
+        if (usable && row_ok) dist_bounds4<N, M>(x, steps, lane, smax, bins[w], lo, hi, q);
+        if (wpr > 1) {
+            double* mine = reinterpret_cast<double*>(bins[w].above);
+            __syncwarp();
+            mine[lane] = lo;
+            mine[32 + lane] = hi;
+            if (lane == 0) mine[64] = (double)q;
+            __syncthreads();
+            lo = hi = 0.0;
+            q = 0.0f;
+            for (int c = 0; c < wpr; ++c) {
+                const double* part = reinterpret_cast<const double*>(bins[row_in_block * wpr + c].above);
+                lo += part[lane];
+                hi += part[32 + lane];
+                q += (float)part[64];
+            }
+            if (ALIAS) __syncthreads();
+        }
+        if constexpr (ALIAS) {
+            static_assert(kKeptBytes<N, M> <= (int)sizeof(DistBins), "kept values in the place of the bins");
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < KN; ++i) kept[i * 32 + lane] = x[i];
+        }
+        // |root of the exact distance - root of the distance of the values as binned| <= slack
+        const float root = sqrtf(fmaxf(q * 1.0000077f + (float)hi, 0.0f) + 1e-3f * slack);
+        const double margin = 1.001 * (double)(slack * (2.0f * root + slack));
+        lo -= margin;
+        hi = lane < ncand ? hi + margin : 1e300;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) hi = fmin(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        left = left && (!usable || lo <= hi);
+    } else {
+        // the row's largest value alone makes candidate j's distance at least (2 j - 1)^2 (its quotient is beyond the end code, 127 or
+        // 128), that of candidate 0 is at most a quarter per kept value
+        const int last = (int)((0.5003f * sqrtf((float)(KS * 32 * steps * wpr)) + 1.0003f) * 0.5f) + 1;
+        const int eval = min(ncand, last + 1);
+        float mine = inf;  // lane j: candidate j's distance in units of s_max^2
+        if (usable && row_ok) {
+            uint64_t y[KN / 2];
+            float lim[KN];
+            {
+                const float r0 = __frcp_rn(smax);
+#pragma unroll
+                for (int i = 0; i < KN; ++i) lim[i] = kMagic + (x[i] < 0.0f ? qend : qend - 1.0f);
+#pragma unroll
+                for (int i = 0; i < KN / 2; ++i) y[i] = ptx::pack_f32x2(fabsf(__fmul_rn(x[2 * i], r0)), fabsf(__fmul_rn(x[2 * i + 1], r0)));
+            }
+            const float my_inv = __frcp_rn((float)(64 - lane) * 0.015625f);  // 64 / (64 - j) of candidate j = lane
+            const uint64_t magic2 = ptx::pack_f32x2(kMagic, kMagic), nmagic2 = ptx::pack_f32x2(-kMagic, -kMagic);
+            // two candidates a trip, their sums over the lanes by a transposing butterfly: lane l ends up with candidate
+            // 2 g + l / 16 of trip g and keeps trip l % 16's
+            constexpr int kTrip = 2, kLanes = 32 / kTrip;
+            float kept = inf;
+#pragma unroll 1
+            for (int g = 0; kTrip * g < eval; ++g) {
+                float e[kTrip];
+#pragma unroll
+                for (int k = 0; k < kTrip; ++k) {
+                    const float inv = __shfl_sync(0xffffffffu, my_inv, kTrip * g + k);
+                    const float na = (float)(kTrip * g + k - 64) * 0.015625f;  // -(64 - j) / 64
+                    const uint64_t inv2 = ptx::pack_f32x2(inv, inv), na2 = ptx::pack_f32x2(na, na);
+                    uint64_t acc = 0;
+                    auto add = [&](int i) {
+                        float t0, t1;
+                        ptx::unpack_f32x2(ptx::fma_f32x2(y[i], inv2, magic2), t0, t1);
+                        const uint64_t code = ptx::add_f32x2(ptx::pack_f32x2(fminf(t0, lim[2 * i]), fminf(t1, lim[2 * i + 1])), nmagic2);
+                        const uint64_t d = ptx::fma_f32x2(na2, code, y[i]);
+                        acc = ptx::fma_f32x2(d, d, acc);
+                    };
+                    if constexpr (KS >= 4) {
+#pragma unroll
+                        for (int st = 0; st < 4; ++st)
+                            if (st < steps) {  // steps beyond the warp's columns hold zeros
+#pragma unroll
+                                for (int i = st * KS / 2; i < (st + 1) * KS / 2; ++i) add(i);
+                            }
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < KN / 2; ++i) add(i);
+                    }
+                    float a0, a1;
+                    ptx::unpack_f32x2(acc, a0, a1);
+                    e[k] = a0 + a1;
+                }
+                const bool up = lane & kLanes;
+                const float keep = up ? e[1] : e[0], give = up ? e[0] : e[1];
+                e[0] = keep + __shfl_xor_sync(0xffffffffu, give, kLanes);
+#pragma unroll
+                for (int o = kLanes / 2; o > 0; o >>= 1) e[0] += __shfl_xor_sync(0xffffffffu, e[0], o);
+                if (lane % kLanes == g) kept = e[0];
+            }
+            mine = __shfl_sync(0xffffffffu, kept, (lane % kTrip) * kLanes + lane / kTrip);  // candidate j to lane j
+        }
+        if (wpr > 1) {
+            float* red_f = reinterpret_cast<float*>(red_e);
+            red_f[w * 32 + lane] = mine;
+            __syncthreads();
+            mine = 0.0f;
+            for (int c = 0; c < wpr; ++c) mine += red_f[(row_in_block * wpr + c) * 32 + lane];
+            __syncthreads();  // the array is used again below
+        }
+        // candidates that the bounds leave
+        const float root = sqrtf(mine), lo = fmaxf(root - slack, 0.0f);
+        float best = lane < ncand ? (root + slack) * (root + slack) * 1.0000153f : inf;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+        left = left && (!usable || lo * lo * 0.9999847f <= best);
+    }
     const unsigned mask = row_ok ? __ballot_sync(0xffffffffu, left) : 1u;
     const bool single = (mask & (mask - 1u)) == 0u;
     if (single && wpr == 1) return __ffs(mask) - 1;
@@ -369,7 +499,7 @@ __device__ __forceinline__ int dist_search(const float* v, int steps, int lane, 
     if (!single) {
         for (unsigned m = mask; m; m &= m - 1u) {
             const int j = __ffs(m) - 1;
-            const double e = dist_exact<N, M, BITS>(v, smax, j);
+            const double e = dist_exact<BITS>(kept + lane, KS * steps, smax, j);
             if (lane == j) exact = e;
         }
     }
@@ -454,7 +584,7 @@ __device__ __forceinline__ float row_max(const float* v, int lane, int w, int wp
                                          uint32_t* status, bool& bad) {
     float amax = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) amax = max_abs_nan(v[2 * i], v[2 * i + 1], amax);
+    for (int i = 0; i < 16; ++i) amax = ptx::max_abs_nan(v[2 * i], v[2 * i + 1], amax);
     bad = __any_sync(0xffffffffu, !(amax <= 3.402823466e+38f));
     if (bad) {
         if (lane == 0 && status) atomicOr(status, NM_STATUS_NONFINITE);
@@ -669,7 +799,7 @@ template <int N, int M, int BITS, bool DENSE_OUT, bool DIST = false>
 __device__ __forceinline__ void pack_finish(const PackJobDev& job, const UnitPos& up, int lane, int w, const float* v,
                                             float* red, const uint16_t* pos48, float* scratch, uint32_t* status,
                                             float* __restrict__ Zout, float* __restrict__ Unext, bool wide, int group_mode, int group_rows,
-                                            double* red_e = nullptr) {
+                                            double* red_e = nullptr, DistBins* bins = nullptr, float* kept = nullptr) {
     const int wpr = 1 << job.wpr_log2;
     bool bad;
     const float amax = row_max(v, lane, w, wpr, up.row_in_block, red, status, bad);
@@ -695,7 +825,7 @@ __device__ __forceinline__ void pack_finish(const PackJobDev& job, const UnitPos
     }
     s = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
     if constexpr (DIST) {  // group_rows carries the number of candidate scales
-        const int best = dist_search<N, M, BITS>(v, up.steps, lane, w, wpr, up.row_in_block, up.row_ok, s, bad, group_rows, red_e);
+        const int best = dist_search<N, M, BITS, false>(v, up.steps, lane, w, wpr, up.row_in_block, up.row_ok, s, bad, group_rows, red_e, bins, kept);
         s = __fmul_rn(s, (float)(64 - best) * 0.015625f);
     }
     if (!up.row_ok) return;
@@ -797,19 +927,19 @@ constexpr int kStagedBlocksPerSm = 3;
 // or six, more of a warp's loads are in flight, but 85 M weights in four formats take 125 / 116 us instead of 104, the
 // 24-layer sweep 436 / 441 instead of 403.  Dense outputs six (738 us; five and four the same).  The search four, and
 // six where a lane keeps at most eight values.
-template <int N, int M, bool DENSE_OUT, bool DIST>
-constexpr int kDirectBlocksPerSm = DIST ? (32 / M * N <= 8 ? 6 : 4) : DENSE_OUT ? 6 : 8;
+template <int N, int M, int BITS, bool DENSE_OUT, bool DIST>
+constexpr int kDirectBlocksPerSm = DIST ? (32 / M * N <= 8 ? 6 : BITS == 4 ? 6 : 4) : DENSE_OUT ? 6 : 8;
 
 constexpr int kFewBlocksPerSm = 5;  // the plain projection of two operands where no SM gets more blocks (see pick_bits)
 
 template <int N, int M, int BITS, int MAXT, bool DENSE_OUT = false, int PIPE = kDirect, bool DIST = false,
-          int PER_SM = kDirectBlocksPerSm<N, M, DENSE_OUT, DIST>>
+          int PER_SM = kDirectBlocksPerSm<N, M, BITS, DENSE_OUT, DIST>>
 __global__ void __launch_bounds__(MAXT, PIPE != kDirect ? kStagedBlocksPerSm : (MAXT == 128 ? PER_SM : 1))
 pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constant__ PackJobInline inl, uint32_t* status,
             float* __restrict__ Zout, float* __restrict__ Unext, const DenseOutDev* __restrict__ dense_jobs,
             int group_mode, int group_rows, unsigned nunits, bool chained) {
     static_assert(PIPE == kDirect || (MAXT == 128 && N <= 2 && !DENSE_OUT && !DIST), "see staged_form");
-    // staged: [warps][2 buffers][W, U][1024] floats.  Then (DIST) [warps][32] doubles, [2][warps] floats for the row maximum, (4:8) the
+    // staged: [warps][2 buffers][W, U][1024] floats.  Then (DIST) [warps][32] doubles, (4 bits) [warps] DistBins, [warps][kept values][32], [2][warps] floats for the row maximum, (4:8) the
     // position table and [warps][8][32] floats, (staged) [warps][2] mbarriers and the abort flag.
     extern __shared__ float4 tile[];
     const int warps = blockDim.x >> 5;
@@ -817,6 +947,10 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
     uint8_t* at = reinterpret_cast<uint8_t*>(tile) + (PIPE == kStaged2 ? warps * 16384 : 0);
     double* red_e = reinterpret_cast<double*>(at);
     if (DIST) at += warps * 256;
+    DistBins* bins = reinterpret_cast<DistBins*>(at);
+    if (DIST && BITS == 4) at += warps * sizeof(DistBins);
+    float* kept = reinterpret_cast<float*>(at) + w * (32 * (32 / M * N));
+    if (DIST) at += warps * kKeptBytes<N, M>;
     float* red = reinterpret_cast<float*>(at);
     at += warps * 8;
     uint16_t* pos48 = nullptr;
@@ -843,7 +977,7 @@ pack_kernel(const PackJobDev* __restrict__ jobs, int njobs, const __grid_constan
         float v[32];
         load_global(job, up, lane, wide, v);
         pack_finish<N, M, BITS, DENSE_OUT, DIST>(job, up, lane, w, v, red, pos48, scratch, status, Zout, Unext, wide, group_mode,
-                                                group_rows, red_e);
+                                                group_rows, red_e, bins, kept);
     } else {
         uint64_t* bars = reinterpret_cast<uint64_t*>(at);                 // [warps][2]
         volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 2 * warps);
@@ -1059,10 +1193,13 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1) dist_scale_kernel(c
                                                                               const __grid_constant__ PackJobInline inl,
                                                                               uint32_t* status, int ncand,
                                                                               int32_t* __restrict__ cand_out) {
-    extern __shared__ float4 tile[];  // [warps][32] doubles, [warps] floats
+    extern __shared__ float4 tile[];  // [warps][32] doubles, (4 bits) [warps] DistBins, [warps][kept values][32], [warps] floats
     const int warps = blockDim.x >> 5;
     double* red_e = reinterpret_cast<double*>(tile);
-    float* red = reinterpret_cast<float*>(red_e + warps * 32);
+    DistBins* bins = reinterpret_cast<DistBins*>(red_e + warps * 32);
+    constexpr bool kAlias = BITS == 4 && MAXT > 128;  // up to 32 warps: room for only one of the two
+    float* kept = kAlias ? reinterpret_cast<float*>(bins + (threadIdx.x >> 5)) : reinterpret_cast<float*>(bins + (BITS == 4 ? warps : 0)) + (threadIdx.x >> 5) * (kKeptBytes<N, M> / 4);
+    float* red = kAlias ? reinterpret_cast<float*>(bins + warps) : reinterpret_cast<float*>(bins + (BITS == 4 ? warps : 0)) + warps * (kKeptBytes<N, M> / 4);
     int index = 0;
     const PackJobDev job = find_job(jobs, njobs, inl, blockIdx.x, index);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1074,7 +1211,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1) dist_scale_kernel(c
     const float amax = row_max(v, lane, w, wpr, up.row_in_block, red, status, bad);
     constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
     const float smax = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
-    const int bj = dist_search<N, M, BITS>(v, up.steps, lane, w, wpr, up.row_in_block, up.row_ok, smax, bad, ncand, red_e);
+    const int bj = dist_search<N, M, BITS, kAlias>(v, up.steps, lane, w, wpr, up.row_in_block, up.row_ok, smax, bad, ncand, red_e, bins, kept);
     if (up.row_ok && up.chunk == 0 && lane == 0) {
         job.scales[up.row] = __fmul_rn(smax, (float)(64 - bj) * 0.015625f);
         if (cand_out) cand_out[up.row] = bj;
@@ -1085,7 +1222,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 4 : 1) dist_scale_kernel(c
 // host side
 // ---------------------------------------------------------------------------------------------
 using PackFnPtr = void (*)(const PackJobDev*, int, const PackJobInline, uint32_t*, float*, float*, const DenseOutDev*, int, int, unsigned, bool);
-struct PackFn { PackFnPtr fn; int form; bool dist = false; };  // kernel, its form (kDirect, kStaged2), with the scale search
+struct PackFn { PackFnPtr fn; int form; size_t search = 0; };  // kernel, its form (kDirect, kStaged2), shared memory of the scale search per warp
 
 // nm_debug_set_option("pack_form"): 0 = automatic, 2 = kStaged2 wherever it exists (blocks of four warps, 1:4, 2:4, 1:8 and 2:8, no
 // dense outputs), anything else = kDirect.
@@ -1186,7 +1323,7 @@ static int launch_table(PackFn k, const PackJobDev* jobs_dev, int njobs, const P
                         const DenseOutDev* dense_jobs, int group_mode, int group_rows, bool chained = false) {
     // buffers and barriers of the staged form, distances of the search, row-maximum slots, the 4:8 tables (see the kernel)
     const bool staged = k.form == kStaged2;
-    const size_t smem = (size_t)warps * ((staged ? 16384 + 16 : 0) + (k.dist ? 32 * sizeof(double) : 0) + 2 * sizeof(float) + 1024) + 512 + 16;
+    const size_t smem = (size_t)warps * ((staged ? 16384 + 16 : 0) + k.search + 2 * sizeof(float) + 1024) + 512 + 16;
     const PackFnPtr fn = k.fn;
     if (smem > 48 * 1024) {  // the attribute is set once per kernel and device
         struct Done { const void* fn; int dev; };
@@ -1297,6 +1434,11 @@ static int launch_grouped_single(const nm_pack_job_t& j, int group_rows, uint32_
                   Z, U_next, nullptr, kGroupScalesGiven, group_rows);
 }
 
+// Shared memory per warp of the scale search.
+static constexpr size_t dist_smem(int bits, int kept_bytes, bool alias = false) {
+    return 32 * sizeof(double) + (bits == 4 ? sizeof(DistBins) : 0) + (alias && bits == 4 ? 0 : (size_t)kept_bytes);
+}
+
 using DistFn = void (*)(const PackJobDev*, int, const PackJobInline, uint32_t*, int, int32_t*);
 
 template <int N, int M>
@@ -1316,9 +1458,10 @@ static DistFn pick_dist(int n, int m, int bits, int warps) {
     return pick_dist_bits<4, 8>(bits, warps);
 }
 
-static int launch_dist(DistFn fn, const PackJobDev* jobs_dev, int njobs, const PackJobDev& single, unsigned blocks,
+static int launch_dist(DistFn fn, size_t search, const PackJobDev* jobs_dev, int njobs, const PackJobDev& single, unsigned blocks,
                        int warps, uint32_t* status, cudaStream_t stream, int ncand, int32_t* cand) {
-    const size_t smem = (size_t)warps * (32 * sizeof(double) + sizeof(float));
+    const size_t smem = (size_t)warps * (search + sizeof(float));
+    if (smem > 48 * 1024) NM_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     PackJobInline inl{};
     inl.j[0] = single;
     fn<<<blocks, warps * 32, smem, stream>>>(jobs_dev, njobs, inl, status, ncand, cand);
@@ -1327,11 +1470,11 @@ static int launch_dist(DistFn fn, const PackJobDev* jobs_dev, int njobs, const P
 }
 
 // Search and projection in one kernel (blocks of four warps): the row stays in registers from the one to the other, so W and U are
-// read once: 85 M weights at 2:4 / 4 bit 533 us against 405 + 156 us for the search followed by the projection.
+// read once.
 template <int N, int M, bool DENSE_OUT>
 static PackFn pick_dist_pack_bits(int bits) {
-    return bits == 8 ? PackFn{(PackFnPtr)pack_kernel<N, M, 8, 128, DENSE_OUT, kDirect, true>, kDirect, true}
-                     : PackFn{(PackFnPtr)pack_kernel<N, M, 4, 128, DENSE_OUT, kDirect, true>, kDirect, true};
+    return bits == 8 ? PackFn{(PackFnPtr)pack_kernel<N, M, 8, 128, DENSE_OUT, kDirect, true>, kDirect, dist_smem(8, kKeptBytes<N, M>)}
+                     : PackFn{(PackFnPtr)pack_kernel<N, M, 4, 128, DENSE_OUT, kDirect, true>, kDirect, dist_smem(4, kKeptBytes<N, M>)};
 }
 
 template <bool DENSE_OUT>
@@ -1349,7 +1492,7 @@ static int launch_dist_single(const nm_pack_job_t& j, int ncand, int32_t* cand, 
     const int warps = std::max(kPackMinWarps, 1 << d.wpr_log2);
     const int rows_per_block = warps >> d.wpr_log2;
     const unsigned blocks = (unsigned)((j.out + rows_per_block - 1) / rows_per_block);
-    return launch_dist(pick_dist(j.n, j.m, j.bits, warps), nullptr, 0, d, blocks, warps, status, stream, ncand, cand);
+    return launch_dist(pick_dist(j.n, j.m, j.bits, warps), dist_smem(j.bits, 32 / (j.n == j.m ? 4 : j.m) * (j.n == j.m ? 4 : j.n) * 128, warps > kPackMinWarps), nullptr, 0, d, blocks, warps, status, stream, ncand, cand);
 }
 
 // One matrix: search and projection.
@@ -1527,7 +1670,7 @@ static int launch_batched(const nm_pack_job_t* jobs, const DenseOutDev* dense, i
                             status, s, nullptr, nullptr, dense_g, kGroupNone, dist_ncand, chained);
         } else {
             if (dist_ncand > 0) {  // the search writes every job's scales, the projection takes them
-                rc = nm::launch_dist(nm::pick_dist(k.n, k.m, k.bits, k.warps), dev, count, nm::PackJobDev{}, group_blocks[g], k.warps,
+                rc = nm::launch_dist(nm::pick_dist(k.n, k.m, k.bits, k.warps), nm::dist_smem(k.bits, 32 / (k.n == k.m ? 4 : k.m) * (k.n == k.m ? 4 : k.n) * 128, k.warps > nm::kPackMinWarps), dev, count, nm::PackJobDev{}, group_blocks[g], k.warps,
                                      status, s, dist_ncand, nullptr);
                 if (rc != NM_OK) return rc;
             }
