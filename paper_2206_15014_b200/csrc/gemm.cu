@@ -59,14 +59,14 @@ constexpr long long kWaitLimit = NM_WAIT_LIMIT;  // SM clocks per device-side wa
 
 // What the epilogue writes: y = fma(acc, sx * sw[o], b[o]) as fp32; the raw int32 accumulators; y re-quantised
 // to 8 bits with a scale fixed ahead of time (Eq. 5, b = 8); y rounded to bfloat16.
-enum { EPI_F32 = 0, EPI_ACC = 1, EPI_Q8 = 2, EPI_BF16 = 3 };
+enum { EPI_F32 = 0, EPI_ACC = 1, EPI_Q8 = 2, EPI_BF16 = 3, EPI_F32MAX = 4 };  // EPI_F32MAX: fp32 and the running max|y|
+template <int EPI> constexpr bool kF32 = EPI == EPI_F32 || EPI == EPI_F32MAX;
 template <int EPI> struct EpiOut { using type = uint32_t; };          // fp32 / int32 move as 32-bit patterns
 template <> struct EpiOut<EPI_Q8> { using type = uint8_t; };
 template <> struct EpiOut<EPI_BF16> { using type = uint16_t; };
-// Narrow outputs leave through [16 tokens][128 channels] tiles that the four warps of a TMEM-lane-quarter
-// group fill together (rows of 128 / 256 bytes instead of 32 / 64): named barriers kNarrowFree + half and
-// kNarrowFull + half order the fills against the one warp that issues the TMA store, kNarrowAgree + half
-// makes the group take a timed-out wait together so that nobody is left alone on a barrier.
+// Narrow outputs leave through [tokens][128 channels] tiles that the four warps of a TMEM-lane-quarter
+// group fill together (rows of 128 / 256 bytes instead of 32 / 64; see narrow_tile): a named barrier per group orders the fills against the
+// one warp that issues the TMA store, kNarrowAgree + half makes the group take a timed-out wait together so that nobody is left alone on it.
 // EPI_Q8 without a branch per value: the code from the reciprocal rsy = RN(1 / sy), exact unless the product sits
 // within 2^-15 of a rounding tie (6 values in 100000), where only the IEEE division decides.  `worst` keeps the largest
 // distance of a product from its rounded integer over a run of values; beyond 0.49996948 the caller fills the run again
@@ -86,7 +86,7 @@ __device__ __forceinline__ uint8_t epi_convert_q8_fast(uint32_t acc, float c_n, 
 __device__ __noinline__ int quantise8_exact_call(float y, float sy) { return quantise8_exact(y, sy); }
 
 template <int EPI> constexpr bool kNarrow = EPI == EPI_Q8 || EPI == EPI_BF16;
-constexpr uint32_t kNarrowFree = 9, kNarrowFull = 11, kNarrowAgree = 13;
+constexpr uint32_t kNarrowGroup = 9, kNarrowAgree = 13;  // named barriers: one per group from kNarrowGroup on
 
 // One output element from an accumulator: fp32 value y, then the narrowing the epilogue kind asks for.
 template <int EPI>
@@ -97,7 +97,7 @@ __device__ __forceinline__ typename EpiOut<EPI>::type epi_convert(uint32_t acc, 
     } else {
         const float y = __fmaf_rn((float)(int)acc, c_n, b_n);
         y_abs = fabsf(y);
-        if constexpr (EPI == EPI_F32) {
+        if constexpr (kF32<EPI>) {
             return __float_as_uint(y);
         } else if constexpr (EPI == EPI_Q8) {
             // the IEEE quotient y / sy rounded half to even and clamped to [-128, 127]
@@ -110,6 +110,160 @@ __device__ __forceinline__ typename EpiOut<EPI>::type epi_convert(uint32_t acc, 
         }
     }
 }
+
+// Four codes of the exact quantiser, for the few values in 10^5 next to a rounding tie: a call, out of the loops' way.
+__device__ __noinline__ uint32_t quantise8_exact4(float y0, float y1, float y2, float y3, float sy) {
+    return (uint32_t)(quantise8_exact(y0, sy) & 0xff) | (uint32_t)(quantise8_exact(y1, sy) & 0xff) << 8 |
+           (uint32_t)(quantise8_exact(y2, sy) & 0xff) << 16 | (uint32_t)(quantise8_exact(y3, sy) & 0xff) << 24;
+}
+
+// One output tile of a group of four epilogue warps (one per TMEM lane quarter q) as int8 or bfloat16.
+//
+// A warp reads 16 tokens of its 32 channels from the accumulator in the fragment layout of stmatrix (a thread has two neighbouring
+// tokens of four channels), converts them in pairs, and writes them transposed, 16 bytes of a token's row at a time, into the group's
+// staging tile [UNIT tokens][128 channels], in the 128-byte swizzle of the store's tensor map, so that no two rows of a matrix meet in a
+// bank.  With a lane per channel every value took a conversion and a store instruction of its own: 4 instructions for a bfloat16, 11 for an
+// exact int8 code, 2.2 and 5.3 so: 1024 -> 3072, 20000 tokens 41.1 -> 38.5 us (bfloat16); 768 -> 768, 16384 tokens 17.1 -> 14.6 (int8); int8
+// outputs over 337 shapes and formats 0.93 of the time, bfloat16 0.97.
+// int8: t = fma(y, rsy, 1.5 * 2^23) rounds the product to the nearest-even integer, which saturates to the code; `d` is the product's
+// distance from it, and within 2^-15 of a tie (or NaN) the IEEE division decides.
+//
+// acc: TMEM address of the tile's first column in this warp's lane quarter.  c, b: scale and bias of channels lane / 4 + 8 i of the quarter.
+// valid: tokens of the tile that exist.  stage: the group's two staging tiles.  release(): this warp has read its accumulator.
+template <int EPI, int UNIT, bool HINT, typename Release>
+__device__ __forceinline__ void narrow_tile(uint32_t acc, int columns, int valid, int group, int groups, uint32_t bar, uint32_t stage,
+                                            uint32_t& n_stores, int q, int lane, const float (&c)[4], const float (&b)[4], float sy, float rsy,
+                                            const CUtensorMap* tmap_y, int n0, int t0, int out, uint64_t policy, Release release) {
+    constexpr uint32_t ROW = 128, BOX = UNIT * ROW, TILE = (EPI == EPI_BF16 ? 2 : 1) * BOX;  // bfloat16: two boxes of 64 channels
+    constexpr float kMagic = 12582912.0f;
+    const int units = (min(valid, columns) + UNIT - 1) / UNIT;  // units that hold tokens (the same for the whole group)
+    const uint64_t c01[2] = {ptx::pack_f32x2(c[0], c[0]), ptx::pack_f32x2(c[2], c[2])}, c23[2] = {ptx::pack_f32x2(c[1], c[1]), ptx::pack_f32x2(c[3], c[3])};
+    const uint64_t b01[2] = {ptx::pack_f32x2(b[0], b[0]), ptx::pack_f32x2(b[2], b[2])}, b23[2] = {ptx::pack_f32x2(b[1], b[1]), ptx::pack_f32x2(b[3], b[3])};
+    if (group >= units) release();
+#pragma unroll 1
+    for (int u = group; u < units; u += groups) {
+        const uint32_t tile = stage + (n_stores & 1u) * TILE;
+#pragma unroll
+        for (int h = 0; h < UNIT / 16; ++h) {
+            uint32_t r[16];
+            ptx::tmem_ld_16x256x2(acc + u * UNIT + 16 * h, r);
+            ptx::tmem_ld_16x256x2(acc + (16u << 16) + u * UNIT + 16 * h, r + 8);
+            ptx::tmem_ld_wait();
+            if (h == UNIT / 16 - 1 && u + groups >= units) release();
+            uint32_t pk[EPI == EPI_Q8 ? 4 : 8];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {  // k = 2 * (lane half) + column group
+                const uint32_t* x = r + 4 * k;
+                const uint64_t y01 = ptx::fma_f32x2(ptx::pack_f32x2((float)(int)x[0], (float)(int)x[1]), c01[k >> 1], b01[k >> 1]);
+                const uint64_t y23 = ptx::fma_f32x2(ptx::pack_f32x2((float)(int)x[2], (float)(int)x[3]), c23[k >> 1], b23[k >> 1]);
+                float y0, y1, y2, y3;
+                ptx::unpack_f32x2(y01, y0, y1);
+                ptx::unpack_f32x2(y23, y2, y3);
+                if constexpr (EPI == EPI_BF16) {
+                    pk[2 * k] = ptx::cvt_bf16x2(y0, y1);
+                    pk[2 * k + 1] = ptx::cvt_bf16x2(y2, y3);
+                } else {
+                    const uint64_t rs2 = ptx::pack_f32x2(rsy, rsy), magic2 = ptx::pack_f32x2(kMagic, kMagic), minus2 = ptx::pack_f32x2(-1.0f, -1.0f);
+                    const uint64_t t01 = ptx::fma_f32x2(y01, rs2, magic2), t23 = ptx::fma_f32x2(y23, rs2, magic2);
+                    float d0, d1, d2, d3, t[4];
+                    ptx::unpack_f32x2(ptx::fma_f32x2(y01, rs2, ptx::fma_f32x2(t01, minus2, magic2)), d0, d1);
+                    ptx::unpack_f32x2(ptx::fma_f32x2(y23, rs2, ptx::fma_f32x2(t23, minus2, magic2)), d2, d3);
+                    ptx::unpack_f32x2(t01, t[0], t[1]);
+                    ptx::unpack_f32x2(t23, t[2], t[3]);
+                    auto code = [&](int i) { return __float_as_int(t[i]) - 0x4B400000; };
+                    pk[k] = ptx::pack_sat_s8(code(0), code(1), ptx::pack_sat_s8(code(2), code(3), 0u));
+                    if (!(ptx::max_abs_nan(d2, d3, ptx::max_abs_nan(d0, d1, 0.0f)) <= 0.49996948f)) pk[k] = quantise8_exact4(y0, y1, y2, y3, sy);
+                }
+            }
+            if (h == 0) {
+                if (q == 0 && lane == 0) ptx::bulk_wait_group_read<1>();  // the store before the last has read this tile
+                ptx::named_bar_sync(bar, 128);
+            }
+            const uint32_t token = lane & 7;
+            if constexpr (EPI == EPI_BF16) {
+#pragma unroll
+                for (int g = 0; g < 2; ++g)  // matrix i: channels 8 i .. 8 i + 7 of the quarter, eight tokens
+                    ptx::stmatrix_trans_b16(tile + (q >> 1) * BOX + (16 * h + 8 * g + token) * ROW + ((((q & 1) * 4 + (lane >> 3)) ^ token) << 4),
+                                            pk[2 * g], pk[2 * g + 1], pk[4 + 2 * g], pk[4 + 2 * g + 1]);
+            } else {  // matrix i: channels 16 (i % 2) .. + 15 of the quarter, tokens 8 (i / 2) .. + 7
+                ptx::stmatrix_trans_b8(tile + (16 * h + 8 * (lane >> 4) + token) * ROW + (((q * 2 + ((lane >> 3) & 1)) ^ token) << 4), pk[0], pk[2], pk[1], pk[3]);
+            }
+        }
+        ptx::fence_proxy_async_smem();
+        ptx::named_bar_sync(bar, 128);
+        if (q == 0 && lane == 0) {
+#pragma unroll
+            for (int x = 0; x < (int)(TILE / BOX); ++x) {
+                if (x && n0 + 64 * x >= out) break;
+                if (HINT) ptx::tma_store_2d_hint(tmap_y, n0 + 64 * x, t0 + u * UNIT, tile + x * BOX, policy);
+                else ptx::tma_store_2d(tmap_y, n0 + 64 * x, t0 + u * UNIT, tile + x * BOX);
+            }
+            ptx::bulk_commit_group();
+        }
+        ++n_stores;
+    }
+}
+
+// One output tile where TMA cannot store the rows of Y (not whole units of 16 bytes): a lane per channel, 32 tokens of an accumulator at a
+// time, stored straight from the registers.  Staged in shared memory and written by rows of 128 channels, with a quarter of the partial
+// sectors, it was slower: bfloat16 1024 -> 1002, 8192 tokens, packed 4-bit codes 28 us against 18, fp32 23 against 17.  Out of the kernels' main
+// loops, so that those stay short.
+template <int EPI, typename Release>
+__device__ __forceinline__ void direct_tile(uint32_t acc, int columns, int valid, int group, int groups, float c_n, float b_n, float sy, float rsy,
+                                            typename EpiOut<EPI>::type* Y, int t0, int n, int out, float& amax, Release release) {
+    using OT = typename EpiOut<EPI>::type;
+    const int chunks = (min(valid, columns) + 31) >> 5;
+    if (group >= chunks) release();
+#pragma unroll 1
+    for (int c = group; c < chunks; c += groups) {
+        uint32_t r[32];
+        ptx::tmem_ld_32x32(acc + c * 32, r);
+        ptx::tmem_ld_wait();
+        if (c + groups >= chunks) release();
+        const int count = min(32, valid - c * 32);
+        OT* dst = Y + (size_t)(t0 + c * 32) * out + n;
+        auto conv = [&](int j) -> OT {
+            float y_abs = 0.0f;
+            OT o;
+            if constexpr (EPI == EPI_Q8) {
+                float worst = 0.0f;
+                o = epi_convert_q8_fast(r[j], c_n, b_n, rsy, worst);
+                if (!(worst <= 0.49996948f)) o = (OT)(int8_t)quantise8_exact_call(__fmaf_rn((float)(int)r[j], c_n, b_n), sy);
+            } else {
+                o = epi_convert<EPI>(r[j], c_n, b_n, sy, rsy, y_abs);
+            }
+            if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, y_abs);
+            return o;
+        };
+        if (n < out) {
+            if (count == 32) {  // no branch per store
+#pragma unroll
+                for (int j = 0; j < 32; ++j) dst[(size_t)j * out] = conv(j);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    if (j < count) dst[(size_t)j * out] = conv(j);
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// Weight scale and bias of the four channels of a thread in narrow_tile; `first` is the lane quarter's first channel.
+__device__ __forceinline__ void narrow_fetch(const float* sw, const float* bias, int first, int lane, int out, float (&s)[4], float (&b)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int n = first + (lane >> 2) + 8 * i;
+        s[i] = n < out ? sw[n] : 0.0f;
+        b[i] = n < out && bias ? bias[n] : 0.0f;
+    }
+}
+__device__ __forceinline__ void narrow_constants(const float* sw, const float* bias, float sx, int first, int lane, int out, float (&c)[4], float (&b)[4]) {
+    narrow_fetch(sw, bias, first, lane, out, c, b);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) c[i] = __fmul_rn(sx, c[i]);
+}
+
 // Pieces of metadata (16 bytes: one row, one 128-wide k-block) that a metadata warp of the one-CTA kernel has in flight (four
 // in the forms with weight-building warps, which are short of registers).  One at a time, each load waited for before its
 // store to TMEM, they held up the first MMA: 384 tokens 1024 -> 3072 7.6 -> 6.6 us, 4096 -> 1024 16.8 -> 14.7, 64 tokens
@@ -466,6 +620,8 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         const float rsy = EPI == EPI_Q8 ? __frcp_rn(p.sy) : 0.0f;
         int scaled_out_tile = -1;
         uint32_t n_stores = 0;
+        int narrow_out_tile = -1;  // whose constants nc, nb are (narrow outputs)
+        float nc[4], nb[4];
         bool ok = true;
 
         // Index metadata of this lane's weight row for the whole reduction; rows past the end get a valid "positions 0,1" pattern,
@@ -522,10 +678,14 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
             const int tile = tile_begin + i, out_tile = tile / p.n_tok_tiles, buf = i & 1;
             const int n0 = out_tile * kBM, n = n0 + row, t0 = (tile % p.n_tok_tiles) * BN;
             if (SPARSE && i == 0 && half == 0) load_meta(out_tile, true);
-            if (!(RES && SPARSE) && EPI != EPI_ACC && out_tile != scaled_out_tile) {  // channel constants: once per output tile
+            if (!(RES && SPARSE) && EPI != EPI_ACC && !(kNarrow<EPI> && p.tma_store) && out_tile != scaled_out_tile) {  // channel constants: once per output tile
                 scaled_out_tile = out_tile;
                 c_n = n < p.out ? __fmul_rn(sx, p.sw[n]) : 0.0f;
                 b_n = n < p.out && p.bias ? p.bias[n] : 0.0f;
+            }
+            if (kNarrow<EPI> && p.tma_store && out_tile != narrow_out_tile) {
+                narrow_out_tile = out_tile;
+                narrow_constants(p.sw, p.bias, sx, n0 + q * 32, lane, p.out, nc, nb);
             }
             bool got = ptx::mbar_wait_bounded(acc_full_bar(buf), (i >> 1) & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
@@ -538,104 +698,72 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 if (next_out_tile != out_tile) load_meta(next_out_tile, false);  // MMAs of this output tile are done
             }
             const bool n_ok = n < p.out;
-            if (RES && SPARSE && EPI != EPI_ACC && out_tile != scaled_out_tile) {  // (see load_meta)
+            if (RES && SPARSE && EPI != EPI_ACC && !(kNarrow<EPI> && p.tma_store) && out_tile != scaled_out_tile) {  // (see load_meta)
                 scaled_out_tile = out_tile;
                 c_n = n_ok ? __fmul_rn(sx, p.sw[n]) : 0.0f;
                 b_n = n_ok && p.bias ? p.bias[n] : 0.0f;
             }
-            const int nact = min(CH, (p.tokens - t0 + 31) >> 5);  // chunks that hold tokens (warp-uniform)
-            // Accumulator chunks are read one ahead of their conversion (two register buffers); the
-            // transform kernels, short of registers with their extra warps, read each chunk when it is due.
-            // narrow outputs: the conversion code of one chunk is long; the chunk loop stays a loop (one copy of that code
-            // instead of CI, which no longer fit the instruction cache) and every chunk is read when it is due
-            constexpr int RB = (XF || kNarrow<EPI>) ? 1 : 2;
-            uint32_t r[RB][32];
-            if (half >= nact) release_acc(buf);
-            else if (RB == 2) ptx::tmem_ld_32x32(lane_taddr + buf * BN + half * 32, r[0]);
-#pragma unroll (kNarrow<EPI> ? 1 : CI)
-            for (int ci = 0; ci < CI; ++ci) {
-                const int c = half + ci * EWH, tc0 = t0 + c * 32;
-                if (c < nact) {
-                    if (RB == 1) ptx::tmem_ld_32x32(lane_taddr + buf * BN + c * 32, r[0]);
-                    ptx::tmem_ld_wait();
-                    if (c + EWH >= nact) release_acc(buf);
-                    else if (RB == 2) ptx::tmem_ld_32x32(lane_taddr + buf * BN + (c + EWH) * 32, r[(ci + 1) & (RB - 1)]);
-                    // conversion of accumulator column j of this chunk; jmax = outputs of this lane that exist
-                    const int jmax = n_ok ? min(32, p.tokens - tc0) : 0;
-                    using OT = typename EpiOut<EPI>::type;
-                    auto conv = [&](int j) -> OT {
-                        float y_abs;
-                        const OT o = epi_convert<EPI>(r[ci & (RB - 1)][j], c_n, b_n, p.sy, rsy, y_abs);
-                        if constexpr (EPI == EPI_F32) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
-                        return o;
-                    };
-                    // The two store paths are separate loops: a branch inside the unrolled loop costs a
-                    // pipeline refill per column (measured ~30 clk each), far more than its arithmetic.
-                    if (p.tma_store) {
+            if (!p.tma_store) {
+                direct_tile<EPI>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, c_n, b_n, p.sy, rsy,
+                                 reinterpret_cast<typename EpiOut<EPI>::type*>(kF32<EPI> ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW), t0, n, p.out, amax,
+                                 [&] { release_acc(buf); });
+                continue;
+            }
+            if constexpr (kNarrow<EPI>) {
+                constexpr uint32_t kPerGroup = (EPI == EPI_BF16 ? 2 : 1) * 4096;
+                narrow_tile<EPI, 16, false>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, kNarrowGroup + half, ptx::smem_u32(store_stage) + half * kPerGroup,
+                                            n_stores, q, lane, nc, nb, p.sy, rsy, &tmap_y, n0, t0, p.out, 0, [&] { release_acc(buf); });
+                continue;
+            }
+            if constexpr (!kNarrow<EPI>) {
+                const int nact = min(CH, (p.tokens - t0 + 31) >> 5);  // chunks that hold tokens (warp-uniform)
+                // Accumulator chunks are read one ahead of their conversion (two register buffers); the
+                // transform kernels, short of registers with their extra warps, read each chunk when it is due.
+                constexpr int RB = XF ? 1 : 2;
+                uint32_t r[RB][32];
+                if (half >= nact) release_acc(buf);
+                else if (RB == 2) ptx::tmem_ld_32x32(lane_taddr + buf * BN + half * 32, r[0]);
+#pragma unroll
+                for (int ci = 0; ci < CI; ++ci) {
+                    const int c = half + ci * EWH, tc0 = t0 + c * 32;
+                    if (c < nact) {
+                        if (RB == 1) ptx::tmem_ld_32x32(lane_taddr + buf * BN + c * 32, r[0]);
+                        ptx::tmem_ld_wait();
+                        if (c + EWH >= nact) release_acc(buf);
+                        else if (RB == 2) ptx::tmem_ld_32x32(lane_taddr + buf * BN + (c + EWH) * 32, r[(ci + 1) & (RB - 1)]);
+                        // conversion of accumulator column j of this chunk; jmax = outputs of this lane that exist
+                        const int jmax = n_ok ? min(32, p.tokens - tc0) : 0;
+                        using OT = typename EpiOut<EPI>::type;
+                        auto conv = [&](int j) -> OT {
+                            float y_abs;
+                            const OT o = epi_convert<EPI>(r[ci & (RB - 1)][j], c_n, b_n, p.sy, 0.0f, y_abs);
+                            if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
+                            return o;
+                        };
                         // two stores of 16 tokens each, through alternating staging tiles: while one is
                         // being read by its TMA store the other is filled
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             if (tc0 + 16 * h >= p.tokens) continue;  // warp-uniform (and the same in all warps of a group)
-                            if constexpr (kNarrow<EPI>) {
-                                OT* sb = reinterpret_cast<OT*>(store_stage) + (half * 2 + (n_stores & 1u)) * (16 * 128);
-                                if (q == 0 && lane == 0) ptx::bulk_wait_group_read<1>();  // the store before the last has read this tile
-                                ptx::named_bar_sync(kNarrowFree + half, 128);
-                                if constexpr (EPI == EPI_Q8) {
-                                    float worst = 0.0f;
+                            OT* sb = reinterpret_cast<OT*>(my_stage + (n_stores & 1u) * 512);
+                            if (lane == 0) ptx::bulk_wait_group_read<1>();  // the store before the last has read this tile
+                            __syncwarp();
 #pragma unroll
-                                    for (int j = 0; j < 16; ++j)
-                                        sb[j * 128 + q * 32 + lane] = epi_convert_q8_fast(r[ci & (RB - 1)][16 * h + j], c_n, b_n, rsy, worst);
-                                    if (__any_sync(0xffffffffu, !(worst <= 0.49996948f))) {  // rare (3 % of the runs)
-                                        // find the values in question again; the exact division decides those
-#pragma unroll
-                                        for (int j = 0; j < 16; ++j) {
-                                            float w1 = 0.0f;
-                                            (void)epi_convert_q8_fast(r[ci & (RB - 1)][16 * h + j], c_n, b_n, rsy, w1);
-                                            if (!(w1 <= 0.49996948f))
-                                                sb[j * 128 + q * 32 + lane] = (uint8_t)(int8_t)quantise8_exact_call(
-                                                    __fmaf_rn((float)(int)r[ci & (RB - 1)][16 * h + j], c_n, b_n), p.sy);
-                                        }
-                                    }
-                                } else {
-#pragma unroll
-                                    for (int j = 0; j < 16; ++j) sb[j * 128 + q * 32 + lane] = conv(16 * h + j);
-                                }
-                                ptx::fence_proxy_async_smem();
-                                ptx::named_bar_sync(kNarrowFull + half, 128);
-                                if (q == 0 && lane == 0) {
-                                    ptx::tma_store_2d(&tmap_y, n0, tc0 + 16 * h, ptx::smem_u32(sb));
-                                    ptx::bulk_commit_group();
-                                }
-                                ++n_stores;
-                            } else {
-                                OT* sb = reinterpret_cast<OT*>(my_stage + (n_stores & 1u) * 512);
-                                if (lane == 0) ptx::bulk_wait_group_read<1>();  // the store before the last has read this tile
-                                __syncwarp();
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) sb[j * 32 + lane] = conv(16 * h + j);
-                                ptx::fence_proxy_async_smem();
-                                __syncwarp();
-                                if (lane == 0) {
-                                    ptx::tma_store_2d(&tmap_y, n0 + q * 32, tc0 + 16 * h, ptx::smem_u32(sb));
-                                    ptx::bulk_commit_group();
-                                }
-                                ++n_stores;
+                            for (int j = 0; j < 16; ++j) sb[j * 32 + lane] = conv(16 * h + j);
+                            ptx::fence_proxy_async_smem();
+                            __syncwarp();
+                            if (lane == 0) {
+                                ptx::tma_store_2d(&tmap_y, n0 + q * 32, tc0 + 16 * h, ptx::smem_u32(sb));
+                                ptx::bulk_commit_group();
                             }
-                        }
-                    } else {  // output rows not 16-byte aligned: lane = channel, j = token
-                        OT* dst = reinterpret_cast<OT*>(EPI == EPI_F32 ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW) + (size_t)tc0 * p.out + n;
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const OT o = conv(j);
-                            if (j < jmax) dst[(size_t)j * p.out] = o;
+                            ++n_stores;
                         }
                     }
                 }
             }
         }
-        if (lane == 0) ptx::bulk_wait_group<0>();
-        if (EPI == EPI_F32 && p.absmax) {
+        if (lane == 0) ptx::bulk_wait_group_read<0>();  // the stores have read the staging tiles
+        if (EPI == EPI_F32MAX) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
             if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(p.absmax), __float_as_uint(amax));
@@ -670,7 +798,6 @@ template <bool BUILD> constexpr int kPairThreadsOf = kPairThreads + (BUILD ? 32 
 // The second eight sit behind the gate warp, where the builder warps of the BUILD form are.
 template <int EPI, bool RES, bool BUILD> constexpr int kPairEpiWarps = (kNarrow<EPI> && RES && !BUILD) ? 16 : kEpiWarps;
 template <int EPI, bool RES, bool BUILD> constexpr int kPairThreadsFor = kPairThreadsOf<BUILD> + 32 * (kPairEpiWarps<EPI, RES, BUILD> - kEpiWarps);
-constexpr uint32_t kNarrowGroup = 9;  // named barriers 9-12: one per group of four epilogue warps in that form
 constexpr int kPairMaxStages = 7;   // the relay cycles through 8 named barriers (ids 1-8; 9-14 serve the narrow-output epilogue)
 
 constexpr int kPairResStages = 4;   // stages of weights a CTA can keep resident (1024 reduction elements at 2:4)
@@ -970,6 +1097,8 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
         const float rsy = EPI == EPI_Q8 ? __frcp_rn(p.sy) : 0.0f;
         int scaled_out_tile = -1;
         uint32_t n_stores = 0;
+        int narrow_out_tile = -1;  // whose constants nc, nb are (narrow outputs)
+        float nc[4], nb[4];
         bool ok = true;
 
         auto load_meta = [&](int out_tile) {
@@ -1005,6 +1134,10 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
             const int out_tile = tc.o, tok_tile = tc.t, buf = i & 1;
             const int n0 = out_tile * (2 * kBM) + (int)rank * kBM, n = n0 + row, t0 = tok_tile * BN;
             if (SPARSE && i == 0 && half == 0) load_meta(out_tile);
+            if (kNarrow<EPI> && p.tma_store && out_tile != narrow_out_tile) {
+                narrow_out_tile = out_tile;
+                narrow_constants(p.sw, p.bias, sx, n0 + q * 32, lane, p.out, nc, nb);
+            }
             bool got = ptx::mbar_wait_bounded(acc_full_bar(buf), (i >> 1) & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
             if (!ok && lane == 0) raise_timeout();
@@ -1019,176 +1152,76 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                 if (next_out_tile != out_tile) load_meta(next_out_tile);
             }
             const bool n_ok = n < p.out;
-            if (EPI != EPI_ACC && out_tile != scaled_out_tile) {  // channel constants: fetched once per output tile
+            if (EPI != EPI_ACC && !(kNarrow<EPI> && p.tma_store) && out_tile != scaled_out_tile) {  // channel constants: fetched once per output tile
                 scaled_out_tile = out_tile;
                 c_n = n_ok ? __fmul_rn(sx, p.sw[n]) : 0.0f;
                 b_n = n_ok && p.bias ? p.bias[n] : 0.0f;
             }
-            if constexpr (EW == 16) {
-                // Four groups of four warps (one per TMEM lane quarter); group g takes the 16-token units g, g + 4, ... of the
-                // tile: reads 16 accumulator columns, fills its quarter of the group's [16 tokens][128 channels] staging tile
-                // (two per group, used alternately), and the group's warp of lane quarter 0 issues the store.
-                using OT = typename EpiOut<EPI>::type;
-                constexpr int UNITS = BN / 16;
-                const int nunits = min(UNITS, (p.tokens - t0 + 15) >> 4);  // units that hold tokens (the same for the whole group)
-                const uint32_t gbar = kNarrowGroup + half;
-                bool released = false;
-#pragma unroll 1
-                for (int u = half; u < nunits; u += 4) {
-                    const int tc0 = t0 + 16 * u;
-                    uint32_t r[16];
-                    ptx::tmem_ld_32x16(lane_taddr + buf * BN + 16 * u, r);
-                    ptx::tmem_ld_wait();
-                    NM_TRACE_EPI_ADD(0);
-                    if (u + 4 >= nunits) { release_acc(buf); released = true; }
-                    if (p.tma_store) {
-                        OT* sb = reinterpret_cast<OT*>(store_stage) + (half * 2 + (n_stores & 1u)) * (16 * 128);
-                        if (q == 0 && lane == 0) ptx::bulk_wait_group_read<1>();  // the store before the last has read this tile
-                        ptx::named_bar_sync(gbar, 128);
-                        NM_TRACE_EPI_ADD(1);
-                        if constexpr (EPI == EPI_Q8) {
-                            float worst = 0.0f;
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) sb[j * 128 + q * 32 + lane] = epi_convert_q8_fast(r[j], c_n, b_n, rsy, worst);
-                            if (__any_sync(0xffffffffu, !(worst <= 0.49996948f))) {  // rare (3 % of the runs)
-                                // find the values in question again; the exact division decides those
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) {
-                                    float w1 = 0.0f;
-                                    (void)epi_convert_q8_fast(r[j], c_n, b_n, rsy, w1);
-                                    if (!(w1 <= 0.49996948f))
-                                        sb[j * 128 + q * 32 + lane] =
-                                            (uint8_t)(int8_t)quantise8_exact_call(__fmaf_rn((float)(int)r[j], c_n, b_n), p.sy);
-                                }
-                            }
-                        } else {
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) {
-                                float y_abs;
-                                sb[j * 128 + q * 32 + lane] = epi_convert<EPI>(r[j], c_n, b_n, p.sy, rsy, y_abs);
-                            }
-                        }
-                        NM_TRACE_EPI_ADD(2);
-                        ptx::fence_proxy_async_smem();
-                        ptx::named_bar_sync(gbar, 128);
-                        NM_TRACE_EPI_ADD(3);
-                        if (q == 0 && lane == 0) {
-                            ptx::tma_store_2d_hint(&tmap_y, n0, tc0, ptx::smem_u32(sb), stream_out);
-                            ptx::bulk_commit_group();
-                        }
-                        NM_TRACE_EPI_ADD(4);
-                        ++n_stores;
-                    } else {
-                        const int jmax = n_ok ? min(16, p.tokens - tc0) : 0;  // outputs of this lane that exist
-                        OT* dst = reinterpret_cast<OT*>(p.NARROW) + (size_t)tc0 * p.out + n;
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            float y_abs;
-                            const OT o = epi_convert<EPI>(r[j], c_n, b_n, p.sy, rsy, y_abs);
-                            if (j < jmax) dst[(size_t)j * p.out] = o;
-                        }
-                    }
-                }
-                if (!released) release_acc(buf);
+            if (!p.tma_store) {
+                direct_tile<EPI>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, c_n, b_n, p.sy, rsy,
+                                 reinterpret_cast<typename EpiOut<EPI>::type*>(kF32<EPI> ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW), t0, n, p.out, amax,
+                                 [&] { release_acc(buf); });
+                continue;
+            }
+            if constexpr (kNarrow<EPI>) {
+                constexpr uint32_t kPerGroup = (EPI == EPI_BF16 ? 2 : 1) * 4096;
+                narrow_tile<EPI, 16, true>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, kNarrowGroup + half, ptx::smem_u32(store_stage) + half * kPerGroup,
+                                           n_stores, q, lane, nc, nb, p.sy, rsy, &tmap_y, n0, t0, p.out, stream_out, [&] { release_acc(buf); });
                 if (ew == 0 && lane == 0) { NM_TRACE_TILE(i, 1); NM_TRACE_EPI_FLUSH(i); }
                 continue;
             }
-            const int nact = min(CH, (p.tokens - t0 + 31) >> 5);
-            // chunks are read one ahead of their conversion; with the builder warps present registers are short and
-            // every chunk is read when it is due
-            constexpr int RB = (BUILD || kNarrow<EPI>) ? 1 : 2;  // narrow outputs: see the one-CTA kernel
-            uint32_t r[RB][32];
-            if (half >= nact) release_acc(buf);
-            else if (RB == 2) ptx::tmem_ld_32x32(lane_taddr + buf * BN + half * 32, r[0]);
-#pragma unroll (kNarrow<EPI> ? 1 : CI)
-            for (int ci = 0; ci < CI; ++ci) {
-                const int c = half + ci * EWH, tc0 = t0 + c * 32;
-                if (c < nact) {
-                    if (RB == 1) ptx::tmem_ld_32x32(lane_taddr + buf * BN + c * 32, r[0]);
-                    ptx::tmem_ld_wait();
-                    NM_TRACE_EPI_ADD(0);
-                    if (c + EWH >= nact) release_acc(buf);
-                    else if (RB == 2) ptx::tmem_ld_32x32(lane_taddr + buf * BN + (c + EWH) * 32, r[(ci + 1) & (RB - 1)]);
-                    const int jmax = n_ok ? min(32, p.tokens - tc0) : 0;  // outputs of this lane that exist
-                    using OT = typename EpiOut<EPI>::type;
-                    auto conv = [&](int j) -> OT {
-                        float y_abs;
-                        const OT o = epi_convert<EPI>(r[ci & (RB - 1)][j], c_n, b_n, p.sy, rsy, y_abs);
-                        if constexpr (EPI == EPI_F32) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
-                        return o;
-                    };
-                    if (p.tma_store) {  // separate branch-free loops for the two store paths
+            if constexpr (!kNarrow<EPI>) {
+                const int nact = min(CH, (p.tokens - t0 + 31) >> 5);
+                // chunks are read one ahead of their conversion; with the builder warps present registers are short and
+                // every chunk is read when it is due
+                constexpr int RB = BUILD ? 1 : 2;
+                uint32_t r[RB][32];
+                if (half >= nact) release_acc(buf);
+                else if (RB == 2) ptx::tmem_ld_32x32(lane_taddr + buf * BN + half * 32, r[0]);
+#pragma unroll
+                for (int ci = 0; ci < CI; ++ci) {
+                    const int c = half + ci * EWH, tc0 = t0 + c * 32;
+                    if (c < nact) {
+                        if (RB == 1) ptx::tmem_ld_32x32(lane_taddr + buf * BN + c * 32, r[0]);
+                        ptx::tmem_ld_wait();
+                        NM_TRACE_EPI_ADD(0);
+                        if (c + EWH >= nact) release_acc(buf);
+                        else if (RB == 2) ptx::tmem_ld_32x32(lane_taddr + buf * BN + (c + EWH) * 32, r[(ci + 1) & (RB - 1)]);
+                        const int jmax = n_ok ? min(32, p.tokens - tc0) : 0;  // outputs of this lane that exist
+                        using OT = typename EpiOut<EPI>::type;
+                        auto conv = [&](int j) -> OT {
+                            float y_abs;
+                            const OT o = epi_convert<EPI>(r[ci & (RB - 1)][j], c_n, b_n, p.sy, 0.0f, y_abs);
+                            if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
+                            return o;
+                        };
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {  // 16 tokens per store, alternating staging tiles
                             if (tc0 + 16 * h >= p.tokens) continue;  // warp-uniform (and the same in all warps of a group)
-                            if constexpr (kNarrow<EPI>) {  // one [16 tokens][128 channels] tile per four warps
-                                OT* sb = reinterpret_cast<OT*>(store_stage) + (half * 2 + (n_stores & 1u)) * (16 * 128);
-                                if (q == 0 && lane == 0) ptx::bulk_wait_group_read<1>();  // the store before the last has read this tile
-                                ptx::named_bar_sync(kNarrowFree + half, 128);
-                                NM_TRACE_EPI_ADD(1);
-                                if constexpr (EPI == EPI_Q8) {
-                                    float worst = 0.0f;
+                            OT* sb = reinterpret_cast<OT*>(my_stage + (NB == 2 ? (n_stores & 1u) * 512 : 0));
+                            if (lane == 0) ptx::bulk_wait_group_read<NB - 1>();  // the store that last used this tile has read it
+                            __syncwarp();
+                            NM_TRACE_EPI_ADD(1);
 #pragma unroll
-                                    for (int j = 0; j < 16; ++j)
-                                        sb[j * 128 + q * 32 + lane] = epi_convert_q8_fast(r[ci & (RB - 1)][16 * h + j], c_n, b_n, rsy, worst);
-                                    if (__any_sync(0xffffffffu, !(worst <= 0.49996948f))) {  // rare (3 % of the runs)
-                                        // find the values in question again; the exact division decides those
-#pragma unroll
-                                        for (int j = 0; j < 16; ++j) {
-                                            float w1 = 0.0f;
-                                            (void)epi_convert_q8_fast(r[ci & (RB - 1)][16 * h + j], c_n, b_n, rsy, w1);
-                                            if (!(w1 <= 0.49996948f))
-                                                sb[j * 128 + q * 32 + lane] = (uint8_t)(int8_t)quantise8_exact_call(
-                                                    __fmaf_rn((float)(int)r[ci & (RB - 1)][16 * h + j], c_n, b_n), p.sy);
-                                        }
-                                    }
-                                } else {
-#pragma unroll
-                                    for (int j = 0; j < 16; ++j) sb[j * 128 + q * 32 + lane] = conv(16 * h + j);
-                                }
-                                NM_TRACE_EPI_ADD(2);
-                                ptx::fence_proxy_async_smem();
-                                ptx::named_bar_sync(kNarrowFull + half, 128);
-                                NM_TRACE_EPI_ADD(3);
-                                if (q == 0 && lane == 0) {
-                                    ptx::tma_store_2d(&tmap_y, n0, tc0 + 16 * h, ptx::smem_u32(sb));
-                                    ptx::bulk_commit_group();
-                                }
-                                NM_TRACE_EPI_ADD(4);
-                                ++n_stores;
-                            } else {
-                                OT* sb = reinterpret_cast<OT*>(my_stage + (NB == 2 ? (n_stores & 1u) * 512 : 0));
-                                if (lane == 0) ptx::bulk_wait_group_read<NB - 1>();  // the store that last used this tile has read it
-                                __syncwarp();
-                                NM_TRACE_EPI_ADD(1);
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) sb[j * 32 + lane] = conv(16 * h + j);
-                                NM_TRACE_EPI_ADD(2);
-                                ptx::fence_proxy_async_smem();
-                                __syncwarp();
-                                NM_TRACE_EPI_ADD(3);
-                                if (lane == 0) {
-                                    ptx::tma_store_2d_hint(&tmap_y, n0 + q * 32, tc0 + 16 * h, ptx::smem_u32(sb), stream_out);
-                                    ptx::bulk_commit_group();
-                                }
-                                NM_TRACE_EPI_ADD(4);
-                                ++n_stores;
+                            for (int j = 0; j < 16; ++j) sb[j * 32 + lane] = conv(16 * h + j);
+                            NM_TRACE_EPI_ADD(2);
+                            ptx::fence_proxy_async_smem();
+                            __syncwarp();
+                            NM_TRACE_EPI_ADD(3);
+                            if (lane == 0) {
+                                ptx::tma_store_2d_hint(&tmap_y, n0 + q * 32, tc0 + 16 * h, ptx::smem_u32(sb), stream_out);
+                                ptx::bulk_commit_group();
                             }
-                        }
-                    } else {
-                        OT* dst = reinterpret_cast<OT*>(EPI == EPI_F32 ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW) + (size_t)tc0 * p.out + n;
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const OT o = conv(j);
-                            if (j < jmax) dst[(size_t)j * p.out] = o;
+                            NM_TRACE_EPI_ADD(4);
+                            ++n_stores;
                         }
                     }
                 }
             }
             if (ew == 0 && lane == 0) { NM_TRACE_TILE(i, 1); NM_TRACE_EPI_FLUSH(i); }
         }
-        if (lane == 0) ptx::bulk_wait_group<0>();
-        if (EPI == EPI_F32 && p.absmax) {
+        if (lane == 0) ptx::bulk_wait_group_read<0>();  // the stores have read the staging tiles
+        if (EPI == EPI_F32MAX) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
             if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(p.absmax), __float_as_uint(amax));
@@ -1264,16 +1297,18 @@ struct LinearArgs {
 // through TMA when the output can be described by a tensor map (16-byte aligned base and row pitch);
 // otherwise *tma_store is cleared, the threads store directly and the map describes X as a stand-in.
 template <int EPI>
-static int make_store_map(CUtensorMap* ty, const LinearArgs& a, bool* tma_store, uint32_t box_rows = 16, uint32_t box_cols = 0) {
+static int make_store_map(CUtensorMap* ty, const LinearArgs& a, bool* tma_store, uint32_t box_rows = 16) {
     const nm_packed_t& W = *a.W;
     constexpr uint32_t es = (uint32_t)sizeof(typename EpiOut<EPI>::type);
-    void* ybase = EPI == EPI_F32 ? (void*)a.Y : EPI == EPI_ACC ? (void*)a.ACC : a.NARROW;
+    void* ybase = kF32<EPI> ? (void*)a.Y : EPI == EPI_ACC ? (void*)a.ACC : a.NARROW;
     *tma_store = aligned(ybase, 16) && ((size_t)W.out * es) % 16 == 0;
-    const CUtensorMapDataType dt = EPI == EPI_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : EPI == EPI_ACC ? CU_TENSOR_MAP_DATA_TYPE_INT32
+    const CUtensorMapDataType dt = kF32<EPI> ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : EPI == EPI_ACC ? CU_TENSOR_MAP_DATA_TYPE_INT32
                                  : EPI == EPI_Q8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     if (!*tma_store)
         return make_map(ty, a.X, (uint64_t)a.tokens, (uint64_t)W.in / 4, 16, 32, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_DATA_TYPE_INT32, 4);
-    return make_map(ty, ybase, (uint64_t)a.tokens, (uint64_t)W.out, box_rows, box_cols ? box_cols : (kNarrow<EPI> ? 128 : 32), CU_TENSOR_MAP_SWIZZLE_NONE, dt, es);
+    // narrow outputs: rows of 128 bytes in the swizzle of narrow_tile
+    return make_map(ty, ybase, (uint64_t)a.tokens, (uint64_t)W.out, box_rows, kNarrow<EPI> ? 128 / es : 32,
+                    kNarrow<EPI> ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, dt, es);
 }
 
 template <bool SPARSE, int BN, int EPI, int WSRC>
@@ -1706,7 +1741,7 @@ static int pick_bn(const LinearArgs& a) {
     } else {
         // Sparse-target formats with a short reduction and work for every SM pair: the CTA-pair kernel with the weights
         // rebuilt once per output tile into its resident region (32-bit outputs).
-        if constexpr (SPARSE && (EPI == EPI_F32 || EPI == EPI_ACC)) {
+        if constexpr (SPARSE && (kF32<EPI> || EPI == EPI_ACC)) {
             const long long pair_tiles = (long long)((a.W->out + 2 * kBM - 1) / (2 * kBM)) * ((a.tokens + 191) / 192);
             if (a.W->in <= kPairResStages * PairCfg<true, 192>::KB && pair_tiles >= sms / 2 && !(pair_tiles > sms / 2 && one_wave(a)) &&
                 !g_opt.no_pair && !g_opt.no_resident)
@@ -1764,7 +1799,7 @@ static int run_linear(const LinearArgs& a, int epi) {
     if (epi == EPI_BF16 && !aligned(a.NARROW, 2)) return NM_ERR_ALIGN;
     if (a.tokens == 0 || W.out == 0) return NM_OK;
     switch (epi) {
-        case EPI_F32: return run_linear_epi<EPI_F32>(a, xform, sparse);
+        case EPI_F32: return a.absmax ? run_linear_epi<EPI_F32MAX>(a, xform, sparse) : run_linear_epi<EPI_F32>(a, xform, sparse);
         case EPI_ACC: return run_linear_epi<EPI_ACC>(a, xform, sparse);
         case EPI_Q8: return run_linear_epi<EPI_Q8>(a, xform, sparse);
         default: return run_linear_epi<EPI_BF16>(a, xform, sparse);

@@ -185,7 +185,7 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
         const float rsy = EPI == EPI_Q8 ? __frcp_rn(p.sy) : 0.0f;
         float amax = 0.0f;
         using OT = typename EpiOut<EPI>::type;
-        OT* const Y = reinterpret_cast<OT*>(EPI == EPI_F32 ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW);
+        OT* const Y = reinterpret_cast<OT*>(kF32<EPI> ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW);
         for (int ch = half; ch < chunks; ch += 2) {
             const int col = rank * slice + ch * 8, t = t0 + col;
             if (t >= p.tokens) break;
@@ -210,12 +210,12 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
                 } else {
                     float y_abs;
                     o = epi_convert<EPI>(r[j], c_n, b_n, p.sy, rsy, y_abs);
-                    if constexpr (EPI == EPI_F32) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
+                    if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
                 }
                 if (j < jmax) dst[(size_t)j * p.out] = o;
             }
         }
-        if (EPI == EPI_F32 && p.absmax) {
+        if (EPI == EPI_F32MAX) {
 #pragma unroll
             for (int s = 16; s > 0; s >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, s));
             if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(p.absmax), __float_as_uint(amax));

@@ -361,9 +361,8 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
         // ------------------------------ epilogue warps (both CTAs) --------------------------------
         // Warps 2-5 read block 0's accumulator, warps 6-9 block 1's; each its TMEM lane quarter, all BN columns.
         constexpr int CH = BN / 32;
-        // narrow outputs leave through staging tiles that a block's four warps share; for 32-bit outputs that form (one
+        // narrow outputs leave through staging tiles that a block's four warps share (narrow_tile); for 32-bit outputs that form (one
         // 16 KB tile per block) was measured slower than a tile per warp (FFN2 alone 44.6 against 42.5 us)
-        constexpr bool kGroupEpi = kNarrow<EPI>;
         const int ew = warp - 2, q = warp & 3, blk = ew >> 2;
         const uint32_t acc_taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)blk * BN;
         uint32_t* my_stage = reinterpret_cast<uint32_t*>(store_stage + ew * 4096);
@@ -373,6 +372,8 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
         float amax = 0.0f, c_n = 0.0f, b_n = 0.0f;
         const float rsy = EPI == EPI_Q8 ? __frcp_rn(p.sy) : 0.0f;
         uint32_t n_stores = 0;
+        int narrow_out_tile = -1;  // whose constants nc, nb are (narrow outputs)
+        float nc[4], nb[4];
         int scaled_out_tile = -1;
         bool ok = true;
         auto release_acc = [&]() {  // this warp has read all it needs from the accumulator
@@ -384,129 +385,72 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
             const TileCoord tc = tile_coord(tile_begin + i, p.n_tok_tiles, p.n_out_tiles, p.band);
             const int nw = tc.o * (2 * Cfg::A_ROWS) + (int)rank * Cfg::A_ROWS + blk * kBM + q * 32;  // first channel of this warp
             const int n = nw + lane, t0 = tc.t * BN;
+            if (kNarrow<EPI> && p.tma_store && tc.o != narrow_out_tile) {
+                narrow_out_tile = tc.o;
+                narrow_constants(p.sw, p.bias, sx, nw, lane, p.out, nc, nb);
+            }
             bool got = ptx::mbar_wait_bounded(acc_full_bar(blk), (uint32_t)i & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
             if (!ok && lane == 0) raise_timeout();
-            if constexpr (kGroupEpi) ok = ptx::named_bar_and(kWideNarrowBar + blk, 128, ok);  // the block's four warps stop together
+            if constexpr (kNarrow<EPI>) ok = ptx::named_bar_and(kWideNarrowBar + blk, 128, ok);  // the block's four warps stop together
             if (!ok) break;
             ptx::tc_fence_after();
             if (ew == 0 && lane == 0) NM_TRACE_TILE(i, 0);
             if (ew == 4 && lane == 0) NM_TRACE_TILE(i, 2);
             const bool n_ok = n < p.out;
-            if (EPI != EPI_ACC && tc.o != scaled_out_tile) {  // channel constants: fetched once per output tile
+            if (EPI != EPI_ACC && !(kNarrow<EPI> && p.tma_store) && tc.o != scaled_out_tile) {  // channel constants: fetched once per output tile
                 scaled_out_tile = tc.o;
                 c_n = n_ok ? __fmul_rn(sx, p.sw[n]) : 0.0f;
                 b_n = n_ok && p.bias ? p.bias[n] : 0.0f;
             }
             const int nact = min(CH, (p.tokens - t0 + 31) >> 5);  // chunks that hold tokens (warp-uniform)
-            if constexpr (kGroupEpi) {
-                // int8 / bfloat16 outputs: the four warps of a block fill one [32 tokens][128 channels] staging tile per chunk
-                // together (two tiles per block, used alternately: rows of 128 / 256 bytes for the store), the warp of lane
-                // quarter 0 issues the store.  One named barrier per block orders the fills against the store.
-                using OT = typename EpiOut<EPI>::type;
-                const uint32_t gbar = kWideNarrowBar + blk;
-                const int n0b = nw - q * 32;  // first channel of the block
-                if (nact == 0) release_acc();
-#pragma unroll 1
-                for (int c = 0; c < nact; ++c) {
-                    const int tc0 = t0 + c * 32;
-                    uint32_t r[32];
-                    ptx::tmem_ld_32x32(acc_taddr + c * 32, r);
-                    ptx::tmem_ld_wait();
-                    if (c + 1 >= nact) release_acc();
-                    if (p.tma_store) {
-                        constexpr int NBUF = sizeof(OT) == 4 ? 1 : 2;  // 32 KB of staging: one 16 KB tile per block, or two smaller ones
-                        OT* sb = reinterpret_cast<OT*>(store_stage) + (blk * NBUF + (NBUF == 2 ? (n_stores & 1u) : 0u)) * (32 * 128);
-                        const int jmax = n_ok ? min(32, p.tokens - tc0) : 0;  // outputs of this lane that exist
-                        if (q == 0 && lane == 0) ptx::bulk_wait_group_read<NBUF - 1>();  // the store that last used this tile has read it
-                        ptx::named_bar_sync(gbar, 128);
-                        OT* mine = sb + q * 32 + lane;
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            if constexpr (EPI == EPI_Q8) {
-                                float worst = 0.0f;
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) mine[(16 * h + j) * 128] = epi_convert_q8_fast(r[16 * h + j], c_n, b_n, rsy, worst);
-                                if (__any_sync(0xffffffffu, !(worst <= 0.49996948f))) {  // rare (3 % of the runs)
-                                    // find the values in question again; the exact division decides those
-#pragma unroll
-                                    for (int j = 0; j < 16; ++j) {
-                                        float w1 = 0.0f;
-                                        (void)epi_convert_q8_fast(r[16 * h + j], c_n, b_n, rsy, w1);
-                                        if (!(w1 <= 0.49996948f))
-                                            mine[(16 * h + j) * 128] =
-                                                (uint8_t)(int8_t)quantise8_exact_call(__fmaf_rn((float)(int)r[16 * h + j], c_n, b_n), p.sy);
-                                    }
-                                }
-                            } else {
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) {
-                                    float y_abs;
-                                    mine[(16 * h + j) * 128] = epi_convert<EPI>(r[16 * h + j], c_n, b_n, p.sy, rsy, y_abs);
-                                    if constexpr (EPI == EPI_F32) amax = fmaxf(amax, 16 * h + j < jmax ? y_abs : 0.0f);
-                                }
-                            }
-                        }
-                        ptx::fence_proxy_async_smem();
-                        ptx::named_bar_sync(gbar, 128);
-                        if (q == 0 && lane == 0) {
-                            ptx::tma_store_2d_hint(&tmap_y, n0b, tc0, ptx::smem_u32(sb), stream_out);
-                            ptx::bulk_commit_group();
-                        }
-                        ++n_stores;
-                    } else {
-                        const int jmax = n_ok ? min(32, p.tokens - tc0) : 0;  // outputs of this lane that exist
-                        OT* dst = reinterpret_cast<OT*>(EPI == EPI_F32 ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW) + (size_t)tc0 * p.out + n;
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            float y_abs;
-                            const OT o = epi_convert<EPI>(r[j], c_n, b_n, p.sy, rsy, y_abs);
-                            if constexpr (EPI == EPI_F32) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
-                            if (j < jmax) dst[(size_t)j * p.out] = o;
-                        }
-                    }
-                }
+            if (!p.tma_store) {
+                direct_tile<EPI>(acc_taddr, BN, p.tokens - t0, 0, 1, c_n, b_n, p.sy, rsy,
+                                 reinterpret_cast<typename EpiOut<EPI>::type*>(kF32<EPI> ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW), t0, n, p.out, amax, release_acc);
+                continue;
+            }
+            if constexpr (kNarrow<EPI>) {
+                constexpr uint32_t kPerBlock = (EPI == EPI_BF16 ? 2 : 1) * 8192;
+                narrow_tile<EPI, 32, true>(acc_taddr, BN, p.tokens - t0, 0, 1, kWideNarrowBar + blk, ptx::smem_u32(store_stage) + blk * kPerBlock, n_stores,
+                                           q, lane, nc, nb, p.sy, rsy, &tmap_y, nw - q * 32, t0, p.out, stream_out, release_acc);
                 if (ew == 0 && lane == 0) NM_TRACE_TILE(i, 1);
                 if (ew == 4 && lane == 0) NM_TRACE_TILE(i, 3);
                 continue;
             }
-            constexpr int RB = W4 ? 1 : 2;  // chunk read one ahead of its conversion, except where registers are short
-            uint32_t r[RB][32];
-            if (nact == 0) release_acc();
-            else if (RB == 2) ptx::tmem_ld_32x32(acc_taddr, r[0]);
+            if constexpr (!kNarrow<EPI>) {
+                constexpr int RB = W4 ? 1 : 2;  // chunk read one ahead of its conversion, except where registers are short
+                uint32_t r[RB][32];
+                if (nact == 0) release_acc();
+                else if (RB == 2) ptx::tmem_ld_32x32(acc_taddr, r[0]);
 #pragma unroll
-            for (int c = 0; c < CH; ++c) {
-                const int tc0 = t0 + c * 32;
-                if (c < nact) {
-                    if (RB == 1) ptx::tmem_ld_32x32(acc_taddr + c * 32, r[0]);
-                    ptx::tmem_ld_wait();
-                    if (c + 1 >= nact) release_acc();
-                    else if (RB == 2) ptx::tmem_ld_32x32(acc_taddr + (c + 1) * 32, r[(c + 1) & (RB - 1)]);
-                    const int jmax = n_ok ? min(32, p.tokens - tc0) : 0;  // outputs of this lane that exist
-                    auto conv = [&](int j) -> uint32_t {
-                        float y_abs;
-                        const uint32_t o = epi_convert<EPI>(r[c & (RB - 1)][j], c_n, b_n, p.sy, 0.0f, y_abs);
-                        if constexpr (EPI == EPI_F32) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
-                        return o;
-                    };
-                    if (p.tma_store) {  // separate branch-free loops for the two store paths
+                for (int c = 0; c < CH; ++c) {
+                    const int tc0 = t0 + c * 32;
+                    if (c < nact) {
+                        if (RB == 1) ptx::tmem_ld_32x32(acc_taddr + c * 32, r[0]);
+                        ptx::tmem_ld_wait();
+                        if (c + 1 >= nact) release_acc();
+                        else if (RB == 2) ptx::tmem_ld_32x32(acc_taddr + (c + 1) * 32, r[(c + 1) & (RB - 1)]);
+                        const int jmax = n_ok ? min(32, p.tokens - tc0) : 0;  // outputs of this lane that exist
+                        using OT = typename EpiOut<EPI>::type;
+                        auto conv = [&](int j) -> OT {
+                            float y_abs;
+                            const OT o = epi_convert<EPI>(r[c & (RB - 1)][j], c_n, b_n, p.sy, 0.0f, y_abs);
+                            if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
+                            return o;
+                        };
                         // rows of the tile past the last token are clipped by the store
                         if (lane == 0) ptx::bulk_wait_group_read<0>();  // the store before this one has read the tile
                         __syncwarp();
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) my_stage[j * 32 + lane] = conv(j);
+                        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) my_stage[(16 * h + j) * 32 + lane] = conv(16 * h + j);
+                        }
                         ptx::fence_proxy_async_smem();
                         __syncwarp();
                         if (lane == 0) {
                             ptx::tma_store_2d_hint(&tmap_y, nw, tc0, ptx::smem_u32(my_stage), stream_out);
                             ptx::bulk_commit_group();
-                        }
-                    } else {
-                        uint32_t* dst = reinterpret_cast<uint32_t*>(EPI == EPI_F32 ? (void*)p.Y : (void*)p.ACC) + (size_t)tc0 * p.out + n;
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const uint32_t o = conv(j);
-                            if (j < jmax) dst[(size_t)j * p.out] = o;
                         }
                     }
                 }
@@ -514,8 +458,8 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
             if (ew == 0 && lane == 0) NM_TRACE_TILE(i, 1);
             if (ew == 4 && lane == 0) NM_TRACE_TILE(i, 3);
         }
-        if (lane == 0) ptx::bulk_wait_group<0>();
-        if (EPI == EPI_F32 && p.absmax) {
+        if (lane == 0) ptx::bulk_wait_group_read<0>();  // the stores have read the staging tiles
+        if (EPI == EPI_F32MAX) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
             if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(p.absmax), __float_as_uint(amax));

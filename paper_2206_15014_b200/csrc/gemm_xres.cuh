@@ -280,7 +280,9 @@ nm_gemm_xres_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
         // channel constants of a tile are fetched while the one before it is converted
         auto scale_of = [&](int tile_o) { const int n = tile_o * (2 * kBM) + (int)rank * kBM + row; return EPI != EPI_ACC && n < p.out ? p.sw[n] : 0.0f; };
         auto bias_of = [&](int tile_o) { const int n = tile_o * (2 * kBM) + (int)rank * kBM + row; return EPI != EPI_ACC && p.bias && n < p.out ? p.bias[n] : 0.0f; };
-        float sw_next = scale_of(o), b_next = bias_of(o);
+        float sw_next = 0.0f, b_next = 0.0f, ns_next[4], nb_next[4];
+        if (kNarrow<EPI> && p.tma_store) narrow_fetch(p.sw, p.bias, o * (2 * kBM) + (int)rank * kBM + q * 32, lane, p.out, ns_next, nb_next);
+        else { sw_next = scale_of(o); b_next = bias_of(o); }
 
         NM_TRACE_EPI_DECL;
         for (int i = 0; i < tile_count && ok; ++i) {
@@ -295,99 +297,49 @@ nm_gemm_xres_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
             if (ew == 0 && lane == 0) NM_TRACE_TILE(i, 0);
             NM_TRACE_EPI_MARK();
             const bool n_ok = n < p.out;
-            const float c_n = __fmul_rn(sx, sw_next), b_n = b_next;
-            sw_next = scale_of(o); b_next = bias_of(o);
-            if constexpr (EW == 16) {
-                // Four groups of four warps (one per TMEM lane quarter); group g takes the 16-token units g, g + 4, ... of the
-                // tile: reads 16 accumulator columns, fills its quarter of the group's [16 tokens][128 channels] staging tile
-                // (two per group, used alternately), and the group's warp of lane quarter 0 issues the store.
-                using OT = typename EpiOut<EPI>::type;
-                constexpr int UNITS = BN / 16;
-                const int nunits = min(UNITS, (p.tokens - t0 + 15) >> 4);  // units that hold tokens (the same for the whole group)
-                const uint32_t gbar = kNarrowGroup + half;
-                bool released = false;
-#pragma unroll 1
-                for (int u = half; u < nunits; u += 4) {
-                    const int tc0 = t0 + 16 * u;
-                    uint32_t r[16];
-                    ptx::tmem_ld_32x16(lane_taddr + buf * BN + 16 * u, r);
-                    ptx::tmem_ld_wait();
-                    NM_TRACE_EPI_ADD(0);
-                    if (u + 4 >= nunits) { release_acc(buf); released = true; }
-                    if (p.tma_store) {
-                        OT* sb = reinterpret_cast<OT*>(store_stage) + (half * 2 + (n_stores & 1u)) * (16 * 128);
-                        if (q == 0 && lane == 0) ptx::bulk_wait_group_read<1>();  // the store before the last has read this tile
-                        ptx::named_bar_sync(gbar, 128);
-                        NM_TRACE_EPI_ADD(1);
-                        if constexpr (EPI == EPI_Q8) {
-                            float worst = 0.0f;
+            if (!p.tma_store) {
+                const float c_n = __fmul_rn(sx, sw_next), b_n = b_next;
+                sw_next = scale_of(o); b_next = bias_of(o);
+                direct_tile<EPI>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, c_n, b_n, p.sy, rsy,
+                                 reinterpret_cast<typename EpiOut<EPI>::type*>(kF32<EPI> ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW), t0, n, p.out, amax,
+                                 [&] { release_acc(buf); });
+                continue;
+            }
+            if constexpr (kNarrow<EPI>) {
+                float nc[4], nb[4];
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) sb[j * 128 + q * 32 + lane] = epi_convert_q8_fast(r[j], c_n, b_n, rsy, worst);
-                            if (__any_sync(0xffffffffu, !(worst <= 0.49996948f))) {  // rare (3 % of the runs)
-                                // find the values in question again; the exact division decides those
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) {
-                                    float w1 = 0.0f;
-                                    (void)epi_convert_q8_fast(r[j], c_n, b_n, rsy, w1);
-                                    if (!(w1 <= 0.49996948f))
-                                        sb[j * 128 + q * 32 + lane] =
-                                            (uint8_t)(int8_t)quantise8_exact_call(__fmaf_rn((float)(int)r[j], c_n, b_n), p.sy);
-                                }
-                            }
-                        } else {
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) {
-                                float y_abs;
-                                sb[j * 128 + q * 32 + lane] = epi_convert<EPI>(r[j], c_n, b_n, p.sy, rsy, y_abs);
-                            }
-                        }
-                        NM_TRACE_EPI_ADD(2);
-                        ptx::fence_proxy_async_smem();
-                        ptx::named_bar_sync(gbar, 128);
-                        NM_TRACE_EPI_ADD(3);
-                        if (q == 0 && lane == 0) {
-                            ptx::tma_store_2d_hint(&tmap_y, n0, tc0, ptx::smem_u32(sb), stream_out);
-                            ptx::bulk_commit_group();
-                        }
-                        NM_TRACE_EPI_ADD(4);
-                        ++n_stores;
-                    } else {
-                        const int jmax = n_ok ? min(16, p.tokens - tc0) : 0;  // outputs of this lane that exist
-                        OT* dst = reinterpret_cast<OT*>(p.NARROW) + (size_t)tc0 * p.out + n;
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            float y_abs;
-                            const OT o = epi_convert<EPI>(r[j], c_n, b_n, p.sy, rsy, y_abs);
-                            if (j < jmax) dst[(size_t)j * p.out] = o;
-                        }
-                    }
-                }
-                if (!released) release_acc(buf);
+                for (int k = 0; k < 4; ++k) { nc[k] = __fmul_rn(sx, ns_next[k]); nb[k] = nb_next[k]; }
+                narrow_fetch(p.sw, p.bias, o * (2 * kBM) + (int)rank * kBM + q * 32, lane, p.out, ns_next, nb_next);
+                constexpr uint32_t kPerGroup = (EPI == EPI_BF16 ? 2 : 1) * 4096;
+                narrow_tile<EPI, 16, true>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, kNarrowGroup + half, ptx::smem_u32(store_stage) + half * kPerGroup,
+                                           n_stores, q, lane, nc, nb, p.sy, rsy, &tmap_y, n0, t0, p.out, stream_out, [&] { release_acc(buf); });
                 if (ew == 0 && lane == 0) { NM_TRACE_TILE(i, 1); NM_TRACE_EPI_FLUSH(i); }
                 continue;
             }
-            const int nact = min(CH, (p.tokens - t0 + 31) >> 5);
-            // chunks are read one ahead of their conversion
-            uint32_t r[2][32];
-            if (half >= nact) release_acc(buf);
-            else ptx::tmem_ld_32x32(lane_taddr + buf * BN + half * 32, r[0]);
+            if constexpr (!kNarrow<EPI>) {
+                const float c_n = __fmul_rn(sx, sw_next), b_n = b_next;
+                sw_next = scale_of(o); b_next = bias_of(o);
+                const int nact = min(CH, (p.tokens - t0 + 31) >> 5);
+                // chunks are read one ahead of their conversion
+                uint32_t r[2][32];
+                if (half >= nact) release_acc(buf);
+                else ptx::tmem_ld_32x32(lane_taddr + buf * BN + half * 32, r[0]);
 #pragma unroll
-            for (int ci = 0; ci < CI; ++ci) {
-                const int c = half + ci * EWH, tc0 = t0 + c * 32;
-                if (c < nact) {
-                    ptx::tmem_ld_wait();
-                    NM_TRACE_EPI_ADD(0);
-                    if (c + EWH >= nact) release_acc(buf);
-                    else ptx::tmem_ld_32x32(lane_taddr + buf * BN + (c + EWH) * 32, r[(ci + 1) & 1]);
-                    const int jmax = n_ok ? min(32, p.tokens - tc0) : 0;  // outputs of this lane that exist
-                    using OT = typename EpiOut<EPI>::type;
-                    auto conv = [&](int j) -> OT {
-                        float y_abs;
-                        const OT o = epi_convert<EPI>(r[ci & 1][j], c_n, b_n, p.sy, rsy, y_abs);
-                        if constexpr (EPI == EPI_F32) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
-                        return o;
-                    };
-                    if (p.tma_store) {  // separate branch-free loops for the two store paths
+                for (int ci = 0; ci < CI; ++ci) {
+                    const int c = half + ci * EWH, tc0 = t0 + c * 32;
+                    if (c < nact) {
+                        ptx::tmem_ld_wait();
+                        NM_TRACE_EPI_ADD(0);
+                        if (c + EWH >= nact) release_acc(buf);
+                        else ptx::tmem_ld_32x32(lane_taddr + buf * BN + (c + EWH) * 32, r[(ci + 1) & 1]);
+                        const int jmax = n_ok ? min(32, p.tokens - tc0) : 0;  // outputs of this lane that exist
+                        using OT = typename EpiOut<EPI>::type;
+                        auto conv = [&](int j) -> OT {
+                            float y_abs;
+                            const OT o = epi_convert<EPI>(r[ci & 1][j], c_n, b_n, p.sy, 0.0f, y_abs);
+                            if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
+                            return o;
+                        };
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {  // 16 tokens per store, alternating staging tiles
                             if (tc0 + 16 * h >= p.tokens) continue;  // warp-uniform (and the same in all warps of a group)
@@ -408,20 +360,13 @@ nm_gemm_xres_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                             NM_TRACE_EPI_ADD(4);
                             ++n_stores;
                         }
-                    } else {
-                        OT* dst = reinterpret_cast<OT*>(EPI == EPI_F32 ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW) + (size_t)tc0 * p.out + n;
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const OT o = conv(j);
-                            if (j < jmax) dst[(size_t)j * p.out] = o;
-                        }
                     }
                 }
             }
             if (ew == 0 && lane == 0) { NM_TRACE_TILE(i, 1); NM_TRACE_EPI_FLUSH(i); }
         }
-        if (lane == 0) ptx::bulk_wait_group<0>();
-        if (EPI == EPI_F32 && p.absmax) {
+        if (lane == 0) ptx::bulk_wait_group_read<0>();  // the stores have read the staging tiles
+        if (EPI == EPI_F32MAX) {
 #pragma unroll
             for (int s = 16; s > 0; s >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, s));
             if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(p.absmax), __float_as_uint(amax));
