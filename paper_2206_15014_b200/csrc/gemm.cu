@@ -1435,12 +1435,12 @@ static int launch_gemm_pair(const LinearArgs& a) {
 // Wide pair kernel (512 channels x BN tokens per pair): 2:4 int8 weights streamed, fp32 / int32 outputs.
 template <int BN, int EPI, bool W4 = false>
 static int launch_gemm_wide(const LinearArgs& a) {
-    using Cfg = WideCfg<BN>;
+    using Cfg = WideCfg<BN, W4>;
     constexpr int SKEW = 0;
     const nm_packed_t& W = *a.W;
     CUtensorMap tw, tx, ty;
-    // packed 4-bit codes are read by the builder warps, not by TMA: the weight map then describes X as a stand-in
-    int rc = W4 ? make_map(&tw, a.X, (uint64_t)a.tokens, (uint64_t)W.in, Cfg::B_ROWS, 128, CU_TENSOR_MAP_SWIZZLE_128B)
+    // packed 4-bit codes: two stages of a row at a time
+    int rc = W4 ? make_map(&tw, W.values, (uint64_t)W.out, (uint64_t)W.in / 4, Cfg::A_ROWS, 64, CU_TENSOR_MAP_SWIZZLE_64B)
                 : make_map(&tw, W.values, (uint64_t)W.out, (uint64_t)W.in / 2, Cfg::A_ROWS, Cfg::A_ROW, CU_TENSOR_MAP_SWIZZLE_64B);
     if (rc != NM_OK) return rc;
     rc = make_map(&tx, a.X, (uint64_t)a.tokens, (uint64_t)W.in, Cfg::B_ROWS, 128, CU_TENSOR_MAP_SWIZZLE_128B);

@@ -27,23 +27,20 @@ constexpr int kWideGateWarp = 2 + kWideEpiWarps;
 constexpr int kWideMetaWarp0 = kWideGateWarp + 1;
 constexpr int kWideThreads = 32 * (kWideMetaWarp0 + 4);  // producer, MMA, epilogue warps, gate, metadata warps
 // W4 (2:4 weights stored as packed 4-bit codes): the weight tile of a stage is not copied by TMA but built in shared
-// memory by eight more warps, one thread per weight row of the CTA: 32 bytes of nibbles per row and stage (fetched one
-// stage ahead) widened to the 64 int8 slot bytes and written in the tile's swizzle; the stage's "full" barrier counts
-// those warps too.  The 2:4 index metadata is the same as for 8-bit codes.  (Measured: a stage then takes ~980 clocks
-// instead of 582, with eight or with sixteen builder warps alike: the generic-proxy stores and fences compete for the
-// shared-memory bandwidth the MMAs and TMA already use up.  Fetching the codes four stages ahead instead of one made it
-// slower still, 59.5 -> 70.7 us on 4096 -> 1024 at 16384 tokens: the loads' latency is not what holds the builders.
-// One builder warp per ring slot, building the slot's whole tile with a single proxy fence, 66.4 us: a lone warp needs
-// about 2.5 k clk per tile, nearly the ring's whole lead.  Two groups of four warps on alternate stages, two rows per
-// thread: 61.0 us.  Fetch distances of two and three stages: 58.6 and 59.5 us.  Six builder warps, none of them on the
-// MMA warp's scheduler: 69.5 us.  Sixteen builder warps in two groups on alternate stages (64 registers per thread): 87.8 us.)
+// memory by eight more warps, one thread per weight row of the CTA: 32 bytes of nibbles per row and stage widened to the 64 int8
+// slot bytes and written in the tile's swizzle; the stage's "full" barrier counts those warps too.  The 2:4 index metadata is the
+// same as for 8-bit codes.  The nibbles come through TMA too, two stages (64 bytes a row) at a time into a ring of two buffers: read by
+// the builders straight from global memory, 32 rows far apart per load, they took 512 tag lookups of the L1 per stage beside the
+// 256 of the index metadata, more than the stage's 448 clocks of MMAs.
+// 12000 tokens 3072 -> 768 bfloat16 43.5 -> 35.2 us, 16384 tokens 4096 -> 1024 int8 59.1 -> 49.1; 0.82 over the shapes with more than one tile a
+// pair.
 constexpr int kWideBuildWarps = 8;
 template <bool W4> constexpr int kWideThreadsOf = kWideThreads + (W4 ? 32 * kWideBuildWarps : 0);
 constexpr uint32_t kWideNarrowBar = 13;  // named barriers 13 and 14: the four epilogue warps of block 0 / block 1 (narrow outputs)
 constexpr uint32_t kWideRelayIds = 12;  // named barriers 1..12 carry the gate's relays in turn; the gate is never more
                                         // than STAGES + SKEW steps ahead of the MMA thread
 
-template <int BN>
+template <int BN, bool W4 = false>
 struct WideCfg {
     static constexpr int KB = 128;                       // reduction elements per stage
     static constexpr int A_ROWS = 2 * kBM;               // weight rows per CTA: two blocks of 128
@@ -58,9 +55,11 @@ struct WideCfg {
     // rows per tile 9.3 k clocks, 56 of 32 rows 6.9 k, with 8 or 16 warps alike), and here the epilogue is exposed, so
     // fewer, taller boxes pay; a second tile per warp would cost a ring stage, which costs more (measured).
     static constexpr int STORE_STAGE = kWideEpiWarps * 4096;
-    static constexpr int FIT = (kSmemLimit - kSmemTail - STORE_STAGE - 1024) / STAGE;
+    static constexpr int CODE_BYTES = A_ROWS * 64;       // W4: packed codes of two stages
+    static constexpr int CODES = W4 ? 2 * CODE_BYTES : 0;
+    static constexpr int FIT = (kSmemLimit - kSmemTail - STORE_STAGE - 1024 - CODES) / STAGE;
     static constexpr int STAGES = FIT < 8 ? FIT : 8;
-    static constexpr int SMEM = STAGES * STAGE + STORE_STAGE + kSmemTail + 1024;
+    static constexpr int SMEM = STAGES * STAGE + CODES + STORE_STAGE + kSmemTail + 1024;
     static constexpr int META_COL = 2 * BN;              // first TMEM column of the metadata ring
     static constexpr int META_SLOT = 8;                  // columns per stage: two blocks x 128 index bits per row
     static_assert(STAGES >= 4, "pipeline too shallow");
@@ -74,13 +73,14 @@ __global__ void __launch_bounds__(kWideThreadsOf<W4>, 1)
 nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                     const __grid_constant__ CUtensorMap tmap_y, const GemmParams p,
                     const __grid_constant__ PairSchedule sched) {
-    using Cfg = WideCfg<BN>;
+    using Cfg = WideCfg<BN, W4>;
     constexpr int S = Cfg::STAGES;
     static_assert(SKEW >= 0 && SKEW < S - 2, "the ring must hold the stages block 1 lags behind plus loads in flight");
     static_assert(S + SKEW < (int)kWideRelayIds, "relay barriers would be reused before the MMA thread has passed them");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t* store_stage = smem + S * Cfg::STAGE;
+    uint8_t* codes = smem + S * Cfg::STAGE;  // W4: two buffers [256 rows][64 bytes]
+    uint8_t* store_stage = codes + Cfg::CODES;
     uint64_t* bars = reinterpret_cast<uint64_t*>(store_stage + Cfg::STORE_STAGE);
     const uint32_t bar0 = ptx::smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };                     // leader: TMA bytes of both CTAs + 8 metadata warps
@@ -88,7 +88,9 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
     auto acc_full_bar = [&](int b) { return bar0 + 8u * (2 * S + b); };       // both CTAs (multicast commit)
     auto acc_empty_bar = [&](int b) { return bar0 + 8u * (2 * S + 2 + b); };  // leader; four warps of each CTA arrive
     const uint32_t drained_bar = bar0 + 8u * (2 * S + 4);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 5);
+    auto code_full_bar = [&](uint32_t b) { return bar0 + 8u * (2 * S + 5 + b); };   // W4, this CTA's: bytes landed
+    auto code_empty_bar = [&](uint32_t b) { return bar0 + 8u * (2 * S + 7 + b); };  // ... the builder warps have read them
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 9);
     volatile uint32_t* abort_flag = tmem_slot + 1;
     volatile uint32_t* never_flag = tmem_slot + 2;
 
@@ -102,7 +104,7 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) { ptx::mbar_init(full_bar(s), 1 + 8 + (W4 ? 2 * kWideBuildWarps : 0)); ptx::mbar_init(empty_bar(s), 1); }
-        for (int b = 0; b < 2; ++b) { ptx::mbar_init(acc_full_bar(b), 1); ptx::mbar_init(acc_empty_bar(b), 8); }
+        for (int b = 0; b < 2; ++b) { ptx::mbar_init(acc_full_bar(b), 1); ptx::mbar_init(acc_empty_bar(b), 8); ptx::mbar_init(code_full_bar(b), 1); ptx::mbar_init(code_empty_bar(b), kWideBuildWarps); }
         ptx::mbar_init(drained_bar, 1);
         *abort_flag = 0;
         *never_flag = 0;
@@ -138,6 +140,7 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
         // ------------------------------ TMA producer (both CTAs) --------------------------------
         if (lane == 0) {
             uint32_t it = 0, parity = 1u;  // the first pass over the ring finds every stage free
+            uint32_t code = 0, code_parity = 1u;
             const uint64_t keep = ptx::policy_evict_last();  // weights and X are read again by other pairs
             int s = 0;
             bool ok = true;
@@ -147,6 +150,15 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                 const int n0 = tc.o * (2 * Cfg::A_ROWS) + (int)rank * Cfg::A_ROWS;
                 const int t0 = tc.t * BN + (int)rank * Cfg::B_ROWS;
                 for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
+                    if (W4 && (kb & 1) == 0) {  // packed codes of this stage and the next; columns past the row are filled with zeros
+                        if (!ptx::mbar_wait_bounded(code_empty_bar(code), code_parity, abort_flag, kWaitLimit)) {
+                            raise_timeout(); ok = false; break;
+                        }
+                        ptx::mbar_expect_tx(code_full_bar(code), Cfg::CODE_BYTES);
+                        ptx::tma_load_2d(ptx::smem_u32(codes) + code * Cfg::CODE_BYTES, &tmap_w, kb * 32, n0, code_full_bar(code));
+                        code ^= 1u;
+                        if (code == 0) code_parity ^= 1u;
+                    }
                     if (!ptx::mbar_wait_bounded(empty_bar(s), parity, abort_flag, kWaitLimit)) {
                         raise_timeout(); ok = false; break;
                     }
@@ -167,45 +179,38 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
     } else if (W4 && warp >= kWideMetaWarp0 + 4) {
         // ------------------------------ weight-tile builders (W4, both CTAs) ---------------------
         // Thread = one of the CTA's 256 weight rows (block = row / 128).  Per stage: the row's 32 bytes of packed
-        // nibbles (128 reduction elements at 2:4 = 64 codes), fetched one stage ahead, become the 64 slot bytes.
+        // nibbles (128 reduction elements at 2:4 = 64 codes) become the 64 slot bytes.
         const int r256 = (warp - (kWideMetaWarp0 + 4)) * 32 + lane;
         uint8_t* const my_rows = smem + (r256 >> 7) * Cfg::A_BLOCK;  // this thread's block within a stage
-        // the row's packed codes: pointer of the current tile, recomputed only when the tile changes (a single
-        // thread's integer divisions cost hundreds of clocks)
-        auto row_of_tile = [&](int i) -> const uint4* {
-            if (i >= tile_count) return nullptr;
-            const TileCoord tc = tile_coord(tile_begin + i, p.n_tok_tiles, p.n_out_tiles, p.band);
-            const int n = tc.o * (2 * Cfg::A_ROWS) + (int)rank * Cfg::A_ROWS + r256;
-            return n < p.out ? reinterpret_cast<const uint4*>(p.values + (size_t)n * p.vrow_bytes) : nullptr;  // rows past the end: zeros
-        };
-        auto fetch = [&](const uint4* row, int kb, uint4 (&raw)[2]) {
-            if (row) { raw[0] = __ldg(row + 2 * kb); raw[1] = __ldg(row + 2 * kb + 1); }
-            else raw[0] = raw[1] = make_uint4(0u, 0u, 0u, 0u);
-        };
-        int i = 0, kb = 0;
-        const uint4* row = row_of_tile(0);
-        uint4 cur[2], nxt[2];
-        fetch(row, 0, nxt);
-        uint32_t parity = 1u;
+        const uint8_t* const my_codes = codes + r256 * 64;
+        const int x = (r256 >> 1) & 3;  // 64-byte swizzle of the code rows
+        uint32_t parity = 1u, code = 0, code_parity = 0;
         int s = 0;
-        while (i < tile_count) {
-            cur[0] = nxt[0]; cur[1] = nxt[1];
-            int ni = i, nkb = kb + 1;
-            const uint4* nrow = row;
-            if (nkb == p.kblocks) { nkb = 0; ++ni; nrow = row_of_tile(ni); }
-            fetch(nrow, nkb, nxt);  // the next stage's codes travel while this one is built
-            bool got = lane != 0 || ptx::mbar_wait_bounded(empty_bar(s), parity, abort_flag, kWaitLimit);
-            if (!__all_sync(0xffffffffu, got)) { if (lane == 0) raise_timeout(); break; }
-            uint32_t w[16];
-            const uint32_t cw[8] = {cur[0].x, cur[0].y, cur[0].z, cur[0].w, cur[1].x, cur[1].y, cur[1].z, cur[1].w};
+        bool ok = true;
+        for (int i = 0; i < tile_count && ok; ++i) {
+            for (int kb = 0; kb < p.kblocks; ++kb) {
+                const int half = kb & 1;
+                bool got = half || ptx::mbar_wait_bounded(code_full_bar(code), code_parity, abort_flag, kWaitLimit);
+                if (!__all_sync(0xffffffffu, got)) { if (lane == 0) raise_timeout(); ok = false; break; }
+                const uint8_t* src = my_codes + code * Cfg::CODE_BYTES;
+                const uint4 lo = *reinterpret_cast<const uint4*>(src + (((2 * half) ^ x) << 4)), hi = *reinterpret_cast<const uint4*>(src + (((2 * half + 1) ^ x) << 4));
+                got = lane != 0 || ptx::mbar_wait_bounded(empty_bar(s), parity, abort_flag, kWaitLimit);
+                if (!__all_sync(0xffffffffu, got)) { if (lane == 0) raise_timeout(); ok = false; break; }
+                uint32_t w[16];
+                const uint32_t cw[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
 #pragma unroll
-            for (int j = 0; j < 8; ++j) xf::widen8(cw[j], w[2 * j], w[2 * j + 1]);
-            xf::store_row<true>(my_rows + (size_t)s * Cfg::STAGE, r256 & 127, w);
-            ptx::fence_proxy_async_smem();  // the MMA reads the tile through the async proxy
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive_cluster(lead_full0 + 8u * s);
-            if (++s == S) { s = 0; parity ^= 1u; }
-            i = ni; kb = nkb; row = nrow;
+                for (int j = 0; j < 8; ++j) xf::widen8(cw[j], w[2 * j], w[2 * j + 1]);
+                xf::store_row<true>(my_rows + (size_t)s * Cfg::STAGE, r256 & 127, w);
+                ptx::fence_proxy_async_smem();  // the MMA reads the tile through the async proxy, and the next copy overwrites the codes through it
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive_cluster(lead_full0 + 8u * s);
+                if (half || kb + 1 == p.kblocks) {  // the buffer has been read (not before the codes have been used: a load may still be queued)
+                    if (lane == 0) ptx::mbar_arrive(code_empty_bar(code));
+                    code ^= 1u;
+                    if (code == 0) code_parity ^= 1u;
+                }
+                if (++s == S) { s = 0; parity ^= 1u; }
+            }
         }
     } else if (warp >= kWideMetaWarp0) {
         // ------------------------------ metadata warps (both CTAs) -------------------------------
