@@ -1522,13 +1522,15 @@ static int launch_gemm_xres(const LinearArgs& a) {
 }
 
 // One-CTA tiles with the reduction split over clusters of `splits` CTAs (gemm_split.cuh).
-template <bool SPARSE, int BN, int EPI>
+template <bool SPARSE, int BN, int EPI, bool XF>
 static int launch_gemm_split(const LinearArgs& a, int splits) {
     using Cfg = SplitCfg<SPARSE, BN>;
     const nm_packed_t& W = *a.W;
     CUtensorMap tw, tx;
-    int rc = make_map(&tw, W.values, (uint64_t)W.out, (uint64_t)(SPARSE ? W.in / 2 : W.in), kBM, Cfg::A_ROW,
-                      SPARSE ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B);
+    // rebuilt weights are not read by TMA: the weight map then describes X as a stand-in
+    int rc = XF ? make_map(&tw, a.X, (uint64_t)a.tokens, (uint64_t)W.in, BN, 128, CU_TENSOR_MAP_SWIZZLE_128B)
+                : make_map(&tw, W.values, (uint64_t)W.out, (uint64_t)(SPARSE ? W.in / 2 : W.in), kBM, Cfg::A_ROW,
+                           SPARSE ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B);
     if (rc != NM_OK) return rc;
     rc = make_map(&tx, a.X, (uint64_t)a.tokens, (uint64_t)W.in, BN, 128, CU_TENSOR_MAP_SWIZZLE_128B);
     if (rc != NM_OK) return rc;
@@ -1538,13 +1540,17 @@ static int launch_gemm_split(const LinearArgs& a, int splits) {
     p.n_tiles = p.n_tok_tiles * ((W.out + kBM - 1) / kBM);
     p.kblocks = W.in / kKB;
     p.meta = (const uint32_t*)W.meta; p.mrow_words = W.in / 32;
+    p.values = (const uint8_t*)W.values;
+    p.vrow_bytes = (int)values_row_bytes(W.in, W.n, W.m, W.bits);
+    p.mrow_bytes = (int)meta_row_words(W.in, W.n, W.m) * 4;
+    p.pat = xf::pattern_of(W.n, W.m, W.bits);
     p.sw = a.sw; p.bias = a.bias; p.sx_dev = a.sx_dev; p.sx_host = a.sx;
     p.Y = a.Y; p.ACC = a.ACC; p.NARROW = a.NARROW; p.sy = a.sy; p.absmax = a.absmax; p.status = a.status;
-    auto fn = nm_gemm_split_kernel<SPARSE, BN, EPI>;
+    auto fn = nm_gemm_split_kernel<SPARSE, BN, EPI, XF>;
     NM_CUDA_TRY(allow_dynamic_smem((const void*)fn, Cfg::SMEM));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p.n_tiles * splits), 1, 1);
-    cfg.blockDim = dim3(kSplitThreads, 1, 1);
+    cfg.blockDim = dim3(kSplitThreadsOf<XF>, 1, 1);
     cfg.dynamicSmemBytes = Cfg::SMEM;
     cfg.stream = a.stream;
     cudaLaunchAttribute attr[2];
@@ -1670,7 +1676,7 @@ static int resident_clusters(int splits) {
     int& n = known[dev][at];
     if (n == 0) {
         using Cfg = SplitCfg<true, 64>;
-        auto fn = nm_gemm_split_kernel<true, 64, EPI_F32>;
+        auto fn = nm_gemm_split_kernel<true, 64, EPI_F32, false>;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)splits, 1, 1);
         cfg.blockDim = dim3(kSplitThreads, 1, 1);
@@ -1693,11 +1699,15 @@ static int resident_clusters(int splits) {
 // at the same rate.  Over 299 shapes (1 to 1000 tokens, reductions of 384 to 8192) 0.70 of the unsplit time in the geometric mean, 1.03 at the
 // worst, the best of all splits 0.697: 384 tokens 4096 -> 1024 11.9 -> 7.3 us, 64 tokens 768 -> 768 4.5 -> 3.6, 1 token 8192 -> 1024 19.7 -> 5.6;
 // not taken: 384 tokens 1024 -> 3072 5.9 / 6.6.
+// Formats rebuilt on the way (xf) pay 384 tokens a k-block for the builders, every cluster more the more of them rebuild the same weights, and
+// the unsplit kernel has an epilogue of its own to be compared with: 0.63 of the unsplit time over 141 shapes, formats and outputs, 1.017 at the
+// worst: 1 token 8192 -> 1536 1:4 / 8 bit 39.9 -> 9.6 us, 384 tokens 1024 -> 1024 1:4 / 8 bit 8.4 -> 7.0, 128 tokens 768 -> 768 2:4 / 4 bit 5.8 -> 4.7;
+// not taken: a reduction of three k-blocks (1 token 384 -> 1536, 4:4 / 4 bit 4.25 / 4.51), 200 tokens 1024 -> 4096, 2:4 / 4 bit 7.3 / 8.3.
 template <bool SPARSE>
-static int split_plan(const LinearArgs& a, int unsplit_bn) {
+static int split_plan(const LinearArgs& a, int unsplit_bn, bool xf = false) {
     if (g_opt.split == 1 || g_opt.one_bn || g_opt.skip_stage) return 0;  // the test hook counts the stages of an unsplit tile
     const int kblocks = a.W->in / kKB, out_tiles = (a.W->out + kBM - 1) / kBM;
-    const long long unsplit = (long long)kblocks * (unsplit_bn + 256);
+    const long long unsplit = xf ? (long long)kblocks * (unsplit_bn + 384) + 4 * unsplit_bn : (long long)kblocks * (unsplit_bn + 256);
     long long best_cost = 0;
     int best = 0;
     for (int splits : {2, 4, 8})
@@ -1707,21 +1717,22 @@ static int split_plan(const LinearArgs& a, int unsplit_bn) {
             if (g_opt.split && plan != g_opt.split) continue;
             const long long clusters = (long long)out_tiles * ((a.tokens + bn - 1) / bn);
             if (clusters * splits > sm_count()) continue;
-            const long long cost = (long long)per * (bn + 256) + 12 * bn;
-            if (!g_opt.split && (10 * cost > 9 * unsplit || clusters > resident_clusters(splits))) continue;
+            const long long cost = xf ? (long long)per * (bn + 384) + 12 * bn + 12 * clusters * splits : (long long)per * (bn + 256) + 12 * bn;
+            const bool gains = xf ? cost <= unsplit && kblocks > 3 : 10 * cost <= 9 * unsplit;
+            if (!g_opt.split && (!gains || clusters > resident_clusters(splits))) continue;
             if (!best || cost < best_cost) { best = plan; best_cost = cost; }
         }
     return best;
 }
 
-template <bool SPARSE, int EPI>
+template <bool SPARSE, int EPI, bool XF>
 static int pick_split(const LinearArgs& a, int plan) {
     const int splits = plan / 1000;
     switch (plan % 1000) {
-        case 128: return launch_gemm_split<SPARSE, 128, EPI>(a, splits);
-        case 96: return launch_gemm_split<SPARSE, 96, EPI>(a, splits);
-        case 64: return launch_gemm_split<SPARSE, 64, EPI>(a, splits);
-        default: return launch_gemm_split<SPARSE, 32, EPI>(a, splits);
+        case 128: return launch_gemm_split<SPARSE, 128, EPI, XF>(a, splits);
+        case 96: return launch_gemm_split<SPARSE, 96, EPI, XF>(a, splits);
+        case 64: return launch_gemm_split<SPARSE, 64, EPI, XF>(a, splits);
+        default: return launch_gemm_split<SPARSE, 32, EPI, XF>(a, splits);
     }
 }
 
@@ -1730,7 +1741,7 @@ static int pick_bn(const LinearArgs& a) {
     const int out_tiles = (a.W->out + kBM - 1) / kBM, sms = sm_count();
     if constexpr (!XF) {
         const int best = one_cta_bn<SPARSE>(a, {192, 128, 96, 64, 32}, 64);
-        if (const int plan = split_plan<SPARSE>(a, best)) return pick_split<SPARSE, EPI>(a, plan);
+        if (const int plan = split_plan<SPARSE>(a, best)) return pick_split<SPARSE, EPI, XF>(a, plan);
         switch (best) {
             case 192: return launch_gemm<SPARSE, 192, EPI, W_TMA>(a);
             case 128: return launch_gemm<SPARSE, 128, EPI, W_TMA>(a);
@@ -1739,6 +1750,7 @@ static int pick_bn(const LinearArgs& a) {
             default: return launch_gemm<SPARSE, 32, EPI, W_TMA>(a);
         }
     } else {
+        if (const int plan = split_plan<SPARSE>(a, one_cta_bn<SPARSE>(a, {192, 128, 64}, 160), true)) return pick_split<SPARSE, EPI, XF>(a, plan);
         // Sparse-target formats with a short reduction and work for every SM pair: the CTA-pair kernel with the weights
         // rebuilt once per output tile into its resident region (32-bit outputs).
         if constexpr (SPARSE && (kF32<EPI> || EPI == EPI_ACC)) {

@@ -1,4 +1,4 @@
-// One-CTA tiles whose reduction is split over a cluster, for weights in tensor-core form and problems with fewer tiles than SMs.
+// One-CTA tiles whose reduction is split over a cluster, for problems with fewer tiles than SMs.
 //
 // A tile is 128 output channels x BN tokens as in nm_gemm_kernel; the `splits` CTAs of a cluster each multiply their share of
 // the k-blocks.  Then CTA r of the cluster gets the tokens [r, r + 1) * BN / splits of everyone's accumulator (int32, 16-byte stores
@@ -9,11 +9,13 @@
 //   warp 0      TMA producer
 //   warp 1      allocates TMEM; one lane waits for the stages and issues the MMAs
 //   warps 2-9   index metadata of the CTA's k-blocks into TMEM (the first four), exchange, epilogue with direct stores
+//   warps 10-21 (XF: weights not in tensor-core form) three groups of four build the weight tiles as in nm_gemm_kernel
 #pragma once
 
 namespace nm {
 
 constexpr int kSplitThreads = 32 * 10;
+template <bool XF> constexpr int kSplitThreadsOf = kSplitThreads + (XF ? 32 * 4 * kBuildGroups : 0);
 constexpr int kSplitMaxKb = 32;   // k-blocks of a CTA: their metadata (4 columns each) lies beside the accumulator
 
 template <bool SPARSE, int BN>
@@ -31,8 +33,8 @@ struct SplitCfg {
     static_assert(STAGE % 1024 == 0 && A_BYTES % 1024 == 0, "swizzle alignment");
 };
 
-template <bool SPARSE, int BN, int EPI>
-__global__ void __launch_bounds__(kSplitThreads, 1)
+template <bool SPARSE, int BN, int EPI, bool XF>
+__global__ void __launch_bounds__(kSplitThreadsOf<XF>, 1)
 nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x, const GemmParams p,
                      const int splits) {
     using Cfg = SplitCfg<SPARSE, BN>;
@@ -48,15 +50,16 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 3);
     volatile uint32_t* abort_flag = tmem_slot + 1;
     volatile uint32_t* never_flag = tmem_slot + 2;  // stays 0: for the drain wait after an abort
+    uint32_t* lut = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(bars) + 512);  // XF: slot tables (xform.cuh)
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)ptx::warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int rank = (int)ptx::cluster_ctarank();
     const int tile = blockIdx.x / splits, out_tile = tile / p.n_tok_tiles;
     const int n0 = out_tile * kBM, t0 = (tile - out_tile * p.n_tok_tiles) * BN;
     const int kb_begin = rank * p.kblocks / splits, kb_count = (rank + 1) * p.kblocks / splits - kb_begin;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < S; ++s) { ptx::mbar_init(full_bar(s), 1); ptx::mbar_init(empty_bar(s), 1); }
+        for (int s = 0; s < S; ++s) { ptx::mbar_init(full_bar(s), XF ? 5 : 1); ptx::mbar_init(empty_bar(s), 1); }
         ptx::mbar_init(acc_full_bar, 1);
         ptx::mbar_init(meta_bar, 4);
         ptx::mbar_init(drained_bar, 1);
@@ -66,6 +69,7 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
         ptx::prefetch_tensormap(&tmap_w);
         ptx::prefetch_tensormap(&tmap_x);
     }
+    if (XF) xf::build_lut(lut, threadIdx.x, blockDim.x);
     if (warp == 1) {
         ptx::tmem_alloc(ptx::smem_u32(tmem_slot), kTmemCols);
         ptx::tmem_relinquish();
@@ -73,7 +77,7 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = ptx::warp_uniform(*tmem_slot);
     ptx::cluster_arrive();  // the others' shared memory may be written once all of them run (waited for before the exchange)
     ptx::grid_dep_wait();   // nothing in global memory is read or written before this point
     ptx::grid_dep_launch();
@@ -94,55 +98,92 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
                 const int s = it % S, kb = kb_begin + it;
                 if (!ptx::mbar_wait_bounded(empty_bar(s), ((it / S) & 1u) ^ 1u, abort_flag, kWaitLimit)) { raise_timeout(); break; }
                 const uint32_t a_dst = ptx::smem_u32(smem + s * Cfg::STAGE);
-                ptx::mbar_expect_tx(full_bar(s), Cfg::STAGE);
-                ptx::tma_load_2d(a_dst, &tmap_w, kb * Cfg::A_ROW, n0, full_bar(s));
+                ptx::mbar_expect_tx(full_bar(s), XF ? Cfg::B_BYTES : Cfg::STAGE);
+                if (!XF) ptx::tma_load_2d(a_dst, &tmap_w, kb * Cfg::A_ROW, n0, full_bar(s));
                 ptx::tma_load_2d(a_dst + Cfg::A_BYTES, &tmap_x, kb * 128, t0, full_bar(s));
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = ptx::idesc_i8(kBM, BN, SPARSE);
-            bool go = true;
-            if (SPARSE) {
-                go = ptx::mbar_wait_bounded(meta_bar, 0, abort_flag, kWaitLimit);
-                ptx::tc_fence_after();
-            }
-            for (int it = 0; it < kb_count && go; ++it) {
-                const int s = it % S;
-                go = ptx::mbar_wait_bounded(full_bar(s), (it / S) & 1u, abort_flag, kWaitLimit);
-                if (!go) break;
-                const uint32_t a_addr = ptx::smem_u32(smem + s * Cfg::STAGE), b_addr = a_addr + Cfg::A_BYTES;
+        constexpr uint32_t idesc = ptx::idesc_i8(kBM, BN, SPARSE);
+        const uint64_t a_desc0 = ptx::smem_desc_kmajor(ptx::smem_u32(smem), SPARSE ? 64 : 128, SPARSE ? ptx::kSwizzle64 : ptx::kSwizzle128);
+        const uint64_t b_desc0 = ptx::smem_desc_kmajor(ptx::smem_u32(smem) + Cfg::A_BYTES, 128, ptx::kSwizzle128);
+        bool go = true;
+        if (SPARSE) {
+            go = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(meta_bar, 0, abort_flag, kWaitLimit));
+            ptx::tc_fence_after();
+        }
+        uint32_t s = 0, parity = 0;
+        for (int it = 0; it < kb_count && go; ++it) {
+            go = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(full_bar(s), parity, abort_flag, kWaitLimit));
+            if (!go) break;
+            if (ptx::elect_one()) {
+                const uint64_t a = ptx::desc_advance(a_desc0, s * Cfg::STAGE), b = ptx::desc_advance(b_desc0, s * Cfg::STAGE);
                 if constexpr (SPARSE) {
 #pragma unroll
                     for (int j = 0; j < 2; ++j)  // 64 logical k each: 32 stored bytes of A, 64 of B
-                        ptx::mma_sp_i8(tmem_base, ptx::smem_desc_kmajor(a_addr + 32 * j, 64, ptx::kSwizzle64),
-                                       ptx::smem_desc_kmajor(b_addr + 64 * j, 128, ptx::kSwizzle128),
+                        ptx::mma_sp_i8(tmem_base, ptx::desc_advance(a, 32 * j), ptx::desc_advance(b, 64 * j),
                                        tmem_base + Cfg::META_COL + it * 4 + 2 * j, idesc, (it | j) != 0);
                 } else {
 #pragma unroll
                     for (int j = 0; j < 4; ++j)  // 32 k each
-                        ptx::mma_i8(tmem_base, ptx::smem_desc_kmajor(a_addr + 32 * j, 128, ptx::kSwizzle128),
-                                    ptx::smem_desc_kmajor(b_addr + 32 * j, 128, ptx::kSwizzle128), idesc, (it | j) != 0);
+                        ptx::mma_i8(tmem_base, ptx::desc_advance(a, 32 * j), ptx::desc_advance(b, 32 * j), idesc, (it | j) != 0);
                 }
                 ptx::tc_commit(empty_bar(s));
             }
+            __syncwarp();
+            if (++s == S) { s = 0; parity ^= 1u; }
+        }
+        if (ptx::elect_one()) {
             if (go) ptx::tc_commit(acc_full_bar);
             else raise_timeout();
             ptx::tc_commit(drained_bar);  // everything issued has retired before TMEM is released
             ptx::mbar_wait_bounded(drained_bar, 0, never_flag, kWaitLimit);
         }
+        __syncwarp();
+    } else if (XF && warp >= kSplitThreads / 32) {
+        // one thread builds one row of a k-block; group g takes k-blocks g, g + G, ... (see nm_gemm_kernel)
+        constexpr int G = kBuildGroups;
+        static_assert(S > G, "every group needs a stage of its own in flight");
+        const int bw = warp - kSplitThreads / 32, grp = bw >> 2, tr = (bw & 3) * 32 + lane, nr = n0 + tr;
+        const int cb = xf::code_bytes(p.pat), mb = xf::meta_bytes(p.pat);
+        const bool row_ok = nr < p.out;
+        const uint8_t* v = p.values + (size_t)(row_ok ? nr : 0) * p.vrow_bytes + (size_t)kb_begin * cb;
+        const uint8_t* m = reinterpret_cast<const uint8_t*>(p.meta) + (size_t)(row_ok ? nr : 0) * p.mrow_bytes + (size_t)kb_begin * mb;
+        xf::Raw cur = xf::load_raw(p.pat, v + (size_t)grp * cb, m + (size_t)grp * mb, row_ok && grp < kb_count);
+        for (int it = grp; it < kb_count; it += G) {
+            const xf::Raw nxt = xf::load_raw(p.pat, v + (size_t)(it + G) * cb, m + (size_t)(it + G) * mb, row_ok && it + G < kb_count);
+            const bool got = lane != 0 || ptx::mbar_wait_bounded(empty_bar(it % S), ((it / S) & 1u) ^ 1u, abort_flag, kWaitLimit);
+            if (!__all_sync(0xffffffffu, got)) { if (lane == 0) raise_timeout(); break; }
+            uint32_t w[SPARSE ? 16 : 32];
+            xf::build_row<SPARSE>(p.pat, cur, lut, w);
+            xf::store_row<SPARSE>(smem + (it % S) * Cfg::STAGE, tr, w);
+            ptx::fence_proxy_async_smem();  // the MMA reads the tile through the async proxy
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(full_bar(it % S));
+            cur = nxt;
+        }
     } else {
         if (SPARSE && half == 0) {
-            // index metadata of this lane's weight row for the CTA's k-blocks, eight pieces in flight together; rows past the end get a
+            // index metadata of this lane's weight row for the CTA's k-blocks, several pieces in flight together; rows past the end get a
             // valid "positions 0,1" pattern, their products are discarded
-            const uint4* src = reinterpret_cast<const uint4*>(p.meta + (size_t)(n < p.out ? n : 0) * p.mrow_words) + kb_begin;
-            for (int c0 = 0; c0 < kb_count; c0 += 8) {
-                uint4 w[8];
+            constexpr int kBatch = XF ? 4 : 8;
+            const uint4 idle = make_uint4(0x44444444u, 0x44444444u, 0x44444444u, 0x44444444u);
+            const int piece = XF ? xf::meta_bytes(p.pat) : 16;  // stored bytes of a k-block
+            const uint8_t* src = reinterpret_cast<const uint8_t*>(p.meta) + (size_t)(n < p.out ? n : 0) * (XF ? p.mrow_bytes : 4 * p.mrow_words) + (size_t)kb_begin * piece;
+            for (int c0 = 0; c0 < kb_count; c0 += kBatch) {
+                uint4 w[kBatch];
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    w[j] = n < p.out && c0 + j < kb_count ? __ldg(src + c0 + j) : make_uint4(0x44444444u, 0x44444444u, 0x44444444u, 0x44444444u);
+                for (int j = 0; j < kBatch; ++j) {
+                    w[j] = idle;
+                    if (n < p.out && c0 + j < kb_count) w[j] = XF ? xf::meta_raw(p.pat, src + (size_t)(c0 + j) * piece) : xf::ldg16(src + (size_t)(c0 + j) * piece);
+                }
+                if constexpr (XF) {
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
+                    for (int j = 0; j < kBatch; ++j)
+                        if (n < p.out && c0 + j < kb_count) w[j] = xf::hw_meta(p.pat, w[j], lut);
+                }
+#pragma unroll
+                for (int j = 0; j < kBatch; ++j)
                     if (c0 + j < kb_count) ptx::tmem_st_32x4(lane_taddr + Cfg::META_COL + 4 * (c0 + j), w[j].x, w[j].y, w[j].z, w[j].w);
             }
             ptx::tmem_st_wait();
@@ -161,7 +202,7 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
     }
     __syncwarp();
     ptx::cluster_wait();
-    if (warp >= 2 && ok) {
+    if (warp >= 2 && warp < kSplitThreads / 32 && ok) {
         // The other CTAs' tokens: [sender][chunk][two halves of four tokens][128 channels] of 16 bytes at the receiver.
         const uint32_t base = ptx::smem_u32(recv) + (uint32_t)row * 16u;
         for (int u = half; u < (splits - 1) * chunks; u += 2) {
@@ -181,7 +222,7 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
     __syncwarp();
     ptx::cluster_arrive();
     ptx::cluster_wait();
-    if (warp >= 2 && ok) {
+    if (warp >= 2 && warp < kSplitThreads / 32 && ok) {
         const float rsy = EPI == EPI_Q8 ? __frcp_rn(p.sy) : 0.0f;
         float amax = 0.0f;
         using OT = typename EpiOut<EPI>::type;

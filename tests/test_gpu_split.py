@@ -12,15 +12,15 @@ pytestmark = pytest.mark.gpu
 PLANS = [(2, 32), (4, 32), (2, 64), (4, 64), (8, 64), (2, 96), (4, 96), (2, 128), (4, 128), (8, 128)]
 
 
-def _run(T, K, out, n):
+def _run(T, K, out, n, m=4, bits=8):
     from gpu_util import PackedOnDevice, gpu_int_linear, gpu_int_linear_q8, gpu_int_linear_bf16
     oracle.set_threads(oracle.max_threads())
     rng = np.random.default_rng(T + K)
     W, b = wl.normal(rng, (out, K), 0.02), wl.normal(rng, (out,), 0.02)
     Xq, sx = oracle.quantize_act(wl.normal(rng, (T, K)))
-    v, meta, s = oracle.project_pack(W, None, n, 4, 8)
-    acc_ref, Y_ref = oracle.int_linear(Xq, oracle.unpack(v, meta, out, K, n, 4, 8), sx, s, b)
-    packed = PackedOnDevice(v, meta, s, out, K, n, 4, 8)
+    v, meta, s = oracle.project_pack(W, None, n, m, bits)
+    acc_ref, Y_ref = oracle.int_linear(Xq, oracle.unpack(v, meta, out, K, n, m, bits), sx, s, b)
+    packed = PackedOnDevice(v, meta, s, out, K, n, m, bits)
     acc, Y = gpu_int_linear(Xq, packed, sx, b)
     assert np.array_equal(acc, acc_ref), f"{(acc != acc_ref).sum()} accumulators differ"
     assert np.array_equal(Y, Y_ref)
@@ -38,6 +38,22 @@ def test_forms(splits, bn, n):
         _run(bn + bn // splits + 3, 128 * (splits + 1), 250, n)  # one CTA has two k-blocks, the second token tile ends early
         if 9 * splits <= 64:
             _run(1, 128 * 9 * splits, 128, n)                    # nine k-blocks in a ring of at most eight, one token
+    finally:
+        nm.nm_debug_set_option("split", 0)
+
+
+@pytest.mark.parametrize("n,m,bits", [(2, 4, 4), (1, 4, 8), (1, 4, 4), (4, 8, 8), (4, 8, 4), (2, 8, 8), (1, 8, 4), (4, 4, 4)])
+def test_formats_rebuilt_on_the_way(n, m, bits):
+    import paper_2206_15014_b200 as nm
+    try:
+        for splits, bn in ((2, 32), (4, 64), (8, 128)):
+            nm.nm_debug_set_option("split", 1000 * splits + bn)
+            _run(bn + bn // splits + 3, 128 * (splits + 1), 250, n, m, bits)
+            if splits < 8:
+                _run(1, 128 * 9 * splits, 128, n, m, bits)
+        nm.nm_debug_set_option("split", 0)
+        for T, K, out in ((5, 1024, 1024), (130, 768, 770), (64, 4096, 300)):  # the library's choice: split
+            _run(T, K, out, n, m, bits)
     finally:
         nm.nm_debug_set_option("split", 0)
 
