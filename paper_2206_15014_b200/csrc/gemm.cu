@@ -64,9 +64,9 @@ template <int EPI> constexpr bool kF32 = EPI == EPI_F32 || EPI == EPI_F32MAX;
 template <int EPI> struct EpiOut { using type = uint32_t; };          // fp32 / int32 move as 32-bit patterns
 template <> struct EpiOut<EPI_Q8> { using type = uint8_t; };
 template <> struct EpiOut<EPI_BF16> { using type = uint16_t; };
-// Narrow outputs leave through [tokens][128 channels] tiles that the four warps of a TMEM-lane-quarter
-// group fill together (rows of 128 / 256 bytes instead of 32 / 64; see narrow_tile): a named barrier per group orders the fills against the
-// one warp that issues the TMA store, kNarrowAgree + half makes the group take a timed-out wait together so that nobody is left alone on it.
+// Narrow outputs leave through [tokens][32 channels] tiles of the warp's own (narrow_tile), or [tokens][128 channels] tiles that the four warps of a
+// TMEM-lane-quarter group fill together (narrow_group_tile): there a named barrier per group orders the fills against the one warp
+// that issues the TMA store, kNarrowAgree + half makes the group take a timed-out wait together so that nobody is left alone on it.
 // EPI_Q8 without a branch per value: the code from the reciprocal rsy = RN(1 / sy), exact unless the product sits
 // within 2^-15 of a rounding tie (6 values in 100000), where only the IEEE division decides.  `worst` keeps the largest
 // distance of a product from its rounded integer over a run of values; beyond 0.49996948 the caller fills the run again
@@ -117,86 +117,161 @@ __device__ __noinline__ uint32_t quantise8_exact4(float y0, float y1, float y2, 
            (uint32_t)(quantise8_exact(y2, sy) & 0xff) << 16 | (uint32_t)(quantise8_exact(y3, sy) & 0xff) << 24;
 }
 
-// One output tile of a group of four epilogue warps (one per TMEM lane quarter q) as int8 or bfloat16.
+// 16 tokens of a warp's 32 channels, as the two loads of the stmatrix layout left them in r, converted: two bfloat16 or four codes a word.
+template <int EPI>
+__device__ __forceinline__ void narrow_convert(const uint32_t* r, uint32_t* pk, const float (&c)[4], const float (&b)[4], float sy, float rsy) {
+    constexpr float kMagic = 12582912.0f;
+    const uint64_t c01[2] = {ptx::pack_f32x2(c[0], c[0]), ptx::pack_f32x2(c[2], c[2])}, c23[2] = {ptx::pack_f32x2(c[1], c[1]), ptx::pack_f32x2(c[3], c[3])};
+    const uint64_t b01[2] = {ptx::pack_f32x2(b[0], b[0]), ptx::pack_f32x2(b[2], b[2])}, b23[2] = {ptx::pack_f32x2(b[1], b[1]), ptx::pack_f32x2(b[3], b[3])};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {  // k = 2 * (lane half) + column group
+        const uint32_t* x = r + 4 * k;
+        const uint64_t y01 = ptx::fma_f32x2(ptx::pack_f32x2((float)(int)x[0], (float)(int)x[1]), c01[k >> 1], b01[k >> 1]);
+        const uint64_t y23 = ptx::fma_f32x2(ptx::pack_f32x2((float)(int)x[2], (float)(int)x[3]), c23[k >> 1], b23[k >> 1]);
+        float y0, y1, y2, y3;
+        ptx::unpack_f32x2(y01, y0, y1);
+        ptx::unpack_f32x2(y23, y2, y3);
+        if constexpr (EPI == EPI_BF16) {
+            pk[2 * k] = ptx::cvt_bf16x2(y0, y1);
+            pk[2 * k + 1] = ptx::cvt_bf16x2(y2, y3);
+        } else {
+            const uint64_t rs2 = ptx::pack_f32x2(rsy, rsy), magic2 = ptx::pack_f32x2(kMagic, kMagic), minus2 = ptx::pack_f32x2(-1.0f, -1.0f);
+            const uint64_t t01 = ptx::fma_f32x2(y01, rs2, magic2), t23 = ptx::fma_f32x2(y23, rs2, magic2);
+            float d0, d1, d2, d3, t[4];
+            ptx::unpack_f32x2(ptx::fma_f32x2(y01, rs2, ptx::fma_f32x2(t01, minus2, magic2)), d0, d1);
+            ptx::unpack_f32x2(ptx::fma_f32x2(y23, rs2, ptx::fma_f32x2(t23, minus2, magic2)), d2, d3);
+            ptx::unpack_f32x2(t01, t[0], t[1]);
+            ptx::unpack_f32x2(t23, t[2], t[3]);
+            auto code = [&](int i) { return __float_as_int(t[i]) - 0x4B400000; };
+            pk[k] = ptx::pack_sat_s8(code(0), code(1), ptx::pack_sat_s8(code(2), code(3), 0u));
+            if (!(ptx::max_abs_nan(d2, d3, ptx::max_abs_nan(d0, d1, 0.0f)) <= 0.49996948f)) pk[k] = quantise8_exact4(y0, y1, y2, y3, sy);
+        }
+    }
+}
+
+// The same words, transposed into a tile [16 tokens][32 channels] in the 64-byte (bfloat16) or 32-byte swizzle of the store's tensor map, so that
+// no two rows of a matrix meet in a bank.
+template <int EPI>
+__device__ __forceinline__ void narrow_fill(uint32_t tile, const uint32_t* pk, int lane) {
+    const uint32_t token = lane & 7;
+    if constexpr (EPI == EPI_BF16) {
+#pragma unroll
+        for (int g = 0; g < 2; ++g)  // matrix i: channels 8 i .. 8 i + 7, eight tokens
+            ptx::stmatrix_trans_b16(tile + (8 * g + token) * 64 + (((lane >> 3) ^ (token >> 1)) << 4), pk[2 * g], pk[2 * g + 1], pk[4 + 2 * g], pk[4 + 2 * g + 1]);
+    } else {  // matrix i: channels 16 (i % 2) .. + 15, tokens 8 (i / 2) .. + 7
+        ptx::stmatrix_trans_b8(tile + (8 * (lane >> 4) + token) * 32 + ((((lane >> 3) & 1) ^ (token >> 2)) << 4), pk[0], pk[2], pk[1], pk[3]);
+    }
+}
+
+// Tiles of 16 tokens that BYTES of staging memory hold, of the SUBS that a warp has to do at most.
+template <int EPI, int BYTES, int SUBS> constexpr int kNarrowStage = BYTES / (EPI == EPI_BF16 ? 1024 : 512) < SUBS ? BYTES / (EPI == EPI_BF16 ? 1024 : 512) : SUBS;
+
+// A warp's 32 channels of an output tile as int8 or bfloat16.  The groups of four warps (one per TMEM lane quarter) share the tile's tokens evenly.
 //
-// A warp reads 16 tokens of its 32 channels from the accumulator in the fragment layout of stmatrix (a thread has two neighbouring
-// tokens of four channels), converts them in pairs, and writes them transposed, 16 bytes of a token's row at a time, into the group's
-// staging tile [UNIT tokens][128 channels], in the 128-byte swizzle of the store's tensor map, so that no two rows of a matrix meet in a
-// bank.  With a lane per channel every value took a conversion and a store instruction of its own: 4 instructions for a bfloat16, 11 for an
-// exact int8 code, 2.2 and 5.3 so: 1024 -> 3072, 20000 tokens 41.1 -> 38.5 us (bfloat16); 768 -> 768, 16384 tokens 17.1 -> 14.6 (int8); int8
-// outputs over 337 shapes and formats 0.93 of the time, bfloat16 0.97.
+// The warp reads 16 tokens from the accumulator in the fragment layout of stmatrix (a thread has two neighbouring tokens of four channels),
+// converts them in pairs, and writes them transposed, 16 bytes of a token's row at a time, into staging tiles of its own, in rounds of
+// as many as its staging memory holds.  With a lane per channel every value took a conversion and a store instruction of its own: 4
+// instructions for a bfloat16, 11 for an exact int8 code, 2.2 and 5.3 so.  No warp waits for another: staging tiles shared by the four
+// warps of a group (rows of 128 channels) took a barrier or two a round, and 300 clocks for the group to agree on an expired wait; 16384
+// tokens 768 -> 3072 bfloat16 31.7 -> 28.9 us (35.0 with a lane per channel), int8 outputs over 263 shapes and formats 0.96 of the time.
 // int8: t = fma(y, rsy, 1.5 * 2^23) rounds the product to the nearest-even integer, which saturates to the code; `d` is the product's
 // distance from it, and within 2^-15 of a tie (or NaN) the IEEE division decides.
 //
 // acc: TMEM address of the tile's first column in this warp's lane quarter.  c, b: scale and bias of channels lane / 4 + 8 i of the quarter.
-// valid: tokens of the tile that exist.  stage: the group's two staging tiles.  release(): this warp has read its accumulator.
-template <int EPI, int UNIT, bool HINT, typename Release>
-__device__ __forceinline__ void narrow_tile(uint32_t acc, int columns, int valid, int group, int groups, uint32_t bar, uint32_t stage,
-                                            uint32_t& n_stores, int q, int lane, const float (&c)[4], const float (&b)[4], float sy, float rsy,
-                                            const CUtensorMap* tmap_y, int n0, int t0, int out, uint64_t policy, Release release) {
-    constexpr uint32_t ROW = 128, BOX = UNIT * ROW, TILE = (EPI == EPI_BF16 ? 2 : 1) * BOX;  // bfloat16: two boxes of 64 channels
-    constexpr float kMagic = 12582912.0f;
-    const int units = (min(valid, columns) + UNIT - 1) / UNIT;  // units that hold tokens (the same for the whole group)
-    const uint64_t c01[2] = {ptx::pack_f32x2(c[0], c[0]), ptx::pack_f32x2(c[2], c[2])}, c23[2] = {ptx::pack_f32x2(c[1], c[1]), ptx::pack_f32x2(c[3], c[3])};
-    const uint64_t b01[2] = {ptx::pack_f32x2(b[0], b[0]), ptx::pack_f32x2(b[2], b[2])}, b23[2] = {ptx::pack_f32x2(b[1], b[1]), ptx::pack_f32x2(b[3], b[3])};
+// valid: tokens of the tile that exist.  n: the warp's first channel.  LD: pieces of 16 tokens that it has in registers together.
+// release(): it has read its accumulator.
+template <int EPI, int SUBS, int STAGE, int BUFS, int LD, bool HINT, typename Release>
+__device__ __forceinline__ void narrow_tile(uint32_t acc, int valid, int group, int groups, uint32_t stage, int lane, const float (&c)[4], const float (&b)[4],
+                                            float sy, float rsy, const CUtensorMap* tmap_y, int n, int t0, int out, uint64_t policy, Release release) {
+    constexpr uint32_t TILE = EPI == EPI_BF16 ? 1024 : 512;
+    const int all = min((valid + 15) >> 4, SUBS * groups), share = (all + groups - 1) / groups;
+    const int first = group * share, last = min(first + share, all);
+    if (first >= last) { release(); return; }
+    uint32_t buf = 0;
+#pragma unroll 1
+    for (int u = first; u < last; u += STAGE) {
+        const uint32_t tile = stage + buf * (STAGE * TILE);
+#pragma unroll
+        for (int h = 0; h < STAGE; h += LD) {
+            if (u + h >= last) break;
+            uint32_t r[LD][16];
+#pragma unroll
+            for (int k = 0; k < LD; ++k) {  // past the last 16 tokens: other columns, not used
+                ptx::tmem_ld_16x256x2(acc + 16 * (u + h + k), r[k]);
+                ptx::tmem_ld_16x256x2(acc + (16u << 16) + 16 * (u + h + k), r[k] + 8);
+            }
+            ptx::tmem_ld_wait();
+            if (u + h + LD >= last) release();
+            uint32_t pk[LD][EPI == EPI_Q8 ? 4 : 8];
+#pragma unroll
+            for (int k = 0; k < LD; ++k) narrow_convert<EPI>(r[k], pk[k], c, b, sy, rsy);
+            if (h == 0) {  // the stores that last used the staging tiles have read them
+                if (lane == 0) {
+                    if (BUFS == 1 || u == first) ptx::bulk_wait_group_read<0>();
+                    else ptx::bulk_wait_group_read<1>();
+                }
+                __syncwarp();
+            }
+#pragma unroll
+            for (int k = 0; k < LD; ++k)
+                if (h + k < STAGE) narrow_fill<EPI>(tile + (h + k) * TILE, pk[k], lane);
+        }
+        ptx::fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0 && n < out) {
+            for (int h = 0; h < min(STAGE, last - u); ++h) {
+                if (HINT) ptx::tma_store_2d_hint(tmap_y, n, t0 + 16 * (u + h), tile + h * TILE, policy);
+                else ptx::tma_store_2d(tmap_y, n, t0 + 16 * (u + h), tile + h * TILE);
+            }
+            ptx::bulk_commit_group();
+        }
+        __syncwarp();
+        if (BUFS == 2) buf ^= 1u;
+    }
+}
+
+// The same for bfloat16 with the four warps of a group sharing staging tiles [UNIT tokens][128 channels], two in turn, so that the rows
+// that leave are whole 128-byte lines and not halves of them: where Y goes to HBM as fast as it can the halves cost more than the group's
+// barriers.  The 512-channel kernel always (with halves 1.008 of the time with packed 4-bit codes, up to 1.038), the pair kernels for shorter reductions from
+// 192 MB of Y on (32768 tokens 1024 -> 3072 64.3 us so, 66.1 with halves; 1024 -> 4096 with 4-bit codes 108.9 / 112.4,
+// with dense weights 104.0 / 112.3; below it the halves are
+// better: 16384 tokens 1024 -> 4096 40.3 / 38.6).
+constexpr size_t kNarrowGroupBytes = (size_t)192 << 20;
+template <int UNIT, typename Release>
+__device__ __forceinline__ void narrow_group_tile(uint32_t acc, int columns, int valid, int group, int groups, uint32_t bar, uint32_t stage, uint32_t& n_stores,
+                                                  int q, int lane, const float (&c)[4], const float (&b)[4], const CUtensorMap* tmap_y, int n0, int t0,
+                                                  int out, uint64_t policy, Release release) {
+    constexpr uint32_t ROW = 128, BOX = UNIT * ROW, TILE = 2 * BOX;  // two boxes of 64 channels
+    const int units = (min(valid, columns) + UNIT - 1) / UNIT;       // units that hold tokens (the same for the whole group)
     if (group >= units) release();
 #pragma unroll 1
     for (int u = group; u < units; u += groups) {
         const uint32_t tile = stage + (n_stores & 1u) * TILE;
 #pragma unroll
         for (int h = 0; h < UNIT / 16; ++h) {
-            uint32_t r[16];
+            uint32_t r[16], pk[8];
             ptx::tmem_ld_16x256x2(acc + u * UNIT + 16 * h, r);
             ptx::tmem_ld_16x256x2(acc + (16u << 16) + u * UNIT + 16 * h, r + 8);
             ptx::tmem_ld_wait();
             if (h == UNIT / 16 - 1 && u + groups >= units) release();
-            uint32_t pk[EPI == EPI_Q8 ? 4 : 8];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {  // k = 2 * (lane half) + column group
-                const uint32_t* x = r + 4 * k;
-                const uint64_t y01 = ptx::fma_f32x2(ptx::pack_f32x2((float)(int)x[0], (float)(int)x[1]), c01[k >> 1], b01[k >> 1]);
-                const uint64_t y23 = ptx::fma_f32x2(ptx::pack_f32x2((float)(int)x[2], (float)(int)x[3]), c23[k >> 1], b23[k >> 1]);
-                float y0, y1, y2, y3;
-                ptx::unpack_f32x2(y01, y0, y1);
-                ptx::unpack_f32x2(y23, y2, y3);
-                if constexpr (EPI == EPI_BF16) {
-                    pk[2 * k] = ptx::cvt_bf16x2(y0, y1);
-                    pk[2 * k + 1] = ptx::cvt_bf16x2(y2, y3);
-                } else {
-                    const uint64_t rs2 = ptx::pack_f32x2(rsy, rsy), magic2 = ptx::pack_f32x2(kMagic, kMagic), minus2 = ptx::pack_f32x2(-1.0f, -1.0f);
-                    const uint64_t t01 = ptx::fma_f32x2(y01, rs2, magic2), t23 = ptx::fma_f32x2(y23, rs2, magic2);
-                    float d0, d1, d2, d3, t[4];
-                    ptx::unpack_f32x2(ptx::fma_f32x2(y01, rs2, ptx::fma_f32x2(t01, minus2, magic2)), d0, d1);
-                    ptx::unpack_f32x2(ptx::fma_f32x2(y23, rs2, ptx::fma_f32x2(t23, minus2, magic2)), d2, d3);
-                    ptx::unpack_f32x2(t01, t[0], t[1]);
-                    ptx::unpack_f32x2(t23, t[2], t[3]);
-                    auto code = [&](int i) { return __float_as_int(t[i]) - 0x4B400000; };
-                    pk[k] = ptx::pack_sat_s8(code(0), code(1), ptx::pack_sat_s8(code(2), code(3), 0u));
-                    if (!(ptx::max_abs_nan(d2, d3, ptx::max_abs_nan(d0, d1, 0.0f)) <= 0.49996948f)) pk[k] = quantise8_exact4(y0, y1, y2, y3, sy);
-                }
-            }
+            narrow_convert<EPI_BF16>(r, pk, c, b, 0.0f, 0.0f);
             if (h == 0) {
                 if (q == 0 && lane == 0) ptx::bulk_wait_group_read<1>();  // the store before the last has read this tile
                 ptx::named_bar_sync(bar, 128);
             }
             const uint32_t token = lane & 7;
-            if constexpr (EPI == EPI_BF16) {
 #pragma unroll
-                for (int g = 0; g < 2; ++g)  // matrix i: channels 8 i .. 8 i + 7 of the quarter, eight tokens
-                    ptx::stmatrix_trans_b16(tile + (q >> 1) * BOX + (16 * h + 8 * g + token) * ROW + ((((q & 1) * 4 + (lane >> 3)) ^ token) << 4),
-                                            pk[2 * g], pk[2 * g + 1], pk[4 + 2 * g], pk[4 + 2 * g + 1]);
-            } else {  // matrix i: channels 16 (i % 2) .. + 15 of the quarter, tokens 8 (i / 2) .. + 7
-                ptx::stmatrix_trans_b8(tile + (16 * h + 8 * (lane >> 4) + token) * ROW + (((q * 2 + ((lane >> 3) & 1)) ^ token) << 4), pk[0], pk[2], pk[1], pk[3]);
-            }
+            for (int g = 0; g < 2; ++g)  // as in narrow_fill
+                ptx::stmatrix_trans_b16(tile + (q >> 1) * BOX + (16 * h + 8 * g + token) * ROW + ((((q & 1) * 4 + (lane >> 3)) ^ token) << 4),
+                                        pk[2 * g], pk[2 * g + 1], pk[4 + 2 * g], pk[4 + 2 * g + 1]);
         }
         ptx::fence_proxy_async_smem();
         ptx::named_bar_sync(bar, 128);
         if (q == 0 && lane == 0) {
 #pragma unroll
-            for (int x = 0; x < (int)(TILE / BOX); ++x) {
+            for (int x = 0; x < 2; ++x) {
                 if (x && n0 + 64 * x >= out) break;
-                if (HINT) ptx::tma_store_2d_hint(tmap_y, n0 + 64 * x, t0 + u * UNIT, tile + x * BOX, policy);
-                else ptx::tma_store_2d(tmap_y, n0 + 64 * x, t0 + u * UNIT, tile + x * BOX);
+                ptx::tma_store_2d_hint(tmap_y, n0 + 64 * x, t0 + u * UNIT, tile + x * BOX, policy);
             }
             ptx::bulk_commit_group();
         }
@@ -290,6 +365,7 @@ struct GemmParams {
     const uint8_t* values; // packed codes (transform modes)
     int vrow_bytes, mrow_bytes, pat;
     int tma_store;         // 1: epilogue writes through shared memory + TMA; 0: direct stores
+    int grouped;           // 1: narrow_group_tile (pair kernels, bfloat16)
     const float* sw;
     const float* bias;
     const float* sx_dev;
@@ -690,7 +766,6 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
             bool got = ptx::mbar_wait_bounded(acc_full_bar(buf), (i >> 1) & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
             if (!ok && lane == 0) raise_timeout();
-            if constexpr (kNarrow<EPI>) ok = ptx::named_bar_and(kNarrowAgree + half, 128, ok);  // the group stops together
             if (!ok) break;
             ptx::tc_fence_after();
             if (SPARSE && half == 0 && i + 1 < tile_count) {
@@ -710,9 +785,9 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 continue;
             }
             if constexpr (kNarrow<EPI>) {
-                constexpr uint32_t kPerGroup = (EPI == EPI_BF16 ? 2 : 1) * 4096;
-                narrow_tile<EPI, 16, false>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, kNarrowGroup + half, ptx::smem_u32(store_stage) + half * kPerGroup,
-                                            n_stores, q, lane, nc, nb, p.sy, rsy, &tmap_y, n0, t0, p.out, 0, [&] { release_acc(buf); });
+                constexpr int SUBS = (BN / 16 + EWH - 1) / EWH;
+                narrow_tile<EPI, SUBS, kNarrowStage<EPI, kStoreStage / kEpiWarps, SUBS>, 1, 1, false>(lane_taddr + buf * BN, p.tokens - t0, half, EWH,
+                    ptx::smem_u32(store_stage) + ew * (kStoreStage / kEpiWarps), lane, nc, nb, p.sy, rsy, &tmap_y, n0 + q * 32, t0, p.out, 0, [&] { release_acc(buf); });
                 continue;
             }
             if constexpr (!kNarrow<EPI>) {
@@ -784,7 +859,7 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
 // the X tile (BN/2 tokens); one MMA issued by the leader CTA (cluster rank 0) spans both CTAs: every
 // CTA's tensor core accumulates its 128 rows over all BN tokens, taking the other half of X from the
 // peer's shared memory.  Per MAC this moves 0.63x the bytes of the one-CTA kernel through L2 and
-// through each SM's shared-memory port, and the sparse MMA is no longer shared-memory bound.
+// through each SM's shared-memory port.
 // Protocol differences: both producers' TMA bytes are counted on the LEADER's "full" barrier; the
 // leader's commits are multicast to the "empty" / "accumulator full" barriers of both CTAs; the
 // peer's epilogue and metadata warps arrive remotely on the leader's barriers; the pair synchronises
@@ -1141,7 +1216,7 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
             bool got = ptx::mbar_wait_bounded(acc_full_bar(buf), (i >> 1) & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
             if (!ok && lane == 0) raise_timeout();
-            if constexpr (kNarrow<EPI>) ok = ptx::named_bar_and(EW == 16 ? kNarrowGroup + half : kNarrowAgree + half, 128, ok);  // the group stops together
+            if (EPI == EPI_BF16 && p.grouped) ok = ptx::named_bar_and(EW == 16 ? kNarrowGroup + half : kNarrowAgree + half, 128, ok);  // the group stops together
             if (!ok) break;
             ptx::tc_fence_after();
             if (ew == 0 && lane == 0) NM_TRACE_TILE(i, 0);
@@ -1164,9 +1239,13 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                 continue;
             }
             if constexpr (kNarrow<EPI>) {
-                constexpr uint32_t kPerGroup = (EPI == EPI_BF16 ? 2 : 1) * 4096;
-                narrow_tile<EPI, 16, true>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, kNarrowGroup + half, ptx::smem_u32(store_stage) + half * kPerGroup,
-                                           n_stores, q, lane, nc, nb, p.sy, rsy, &tmap_y, n0, t0, p.out, stream_out, [&] { release_acc(buf); });
+                constexpr int SUBS = BN / 16 / EWH, PER = Cfg::STORE_STAGE / EW;
+                if (EPI == EPI_BF16 && p.grouped)
+                    narrow_group_tile<16>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, kNarrowGroup + half, ptx::smem_u32(store_stage) + half * 8192, n_stores,
+                                          q, lane, nc, nb, &tmap_y, n0, t0, p.out, stream_out, [&] { release_acc(buf); });
+                else
+                narrow_tile<EPI, SUBS, kNarrowStage<EPI, PER, SUBS>, 1, 1, true>(lane_taddr + buf * BN, p.tokens - t0, half, EWH, ptx::smem_u32(store_stage) + ew * PER,
+                    lane, nc, nb, p.sy, rsy, &tmap_y, n0 + q * 32, t0, p.out, stream_out, [&] { release_acc(buf); });
                 if (ew == 0 && lane == 0) { NM_TRACE_TILE(i, 1); NM_TRACE_EPI_FLUSH(i); }
                 continue;
             }
@@ -1297,7 +1376,7 @@ struct LinearArgs {
 // through TMA when the output can be described by a tensor map (16-byte aligned base and row pitch);
 // otherwise *tma_store is cleared, the threads store directly and the map describes X as a stand-in.
 template <int EPI>
-static int make_store_map(CUtensorMap* ty, const LinearArgs& a, bool* tma_store, uint32_t box_rows = 16) {
+static int make_store_map(CUtensorMap* ty, const LinearArgs& a, bool* tma_store, uint32_t box_rows = 16, bool grouped = false) {
     const nm_packed_t& W = *a.W;
     constexpr uint32_t es = (uint32_t)sizeof(typename EpiOut<EPI>::type);
     void* ybase = kF32<EPI> ? (void*)a.Y : EPI == EPI_ACC ? (void*)a.ACC : a.NARROW;
@@ -1306,9 +1385,9 @@ static int make_store_map(CUtensorMap* ty, const LinearArgs& a, bool* tma_store,
                                  : EPI == EPI_Q8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     if (!*tma_store)
         return make_map(ty, a.X, (uint64_t)a.tokens, (uint64_t)W.in / 4, 16, 32, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_DATA_TYPE_INT32, 4);
-    // narrow outputs: rows of 128 bytes in the swizzle of narrow_tile
-    return make_map(ty, ybase, (uint64_t)a.tokens, (uint64_t)W.out, box_rows, kNarrow<EPI> ? 128 / es : 32,
-                    kNarrow<EPI> ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, dt, es);
+    // narrow outputs: in the swizzle of narrow_fill or narrow_group_tile
+    return make_map(ty, ybase, (uint64_t)a.tokens, (uint64_t)W.out, box_rows, grouped ? 64 : 32,
+                    grouped ? CU_TENSOR_MAP_SWIZZLE_128B : EPI == EPI_BF16 ? CU_TENSOR_MAP_SWIZZLE_64B : EPI == EPI_Q8 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE, dt, es);
 }
 
 template <bool SPARSE, int BN, int EPI, int WSRC>
@@ -1389,10 +1468,12 @@ static int launch_gemm_pair(const LinearArgs& a) {
     rc = make_map_x3(&tx, a.X, (uint64_t)a.tokens, (uint64_t)W.in, Cfg::B_ROWS, Cfg::KB / 128);
     if (rc != NM_OK) return rc;
     bool tma_store = false;
-    rc = make_store_map<EPI>(&ty, a, &tma_store);
+    const bool grouped = EPI == EPI_BF16 && (size_t)a.tokens * W.out * 2 >= kNarrowGroupBytes;
+    rc = make_store_map<EPI>(&ty, a, &tma_store, 16, grouped);
     if (rc != NM_OK) return rc;
     GemmParams p{};
     p.tma_store = tma_store ? 1 : 0;
+    p.grouped = grouped ? 1 : 0;
     p.tokens = a.tokens; p.out = W.out; p.in = W.in;
     p.n_tok_tiles = (a.tokens + BN - 1) / BN;
     p.n_out_tiles = (W.out + 2 * kBM - 1) / (2 * kBM);
@@ -1446,7 +1527,7 @@ static int launch_gemm_wide(const LinearArgs& a) {
     rc = make_map(&tx, a.X, (uint64_t)a.tokens, (uint64_t)W.in, Cfg::B_ROWS, 128, CU_TENSOR_MAP_SWIZZLE_128B);
     if (rc != NM_OK) return rc;
     bool tma_store = false;
-    rc = make_store_map<EPI>(&ty, a, &tma_store, 32);
+    rc = make_store_map<EPI>(&ty, a, &tma_store, EPI == EPI_Q8 ? 16 : 32, EPI == EPI_BF16);
     if (rc != NM_OK) return rc;
     GemmParams p{};
     p.tma_store = tma_store ? 1 : 0;
@@ -1491,10 +1572,12 @@ static int launch_gemm_xres(const LinearArgs& a) {
     rc = make_map_x3(&tx, a.X, (uint64_t)a.tokens, (uint64_t)W.in, Cfg::B_ROWS, Cfg::SLICES);
     if (rc != NM_OK) return rc;
     bool tma_store = false;
-    rc = make_store_map<EPI>(&ty, a, &tma_store);
+    const bool grouped = EPI == EPI_BF16 && (size_t)a.tokens * W.out * 2 >= kNarrowGroupBytes;
+    rc = make_store_map<EPI>(&ty, a, &tma_store, 16, grouped);
     if (rc != NM_OK) return rc;
     GemmParams p{};
     p.tma_store = tma_store ? 1 : 0;
+    p.grouped = grouped ? 1 : 0;
     p.tokens = a.tokens; p.out = W.out; p.in = W.in;
     p.n_tok_tiles = (a.tokens + Cfg::BN - 1) / Cfg::BN;
     p.n_out_tiles = (W.out + 2 * kBM - 1) / (2 * kBM);

@@ -15,9 +15,8 @@
 //   * The accumulators are single-buffered.  The MMA thread runs block 1 SKEW stages behind block 0, so that
 //     block 0's accumulator is handed to its four epilogue warps SKEW stages before block 1's and the next
 //     tile's block-0 MMAs can start while block 1's accumulator is still being read.
-//   * The MMA thread's instruction stream is kept short: descriptors are advanced with one add from values
-//     formed once, ring positions are carried instead of divided out (a single thread's dependent
-//     instructions cost several clocks each; 4 MMAs + commit took ~430 clocks in the 256 x 192 kernel).
+//   * The MMAs are issued from one elected lane of a warp-uniform path: descriptors are advanced with one add from values formed once, ring
+//     positions are carried instead of divided out.  What bounds it: the epilogue, exposed between two tiles, and the loads' latency.
 #pragma once
 
 namespace nm {
@@ -397,7 +396,7 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
             bool got = ptx::mbar_wait_bounded(acc_full_bar(blk), (uint32_t)i & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
             if (!ok && lane == 0) raise_timeout();
-            if constexpr (kNarrow<EPI>) ok = ptx::named_bar_and(kWideNarrowBar + blk, 128, ok);  // the block's four warps stop together
+            if constexpr (EPI == EPI_BF16) ok = ptx::named_bar_and(kWideNarrowBar + blk, 128, ok);  // the block's four warps stop together
             if (!ok) break;
             ptx::tc_fence_after();
             if (ew == 0 && lane == 0) NM_TRACE_TILE(i, 0);
@@ -415,9 +414,14 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                 continue;
             }
             if constexpr (kNarrow<EPI>) {
-                constexpr uint32_t kPerBlock = (EPI == EPI_BF16 ? 2 : 1) * 8192;
-                narrow_tile<EPI, 32, true>(acc_taddr, BN, p.tokens - t0, 0, 1, kWideNarrowBar + blk, ptx::smem_u32(store_stage) + blk * kPerBlock, n_stores,
-                                           q, lane, nc, nb, p.sy, rsy, &tmap_y, nw - q * 32, t0, p.out, stream_out, release_acc);
+                if constexpr (EPI == EPI_BF16) {
+                    narrow_group_tile<32>(acc_taddr, BN, p.tokens - t0, 0, 1, kWideNarrowBar + blk, ptx::smem_u32(store_stage) + blk * 16384, n_stores,
+                                          q, lane, nc, nb, &tmap_y, nw - q * 32, t0, p.out, stream_out, release_acc);
+                } else {
+                    constexpr int SUBS = BN / 16, PER = Cfg::STORE_STAGE / kWideEpiWarps;
+                    narrow_tile<EPI, SUBS, kNarrowStage<EPI, PER / 2, SUBS>, 2, W4 ? 1 : 2, true>(acc_taddr, p.tokens - t0, 0, 1, ptx::smem_u32(store_stage) + ew * PER,
+                        lane, nc, nb, p.sy, rsy, &tmap_y, nw, t0, p.out, stream_out, release_acc);
+                }
                 if (ew == 0 && lane == 0) NM_TRACE_TILE(i, 1);
                 if (ew == 4 && lane == 0) NM_TRACE_TILE(i, 3);
                 continue;

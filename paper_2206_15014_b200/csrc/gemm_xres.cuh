@@ -9,12 +9,10 @@
 // The index metadata changes with every tile: four metadata warps (one per TMEM lane quarter, both CTAs) keep a ring of
 // four buffers of 32 TMEM columns filled, one tile's reduction each.  A token tile's slices are replaced one by one as the
 // last output tile's MMAs are done with them.
-// What bounds it: with fp32 and int8 outputs the epilogue (stores; conversion): 2-3 k of a tile's 5.5-7 k clocks go by waiting for
-// an accumulator.  With bfloat16 the stages: about 1.1 k clocks each, 800 inside a tile with the other outputs, evenly over the
-// k-blocks, for 384 of MMAs at the tensor rate and 448 of shared memory (16 KB written, 40 KB read, counted, at 128 B/clk); 870 without any
-// epilogue, here and in nm_gemm_pair_kernel alike.  What makes the difference is not known: two MMAs of half the width instead, which
-// read the weights twice, add 230 clocks per 16 KB, alternating accumulators change nothing, and weights in 64-byte rows are
-// slower (16384 tokens 1024 -> 4096 64.6 / 62.0 us).
+// What bounds it: the epilogue.  A stage takes 370-480 clocks for 384 of MMAs (800-1100 while the MMAs' operands were built per thread, see
+// elect_one), a tile 3.4-5 k: fp32 by its stores, int8 by its conversion.  16384 tokens 768 -> 3072: bfloat16 31.7 -> 28.9 us
+// with staging tiles of each warp's own (narrow_tile).  Measured without gain: two MMAs of half the
+// width, alternating accumulators, weights in 64-byte rows (16384 tokens 1024 -> 4096 64.6 / 62.0 us).
 #pragma once
 
 namespace nm {
@@ -291,7 +289,7 @@ nm_gemm_xres_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
             bool got = ptx::mbar_wait_bounded(acc_full_bar(buf), (i >> 1) & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
             if (!ok && lane == 0) raise_timeout();
-            if constexpr (kNarrow<EPI>) ok = ptx::named_bar_and(kNarrowGroup + half, 128, ok);  // the group stops together
+            if (EPI == EPI_BF16 && p.grouped) ok = ptx::named_bar_and(kNarrowGroup + half, 128, ok);  // the group stops together
             if (!ok) break;
             ptx::tc_fence_after();
             if (ew == 0 && lane == 0) NM_TRACE_TILE(i, 0);
@@ -310,9 +308,13 @@ nm_gemm_xres_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
 #pragma unroll
                 for (int k = 0; k < 4; ++k) { nc[k] = __fmul_rn(sx, ns_next[k]); nb[k] = nb_next[k]; }
                 narrow_fetch(p.sw, p.bias, o * (2 * kBM) + (int)rank * kBM + q * 32, lane, p.out, ns_next, nb_next);
-                constexpr uint32_t kPerGroup = (EPI == EPI_BF16 ? 2 : 1) * 4096;
-                narrow_tile<EPI, 16, true>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, kNarrowGroup + half, ptx::smem_u32(store_stage) + half * kPerGroup,
-                                           n_stores, q, lane, nc, nb, p.sy, rsy, &tmap_y, n0, t0, p.out, stream_out, [&] { release_acc(buf); });
+                constexpr int SUBS = BN / 16 / EWH, PER = Cfg::STORE_STAGE / EW;
+                if (EPI == EPI_BF16 && p.grouped)
+                    narrow_group_tile<16>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, kNarrowGroup + half, ptx::smem_u32(store_stage) + half * 8192, n_stores,
+                                          q, lane, nc, nb, &tmap_y, n0, t0, p.out, stream_out, [&] { release_acc(buf); });
+                else
+                narrow_tile<EPI, SUBS, kNarrowStage<EPI, PER, SUBS>, 1, 1, true>(lane_taddr + buf * BN, p.tokens - t0, half, EWH, ptx::smem_u32(store_stage) + ew * PER,
+                    lane, nc, nb, p.sy, rsy, &tmap_y, n0 + q * 32, t0, p.out, stream_out, [&] { release_acc(buf); });
                 if (ew == 0 && lane == 0) { NM_TRACE_TILE(i, 1); NM_TRACE_EPI_FLUSH(i); }
                 continue;
             }

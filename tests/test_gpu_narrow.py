@@ -123,3 +123,27 @@ def test_narrow_outputs_reject_bad_arguments():
     with pytest.raises(nm.NmError):  # bfloat16 output on an odd byte address
         buf = torch.zeros(16 * 128 * 2 + 2, dtype=torch.uint8, device="cuda")
         nm.nm_int_linear_bf16(X, 16, packed.desc, 1.0, packed.scales, None, buf[1:], None)
+
+
+@pytest.mark.parametrize("n,m,bits,out", [(2, 4, 8, 3072), (2, 4, 4, 3080), (4, 4, 8, 3080), (2, 8, 4, 3072)])
+def test_bfloat16_too_large_for_the_cache(n, m, bits, out):
+    """At 192 MB of Y the pair kernels store whole lines, shared by four warps: the same bits as pieces of the same tokens."""
+    import torch
+    import paper_2206_15014_b200 as nm
+    from gpu_util import DEV
+    T, K = 34000, 1024  # the last tile ends inside a unit of 16 tokens
+    g = torch.Generator(device=DEV).manual_seed(out)
+    W = torch.randn((out, K), generator=g, device=DEV) * 0.02
+    vb, mb = nm.nm_packed_sizes(out, K, n, m, bits)
+    values, scales = torch.zeros(vb, dtype=torch.uint8, device=DEV), torch.zeros(out, device=DEV)
+    meta = torch.zeros(mb // 4, dtype=torch.int32, device=DEV) if n != m else None
+    nm.nm_project_pack(W, None, out, K, n, m, bits, values, meta, scales)
+    desc = nm.make_packed(out, K, n, m, bits, values, meta)
+    X = torch.randint(-128, 128, (T, K), generator=g, device=DEV, dtype=torch.int8)
+    Y, P = (torch.zeros((T, out), dtype=torch.bfloat16, device=DEV) for _ in range(2))
+    nm.nm_int_linear_bf16(X, T, desc, 0.02, scales, None, Y)
+    for a in range(0, T, 5000):
+        b = min(T, a + 5000)
+        nm.nm_int_linear_bf16(X[a:b], b - a, desc, 0.02, scales, None, P[a:b])
+    assert torch.equal(Y.view(torch.int16), P.view(torch.int16))
+    assert Y.any()
