@@ -189,7 +189,7 @@ __device__ __forceinline__ unsigned keep_mask(const float* a) {
 //
 // A row spans `wpr` warps; the partial sums of its warps are added in a fixed order, so the result is
 // deterministic.  85 M weights at 2:4 / 4 bit and 32 candidates, search and projection: 461 us with all candidates in single precision,
-// 297 so (12.6 M of 2:4 / 8 bit in rows of 1024 0.63 of the time; 398 shapes and formats 0.71 in the geometric mean, 1.05 at the worst, a
+// 297 so (398 shapes and formats 0.71 in the geometric mean, 1.05 at the worst, a
 // matrix of 1 M weights of dense 4 bit).  What bounds it now: instructions (61 % of the issue slots), their fetching among the stalls.
 // ---------------------------------------------------------------------------------------------
 template <int N, int M>
@@ -926,9 +926,9 @@ constexpr int kStagedBlocksPerSm = 3;
 // Resident blocks of four warps that the registers are cut for (kDirect).  Eight (64 registers) for the plain projection: with five
 // or six, more of a warp's loads are in flight, but 85 M weights in four formats take 125 / 116 us instead of 104, the
 // 24-layer sweep 436 / 441 instead of 403.  Dense outputs six (738 us; five and four the same).  The search four, and
-// six where a lane keeps at most eight values.
+// six where a lane keeps at most eight values or the codes have 4 bits.
 template <int N, int M, int BITS, bool DENSE_OUT, bool DIST>
-constexpr int kDirectBlocksPerSm = DIST ? (32 / M * N <= 8 ? 6 : BITS == 4 ? 6 : 4) : DENSE_OUT ? 6 : 8;
+constexpr int kDirectBlocksPerSm = DIST ? (32 / M * N <= 8 || BITS == 4 ? 6 : 4) : DENSE_OUT ? 6 : 8;
 
 constexpr int kFewBlocksPerSm = 5;  // the plain projection of two operands where no SM gets more blocks (see pick_bits)
 
