@@ -175,7 +175,8 @@ template <int EPI, int BYTES, int SUBS> constexpr int kNarrowStage = BYTES / (EP
 // warps of a group (rows of 128 channels) took a barrier or two a round, and 300 clocks for the group to agree on an expired wait; 16384
 // tokens 768 -> 3072 bfloat16 31.7 -> 28.9 us (35.0 with a lane per channel), int8 outputs over 263 shapes and formats 0.96 of the time.
 // int8: t = fma(y, rsy, 1.5 * 2^23) rounds the product to the nearest-even integer, which saturates to the code; `d` is the product's
-// distance from it, and within 2^-15 of a tie (or NaN) the IEEE division decides.
+// distance from it, and within 2^-15 of a tie (or NaN) the IEEE division decides.  Below -1.5 * 2^23 t turns negative and the integer
+// that its bits give, less those of 1.5 * 2^23, wraps round to the other end: rsy comes from narrow_rsy.
 //
 // acc: TMEM address of the tile's first column in this warp's lane quarter.  c, b: scale and bias of channels lane / 4 + 8 i of the quarter.
 // valid: tokens of the tile that exist.  n: the warp's first channel.  LD: pieces of 16 tokens that it has in registers together.
@@ -337,6 +338,16 @@ __device__ __forceinline__ void narrow_constants(const float* sw, const float* b
     narrow_fetch(sw, bias, first, lane, out, c, b);
 #pragma unroll
     for (int i = 0; i < 4; ++i) c[i] = __fmul_rn(sx, c[i]);
+}
+// The reciprocal of an int8 output scale for a thread's four channels in narrow_tile, or NaN (every code from the exact division) where a
+// product could leave the range in which the codes are taken from bits: an accumulator is at most in * 2^14, a product then below 2^23.
+// A bound per tile instead of a clamp per value: a scale that small (200 times under one that spreads the outputs over the codes)
+// saturates nearly every output.
+template <int EPI>
+__device__ __forceinline__ float narrow_rsy(float rsy, const float (&c)[4], const float (&b)[4], int in) {
+    if (EPI != EPI_Q8) return 0.0f;
+    const float c_max = ptx::max_abs_nan(c[0], c[1], ptx::max_abs_nan(c[2], c[3], 0.0f)), b_max = ptx::max_abs_nan(b[0], b[1], ptx::max_abs_nan(b[2], b[3], 0.0f));
+    return (c_max * ((float)in * 16384.0f) + b_max) * rsy < 8388608.0f ? rsy : __int_as_float(0x7fffffff);
 }
 
 // Pieces of metadata (16 bytes: one row, one 128-wide k-block) that a metadata warp of the one-CTA kernel has in flight (four
@@ -697,7 +708,7 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         int scaled_out_tile = -1;
         uint32_t n_stores = 0;
         int narrow_out_tile = -1;  // whose constants nc, nb are (narrow outputs)
-        float nc[4], nb[4];
+        float nc[4], nb[4], nrs = 0.0f;
         bool ok = true;
 
         // Index metadata of this lane's weight row for the whole reduction; rows past the end get a valid "positions 0,1" pattern,
@@ -762,6 +773,7 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
             if (kNarrow<EPI> && p.tma_store && out_tile != narrow_out_tile) {
                 narrow_out_tile = out_tile;
                 narrow_constants(p.sw, p.bias, sx, n0 + q * 32, lane, p.out, nc, nb);
+                nrs = narrow_rsy<EPI>(rsy, nc, nb, p.in);
             }
             bool got = ptx::mbar_wait_bounded(acc_full_bar(buf), (i >> 1) & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
@@ -787,7 +799,7 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
             if constexpr (kNarrow<EPI>) {
                 constexpr int SUBS = (BN / 16 + EWH - 1) / EWH;
                 narrow_tile<EPI, SUBS, kNarrowStage<EPI, kStoreStage / kEpiWarps, SUBS>, 1, 1, false>(lane_taddr + buf * BN, p.tokens - t0, half, EWH,
-                    ptx::smem_u32(store_stage) + ew * (kStoreStage / kEpiWarps), lane, nc, nb, p.sy, rsy, &tmap_y, n0 + q * 32, t0, p.out, 0, [&] { release_acc(buf); });
+                    ptx::smem_u32(store_stage) + ew * (kStoreStage / kEpiWarps), lane, nc, nb, p.sy, nrs, &tmap_y, n0 + q * 32, t0, p.out, 0, [&] { release_acc(buf); });
                 continue;
             }
             if constexpr (!kNarrow<EPI>) {
@@ -1173,7 +1185,7 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
         int scaled_out_tile = -1;
         uint32_t n_stores = 0;
         int narrow_out_tile = -1;  // whose constants nc, nb are (narrow outputs)
-        float nc[4], nb[4];
+        float nc[4], nb[4], nrs = 0.0f;
         bool ok = true;
 
         auto load_meta = [&](int out_tile) {
@@ -1212,6 +1224,7 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
             if (kNarrow<EPI> && p.tma_store && out_tile != narrow_out_tile) {
                 narrow_out_tile = out_tile;
                 narrow_constants(p.sw, p.bias, sx, n0 + q * 32, lane, p.out, nc, nb);
+                nrs = narrow_rsy<EPI>(rsy, nc, nb, p.in);
             }
             bool got = ptx::mbar_wait_bounded(acc_full_bar(buf), (i >> 1) & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
@@ -1245,7 +1258,7 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                                           q, lane, nc, nb, &tmap_y, n0, t0, p.out, stream_out, [&] { release_acc(buf); });
                 else
                 narrow_tile<EPI, SUBS, kNarrowStage<EPI, PER, SUBS>, 1, 1, true>(lane_taddr + buf * BN, p.tokens - t0, half, EWH, ptx::smem_u32(store_stage) + ew * PER,
-                    lane, nc, nb, p.sy, rsy, &tmap_y, n0 + q * 32, t0, p.out, stream_out, [&] { release_acc(buf); });
+                    lane, nc, nb, p.sy, nrs, &tmap_y, n0 + q * 32, t0, p.out, stream_out, [&] { release_acc(buf); });
                 if (ew == 0 && lane == 0) { NM_TRACE_TILE(i, 1); NM_TRACE_EPI_FLUSH(i); }
                 continue;
             }

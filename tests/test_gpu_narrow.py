@@ -125,6 +125,44 @@ def test_narrow_outputs_reject_bad_arguments():
         nm.nm_int_linear_bf16(X, 16, packed.desc, 1.0, packed.scales, None, buf[1:], None)
 
 
+# (tokens, K, out, n, m, bits, options): every kernel that stores int8 tiles, and the split one
+SCALE_CASES = [
+    (77, 128, 208, 2, 4, 8, {"split": 1}),         # one-CTA kernel, weights through TMA
+    (77, 256, 208, 4, 4, 8, {"split": 2032}),      # split reduction: stores of its own
+    (4096 + 37, 512, 1280, 2, 4, 4, {}),           # one-CTA kernel, weights rebuilt and resident
+    (300, 2048, 640, 1, 8, 4, {"split": 1}),       # ... rebuilt for every k-block
+    (3000, 1024, 1296, 2, 4, 8, {"xres": 1}),      # pair kernel with resident activations
+    (3000, 1024, 1296, 4, 4, 8, {"xres": 1}),
+    (3000, 1024, 1296, 2, 4, 8, {"xres": 2}),      # ... with resident weights
+    (6003, 2048, 640, 4, 4, 8, {}),                # ... with both streamed
+    (6003, 2048, 640, 2, 4, 8, {"no_wide": 1}),
+    (6003, 2048, 640, 2, 4, 8, {}),                # 512-channel kernel
+    (6003, 2048, 640, 2, 4, 4, {}),
+]
+
+
+@pytest.mark.parametrize("T,K,out,n,m,bits,options", SCALE_CASES)
+def test_int8_output_at_any_scale(T, K, out, n, m, bits, options):
+    """Quotients y / sy from far inside one code to far beyond the integers that single precision holds, both signs: every
+    power of two around 2^23, where codes taken from bits of a sum could leave their range, and 1e-9 to 1e9 of the largest |Y|."""
+    import paper_2206_15014_b200 as nm
+    from gpu_util import PackedOnDevice, gpu_int_linear_q8
+    Xq, sx, v, meta, s, b, Y = _setup(T + K, T, K, out, n, m, bits)
+    packed = PackedOnDevice(v, meta, s, out, K, n, m, bits)
+    amax = np.float32(np.abs(Y).max())
+    try:
+        for k, x in options.items():
+            nm.nm_debug_set_option(k, x)
+        for quotient in [2.0 ** e for e in range(20, 29)] + [1e9, 1e-9, 1e5, 1e36]:
+            sy = np.float32(float(amax) / quotient)
+            ref = oracle.requantize_static(Y, sy)
+            got = gpu_int_linear_q8(Xq, packed, sx, b, sy)
+            assert np.array_equal(got, ref), f"{(got != ref).sum()} of {ref.size} codes differ at max|Y| / sy = {quotient}"
+    finally:
+        for k in options:
+            nm.nm_debug_set_option(k, 0)
+
+
 @pytest.mark.parametrize("n,m,bits,out", [(2, 4, 8, 3072), (2, 4, 4, 3080), (4, 4, 8, 3080), (2, 8, 4, 3072)])
 def test_bfloat16_too_large_for_the_cache(n, m, bits, out):
     """At 192 MB of Y the pair kernels store whole lines, shared by four warps: the same bits as pieces of the same tokens."""
