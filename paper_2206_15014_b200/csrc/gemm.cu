@@ -1641,7 +1641,7 @@ static int launch_gemm_split(const LinearArgs& a, int splits) {
     p.mrow_bytes = (int)meta_row_words(W.in, W.n, W.m) * 4;
     p.pat = xf::pattern_of(W.n, W.m, W.bits);
     p.sw = a.sw; p.bias = a.bias; p.sx_dev = a.sx_dev; p.sx_host = a.sx;
-    p.Y = a.Y; p.ACC = a.ACC; p.NARROW = a.NARROW; p.sy = a.sy; p.absmax = a.absmax; p.status = a.status;
+    p.Y = a.Y; p.ACC = a.ACC; p.NARROW = a.NARROW; p.sy = a.sy; p.absmax = a.absmax; p.status = a.status; p.skip_stage = g_opt.skip_stage - 1;
     auto fn = nm_gemm_split_kernel<SPARSE, BN, EPI, XF>;
     NM_CUDA_TRY(allow_dynamic_smem((const void*)fn, Cfg::SMEM));
     cudaLaunchConfig_t cfg = {};
@@ -1801,7 +1801,7 @@ static int resident_clusters(int splits) {
 // not taken: a reduction of three k-blocks (1 token 384 -> 1536, 4:4 / 4 bit 4.25 / 4.51), 200 tokens 1024 -> 4096, 2:4 / 4 bit 7.3 / 8.3.
 template <bool SPARSE>
 static int split_plan(const LinearArgs& a, int unsplit_bn, bool xf = false) {
-    if (g_opt.split == 1 || g_opt.one_bn || g_opt.skip_stage) return 0;  // the test hook counts the stages of an unsplit tile
+    if (g_opt.split == 1 || g_opt.one_bn || (g_opt.skip_stage && !g_opt.split)) return 0;  // the test hook counts the stages of an unsplit tile
     const int kblocks = a.W->in / kKB, out_tiles = (a.W->out + kBM - 1) / kBM;
     const long long unsplit = xf ? (long long)kblocks * (unsplit_bn + 384) + 4 * unsplit_bn : (long long)kblocks * (unsplit_bn + 256);
     long long best_cost = 0;

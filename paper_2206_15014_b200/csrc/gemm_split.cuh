@@ -10,6 +10,9 @@
 //   warp 1      allocates TMEM; one lane waits for the stages and issues the MMAs
 //   warps 2-9   index metadata of the CTA's k-blocks into TMEM (the first four), exchange, epilogue with direct stores
 //   warps 10-21 (XF: weights not in tensor-core form) three groups of four build the weight tiles as in nm_gemm_kernel
+// An expired wait: the MMA warp issues nothing more, so no stage comes free after the one that was missed and nobody goes round the ring
+// beyond it; the epilogue warps, which wait in vain for the accumulator, set the flag of every CTA of the cluster between its two
+// barriers, and no CTA of it writes outputs.
 #pragma once
 
 namespace nm {
@@ -97,6 +100,7 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
             for (int it = 0; it < kb_count; ++it) {
                 const int s = it % S, kb = kb_begin + it;
                 if (!ptx::mbar_wait_bounded(empty_bar(s), ((it / S) & 1u) ^ 1u, abort_flag, kWaitLimit)) { raise_timeout(); break; }
+                if (NM_SKIP_STAGE((uint32_t)it)) continue;
                 const uint32_t a_dst = ptx::smem_u32(smem + s * Cfg::STAGE);
                 ptx::mbar_expect_tx(full_bar(s), XF ? Cfg::B_BYTES : Cfg::STAGE);
                 if (!XF) ptx::tma_load_2d(a_dst, &tmap_w, kb * Cfg::A_ROW, n0, full_bar(s));
@@ -218,10 +222,14 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
             ptx::st_cluster_v4(dst, r[0], r[1], r[2], r[3]);
             ptx::st_cluster_v4(dst + kBM * 16u, r[4], r[5], r[6], r[7]);
         }
+    } else if (!ok && lane < splits) {
+        // no sums from here: everyone's flag, so that nobody finishes tokens from what was never sent
+        ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32((const void*)abort_flag), (uint32_t)lane), 1u);
     }
     __syncwarp();
     ptx::cluster_arrive();
     ptx::cluster_wait();
+    ok = ok && *abort_flag == 0u;
     if (warp >= 2 && warp < kSplitThreads / 32 && ok) {
         const float rsy = EPI == EPI_Q8 ? __frcp_rn(p.sy) : 0.0f;
         float amax = 0.0f;

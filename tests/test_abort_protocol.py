@@ -133,3 +133,81 @@ def test_the_model_sees_the_fault_when_the_gate_goes_on_at_once():
     with pytest.raises(AssertionError, match="pending count of zero"):
         for seed in range(200):
             _run(seed, gate_waits=False)
+
+
+def _run_split(seed, kblocks=9, stages=4, skipped=1, ctas=3, builders=4, tells=True):
+    """The split kernel: CTA 0's producer leaves one stage out.  No gate: the MMA thread waits itself and stops for good, its epilogue warps
+    then fail.  Returns, per CTA, whether it writes outputs, and which CTAs' sums it has."""
+    rng = random.Random(seed)
+    full = [[Full(1 + builders) for _ in range(stages)] for _ in range(ctas)]
+    empty = [[0] * stages for _ in range(ctas)]
+    abort, acc, failed = [False] * ctas, [False] * ctas, [False] * ctas
+    met, sums, wrote = [0, 0], [set() for _ in range(ctas)], [None] * ctas
+
+    def ready(c, cond, patience=4000):
+        spins = 0
+        while not cond():
+            spins += 1
+            if (abort[c] and rng.random() < 0.3) or spins > patience:
+                return False
+            yield
+        return True
+
+    def producer(c, expects):  # of X, with bytes to come, or a builder warp
+        for it in range(kblocks):
+            s = it % stages
+            if not (yield from ready(c, lambda: empty[c][s] >= it // stages)):
+                abort[c] = True
+                return
+            if c == 0 and it == skipped and expects:
+                continue
+            full[c][s].arrive(expect=1 if expects else 0)
+            yield
+            if expects:
+                full[c][s].bytes(1)
+
+    def mma(c):
+        for it in range(kblocks):
+            if not (yield from ready(c, lambda: full[c][it % stages].phase > it // stages, 600)):
+                abort[c] = True
+                return
+            empty[c][it % stages] += 1
+            yield
+        acc[c] = True
+
+    def epilogue(c):
+        ok = yield from ready(c, lambda: acc[c])
+        abort[c] = abort[c] or not ok
+        for step in range(2):
+            met[step] += 1
+            while met[step] < ctas:           # the cluster's barriers: everyone arrives, flag or not
+                yield
+            if step == 0:
+                for r in range(ctas):
+                    if ok:
+                        sums[r].add(c)
+                    elif tells:
+                        abort[r] = True
+                yield
+        wrote[c] = ok and not abort[c]
+
+    roles = [g for c in range(ctas) for g in [producer(c, True), mma(c), epilogue(c)] + [producer(c, False) for _ in range(builders)]]
+    while roles:
+        r = rng.choice(roles)
+        try:
+            next(r)
+        except StopIteration:
+            roles.remove(r)
+    return wrote, sums
+
+
+def test_split_kernel_writes_nothing_once_a_cta_has_given_up():
+    src = open(os.path.join(CSRC, "gemm_split.cuh")).read()
+    tells = re.search(r"else if \(!ok[^{]*\{[^}]*st_cluster_u32\(ptx::map_to_cta\([^;]*abort_flag[^;]*;\s*\}\s*__syncwarp\(\);\s*ptx::cluster_arrive\(\);"
+                      r"\s*ptx::cluster_wait\(\);\s*ok = ok && \*abort_flag == 0u;", src) is not None
+    for seed in range(30):
+        wrote, sums = _run_split(seed, tells=tells)
+        assert not any(w and len(s) < len(sums) for w, s in zip(wrote, sums)), "outputs from sums that were never sent"
+    assert any(any(_run_split(seed, tells=False)[0]) for seed in range(30))  # the model sees the fault
+    wrote, sums = _run_split(1, skipped=-1)
+    assert all(wrote) and all(len(s) == 3 for s in sums)

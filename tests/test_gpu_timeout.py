@@ -24,7 +24,7 @@ def _shortwait_lib():
     return mod.build(variant="shortwait")
 
 
-@pytest.mark.parametrize("family", ["one_cta", "one_cta_narrow", "pair", "pair_streamed", "pack_staged"])
+@pytest.mark.parametrize("family", ["one_cta", "one_cta_narrow", "pair", "pair_streamed", "split", "split_rebuilt", "pack_staged"])
 def test_expired_wait_reports_timeout_and_leaves_the_context_usable(family):
     env = dict(os.environ, NMSPARSE_LIB=_shortwait_lib())
     r = subprocess.run([sys.executable, os.path.join(ROOT, "tests", "timeout_case.py"), family], env=env,

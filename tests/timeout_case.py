@@ -14,12 +14,14 @@ import oracle  # noqa: E402
 import workloads as wl  # noqa: E402
 import paper_2206_15014_b200 as nm  # noqa: E402
 
-# family -> (tokens, K, out, options, int8 output?)
+# family -> (tokens, K, out, weight bits, options, int8 output?)
 FAMILIES = {
-    "one_cta": (64, 512, 128, {}, False),                       # one tile, four stages, nm_gemm_kernel
-    "one_cta_narrow": (64, 512, 128, {}, True),                 # the same through the int8-output epilogue's group agreement
-    "pair": (74 * 192, 1024, 256, {}, False),                   # one tile of four stages per SM pair, resident weights: pair 0 stalls alone
-    "pair_streamed": (74 * 192, 1024, 256, {"no_resident": 1}, False),
+    "one_cta": (64, 512, 128, 8, {"split": 1}, False),             # one tile, four stages, nm_gemm_kernel
+    "one_cta_narrow": (64, 512, 128, 8, {"split": 1}, True),       # the same with int8 outputs (staging tiles of each warp's own)
+    "pair": (74 * 192, 1024, 256, 8, {}, False),                   # one tile of four stages per SM pair, resident weights: pair 0 stalls alone
+    "pair_streamed": (74 * 192, 1024, 256, 8, {"no_resident": 1}, False),
+    "split": (64, 4096, 128, 8, {"split": 4064}, False),           # one tile over a cluster of four CTAs, eight stages each: CTA 0 stalls alone
+    "split_rebuilt": (32, 6144, 128, 4, {"split": 2032}, False),   # ... of two, 24 stages in a shorter ring, weights built on the way
 }
 
 
@@ -62,20 +64,20 @@ def pack_staged():
 def main(family):
     if family == "pack_staged":
         return pack_staged()
-    T, K, out, options, narrow = FAMILIES[family]
+    T, K, out, bits, options, narrow = FAMILIES[family]
     dev = torch.device("cuda:0")
     oracle.set_threads(oracle.max_threads())
     rng = np.random.default_rng(7)
     W = wl.normal(rng, (out, K), 0.02)
     b = wl.normal(rng, (out,), 0.02)
     Xq, sx = oracle.quantize_act(wl.normal(rng, (T, K)))
-    v, meta, s = oracle.project_pack(W, None, 2, 4, 8)
-    D = oracle.unpack(v, meta, out, K, 2, 4, 8)
+    v, meta, s = oracle.project_pack(W, None, 2, 4, bits)
+    D = oracle.unpack(v, meta, out, K, 2, 4, bits)
     _, Y_ref = oracle.int_linear(Xq, D, sx, s, b, want_acc=False)
     sy = np.float32(np.abs(Y_ref).max()) / np.float32(127.0)
     td = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev)
     Xd, vd, md, sd, bd = td(Xq), td(v.reshape(-1)), td(meta.reshape(-1).view(np.int32)), td(s), td(b)
-    desc = nm.make_packed(out, K, 2, 4, 8, vd, md)
+    desc = nm.make_packed(out, K, 2, 4, bits, vd, md)
     status = torch.zeros(1, dtype=torch.int32, device=dev)
     for k_, v_ in options.items():
         nm.nm_debug_set_option(k_, v_)
@@ -90,9 +92,11 @@ def main(family):
         return Y
 
     nm.nm_debug_set_option("skip_stage", 2)   # CTA 0 never issues its second pipeline stage
-    launch()
+    Y = launch()
     rc = nm.nm_poll_status(status)
     assert rc == nm.NM_ERR_TIMEOUT, f"expected a timeout, got {nm.nm_strerror(rc)} {nm.nm_last_cuda_error()}"
+    if family.startswith("split"):            # the cluster's other CTAs know: nobody writes sums that lack a part
+        assert not Y.any()
     nm.nm_debug_set_option("skip_stage", 0)
     status.zero_()
     Y = launch()                              # same stream, same context: a normal call works and is right
