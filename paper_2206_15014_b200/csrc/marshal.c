@@ -45,6 +45,7 @@ typedef struct {
     PyObject* twin;                    /* the Python function */
     PyObject* packed_type;             /* class of the weight descriptor */
     PyObject* check;                   /* check(code, name) raises the library's error */
+    PyObject *dict, *weakrefs;
 } Entry;
 
 static PyObject *s_data_ptr, *current_device, *raw_stream;
@@ -180,20 +181,37 @@ twin:
 
 static int entry_traverse(PyObject* self, visitproc visit, void* arg) {
     Entry* e = (Entry*)self;
-    Py_VISIT(e->twin); Py_VISIT(e->packed_type); Py_VISIT(e->check);
+    Py_VISIT(e->twin); Py_VISIT(e->packed_type); Py_VISIT(e->check); Py_VISIT(e->dict);
     return 0;
 }
+/* The cycle through the twin's globals is broken there: an entry that a finaliser calls late still has all it needs. */
 static int entry_clear(PyObject* self) {
-    Entry* e = (Entry*)self;
-    Py_CLEAR(e->twin); Py_CLEAR(e->packed_type); Py_CLEAR(e->check);
+    Py_CLEAR(((Entry*)self)->dict);
     return 0;
 }
 static void entry_dealloc(PyObject* self) {
+    Entry* e = (Entry*)self;
     PyObject_GC_UnTrack(self);
-    entry_clear(self);
+    if (e->weakrefs) PyObject_ClearWeakRefs(self);
+    Py_CLEAR(e->dict);
+    Py_DECREF(e->twin); Py_DECREF(e->packed_type); Py_DECREF(e->check);
     PyObject_GC_Del(self);
 }
-/* __name__, __doc__ and the signature (through __wrapped__) are the twin's. */
+/* Everything else that a Python function can do: __name__, __doc__ and the signature (through __wrapped__) are the twin's, and so is
+ * every attribute not set here; an entry pickles and copies by its name, binds as a method and takes attributes and weak references. */
+static PyObject* entry_getattro(PyObject* self, PyObject* name) {
+    PyObject* v = PyObject_GenericGetAttr(self, name);
+    if (v || !PyErr_ExceptionMatches(PyExc_AttributeError)) return v;
+    PyErr_Clear();
+    return PyObject_GetAttr(((Entry*)self)->twin, name);
+}
+static PyObject* entry_repr(PyObject* self) { return PyObject_Repr(((Entry*)self)->twin); }
+static PyObject* entry_bind(PyObject* self, PyObject* obj, PyObject* type) {
+    (void)type;
+    return obj ? PyMethod_New(self, obj) : Py_NewRef(self);
+}
+static PyObject* entry_reduce(PyObject* self, PyObject* none) { (void)none; return PyObject_GetAttrString(((Entry*)self)->twin, "__qualname__"); }
+static PyMethodDef entry_methods[] = {{"__reduce__", entry_reduce, METH_NOARGS, NULL}, {NULL, NULL, 0, NULL}};
 static PyObject* get_wrapped(PyObject* self, void* c) { (void)c; return Py_NewRef(((Entry*)self)->twin); }
 static PyObject* get_of_twin(PyObject* self, void* attr) { return PyObject_GetAttrString(((Entry*)self)->twin, (const char*)attr); }
 static PyGetSetDef entry_getset[] = {{"__wrapped__", get_wrapped, NULL, NULL, NULL},
@@ -201,6 +219,7 @@ static PyGetSetDef entry_getset[] = {{"__wrapped__", get_wrapped, NULL, NULL, NU
                                      {"__qualname__", get_of_twin, NULL, NULL, "__qualname__"},
                                      {"__module__", get_of_twin, NULL, NULL, "__module__"},
                                      {"__doc__", get_of_twin, NULL, NULL, "__doc__"},
+                                     {"__dict__", PyObject_GenericGetDict, PyObject_GenericSetDict, NULL, NULL},
                                      {NULL, NULL, NULL, NULL, NULL}};
 static PyTypeObject EntryType = {
     PyVarObject_HEAD_INIT(NULL, 0).tp_name = "_marshal.Entry",
@@ -212,6 +231,13 @@ static PyTypeObject EntryType = {
     .tp_traverse = entry_traverse,
     .tp_clear = entry_clear,
     .tp_getset = entry_getset,
+    .tp_methods = entry_methods,
+    .tp_getattro = entry_getattro,
+    .tp_setattro = PyObject_GenericSetAttr,
+    .tp_repr = entry_repr,
+    .tp_descr_get = entry_bind,
+    .tp_dictoffset = offsetof(Entry, dict),
+    .tp_weaklistoffset = offsetof(Entry, weakrefs),
 };
 
 /* entry(name, address of the C entry point, Python twin, weight descriptor class, check) */
@@ -231,6 +257,7 @@ static PyObject* entry(PyObject* self, PyObject* args) {
         e->twin = Py_NewRef(twin);
         e->packed_type = Py_NewRef(cls);
         e->check = Py_NewRef(check);
+        e->dict = e->weakrefs = NULL;
         PyObject_GC_Track((PyObject*)e);
         return (PyObject*)e;
     }

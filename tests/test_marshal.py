@@ -1,7 +1,11 @@
 """The extension module of the binding takes every call form that its Python twins take, with the same results and errors
 (no GPU needed: calls that return before a launch)."""
+import copy
 import ctypes
 import inspect
+import pickle
+import types
+import weakref
 
 import numpy as np
 import pytest
@@ -58,3 +62,23 @@ def test_error_codes_and_descriptor_checks():
 
     with pytest.raises(ctypes.ArgumentError):
         nm.nm_int_linear(t, 0, Other(), 0.5, t, None, t, stream=0)
+
+
+@pytest.mark.parametrize("name", NAMES)
+def test_an_entry_does_what_a_function_does(name):
+    fast, twin = getattr(nm, name), inspect.unwrap(getattr(nm, name))
+    assert pickle.loads(pickle.dumps(fast)) is fast and copy.copy(fast) is fast
+    held = types.SimpleNamespace(call=fast, other=[fast])
+    again = copy.deepcopy(held)
+    assert again.call is fast and again.other[0] is fast
+    assert weakref.ref(fast)() is fast
+    assert fast.__defaults__ == twin.__defaults__ and fast.__code__ is twin.__code__ and name in repr(fast)
+    with pytest.raises(AttributeError):
+        fast.no_such_attribute
+    fast.note = 1
+    try:
+        assert fast.note == 1 and not hasattr(twin, "note")
+    finally:
+        del fast.note
+    bound = type("Holder", (), {"call": fast})().call
+    assert isinstance(bound, types.MethodType) and bound.__func__ is fast
