@@ -8,6 +8,7 @@ library has not been built (run ``python paper_2206_15014_b200/build.py``).
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
 import importlib.util
 import os
 
@@ -360,9 +361,12 @@ def nm_poll_status(status=None, stream=None):
 
 
 # The calls that a program makes once per layer go through a small extension module (csrc/marshal.c), which converts plain
-# arguments itself and hands anything else to the functions above.
+# arguments itself and hands anything else to the functions above.  Where it has not been built for this interpreter they stay as they are.
 def _fast_entries():
-    spec = importlib.util.spec_from_file_location("_marshal", os.path.join(_HERE, "_marshal.so"))
+    path = os.path.join(_HERE, "_marshal" + importlib.machinery.EXTENSION_SUFFIXES[0])
+    if not os.path.exists(path):
+        return
+    spec = importlib.util.spec_from_file_location("_marshal", path)
     marshal = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(marshal)
     for name in ("nm_int_linear", "nm_int_linear_dsx", "nm_int_linear_q8", "nm_int_linear_bf16", "nm_absmax", "nm_quantize_act"):

@@ -1,6 +1,7 @@
 """Builds libnmsparse.so (the C-ABI library) in-tree with nvcc for sm_100a."""
 from __future__ import annotations
 
+import importlib.machinery
 import os
 import subprocess
 import sys
@@ -20,17 +21,22 @@ FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std
 VARIANTS = {"": [], "trace": ["-DNM_TRACE"], "shortwait": ["-DNM_WAIT_LIMIT=(1ll<<21)", "-DNM_TEST_HOOKS"]}
 
 
-# Extension module of the Python binding (csrc/marshal.c): plain C against the interpreter's headers.
-MARSHAL = os.path.join(HERE, "_marshal.so")
+# Extension module of the Python binding (csrc/marshal.c): plain C against the interpreter's headers, under this interpreter's tag, so that
+# no other one loads it.  The binding is complete without it, and the library is built where it cannot be.
+MARSHAL = os.path.join(HERE, "_marshal" + importlib.machinery.EXTENSION_SUFFIXES[0])
 
 
-def build_marshal(force: bool = False) -> str:
-    src, header = os.path.join(CSRC, "marshal.c"), os.path.join(os.path.dirname(HERE), "include", "nmsparse.h")
-    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= max(os.path.getmtime(src), os.path.getmtime(header)):
+def build_marshal(force: bool = False) -> str | None:
+    deps = (os.path.join(CSRC, "marshal.c"), os.path.join(os.path.dirname(HERE), "include", "nmsparse.h"), os.path.abspath(__file__))
+    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= max(map(os.path.getmtime, deps)):
         return MARSHAL
     tmp = MARSHAL + f".tmp{os.getpid()}"
-    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"],
-                           src, "-o", tmp])
+    try:
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"],
+                               deps[0], "-o", tmp])
+    except (OSError, subprocess.CalledProcessError) as e:
+        sys.stderr.write(f"{os.path.basename(MARSHAL)} not built ({e}): calls go through ctypes\n")
+        return None
     os.replace(tmp, MARSHAL)
     return MARSHAL
 

@@ -2,8 +2,14 @@
 (no GPU needed: calls that return before a launch)."""
 import copy
 import ctypes
+import importlib.machinery
+import importlib.util
 import inspect
+import os
 import pickle
+import shutil
+import subprocess
+import sys
 import types
 import weakref
 
@@ -12,6 +18,9 @@ import pytest
 import torch
 
 import paper_2206_15014_b200 as nm
+
+PACKAGE = os.path.dirname(os.path.abspath(nm.__file__))
+SUFFIX = importlib.machinery.EXTENSION_SUFFIXES[0]
 
 NAMES = ("nm_int_linear", "nm_int_linear_dsx", "nm_int_linear_q8", "nm_int_linear_bf16", "nm_absmax", "nm_quantize_act")
 
@@ -82,3 +91,44 @@ def test_an_entry_does_what_a_function_does(name):
         del fast.note
     bound = type("Holder", (), {"call": fast})().call
     assert isinstance(bound, types.MethodType) and bound.__func__ is fast
+
+
+def _imported_from(tmp_path, files):
+    """The package with only the given files beside __init__.py, imported by another process: the type of an entry."""
+    home = tmp_path / "paper_2206_15014_b200"
+    home.mkdir()
+    shutil.copy(os.path.join(PACKAGE, "__init__.py"), home)
+    for name, source in files.items():
+        if source is None:
+            (home / name).write_bytes(b"not for this interpreter")
+        else:
+            shutil.copy(source, home / name)
+    env = dict(os.environ, NMSPARSE_LIB=nm.LIB_PATH, PYTHONPATH=str(tmp_path))
+    r = subprocess.run([sys.executable, "-c", "import paper_2206_15014_b200 as nm; assert nm.nm_version(); print(type(nm.nm_int_linear).__name__)"],
+                       env=env, cwd=tmp_path, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    return r.stdout.split()[-1]
+
+
+def test_the_package_is_complete_without_the_extension(tmp_path):
+    assert _imported_from(tmp_path, {}) == "function"
+
+
+def test_only_the_extension_of_this_interpreter_is_loaded(tmp_path):
+    assert os.path.exists(os.path.join(PACKAGE, "_marshal" + SUFFIX)) and "." in SUFFIX[1:]
+    assert _imported_from(tmp_path, {"_marshal.so": None, "_marshal.cpython-39-x86_64-linux-gnu.so": None}) == "function"
+
+
+def test_the_library_is_built_where_the_extension_cannot_be(monkeypatch, tmp_path, capsys):
+    spec = importlib.util.spec_from_file_location("nm_build", os.path.join(PACKAGE, "build.py"))
+    build = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(build)
+    built = []
+    monkeypatch.setattr(build, "MARSHAL", str(tmp_path / "_marshal.so"))
+    monkeypatch.setattr(build, "LIB", str(tmp_path / "lib.so"))
+    monkeypatch.setattr(build, "CSRC", shutil.copytree(build.CSRC, tmp_path / "csrc"))
+    monkeypatch.setenv("CC", str(tmp_path / "no_such_compiler"))
+    monkeypatch.setenv("NVCC", shutil.which("true"))  # stands in for nvcc
+    monkeypatch.setattr(build.os, "replace", lambda a, b: built.append(b))
+    assert build.build() == build.LIB and built == [build.LIB]
+    assert "not built" in capsys.readouterr().err
