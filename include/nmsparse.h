@@ -314,6 +314,13 @@ int nm_pair_tile_plan(int n_tok_tiles, int n_out_tiles, int pairs, int resident,
                       int *start, int *tile_out, int *tile_tok);
 
 /*
+ * Host-only: whether nm_int_linear and its variants split the reduction of a problem over a cluster (for inspection and tests; it
+ * launches nothing): 1000 * CTAs of a cluster + token-tile width, 0 = not split, or a negative error.  clusters (nullable): how many
+ * clusters of 2, 4 and 8 CTAs run at a time; NULL asks the current device.
+ */
+int nm_split_plan(int tokens, int out, int in, int n, int m, int bits, const int *clusters /* [3], host */);
+
+/*
  * Measurement aid (the paper has no counterpart): the memory traffic of the CTA-pair kernel of nm_int_linear
  * without its arithmetic.  Every CTA pair walks the tiles nm_pair_tile_plan gives it (streamed form); per
  * pipeline stage each CTA loads a box of `a_rows` x `a_row_bytes` (64 or 128) from W, a row-major byte matrix
@@ -347,8 +354,8 @@ int nm_probe_tma_stream(const void *W, int w_rows, int w_row_bytes, const void *
  * dependent-launch attribute), "no_pair" (one-CTA kernels only), "no_resident" (always stream the weights),
  * "no_wide" (never the 512-channel pair kernel), "wide_any" (the 512-channel pair kernel whenever the shape
  * allows it, however few tiles there are), "wide_bn" (its token-tile width, 224 or 192), "band" (band size of the streamed pair kernel's tile order),
- * "split" (one-CTA tiles with the reduction split over a cluster: 1000 * CTAs + token-tile width, for instance 4096, where that
- * fits, 1 = never), "one_bn" (token-tile width of the one-CTA kernel: 192, 128, 96, 64 or 32 where it exists), "xres" (the pair kernel with resident
+ * "split" (one-CTA tiles with the reduction split over a cluster: 1000 * CTAs + token-tile width, for instance 4096,
+ * 1 = never; a call that would run on one-CTA tiles and cannot have that split returns NM_ERR_UNSUPPORTED), "one_bn" (token-tile width of the one-CTA kernel: 192, 128, 96, 64 or 32 where it exists), "xres" (the pair kernel with resident
  * activations: 1 = wherever a pair kernel with a reduction of at most 1024 runs, 2 = never),
  * "pack_form" (form of the projection kernel in blocks of four warps: 2 = persistent with the next rows staged in shared
  * memory by bulk copies, where that form exists: 1:4, 2:4, 1:8 and 2:8 without dense outputs; 1 or 3 = one unit per block).

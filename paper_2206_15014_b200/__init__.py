@@ -37,7 +37,7 @@ EXPORTS = (
     "nm_int_linear", "nm_int_linear_dsx", "nm_int_linear_acc", "nm_int_linear_q8", "nm_int_linear_bf16",
     "nm_int_linear_workspace_bytes",
     "nm_int_linear_check", "nm_absmax", "nm_quantize_act", "nm_poll_status", "nm_strerror",
-    "nm_last_cuda_error", "nm_version", "nm_bits_per_param", "nm_encoder_cost", "nm_pair_tile_plan",
+    "nm_last_cuda_error", "nm_version", "nm_bits_per_param", "nm_encoder_cost", "nm_pair_tile_plan", "nm_split_plan",
     "nm_probe_tma_stream", "nm_debug_set_trace", "nm_debug_set_option",
 )
 
@@ -309,6 +309,14 @@ def nm_pair_tile_plan(n_tok_tiles, n_out_tiles, pairs, resident, band_request=0)
     band = _lib.nm_pair_tile_plan(n_tok_tiles, n_out_tiles, pairs, int(bool(resident)), band_request, start, to, tt)
     _chk(min(band, 0), "nm_pair_tile_plan")
     return band, list(start), list(to)[:n], list(tt)[:n]
+
+
+def nm_split_plan(tokens, out, in_, n, m, bits, clusters=None):
+    """-> 1000 * CTAs + token-tile width of the split reduction the linear layer takes, 0 = not split (host only; `clusters`:
+    how many clusters of 2, 4 and 8 CTAs run at a time, None = as the current device says)."""
+    plan = _lib.nm_split_plan(tokens, out, in_, n, m, bits, None if clusters is None else (ctypes.c_int * 3)(*clusters))
+    _chk(min(plan, 0), "nm_split_plan")
+    return plan
 
 
 def nm_bits_per_param(n, m, bits, index_bits=-1):

@@ -1699,7 +1699,6 @@ static bool one_wave(const LinearArgs& a) {
 // up, times the tile width); 0 = the wide kernel does not apply (short reductions keep their weights resident in
 // the 256-channel kernel; a matrix of at most 256 channels would leave one of the two blocks idle; narrow outputs
 // and small problems stay on the other kernels).
-template <int EPI>
 static int wide_bn(const LinearArgs& a) {
     if (g_opt.no_wide || g_opt.no_pair) return 0;
     const nm_packed_t& W = *a.W;
@@ -1719,7 +1718,7 @@ static int wide_bn(const LinearArgs& a) {
 }
 
 // The pair kernel pays off when there is enough work for every SM pair; small problems stay on one CTA.
-template <bool SPARSE, int EPI>
+template <bool SPARSE>
 static bool use_pair(const LinearArgs& a) {
     if (g_opt.no_pair) return false;
     const long long tiles = (long long)((a.W->out + 2 * kBM - 1) / (2 * kBM)) * ((a.tokens + 191) / 192);
@@ -1760,11 +1759,11 @@ static int one_cta_bn(const LinearArgs& a, std::initializer_list<int> widths, in
     return best;
 }
 
-// Clusters of `splits` one-CTA tiles that the current device runs at a time (asked once per device; 74, 33 and 14 for 2, 4 and 8 CTAs where
-// the query fails): one more goes into a second round, which costs what the split gains.
+// Clusters of `splits` one-CTA tiles that the current device runs at a time (74, 33 and 14 of 2, 4 and 8 CTAs): one more goes into a second
+// round, which costs what the split gains.  Asked once per device; 0, that is no split, also where the device does not say.
 static int resident_clusters(int splits) {
     static std::mutex mu;
-    static int known[64][3] = {};
+    static int known[64][3] = {};  // 1 + the answer
     const int at = splits == 2 ? 0 : splits == 4 ? 1 : 2;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
@@ -1781,13 +1780,14 @@ static int resident_clusters(int splits) {
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = (unsigned)splits; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
-        if (allow_dynamic_smem((const void*)fn, Cfg::SMEM) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&n, (const void*)fn, &cfg) != cudaSuccess || n < 1) {
+        int fit = 0;
+        if (allow_dynamic_smem((const void*)fn, Cfg::SMEM) != cudaSuccess || cudaOccupancyMaxActiveClusters(&fit, (const void*)fn, &cfg) != cudaSuccess) {
             (void)cudaGetLastError();
-            n = splits == 2 ? 74 : splits == 4 ? 33 : 14;
+            return 0;
         }
+        n = 1 + std::max(fit, 0);
     }
-    return n;
+    return n - 1;
 }
 
 // Where the reduction is split, and how: 1000 * CTAs + token-tile width, or 0.  A split costs its k-blocks, each the tile's width
@@ -1799,8 +1799,11 @@ static int resident_clusters(int splits) {
 // the unsplit kernel has an epilogue of its own to be compared with: 0.63 of the unsplit time over 141 shapes, formats and outputs, 1.017 at the
 // worst: 1 token 8192 -> 1536 1:4 / 8 bit 39.9 -> 9.6 us, 384 tokens 1024 -> 1024 1:4 / 8 bit 8.4 -> 7.0, 128 tokens 768 -> 768 2:4 / 4 bit 5.8 -> 4.7;
 // not taken: a reduction of three k-blocks (1 token 384 -> 1536, 4:4 / 4 bit 4.25 / 4.51), 200 tokens 1024 -> 4096, 2:4 / 4 bit 7.3 / 8.3.
-template <bool SPARSE>
-static int split_plan(const LinearArgs& a, int unsplit_bn, bool xf = false) {
+// `resident(splits)`: clusters of that size that run at a time.
+template <bool SPARSE, bool XF, typename Resident>
+static int split_plan(const LinearArgs& a, Resident resident) {
+    constexpr bool xf = XF;
+    const int unsplit_bn = XF ? one_cta_bn<SPARSE>(a, {192, 128, 64}, 160) : one_cta_bn<SPARSE>(a, {192, 128, 96, 64, 32}, 64);
     if (g_opt.split == 1 || g_opt.one_bn || (g_opt.skip_stage && !g_opt.split)) return 0;  // the test hook counts the stages of an unsplit tile
     const int kblocks = a.W->in / kKB, out_tiles = (a.W->out + kBM - 1) / kBM;
     const long long unsplit = xf ? (long long)kblocks * (unsplit_bn + 384) + 4 * unsplit_bn : (long long)kblocks * (unsplit_bn + 256);
@@ -1815,7 +1818,7 @@ static int split_plan(const LinearArgs& a, int unsplit_bn, bool xf = false) {
             if (clusters * splits > sm_count()) continue;
             const long long cost = xf ? (long long)per * (bn + 384) + 12 * bn + 12 * clusters * splits : (long long)per * (bn + 256) + 12 * bn;
             const bool gains = xf ? cost <= unsplit && kblocks > 3 : 10 * cost <= 9 * unsplit;
-            if (!g_opt.split && (!gains || clusters > resident_clusters(splits))) continue;
+            if (g_opt.split ? resident(splits) < 1 : !gains || clusters > resident(splits)) continue;
             if (!best || cost < best_cost) { best = plan; best_cost = cost; }
         }
     return best;
@@ -1834,11 +1837,11 @@ static int pick_split(const LinearArgs& a, int plan) {
 
 template <bool SPARSE, int EPI, bool XF>
 static int pick_bn(const LinearArgs& a) {
+    if (const int plan = split_plan<SPARSE, XF>(a, resident_clusters)) return pick_split<SPARSE, EPI, XF>(a, plan);
+    if (g_opt.split > 1) return NM_ERR_UNSUPPORTED;  // a split was asked for that this problem cannot have
     const int out_tiles = (a.W->out + kBM - 1) / kBM, sms = sm_count();
     if constexpr (!XF) {
-        const int best = one_cta_bn<SPARSE>(a, {192, 128, 96, 64, 32}, 64);
-        if (const int plan = split_plan<SPARSE>(a, best)) return pick_split<SPARSE, EPI, XF>(a, plan);
-        switch (best) {
+        switch (one_cta_bn<SPARSE>(a, {192, 128, 96, 64, 32}, 64)) {
             case 192: return launch_gemm<SPARSE, 192, EPI, W_TMA>(a);
             case 128: return launch_gemm<SPARSE, 128, EPI, W_TMA>(a);
             case 96: return launch_gemm<SPARSE, 96, EPI, W_TMA>(a);
@@ -1846,7 +1849,6 @@ static int pick_bn(const LinearArgs& a) {
             default: return launch_gemm<SPARSE, 32, EPI, W_TMA>(a);
         }
     } else {
-        if (const int plan = split_plan<SPARSE>(a, one_cta_bn<SPARSE>(a, {192, 128, 64}, 160), true)) return pick_split<SPARSE, EPI, XF>(a, plan);
         // Sparse-target formats with a short reduction and work for every SM pair: the CTA-pair kernel with the weights
         // rebuilt once per output tile into its resident region (32-bit outputs).
         if constexpr (SPARSE && (kF32<EPI> || EPI == EPI_ACC)) {
@@ -1876,16 +1878,20 @@ static int check_linear(int tokens, int out, int in, int n, int m, int bits) {
     return NM_OK;
 }
 
+// Token-tile width of the 512-channel kernel where it takes the problem (2:4 with 8-bit or packed 4-bit codes), or 0.
+static int takes_wide(const LinearArgs& a, bool xform, bool sparse) {
+    return sparse && (!xform || xf::pattern_of(a.W->n, a.W->m, a.W->bits) == xf::P24_4) ? wide_bn(a) : 0;
+}
+
 template <int EPI>
 static int run_linear_epi(const LinearArgs& a, bool xform, bool sparse) {
-    if (sparse && (!xform || xf::pattern_of(a.W->n, a.W->m, a.W->bits) == xf::P24_4)) {  // 2:4 with 8-bit or packed 4-bit codes
-        const int bn = wide_bn<EPI>(a);
+    if (const int bn = takes_wide(a, xform, sparse)) {
         if (bn == 224) return xform ? launch_gemm_wide<224, EPI, true>(a) : launch_gemm_wide<224, EPI>(a);
-        if (bn == 192) return xform ? launch_gemm_wide<192, EPI, true>(a) : launch_gemm_wide<192, EPI>(a);
+        return xform ? launch_gemm_wide<192, EPI, true>(a) : launch_gemm_wide<192, EPI>(a);
     }
     if (xform) return sparse ? pick_bn<true, EPI, true>(a) : pick_bn<false, EPI, true>(a);
-    if (sparse) return use_pair<true, EPI>(a) ? pick_pair<true, EPI>(a) : pick_bn<true, EPI, false>(a);
-    return use_pair<false, EPI>(a) ? pick_pair<false, EPI>(a) : pick_bn<false, EPI, false>(a);
+    if (sparse) return use_pair<true>(a) ? pick_pair<true, EPI>(a) : pick_bn<true, EPI, false>(a);
+    return use_pair<false>(a) ? pick_pair<false, EPI>(a) : pick_bn<false, EPI, false>(a);
 }
 
 static int run_linear(const LinearArgs& a, int epi) {
@@ -1931,6 +1937,22 @@ int nm_pair_tile_plan(int n_tok_tiles, int n_out_tiles, int pairs, int resident,
         if (tile_tok) tile_tok[t] = c.t;
     }
     return band;
+}
+
+int nm_split_plan(int tokens, int out, int in, int n, int m, int bits, const int* clusters) {
+    const int rc = nm::check_linear(tokens, out, in, n, m, bits);
+    if (rc != NM_OK) return rc;
+    if (tokens == 0 || out == 0) return 0;
+    const nm_packed_t W{out, in, n, m, bits, nullptr, nullptr};
+    nm::LinearArgs a{};
+    a.tokens = tokens; a.W = &W;
+    const int pat = nm::xf::pattern_of(n, m, bits);
+    const bool xform = pat != nm::xf::PNONE, sparse = xform ? nm::xf::sparse_target(pat) : n != m;
+    auto resident = [&](int splits) { return clusters ? clusters[splits == 2 ? 0 : splits == 4 ? 1 : 2] : nm::resident_clusters(splits); };
+    if (nm::takes_wide(a, xform, sparse)) return 0;
+    if (xform) return sparse ? nm::split_plan<true, true>(a, resident) : nm::split_plan<false, true>(a, resident);
+    if (sparse) return nm::use_pair<true>(a) ? 0 : nm::split_plan<true, false>(a, resident);
+    return nm::use_pair<false>(a) ? 0 : nm::split_plan<false, false>(a, resident);
 }
 
 int nm_debug_set_option(const char* name, int value) {

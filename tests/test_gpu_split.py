@@ -12,8 +12,12 @@ pytestmark = pytest.mark.gpu
 PLANS = [(2, 32), (4, 32), (2, 64), (4, 64), (8, 64), (2, 96), (4, 96), (2, 128), (4, 128), (8, 128)]
 
 
-def _run(T, K, out, n, m=4, bits=8):
+def _run(T, K, out, n, m=4, bits=8, plan=None):
+    """plan: the split that must be taken; None: the library's choice, which must be one."""
+    import paper_2206_15014_b200 as nm
     from gpu_util import PackedOnDevice, gpu_int_linear, gpu_int_linear_q8, gpu_int_linear_bf16
+    taken = nm.nm_split_plan(T, out, K, n, m, bits)
+    assert taken == plan if plan else taken > 1000
     oracle.set_threads(oracle.max_threads())
     rng = np.random.default_rng(T + K)
     W, b = wl.normal(rng, (out, K), 0.02), wl.normal(rng, (out,), 0.02)
@@ -35,9 +39,9 @@ def test_forms(splits, bn, n):
     import paper_2206_15014_b200 as nm
     nm.nm_debug_set_option("split", 1000 * splits + bn)
     try:
-        _run(bn + bn // splits + 3, 128 * (splits + 1), 250, n)  # one CTA has two k-blocks, the second token tile ends early
+        _run(bn + bn // splits + 3, 128 * (splits + 1), 250, n, plan=1000 * splits + bn)  # one CTA has two k-blocks, the second token tile ends early
         if 9 * splits <= 64:
-            _run(1, 128 * 9 * splits, 128, n)                    # nine k-blocks in a ring of at most eight, one token
+            _run(1, 128 * 9 * splits, 128, n, plan=1000 * splits + bn)                    # nine k-blocks in a ring of at most eight, one token
     finally:
         nm.nm_debug_set_option("split", 0)
 
@@ -48,9 +52,9 @@ def test_formats_rebuilt_on_the_way(n, m, bits):
     try:
         for splits, bn in ((2, 32), (4, 64), (8, 128)):
             nm.nm_debug_set_option("split", 1000 * splits + bn)
-            _run(bn + bn // splits + 3, 128 * (splits + 1), 250, n, m, bits)
+            _run(bn + bn // splits + 3, 128 * (splits + 1), 250, n, m, bits, 1000 * splits + bn)
             if splits < 8:
-                _run(1, 128 * 9 * splits, 128, n, m, bits)
+                _run(1, 128 * 9 * splits, 128, n, m, bits, 1000 * splits + bn)
         nm.nm_debug_set_option("split", 0)
         for T, K, out in ((5, 1024, 1024), (130, 768, 770), (64, 4096, 300)):  # the library's choice: split
             _run(T, K, out, n, m, bits)
@@ -73,8 +77,10 @@ def test_library_choice_matches_the_unsplit_kernel(T, K, out, n):
     desc = nm.make_packed(out, K, n, 4, 8, values, meta)
     X = torch.randint(-128, 128, (T, K), generator=g, device=DEV, dtype=torch.int8)
     got = []
-    for choice in (0, 1, 2064):
+    for choice in (0, 1, 2128):
         nm.nm_debug_set_option("split", choice)
+        taken = nm.nm_split_plan(T, out, K, n, 4, 8)
+        assert taken == (0 if choice == 1 else choice) if choice else taken > 1000
         amax, sx = torch.zeros(1, device=DEV), torch.full((1,), 0.01, device=DEV)
         Y, status = torch.zeros((T, out), device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
         try:
@@ -85,3 +91,18 @@ def test_library_choice_matches_the_unsplit_kernel(T, K, out, n):
         assert amax.item() == Y.abs().max().item()
         got.append(Y)
     assert torch.equal(got[0], got[1]) and torch.equal(got[0], got[2])
+
+
+def test_a_split_that_does_not_fit_is_refused():
+    import torch
+    import paper_2206_15014_b200 as nm
+    t = torch.zeros(1 << 22, dtype=torch.uint8, device="cuda")
+    desc = nm.make_packed(770, 3072, 2, 4, 8, t, t)
+    try:
+        for forced in (2064, 8192, 7):  # 154 CTAs; no such width; no such number of CTAs
+            nm.nm_debug_set_option("split", forced)
+            with pytest.raises(nm.NmError) as e:
+                nm.nm_int_linear(t, 700, desc, 1.0, t, None, t)
+            assert e.value.code == nm.NM_ERR_UNSUPPORTED
+    finally:
+        nm.nm_debug_set_option("split", 0)
