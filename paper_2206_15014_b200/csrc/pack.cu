@@ -225,7 +225,9 @@ __device__ __forceinline__ void kept_values(const float* v, float* sel) {
 
 // Distance of candidate j in double over the warp's part of the row (every lane returns the sum over the lanes), from the lane's `count` kept
 // values, value i at x[32 i].  A short loop over shared memory: few rows come here, and unrolled over registers its code kept the
-// rest of the kernel out of the instruction cache.  Codes from RN(1 / s_j) as in pack_row, the IEEE division only next to a tie.
+// rest of the kernel out of the instruction cache.  Codes from RN(1 / s_j) as in pack_row, the IEEE division only next to a tie.  Four values
+// at a time, their codes and distances independent of one another: a row with several candidates left is a small matrix's last one, and
+// value by value it took the latency of every step: 256 x 1024 dense 4 bit 13.8 -> 11.1 us, 1024 x 1024 14.9 -> 12.2, 4096 x 1024 2:4 17.7 -> 15.9.
 template <int BITS>
 __device__ __noinline__ double dist_exact(const float* x, int count, float smax, int j) {
     constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
@@ -235,18 +237,26 @@ __device__ __noinline__ double dist_exact(const float* x, int count, float smax,
     const bool fast_ok = sj >= 1.17549435e-38f && sj <= 4.25e37f;
     const double nsd = -(double)sj;
     double e[2] = {0.0, 0.0};
-    for (int i = 0; i < count; i += 2) {
+    for (int i = 0; i < count; i += 4) {  // values past `count` are zeros and add nothing
+        float xi[4], t[4], worst = 0.0f;
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const float xi = x[32 * (i + k)];
-            float t = __fmaf_rn(xi, rs, kMagic);
-            const float f = fabsf(__fmaf_rn(xi, rs, -__fsub_rn(t, kMagic)));
-            t = fminf(fmaxf(t, kMagic - qmax - 1.0f), kMagic + qmax);
-            if (!(f <= 0.49996948f) || !fast_ok) t = __fadd_rn(fminf(fmaxf(__fdiv_rn(xi, sj), kLo), kHi), kMagic);
+        for (int k = 0; k < 4; ++k) xi[k] = x[32 * (i + k)];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            t[k] = __fmaf_rn(xi[k], rs, kMagic);
+            worst = ptx::max_abs_nan(__fmaf_rn(xi[k], rs, -__fsub_rn(t[k], kMagic)), 0.0f, worst);
+            t[k] = fminf(fmaxf(t[k], kMagic - qmax - 1.0f), kMagic + qmax);
+        }
+        if (!(worst <= 0.49996948f) || !fast_ok) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) t[k] = __fadd_rn(fminf(fmaxf(__fdiv_rn(xi[k], sj), kLo), kHi), kMagic);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
             // the code as a double: 2^52 + 2^31 + code is whole
-            const double r = __dsub_rn(__hiloint2double(0x43300000, (__float_as_int(t) - 0x4B400000) ^ (int)0x80000000), 4503601774854144.0);
-            const double d = fma(nsd, r, (double)xi);
-            e[k] = fma(d, d, e[k]);
+            const double r = __dsub_rn(__hiloint2double(0x43300000, (__float_as_int(t[k]) - 0x4B400000) ^ (int)0x80000000), 4503601774854144.0);
+            const double d = fma(nsd, r, (double)xi[k]);
+            e[k & 1] = fma(d, d, e[k & 1]);
         }
     }
     double sum = e[0] + e[1];
