@@ -89,11 +89,6 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
         *abort_flag = 1;
         if (p.status) atomicOr(p.status, NM_STATUS_TIMEOUT);
     };
-    const int ew = warp - 2, q = warp & 3, half = ew >> 2, row = q * 32 + lane, n = n0 + row;
-    const uint32_t lane_taddr = tmem_base + ((uint32_t)(q * 32) << 16);
-    const int slice = BN / splits, chunks = slice >> 3;  // tokens that a CTA finishes, in chunks of eight
-    float c_n = 0.0f, b_n = 0.0f;
-    bool ok = true;
 
     if (warp == 0) {
         if (lane == 0) {
@@ -167,6 +162,10 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
             cur = nxt;
         }
     } else {
+        const int ew = warp - 2, q = warp & 3, half = ew >> 2, row = q * 32 + lane, n = n0 + row;
+        const uint32_t lane_taddr = tmem_base + ((uint32_t)(q * 32) << 16);
+        const int slice = BN / splits, chunks = slice >> 3;  // tokens that a CTA finishes, in chunks of eight
+        float c_n = 0.0f, b_n = 0.0f;
         if (SPARSE && half == 0) {
             // index metadata of this lane's weight row for the CTA's k-blocks, several pieces in flight together; rows past the end get a
             // valid "positions 0,1" pattern, their products are discarded
@@ -200,75 +199,80 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
             c_n = n < p.out ? __fmul_rn(sx, p.sw[n]) : 0.0f;
             b_n = n < p.out && p.bias ? p.bias[n] : 0.0f;
         }
-        ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(acc_full_bar, 0, abort_flag, kWaitLimit));
+        const bool ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(acc_full_bar, 0, abort_flag, kWaitLimit));
         if (!ok && lane == 0) raise_timeout();
         ptx::tc_fence_after();
-    }
-    __syncwarp();
-    ptx::cluster_wait();
-    if (warp >= 2 && warp < kSplitThreads / 32 && ok) {
-        // The other CTAs' tokens: [sender][chunk][two halves of four tokens][128 channels] of 16 bytes at the receiver.
-        const uint32_t base = ptx::smem_u32(recv) + (uint32_t)row * 16u;
-        for (int u = half; u < (splits - 1) * chunks; u += 2) {
-            const int d = u / chunks, ch = u - d * chunks;
-            const int to = rank + 1 + d < splits ? rank + 1 + d : rank + 1 + d - splits;
-            const int col = to * slice + ch * 8;
-            if (t0 + col >= p.tokens) continue;  // nobody will read them (the same for the whole warp)
-            uint32_t r[8];
-            ptx::tmem_ld_32x8(lane_taddr + col, r);
-            ptx::tmem_ld_wait();
-            // this CTA is the receiver's number splits - 2 - d
-            const uint32_t dst = ptx::map_to_cta(base + (uint32_t)(((splits - 2 - d) * chunks + ch) * 2) * (kBM * 16u), (uint32_t)to);
-            ptx::st_cluster_v4(dst, r[0], r[1], r[2], r[3]);
-            ptx::st_cluster_v4(dst + kBM * 16u, r[4], r[5], r[6], r[7]);
-        }
-    } else if (!ok && lane < splits) {
-        // no sums from here: everyone's flag, so that nobody finishes tokens from what was never sent
-        ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32((const void*)abort_flag), (uint32_t)lane), 1u);
-    }
-    __syncwarp();
-    ptx::cluster_arrive();
-    ptx::cluster_wait();
-    ok = ok && *abort_flag == 0u;
-    if (warp >= 2 && warp < kSplitThreads / 32 && ok) {
-        const float rsy = EPI == EPI_Q8 ? __frcp_rn(p.sy) : 0.0f;
-        float amax = 0.0f;
-        using OT = typename EpiOut<EPI>::type;
-        OT* const Y = reinterpret_cast<OT*>(kF32<EPI> ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW);
-        for (int ch = half; ch < chunks; ch += 2) {
-            const int col = rank * slice + ch * 8, t = t0 + col;
-            if (t >= p.tokens) break;
-            uint32_t r[8];
-            ptx::tmem_ld_32x8(lane_taddr + col, r);
-            ptx::tmem_ld_wait();
-            for (int d = 0; d < splits - 1; ++d) {
-                const uint4* part = reinterpret_cast<const uint4*>(recv) + (size_t)((d * chunks + ch) * 2) * kBM + row;
-                const uint4 a = part[0], b = part[kBM];
-                r[0] += a.x; r[1] += a.y; r[2] += a.z; r[3] += a.w;
-                r[4] += b.x; r[5] += b.y; r[6] += b.z; r[7] += b.w;
+        __syncwarp();
+        ptx::cluster_wait();
+        if (__builtin_expect(ok, 1)) {
+            // The other CTAs' tokens: [sender][chunk][two halves of four tokens][128 channels] of 16 bytes at the receiver.
+            const uint32_t base = ptx::smem_u32(recv) + (uint32_t)row * 16u;
+            for (int u = half; u < (splits - 1) * chunks; u += 2) {
+                const int d = u / chunks, ch = u - d * chunks;
+                const int to = rank + 1 + d < splits ? rank + 1 + d : rank + 1 + d - splits;
+                const int col = to * slice + ch * 8;
+                if (t0 + col >= p.tokens) continue;  // nobody will read them (the same for the whole warp)
+                uint32_t r[8];
+                ptx::tmem_ld_32x8(lane_taddr + col, r);
+                ptx::tmem_ld_wait();
+                // this CTA is the receiver's number splits - 2 - d
+                const uint32_t dst = ptx::map_to_cta(base + (uint32_t)(((splits - 2 - d) * chunks + ch) * 2) * (kBM * 16u), (uint32_t)to);
+                ptx::st_cluster_v4(dst, r[0], r[1], r[2], r[3]);
+                ptx::st_cluster_v4(dst + kBM * 16u, r[4], r[5], r[6], r[7]);
             }
-            const int jmax = n < p.out ? min(8, p.tokens - t) : 0;
-            OT* dst = Y + (size_t)t * p.out + n;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                OT o;
-                if constexpr (EPI == EPI_Q8) {
-                    float worst = 0.0f;
-                    o = epi_convert_q8_fast(r[j], c_n, b_n, rsy, worst);
-                    if (!(worst <= 0.49996948f)) o = (OT)(int8_t)quantise8_exact_call(__fmaf_rn((float)(int)r[j], c_n, b_n), p.sy);
-                } else {
-                    float y_abs;
-                    o = epi_convert<EPI>(r[j], c_n, b_n, p.sy, rsy, y_abs);
-                    if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
+        } else if (lane < splits) {
+            // no sums from here: everyone's flag, so that nobody finishes tokens from what was never sent
+            ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32((const void*)abort_flag), (uint32_t)lane), 1u);
+        }
+        __syncwarp();
+        ptx::cluster_arrive();
+        ptx::cluster_wait();
+        if (*abort_flag == 0u) {
+            const float rsy = EPI == EPI_Q8 ? __frcp_rn(p.sy) : 0.0f;
+            float amax = 0.0f;
+            using OT = typename EpiOut<EPI>::type;
+            OT* const Y = reinterpret_cast<OT*>(kF32<EPI> ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW);
+            for (int ch = half; ch < chunks; ch += 2) {
+                const int col = rank * slice + ch * 8, t = t0 + col;
+                if (t >= p.tokens) break;
+                uint32_t r[8];
+                ptx::tmem_ld_32x8(lane_taddr + col, r);
+                ptx::tmem_ld_wait();
+                for (int d = 0; d < splits - 1; ++d) {
+                    const uint4* part = reinterpret_cast<const uint4*>(recv) + (size_t)((d * chunks + ch) * 2) * kBM + row;
+                    const uint4 a = part[0], b = part[kBM];
+                    r[0] += a.x; r[1] += a.y; r[2] += a.z; r[3] += a.w;
+                    r[4] += b.x; r[5] += b.y; r[6] += b.z; r[7] += b.w;
                 }
-                if (j < jmax) dst[(size_t)j * p.out] = o;
+                const int jmax = n < p.out ? min(8, p.tokens - t) : 0;
+                OT* dst = Y + (size_t)t * p.out + n;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    OT o;
+                    if constexpr (EPI == EPI_Q8) {
+                        float worst = 0.0f;
+                        o = epi_convert_q8_fast(r[j], c_n, b_n, rsy, worst);
+                        if (!(worst <= 0.49996948f)) o = (OT)(int8_t)quantise8_exact_call(__fmaf_rn((float)(int)r[j], c_n, b_n), p.sy);
+                    } else {
+                        float y_abs;
+                        o = epi_convert<EPI>(r[j], c_n, b_n, p.sy, rsy, y_abs);
+                        if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
+                    }
+                    if (j < jmax) dst[(size_t)j * p.out] = o;
+                }
+            }
+            if (EPI == EPI_F32MAX) {
+#pragma unroll
+                for (int s = 16; s > 0; s >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, s));
+                if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(p.absmax), __float_as_uint(amax));
             }
         }
-        if (EPI == EPI_F32MAX) {
-#pragma unroll
-            for (int s = 16; s > 0; s >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, s));
-            if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(p.absmax), __float_as_uint(amax));
-        }
+    }
+    if (warp < 2 || warp >= kSplitThreads / 32) {  // the cluster's barriers of the others; apart, so that the builders hold nothing of the epilogue's
+        __syncwarp();
+        ptx::cluster_wait();
+        ptx::cluster_arrive();
+        ptx::cluster_wait();
     }
     // after an expired wait copies may still be on their way into this CTA's shared memory
     if (threadIdx.x == 0 && *abort_flag) ptx::wait_clocks(kAbortDrain);

@@ -203,8 +203,9 @@ def _run_split(seed, kblocks=9, stages=4, skipped=1, ctas=3, builders=4, tells=T
 
 def test_split_kernel_writes_nothing_once_a_cta_has_given_up():
     src = open(os.path.join(CSRC, "gemm_split.cuh")).read()
-    tells = re.search(r"else if \(!ok[^{]*\{[^}]*st_cluster_u32\(ptx::map_to_cta\([^;]*abort_flag[^;]*;\s*\}\s*__syncwarp\(\);\s*ptx::cluster_arrive\(\);"
-                      r"\s*ptx::cluster_wait\(\);\s*ok = ok && \*abort_flag == 0u;", src) is not None
+    exchange = src[src.index("ptx::cluster_wait();"):src.index("const float rsy")]  # from the first cluster barrier to the outputs
+    send, finish = exchange.split("ptx::cluster_arrive();")
+    tells = "st_cluster_u32(ptx::map_to_cta(ptx::smem_u32((const void*)abort_flag)" in send and "*abort_flag == 0u) {" in finish
     for seed in range(30):
         wrote, sums = _run_split(seed, tells=tells)
         assert not any(w and len(s) < len(sums) for w, s in zip(wrote, sums)), "outputs from sums that were never sent"
