@@ -119,7 +119,7 @@ __device__ __noinline__ uint32_t quantise8_exact4(float y0, float y1, float y2, 
 
 // 16 tokens of a warp's 32 channels, as the two loads of the stmatrix layout left them in r, converted: two bfloat16 or four codes a word.
 template <int EPI>
-__device__ __forceinline__ void narrow_convert(const uint32_t* r, uint32_t* pk, const float (&c)[4], const float (&b)[4], float sy, float rsy) {
+__device__ __forceinline__ void narrow_convert(const uint32_t* r, uint32_t* pk, const float (&c)[4], const float (&b)[4], float sy, float rsy, float far) {
     constexpr float kMagic = 12582912.0f;
     const uint64_t c01[2] = {ptx::pack_f32x2(c[0], c[0]), ptx::pack_f32x2(c[2], c[2])}, c23[2] = {ptx::pack_f32x2(c[1], c[1]), ptx::pack_f32x2(c[3], c[3])};
     const uint64_t b01[2] = {ptx::pack_f32x2(b[0], b[0]), ptx::pack_f32x2(b[2], b[2])}, b23[2] = {ptx::pack_f32x2(b[1], b[1]), ptx::pack_f32x2(b[3], b[3])};
@@ -144,7 +144,7 @@ __device__ __forceinline__ void narrow_convert(const uint32_t* r, uint32_t* pk, 
             ptx::unpack_f32x2(t23, t[2], t[3]);
             auto code = [&](int i) { return __float_as_int(t[i]) - 0x4B400000; };
             pk[k] = ptx::pack_sat_s8(code(0), code(1), ptx::pack_sat_s8(code(2), code(3), 0u));
-            if (!(ptx::max_abs_nan(d2, d3, ptx::max_abs_nan(d0, d1, 0.0f)) <= 0.49996948f)) pk[k] = quantise8_exact4(y0, y1, y2, y3, sy);
+            if (!(ptx::max_abs_nan(d2, d3, ptx::max_abs_nan(d0, d1, far)) <= 0.49996948f)) pk[k] = quantise8_exact4(y0, y1, y2, y3, sy);
         }
     }
 }
@@ -163,6 +163,17 @@ __device__ __forceinline__ void narrow_fill(uint32_t tile, const uint32_t* pk, i
     }
 }
 
+// 1 where a product of a thread's four channels in narrow_tile could leave the range in which int8 codes are taken from bits (then every
+// code comes from the exact division), 0 otherwise: an accumulator is at most in * 2^14, a product then below 2^23.  A bound per tile, which
+// nothing waits for before the first check, instead of a clamp per value: a scale that small (200 times under one that spreads the
+// outputs over the codes) saturates nearly every output.
+template <int EPI>
+__device__ __forceinline__ float narrow_far(float rsy, const float (&c)[4], const float (&b)[4], int in) {
+    if (EPI != EPI_Q8) return 0.0f;
+    const float c_max = ptx::max_abs_nan(c[0], c[1], ptx::max_abs_nan(c[2], c[3], 0.0f)), b_max = ptx::max_abs_nan(b[0], b[1], ptx::max_abs_nan(b[2], b[3], 0.0f));
+    return (c_max * ((float)in * 16384.0f) + b_max) * rsy < 8388608.0f ? 0.0f : 1.0f;
+}
+
 // Tiles of 16 tokens that BYTES of staging memory hold, of the SUBS that a warp has to do at most.
 template <int EPI, int BYTES, int SUBS> constexpr int kNarrowStage = BYTES / (EPI == EPI_BF16 ? 1024 : 512) < SUBS ? BYTES / (EPI == EPI_BF16 ? 1024 : 512) : SUBS;
 
@@ -176,15 +187,16 @@ template <int EPI, int BYTES, int SUBS> constexpr int kNarrowStage = BYTES / (EP
 // tokens 768 -> 3072 bfloat16 31.7 -> 28.9 us (35.0 with a lane per channel), int8 outputs over 263 shapes and formats 0.96 of the time.
 // int8: t = fma(y, rsy, 1.5 * 2^23) rounds the product to the nearest-even integer, which saturates to the code; `d` is the product's
 // distance from it, and within 2^-15 of a tie (or NaN) the IEEE division decides.  Below -1.5 * 2^23 t turns negative and the integer
-// that its bits give, less those of 1.5 * 2^23, wraps round to the other end: rsy comes from narrow_rsy.
+// that its bits give, less those of 1.5 * 2^23, wraps round to the other end: narrow_far.
 //
 // acc: TMEM address of the tile's first column in this warp's lane quarter.  c, b: scale and bias of channels lane / 4 + 8 i of the quarter.
 // valid: tokens of the tile that exist.  n: the warp's first channel.  LD: pieces of 16 tokens that it has in registers together.
 // release(): it has read its accumulator.
 template <int EPI, int SUBS, int STAGE, int BUFS, int LD, bool HINT, typename Release>
 __device__ __forceinline__ void narrow_tile(uint32_t acc, int valid, int group, int groups, uint32_t stage, int lane, const float (&c)[4], const float (&b)[4],
-                                            float sy, float rsy, const CUtensorMap* tmap_y, int n, int t0, int out, uint64_t policy, Release release) {
+                                            float sy, float rsy, int in, const CUtensorMap* tmap_y, int n, int t0, int out, uint64_t policy, Release release) {
     constexpr uint32_t TILE = EPI == EPI_BF16 ? 1024 : 512;
+    const float far = narrow_far<EPI>(rsy, c, b, in);
     const int all = min((valid + 15) >> 4, SUBS * groups), share = (all + groups - 1) / groups;
     const int first = group * share, last = min(first + share, all);
     if (first >= last) { release(); return; }
@@ -205,7 +217,7 @@ __device__ __forceinline__ void narrow_tile(uint32_t acc, int valid, int group, 
             if (u + h + LD >= last) release();
             uint32_t pk[LD][EPI == EPI_Q8 ? 4 : 8];
 #pragma unroll
-            for (int k = 0; k < LD; ++k) narrow_convert<EPI>(r[k], pk[k], c, b, sy, rsy);
+            for (int k = 0; k < LD; ++k) narrow_convert<EPI>(r[k], pk[k], c, b, sy, rsy, far);
             if (h == 0) {  // the stores that last used the staging tiles have read them
                 if (lane == 0) {
                     if (BUFS == 1 || u == first) ptx::bulk_wait_group_read<0>();
@@ -255,7 +267,7 @@ __device__ __forceinline__ void narrow_group_tile(uint32_t acc, int columns, int
             ptx::tmem_ld_16x256x2(acc + (16u << 16) + u * UNIT + 16 * h, r + 8);
             ptx::tmem_ld_wait();
             if (h == UNIT / 16 - 1 && u + groups >= units) release();
-            narrow_convert<EPI_BF16>(r, pk, c, b, 0.0f, 0.0f);
+            narrow_convert<EPI_BF16>(r, pk, c, b, 0.0f, 0.0f, 0.0f);
             if (h == 0) {
                 if (q == 0 && lane == 0) ptx::bulk_wait_group_read<1>();  // the store before the last has read this tile
                 ptx::named_bar_sync(bar, 128);
@@ -339,17 +351,6 @@ __device__ __forceinline__ void narrow_constants(const float* sw, const float* b
 #pragma unroll
     for (int i = 0; i < 4; ++i) c[i] = __fmul_rn(sx, c[i]);
 }
-// The reciprocal of an int8 output scale for a thread's four channels in narrow_tile, or NaN (every code from the exact division) where a
-// product could leave the range in which the codes are taken from bits: an accumulator is at most in * 2^14, a product then below 2^23.
-// A bound per tile instead of a clamp per value: a scale that small (200 times under one that spreads the outputs over the codes)
-// saturates nearly every output.
-template <int EPI>
-__device__ __forceinline__ float narrow_rsy(float rsy, const float (&c)[4], const float (&b)[4], int in) {
-    if (EPI != EPI_Q8) return 0.0f;
-    const float c_max = ptx::max_abs_nan(c[0], c[1], ptx::max_abs_nan(c[2], c[3], 0.0f)), b_max = ptx::max_abs_nan(b[0], b[1], ptx::max_abs_nan(b[2], b[3], 0.0f));
-    return (c_max * ((float)in * 16384.0f) + b_max) * rsy < 8388608.0f ? rsy : __int_as_float(0x7fffffff);
-}
-
 // Pieces of metadata (16 bytes: one row, one 128-wide k-block) that a metadata warp of the one-CTA kernel has in flight (four
 // in the forms with weight-building warps, which are short of registers).  One at a time, each load waited for before its
 // store to TMEM, they held up the first MMA: 384 tokens 1024 -> 3072 7.6 -> 6.6 us, 4096 -> 1024 16.8 -> 14.7, 64 tokens
@@ -708,7 +709,7 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         int scaled_out_tile = -1;
         uint32_t n_stores = 0;
         int narrow_out_tile = -1;  // whose constants nc, nb are (narrow outputs)
-        float nc[4], nb[4], nrs = 0.0f;
+        float nc[4], nb[4];
         bool ok = true;
 
         // Index metadata of this lane's weight row for the whole reduction; rows past the end get a valid "positions 0,1" pattern,
@@ -773,7 +774,6 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
             if (kNarrow<EPI> && p.tma_store && out_tile != narrow_out_tile) {
                 narrow_out_tile = out_tile;
                 narrow_constants(p.sw, p.bias, sx, n0 + q * 32, lane, p.out, nc, nb);
-                nrs = narrow_rsy<EPI>(rsy, nc, nb, p.in);
             }
             bool got = ptx::mbar_wait_bounded(acc_full_bar(buf), (i >> 1) & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
@@ -799,7 +799,7 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
             if constexpr (kNarrow<EPI>) {
                 constexpr int SUBS = (BN / 16 + EWH - 1) / EWH;
                 narrow_tile<EPI, SUBS, kNarrowStage<EPI, kStoreStage / kEpiWarps, SUBS>, 1, 1, false>(lane_taddr + buf * BN, p.tokens - t0, half, EWH,
-                    ptx::smem_u32(store_stage) + ew * (kStoreStage / kEpiWarps), lane, nc, nb, p.sy, nrs, &tmap_y, n0 + q * 32, t0, p.out, 0, [&] { release_acc(buf); });
+                    ptx::smem_u32(store_stage) + ew * (kStoreStage / kEpiWarps), lane, nc, nb, p.sy, rsy, p.in, &tmap_y, n0 + q * 32, t0, p.out, 0, [&] { release_acc(buf); });
                 continue;
             }
             if constexpr (!kNarrow<EPI>) {
@@ -1185,7 +1185,7 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
         int scaled_out_tile = -1;
         uint32_t n_stores = 0;
         int narrow_out_tile = -1;  // whose constants nc, nb are (narrow outputs)
-        float nc[4], nb[4], nrs = 0.0f;
+        float nc[4], nb[4];
         bool ok = true;
 
         auto load_meta = [&](int out_tile) {
@@ -1224,7 +1224,6 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
             if (kNarrow<EPI> && p.tma_store && out_tile != narrow_out_tile) {
                 narrow_out_tile = out_tile;
                 narrow_constants(p.sw, p.bias, sx, n0 + q * 32, lane, p.out, nc, nb);
-                nrs = narrow_rsy<EPI>(rsy, nc, nb, p.in);
             }
             bool got = ptx::mbar_wait_bounded(acc_full_bar(buf), (i >> 1) & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
@@ -1258,7 +1257,7 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                                           q, lane, nc, nb, &tmap_y, n0, t0, p.out, stream_out, [&] { release_acc(buf); });
                 else
                 narrow_tile<EPI, SUBS, kNarrowStage<EPI, PER, SUBS>, 1, 1, true>(lane_taddr + buf * BN, p.tokens - t0, half, EWH, ptx::smem_u32(store_stage) + ew * PER,
-                    lane, nc, nb, p.sy, nrs, &tmap_y, n0 + q * 32, t0, p.out, stream_out, [&] { release_acc(buf); });
+                    lane, nc, nb, p.sy, rsy, p.in, &tmap_y, n0 + q * 32, t0, p.out, stream_out, [&] { release_acc(buf); });
                 if (ew == 0 && lane == 0) { NM_TRACE_TILE(i, 1); NM_TRACE_EPI_FLUSH(i); }
                 continue;
             }

@@ -377,7 +377,7 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
         const float rsy = EPI == EPI_Q8 ? __frcp_rn(p.sy) : 0.0f;
         uint32_t n_stores = 0;
         int narrow_out_tile = -1;  // whose constants nc, nb are (narrow outputs)
-        float nc[4], nb[4], nrs = 0.0f;
+        float nc[4], nb[4];
         int scaled_out_tile = -1;
         bool ok = true;
         auto release_acc = [&]() {  // this warp has read all it needs from the accumulator
@@ -392,7 +392,6 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
             if (kNarrow<EPI> && p.tma_store && tc.o != narrow_out_tile) {
                 narrow_out_tile = tc.o;
                 narrow_constants(p.sw, p.bias, sx, nw, lane, p.out, nc, nb);
-                nrs = narrow_rsy<EPI>(rsy, nc, nb, p.in);
             }
             bool got = ptx::mbar_wait_bounded(acc_full_bar(blk), (uint32_t)i & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
@@ -421,7 +420,7 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                 } else {
                     constexpr int SUBS = BN / 16, PER = Cfg::STORE_STAGE / kWideEpiWarps;
                     narrow_tile<EPI, SUBS, kNarrowStage<EPI, PER / 2, SUBS>, 2, W4 ? 1 : 2, true>(acc_taddr, p.tokens - t0, 0, 1, ptx::smem_u32(store_stage) + ew * PER,
-                        lane, nc, nb, p.sy, nrs, &tmap_y, nw, t0, p.out, stream_out, release_acc);
+                        lane, nc, nb, p.sy, rsy, p.in, &tmap_y, nw, t0, p.out, stream_out, release_acc);
                 }
                 if (ew == 0 && lane == 0) NM_TRACE_TILE(i, 1);
                 if (ew == 4 && lane == 0) NM_TRACE_TILE(i, 3);

@@ -314,7 +314,7 @@ nm_gemm_xres_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                                           q, lane, nc, nb, &tmap_y, n0, t0, p.out, stream_out, [&] { release_acc(buf); });
                 else
                 narrow_tile<EPI, SUBS, kNarrowStage<EPI, PER, SUBS>, 1, 1, true>(lane_taddr + buf * BN, p.tokens - t0, half, EWH, ptx::smem_u32(store_stage) + ew * PER,
-                    lane, nc, nb, p.sy, narrow_rsy<EPI>(rsy, nc, nb, p.in), &tmap_y, n0 + q * 32, t0, p.out, stream_out, [&] { release_acc(buf); });
+                    lane, nc, nb, p.sy, rsy, p.in, &tmap_y, n0 + q * 32, t0, p.out, stream_out, [&] { release_acc(buf); });
                 if (ew == 0 && lane == 0) { NM_TRACE_TILE(i, 1); NM_TRACE_EPI_FLUSH(i); }
                 continue;
             }
