@@ -295,8 +295,10 @@ __device__ __forceinline__ void narrow_group_tile(uint32_t acc, int columns, int
 // One output tile where TMA cannot store the rows of Y (not whole units of 16 bytes): a lane per channel, 32 tokens of an accumulator at a
 // time, stored straight from the registers.  Staged in shared memory and written by rows of 128 channels, with a quarter of the partial
 // sectors, it was slower: bfloat16 1024 -> 1002, 8192 tokens, packed 4-bit codes 28 us against 18, fp32 23 against 17.  Out of the kernels' main
-// loops, so that those stay short.
-template <int EPI, typename Release>
+// loops, so that those stay short.  EIGHTS: of the last tokens no more than there are, to eight, in the one-CTA kernel without builder warps: 18
+// tokens 128 -> 2687 bfloat16, dense weights 2.63 -> 2.39 us, 2:4 2.78 -> 2.55.  The kernels with builder warps pay for more code with fetching it
+// (1 % of every other call), int8 codes gain nothing, being a branch each.
+template <int EPI, bool EIGHTS = false, typename Release>
 __device__ __forceinline__ void direct_tile(uint32_t acc, int columns, int valid, int group, int groups, float c_n, float b_n, float sy, float rsy,
                                             typename EpiOut<EPI>::type* Y, int t0, int n, int out, float& amax, Release release) {
     using OT = typename EpiOut<EPI>::type;
@@ -329,8 +331,12 @@ __device__ __forceinline__ void direct_tile(uint32_t acc, int columns, int valid
                 for (int j = 0; j < 32; ++j) dst[(size_t)j * out] = conv(j);
             } else {
 #pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (j < count) dst[(size_t)j * out] = conv(j);
+                for (int g = 0; g < 32; g += 8) {
+                    if (EIGHTS && g >= count) break;
+#pragma unroll
+                    for (int j = g; j < g + 8; ++j)
+                        if (j < count) dst[(size_t)j * out] = conv(j);
+                }
             }
         }
         __syncwarp();
@@ -791,7 +797,7 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                 b_n = n_ok && p.bias ? p.bias[n] : 0.0f;
             }
             if (!p.tma_store) {
-                direct_tile<EPI>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, c_n, b_n, p.sy, rsy,
+                direct_tile<EPI, !XF && EPI != EPI_Q8>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, c_n, b_n, p.sy, rsy,
                                  reinterpret_cast<typename EpiOut<EPI>::type*>(kF32<EPI> ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW), t0, n, p.out, amax,
                                  [&] { release_acc(buf); });
                 continue;
