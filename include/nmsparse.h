@@ -357,6 +357,7 @@ int nm_probe_tma_stream(const void *W, int w_rows, int w_row_bytes, const void *
  * "split" (one-CTA tiles with the reduction split over a cluster: 1000 * CTAs + token-tile width, for instance 4096,
  * 1 = never; a call that would run on one-CTA tiles and cannot have that split returns NM_ERR_UNSUPPORTED), "one_bn" (token-tile width of the one-CTA kernel: 192, 128, 96, 64 or 32 where it exists), "xres" (the pair kernel with resident
  * activations: 1 = wherever a pair kernel with a reduction of at most 1024 runs, 2 = never),
+ * "grouped" (bfloat16 output tiles shared by four warps, where the kernel has that form: 1 = always, 2 = never),
  * "pack_form" (form of the projection kernel in blocks of four warps: 2 = persistent with the next rows staged in shared
  * memory by bulk copies, where that form exists: 1:4, 2:4, 1:8 and 2:8 without dense outputs; 1 or 3 = one unit per block).
  * Results never depend on them.  Returns NM_ERR_UNSUPPORTED for an unknown name.  A library built with

@@ -448,11 +448,13 @@ struct GemmCfg {
     static_assert(BN % 32 == 0 && BN >= 32 && BN <= 256, "token tile");
 };
 
-template <bool SPARSE, int BN, int EPI, int WSRC>
+// GROUPED: bfloat16 tiles through narrow_group_tile; a kernel of its own, since its code beside the other's cost every call 1 %.
+template <bool SPARSE, int BN, int EPI, int WSRC, bool GROUPED = false>
 __global__ void __launch_bounds__(WSRC != W_TMA ? kXformThreads : kGemmThreads, 1)
 nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                const __grid_constant__ CUtensorMap tmap_y, const GemmParams p) {
     constexpr bool XF = WSRC != W_TMA, RES = WSRC == W_RESIDENT;
+    static_assert(!GROUPED || (EPI == EPI_BF16 && RES), "see store_grouped");
     using Cfg = GemmCfg<SPARSE, BN, RES>;
     constexpr int S = Cfg::STAGES;
     extern __shared__ uint8_t smem_raw[];
@@ -784,6 +786,7 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
             bool got = ptx::mbar_wait_bounded(acc_full_bar(buf), (i >> 1) & 1u, abort_flag, kWaitLimit);
             ok = __all_sync(0xffffffffu, got);
             if (!ok && lane == 0) raise_timeout();
+            if constexpr (GROUPED) ok = ptx::named_bar_and(kNarrowAgree + half, 128, ok);  // the group stops together
             if (!ok) break;
             ptx::tc_fence_after();
             if (SPARSE && half == 0 && i + 1 < tile_count) {
@@ -802,7 +805,11 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                                  [&] { release_acc(buf); });
                 continue;
             }
-            if constexpr (kNarrow<EPI>) {
+            if constexpr (GROUPED) {
+                narrow_group_tile<16>(lane_taddr + buf * BN, BN, p.tokens - t0, half, EWH, kNarrowGroup + half, ptx::smem_u32(store_stage) + half * 8192, n_stores,
+                                      q, lane, nc, nb, &tmap_y, n0, t0, p.out, ptx::policy_evict_first(), [&] { release_acc(buf); });
+                continue;
+            } else if constexpr (kNarrow<EPI>) {
                 constexpr int SUBS = (BN / 16 + EWH - 1) / EWH;
                 narrow_tile<EPI, SUBS, kNarrowStage<EPI, kStoreStage / kEpiWarps, SUBS>, 1, 1, false>(lane_taddr + buf * BN, p.tokens - t0, half, EWH,
                     ptx::smem_u32(store_stage) + ew * (kStoreStage / kEpiWarps), lane, nc, nb, p.sy, rsy, p.in, &tmap_y, n0 + q * 32, t0, p.out, 0, [&] { release_acc(buf); });
@@ -1356,6 +1363,7 @@ struct DebugOptions {
     int wide_bn;      // token-tile width of that kernel: 224 or 192 (0 = automatic)
     int xres;         // the pair kernel with resident activations: 1 = whenever the shape allows it, 2 = never
     int split;        // reduction split over a cluster: 1000 * CTAs + token-tile width, 1 = never (0 = automatic)
+    int grouped;      // bfloat16 tiles shared by four warps: 1 = always, 2 = never
     int one_bn;       // token-tile width of the one-CTA kernel (0 = automatic)
     int band;         // band size of the streamed pair kernel's tile order (0 = automatic)
     int skip_stage;   // NM_TEST_HOOKS builds: 1 + the pipeline stage CTA 0's producer leaves out (0 = none)
@@ -1408,6 +1416,20 @@ static int make_store_map(CUtensorMap* ty, const LinearArgs& a, bool* tma_store,
                     grouped ? CU_TENSOR_MAP_SWIZZLE_128B : EPI == EPI_BF16 ? CU_TENSOR_MAP_SWIZZLE_64B : EPI == EPI_Q8 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE, dt, es);
 }
 
+// Whether bfloat16 outputs leave through narrow_group_tile.  The one-CTA kernel with resident weights: from 80 MB of Y at eight k-blocks
+// (weights for the sparse form), or 24 MB at six and more (for the dense one); below, and with shorter reductions, whose tiles follow one another
+// faster, the warps' own tiles are the better ones.  Over 800 shapes, shared / own in us: 16384 tokens 1024 -> 3072 2:4 / 4 bit 41.4 / 43.8, 32768
+// tokens 1024 -> 4096 109 / 118, 24000 tokens 896 -> 4096 4:8 / 4 bit 94 / 115, 16384 tokens 768 -> 2304 4:4 / 4 bit 33.6 / 38.7; not taken:
+// 16384 tokens 896 -> 3072 2:4 / 4 bit 42.3 / 39.8, 8192 tokens 640 -> 3072 4:4 / 4 bit 24.9 / 23.7, 16384 tokens 256 -> 4096 2:4 / 4 bit 45.6 / 33.7.
+template <int EPI, bool RES = false, bool SPARSE = false>
+static bool store_grouped(const LinearArgs& a) {
+    if (EPI != EPI_BF16 || g_opt.grouped == 2) return false;
+    if (g_opt.grouped == 1) return true;
+    const size_t bytes = (size_t)a.tokens * a.W->out * 2;
+    if (!RES) return bytes >= kNarrowGroupBytes;
+    return SPARSE ? a.W->in >= 1024 && bytes >= (size_t)80 << 20 : a.W->in >= 768 && bytes >= (size_t)24 << 20;
+}
+
 template <bool SPARSE, int BN, int EPI, int WSRC>
 static int launch_gemm(const LinearArgs& a) {
     constexpr bool XF = WSRC != W_TMA;
@@ -1422,7 +1444,9 @@ static int launch_gemm(const LinearArgs& a) {
     rc = make_map(&tx, a.X, (uint64_t)a.tokens, (uint64_t)W.in, BN, 128, CU_TENSOR_MAP_SWIZZLE_128B);
     if (rc != NM_OK) return rc;
     bool tma_store = false;
-    rc = make_store_map<EPI>(&ty, a, &tma_store);
+    constexpr bool kBothForms = WSRC == W_RESIDENT && EPI == EPI_BF16;
+    const bool grouped = kBothForms && store_grouped<EPI, true, SPARSE>(a);
+    rc = make_store_map<EPI>(&ty, a, &tma_store, 16, grouped);
     if (rc != NM_OK) return rc;
     GemmParams p{};
     p.tma_store = tma_store ? 1 : 0;
@@ -1438,6 +1462,9 @@ static int launch_gemm(const LinearArgs& a) {
     p.sw = a.sw; p.bias = a.bias; p.sx_dev = a.sx_dev; p.sx_host = a.sx;
     p.Y = a.Y; p.ACC = a.ACC; p.NARROW = a.NARROW; p.sy = a.sy; p.absmax = a.absmax; p.status = a.status; p.trace = g_trace_buffer; p.skip_stage = g_opt.skip_stage - 1;
     auto fn = nm_gemm_kernel<SPARSE, BN, EPI, WSRC>;
+    if constexpr (kBothForms) {
+        if (grouped && tma_store) fn = nm_gemm_kernel<SPARSE, BN, EPI, WSRC, true>;
+    }
     NM_CUDA_TRY(allow_dynamic_smem((const void*)fn, Cfg::SMEM));
     const int grid = p.n_tiles < sm_count() ? p.n_tiles : sm_count();
     cudaLaunchConfig_t cfg = {};
@@ -1486,7 +1513,7 @@ static int launch_gemm_pair(const LinearArgs& a) {
     rc = make_map_x3(&tx, a.X, (uint64_t)a.tokens, (uint64_t)W.in, Cfg::B_ROWS, Cfg::KB / 128);
     if (rc != NM_OK) return rc;
     bool tma_store = false;
-    const bool grouped = EPI == EPI_BF16 && (size_t)a.tokens * W.out * 2 >= kNarrowGroupBytes;
+    const bool grouped = store_grouped<EPI>(a);
     rc = make_store_map<EPI>(&ty, a, &tma_store, 16, grouped);
     if (rc != NM_OK) return rc;
     GemmParams p{};
@@ -1590,7 +1617,7 @@ static int launch_gemm_xres(const LinearArgs& a) {
     rc = make_map_x3(&tx, a.X, (uint64_t)a.tokens, (uint64_t)W.in, Cfg::B_ROWS, Cfg::SLICES);
     if (rc != NM_OK) return rc;
     bool tma_store = false;
-    const bool grouped = EPI == EPI_BF16 && (size_t)a.tokens * W.out * 2 >= kNarrowGroupBytes;
+    const bool grouped = store_grouped<EPI>(a);
     rc = make_store_map<EPI>(&ty, a, &tma_store, 16, grouped);
     if (rc != NM_OK) return rc;
     GemmParams p{};
@@ -1965,7 +1992,7 @@ int nm_debug_set_option(const char* name, int value) {
     struct { const char* name; int* slot; } table[] = {
         {"no_pdl", &nm::g_no_pdl}, {"no_pair", &nm::g_opt.no_pair}, {"no_resident", &nm::g_opt.no_resident},
         {"no_wide", &nm::g_opt.no_wide}, {"wide_any", &nm::g_opt.wide_any}, {"wide_bn", &nm::g_opt.wide_bn},
-        {"one_bn", &nm::g_opt.one_bn}, {"split", &nm::g_opt.split}, {"xres", &nm::g_opt.xres}, {"band", &nm::g_opt.band}, {"pack_form", &nm::g_pack_form}};
+        {"one_bn", &nm::g_opt.one_bn}, {"split", &nm::g_opt.split}, {"xres", &nm::g_opt.xres}, {"grouped", &nm::g_opt.grouped}, {"band", &nm::g_opt.band}, {"pack_form", &nm::g_pack_form}};
     for (auto& e : table)
         if (!strcmp(name, e.name)) { *e.slot = value; return NM_OK; }
 #ifdef NM_TEST_HOOKS

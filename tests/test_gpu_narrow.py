@@ -163,9 +163,36 @@ def test_int8_output_at_any_scale(T, K, out, n, m, bits, options):
             nm.nm_debug_set_option(k, 0)
 
 
+# every kernel that has both forms of bfloat16 tiles: the last token unit is cut short, the last 128 channels too
+@pytest.mark.parametrize("K,n,m,bits,options", [
+    (1152, 4, 4, 8, {}),            # pair kernel with eight epilogue warps, weights streamed
+    (1024, 2, 4, 8, {"xres": 2}),   # ... with sixteen, weights resident
+    (768, 2, 4, 8, {"xres": 1}),    # resident activations
+    (896, 4, 4, 8, {"xres": 1}),
+    (1024, 2, 4, 4, {}),            # one-CTA kernel, weights rebuilt and resident, sparse and dense form
+    (768, 4, 8, 4, {}),
+])
+@pytest.mark.parametrize("grouped", [1, 2])
+def test_bfloat16_tiles_shared_or_own(K, n, m, bits, options, grouped):
+    import paper_2206_15014_b200 as nm
+    from gpu_util import PackedOnDevice, gpu_int_linear_bf16
+    T, out = 2900, 1288
+    Xq, sx, v, meta, s, b, Y = _setup(K, T, K, out, n, m, bits)
+    packed = PackedOnDevice(v, meta, s, out, K, n, m, bits)
+    options = dict(options, grouped=grouped)
+    try:
+        for k, x in options.items():
+            nm.nm_debug_set_option(k, x)
+        assert np.array_equal(gpu_int_linear_bf16(Xq, packed, sx, b), oracle.to_bf16(Y))
+    finally:
+        for k in options:
+            nm.nm_debug_set_option(k, 0)
+
+
 @pytest.mark.parametrize("n,m,bits,out", [(2, 4, 8, 3072), (2, 4, 4, 3080), (4, 4, 8, 3080), (2, 8, 4, 3072)])
 def test_bfloat16_too_large_for_the_cache(n, m, bits, out):
-    """At 192 MB of Y the pair kernels store whole lines, shared by four warps: the same bits as pieces of the same tokens."""
+    """At 192 MB of Y the pair kernels, and the one-CTA kernel with resident weights, store whole lines, shared by four warps: the same
+    bits as pieces of the same tokens, which do not."""
     import torch
     import paper_2206_15014_b200 as nm
     from gpu_util import DEV
