@@ -1,5 +1,6 @@
 // Host-only entry points of the nmsparse C ABI: sizes, validation, status polling, error text.
 #include "common.cuh"
+#include "once.cuh"
 #include <stdio.h>
 #include <string.h>
 
@@ -16,6 +17,14 @@ int record_cuda_error(cudaError_t e, const char* where) {
 int record_text_error(const char* text) {
     snprintf(g_last_error, sizeof(g_last_error), "%s", text);
     return NM_ERR_CUDA;
+}
+
+cudaError_t allow_dynamic_smem(const void* fn, int bytes) {
+    static OncePerDevice once;
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return (cudaError_t)once.run(fn, dev, [&] { return (int)cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
 }
 
 int sm_count() {

@@ -40,6 +40,9 @@ extern int g_no_pdl;
 int pack_set_skip_unit(int unit);
 #endif
 
+// cudaFuncSetAttribute(max dynamic shared memory) once per kernel and device instead of on every launch; `bytes`: the most that a launch of `fn` takes.
+cudaError_t allow_dynamic_smem(const void* fn, int bytes);
+
 // Multiprocessors of the current device (cached per device; 148 when the query fails).
 int sm_count();
 

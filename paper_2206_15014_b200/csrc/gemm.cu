@@ -1374,23 +1374,6 @@ int g_no_pdl = 0;
 // Trace buffer of NM_TRACE builds (device, kTraceStages + kTraceTiles rows of 8 u64), handed to every GEMM launch.
 static unsigned long long* g_trace_buffer = nullptr;
 
-// cudaFuncSetAttribute(max dynamic shared memory) once per kernel and device instead of on every launch.
-static cudaError_t allow_dynamic_smem(const void* fn, int bytes) {
-    struct Done { const void* fn; int dev; };
-    static Done done[256];
-    static int n_done = 0;
-    static std::mutex mu;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lock(mu);
-    for (int i = 0; i < n_done; ++i)
-        if (done[i].fn == fn && done[i].dev == dev) return cudaSuccess;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess && n_done < 256) done[n_done++] = Done{fn, dev};
-    return e;
-}
-
 struct LinearArgs {
     const int8_t* X; int tokens; const nm_packed_t* W;
     float sx; const float* sx_dev; const float* sw; const float* bias;

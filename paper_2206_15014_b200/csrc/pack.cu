@@ -1335,20 +1335,7 @@ static int launch_table(PackFn k, const PackJobDev* jobs_dev, int njobs, const P
     const bool staged = k.form == kStaged2;
     const size_t smem = (size_t)warps * ((staged ? 16384 + 16 : 0) + k.search + 2 * sizeof(float) + 1024) + 512 + 16;
     const PackFnPtr fn = k.fn;
-    if (smem > 48 * 1024) {  // the attribute is set once per kernel and device
-        struct Done { const void* fn; int dev; };
-        static std::mutex mu;
-        static std::vector<Done> done;
-        int dev = 0;
-        NM_CUDA_TRY(cudaGetDevice(&dev));
-        std::lock_guard<std::mutex> lock(mu);
-        bool found = false;
-        for (const Done& d : done) found = found || (d.fn == (const void*)fn && d.dev == dev);
-        if (!found) {
-            NM_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-            done.push_back(Done{(const void*)fn, dev});
-        }
-    }
+    if (smem > 48 * 1024) NM_CUDA_TRY(allow_dynamic_smem((const void*)fn, 227 * 1024));
     const unsigned grid = staged ? std::min(blocks, (unsigned)(sm_count() * kStagedBlocksPerSm)) : blocks;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, 1, 1);
@@ -1471,7 +1458,8 @@ static DistFn pick_dist(int n, int m, int bits, int warps) {
 static int launch_dist(DistFn fn, size_t search, const PackJobDev* jobs_dev, int njobs, const PackJobDev& single, unsigned blocks,
                        int warps, uint32_t* status, cudaStream_t stream, int ncand, int32_t* cand) {
     const size_t smem = (size_t)warps * (search + sizeof(float));
-    if (smem > 48 * 1024) NM_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int most = warps <= kPackMinWarps ? kPackMinWarps : warps <= 16 ? 16 : 32;  // warps that share this kernel (pick_dist_bits)
+    if (smem > 48 * 1024) NM_CUDA_TRY(allow_dynamic_smem((const void*)fn, most * (int)(search + sizeof(float))));
     PackJobInline inl{};
     inl.j[0] = single;
     fn<<<blocks, warps * 32, smem, stream>>>(jobs_dev, njobs, inl, status, ncand, cand);
