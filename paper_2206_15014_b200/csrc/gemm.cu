@@ -90,7 +90,8 @@ constexpr uint32_t kNarrowGroup = 9, kNarrowAgree = 13;  // named barriers: one 
 
 // One output element from an accumulator: fp32 value y, then the narrowing the epilogue kind asks for.
 template <int EPI>
-__device__ __forceinline__ typename EpiOut<EPI>::type epi_convert(uint32_t acc, float c_n, float b_n, float sy, float rsy, float& y_abs) {
+__device__ __forceinline__ typename EpiOut<EPI>::type epi_convert(uint32_t acc, float c_n, float b_n, float& y_abs) {
+    static_assert(EPI != EPI_Q8, "epi_convert_q8_fast or narrow_convert");
     if constexpr (EPI == EPI_ACC) {
         y_abs = 0.0f;
         return acc;
@@ -99,10 +100,6 @@ __device__ __forceinline__ typename EpiOut<EPI>::type epi_convert(uint32_t acc, 
         y_abs = fabsf(y);
         if constexpr (kF32<EPI>) {
             return __float_as_uint(y);
-        } else if constexpr (EPI == EPI_Q8) {
-            // the IEEE quotient y / sy rounded half to even and clamped to [-128, 127]
-            (void)rsy;
-            return (uint8_t)(int8_t)quantise8_exact(y, sy);
         } else {
             uint16_t h;
             asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(h) : "f"(y));
@@ -320,7 +317,7 @@ __device__ __forceinline__ void direct_tile(uint32_t acc, int columns, int valid
                 o = epi_convert_q8_fast(r[j], c_n, b_n, rsy, worst);
                 if (!(worst <= 0.49996948f)) o = (OT)(int8_t)quantise8_exact_call(__fmaf_rn((float)(int)r[j], c_n, b_n), sy);
             } else {
-                o = epi_convert<EPI>(r[j], c_n, b_n, sy, rsy, y_abs);
+                o = epi_convert<EPI>(r[j], c_n, b_n, y_abs);
             }
             if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, y_abs);
             return o;
@@ -836,7 +833,7 @@ nm_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
                         using OT = typename EpiOut<EPI>::type;
                         auto conv = [&](int j) -> OT {
                             float y_abs;
-                            const OT o = epi_convert<EPI>(r[ci & (RB - 1)][j], c_n, b_n, p.sy, 0.0f, y_abs);
+                            const OT o = epi_convert<EPI>(r[ci & (RB - 1)][j], c_n, b_n, y_abs);
                             if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
                             return o;
                         };
@@ -1295,7 +1292,7 @@ nm_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                         using OT = typename EpiOut<EPI>::type;
                         auto conv = [&](int j) -> OT {
                             float y_abs;
-                            const OT o = epi_convert<EPI>(r[ci & (RB - 1)][j], c_n, b_n, p.sy, 0.0f, y_abs);
+                            const OT o = epi_convert<EPI>(r[ci & (RB - 1)][j], c_n, b_n, y_abs);
                             if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
                             return o;
                         };
@@ -1541,11 +1538,10 @@ static int launch_gemm_pair(const LinearArgs& a) {
     return NM_OK;
 }
 
-// Wide pair kernel (512 channels x BN tokens per pair): 2:4 int8 weights streamed, fp32 / int32 outputs.
+// Wide pair kernel (512 channels x BN tokens per pair): 2:4 weights streamed, 8-bit codes or (W4) packed 4-bit ones.
 template <int BN, int EPI, bool W4 = false>
 static int launch_gemm_wide(const LinearArgs& a) {
     using Cfg = WideCfg<BN, W4>;
-    constexpr int SKEW = 0;
     const nm_packed_t& W = *a.W;
     CUtensorMap tw, tx, ty;
     // packed 4-bit codes: two stages of a row at a time
@@ -1568,7 +1564,7 @@ static int launch_gemm_wide(const LinearArgs& a) {
     p.values = (const uint8_t*)W.values; p.vrow_bytes = (int)values_row_bytes(W.in, W.n, W.m, W.bits);
     p.sw = a.sw; p.bias = a.bias; p.sx_dev = a.sx_dev; p.sx_host = a.sx;
     p.Y = a.Y; p.ACC = a.ACC; p.NARROW = a.NARROW; p.sy = a.sy; p.absmax = a.absmax; p.status = a.status; p.trace = g_trace_buffer; p.skip_stage = g_opt.skip_stage - 1;
-    auto fn = nm_gemm_wide_kernel<BN, EPI, SKEW, W4>;
+    auto fn = nm_gemm_wide_kernel<BN, EPI, W4>;
     NM_CUDA_TRY(allow_dynamic_smem((const void*)fn, Cfg::SMEM));
     int pairs = p.n_tiles < sm_count() / 2 ? p.n_tiles : sm_count() / 2;
     if (pairs > kMaxPairs) pairs = kMaxPairs;

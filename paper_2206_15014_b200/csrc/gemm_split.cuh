@@ -255,7 +255,7 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
                         if (!(worst <= 0.49996948f)) o = (OT)(int8_t)quantise8_exact_call(__fmaf_rn((float)(int)r[j], c_n, b_n), p.sy);
                     } else {
                         float y_abs;
-                        o = epi_convert<EPI>(r[j], c_n, b_n, p.sy, rsy, y_abs);
+                        o = epi_convert<EPI>(r[j], c_n, b_n, y_abs);
                         if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
                     }
                     if (j < jmax) dst[(size_t)j * p.out] = o;

@@ -12,9 +12,8 @@
 //     per TMEM lane quarter, both CTAs) copy the 16 bytes per weight row and block that a stage needs from
 //     the canonical metadata in global memory into a ring of TMEM slots (8 columns per stage, same slot
 //     index as the shared-memory stage) with tcgen05.st; the stage's "full" barrier also counts them.
-//   * The accumulators are single-buffered.  The MMA thread runs block 1 SKEW stages behind block 0, so that
-//     block 0's accumulator is handed to its four epilogue warps SKEW stages before block 1's and the next
-//     tile's block-0 MMAs can start while block 1's accumulator is still being read.
+//   * The accumulators are single-buffered: the next tile's MMAs start once both have been read.  (Block 1 a stage or more behind
+//     block 0, whose accumulator would be free that much earlier, was slower.)
 //   * The MMAs are issued from one elected lane of a warp-uniform path: descriptors are advanced with one add from values formed once, ring
 //     positions are carried instead of divided out.  What bounds it: the epilogue, exposed between two tiles, and the loads' latency.
 #pragma once
@@ -37,7 +36,7 @@ constexpr int kWideBuildWarps = 8;
 template <bool W4> constexpr int kWideThreadsOf = kWideThreads + (W4 ? 32 * kWideBuildWarps : 0);
 constexpr uint32_t kWideNarrowBar = 13;  // named barriers 13 and 14: the four epilogue warps of block 0 / block 1 (narrow outputs)
 constexpr uint32_t kWideRelayIds = 12;  // named barriers 1..12 carry the gate's relays in turn; the gate is never more
-                                        // than STAGES + SKEW steps ahead of the MMA thread
+                                        // than STAGES steps ahead of the MMA thread
 
 template <int BN, bool W4 = false>
 struct WideCfg {
@@ -67,15 +66,14 @@ struct WideCfg {
     static_assert(BN % 32 == 0 && BN <= 256, "token tile");
 };
 
-template <int BN, int EPI, int SKEW, bool W4>
+template <int BN, int EPI, bool W4>
 __global__ void __launch_bounds__(kWideThreadsOf<W4>, 1)
 nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                     const __grid_constant__ CUtensorMap tmap_y, const GemmParams p,
                     const __grid_constant__ PairSchedule sched) {
     using Cfg = WideCfg<BN, W4>;
     constexpr int S = Cfg::STAGES;
-    static_assert(SKEW >= 0 && SKEW < S - 2, "the ring must hold the stages block 1 lags behind plus loads in flight");
-    static_assert(S + SKEW < (int)kWideRelayIds, "relay barriers would be reused before the MMA thread has passed them");
+    static_assert(S < (int)kWideRelayIds, "relay barriers would be reused before the MMA thread has passed them");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* codes = smem + S * Cfg::STAGE;  // W4: two buffers [256 rows][64 bytes]
@@ -276,8 +274,7 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
         }
     } else if (warp == kWideGateWarp) {
         // ------------------------------ gate (leader): mbarrier waits relayed to the MMA warp ------
-        // One relay per step g of the MMA thread: step g issues block 0 on stage g and block 1 on stage
-        // g - SKEW.  Runs its full trip count even after a timeout (then without waiting).
+        // One relay per stage.  Runs its full trip count even after a timeout (then without waiting).
         if (leader) {
             bool ok = true;
             auto wait = [&](uint32_t bar, uint32_t parity) {
@@ -287,20 +284,15 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                     ok = false;
                 }
             };
-            int s = 0, kb_l = 0, kb_t = 0;
-            uint32_t parity = 0u, tile_l = 0, tile_t = 0, relay = 1;
-            for (uint32_t g = 0; g < total + SKEW; ++g) {
-                if (g < total) {
-                    if (kb_l == 0) wait(acc_empty_bar(0), (tile_l & 1u) ^ 1u);  // block 0's accumulator read out
-                    wait(full_bar(s), parity);
-                    if (lane == 0) NM_TRACE_STAGE(g, 2);
-                    if (++s == S) { s = 0; parity ^= 1u; }
-                    if (++kb_l == p.kblocks) { kb_l = 0; ++tile_l; }
-                }
-                if (g >= (uint32_t)SKEW) {
-                    if (kb_t == 0) wait(acc_empty_bar(1), (tile_t & 1u) ^ 1u);
-                    if (++kb_t == p.kblocks) { kb_t = 0; ++tile_t; }
-                }
+            int s = 0, kb = 0;
+            uint32_t parity = 0u, tile = 0, relay = 1;
+            for (uint32_t g = 0; g < total; ++g) {
+                if (kb == 0) wait(acc_empty_bar(0), (tile & 1u) ^ 1u);  // block 0's accumulator read out
+                wait(full_bar(s), parity);
+                if (lane == 0) NM_TRACE_STAGE(g, 2);
+                if (++s == S) { s = 0; parity ^= 1u; }
+                if (kb == 0) wait(acc_empty_bar(1), (tile & 1u) ^ 1u);
+                if (++kb == p.kblocks) { kb = 0; ++tile; }
                 __syncwarp();
                 ptx::relay_step(relay, abort_flag);
                 relay = relay == kWideRelayIds ? 1 : relay + 1;
@@ -315,44 +307,29 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
             const uint64_t b_desc0 = ptx::smem_desc_kmajor(smem0 + Cfg::A_BYTES, 128, ptx::kSwizzle128);
             const uint32_t meta0 = tmem_base + Cfg::META_COL;
             const uint32_t last_kb = (uint32_t)p.kblocks - 1;
-            // ring position of block 0 (lead) and block 1 (trail): byte offset of the stage and metadata slot
-            uint32_t off_l = 0, off_t = 0, slot_l = 0, slot_t = 0, kb_l = 0, kb_t = 0, relay = 1;
-            for (uint32_t g = 0; g < total + SKEW; ++g) {
+            uint32_t off = 0, slot = 0, kb = 0, relay = 1;  // byte offset of the stage, metadata slot
+            for (uint32_t g = 0; g < total; ++g) {
                 ptx::named_bar_sync(relay, 64);
                 relay = relay == kWideRelayIds ? 1 : relay + 1;
                 ptx::tc_fence_after();  // orders the MMAs after the metadata stores and accumulator reads of other threads
                 if (ptx::elect_one()) {
                     NM_TRACE_STAGE(g, 3);
-                    if (g < total) {
-                        const uint64_t a = ptx::desc_advance(a_desc0, off_l), b = ptx::desc_advance(b_desc0, off_l);
-                        const uint32_t e = meta0 + slot_l;
-                        ptx::mma_sp_i8_pair(tmem_base, a, b, e, idesc, kb_l != 0);
-                        ptx::mma_sp_i8_pair(tmem_base, ptx::desc_advance(a, 32), ptx::desc_advance(b, 64), e + 2, idesc, 1u);
-                        if (SKEW != 0 && kb_l == last_kb) ptx::tc_commit_pair(acc_full_bar(0), 3);
-                    }
-                    if (g >= (uint32_t)SKEW) {
-                        const uint64_t a = ptx::desc_advance(a_desc0, off_t + Cfg::A_BLOCK), b = ptx::desc_advance(b_desc0, off_t);
-                        const uint32_t e = meta0 + slot_t + 4;
-                        ptx::mma_sp_i8_pair(tmem_base + BN, a, b, e, idesc, kb_t != 0);
-                        ptx::mma_sp_i8_pair(tmem_base + BN, ptx::desc_advance(a, 32), ptx::desc_advance(b, 64), e + 2, idesc, 1u);
-                        ptx::tc_commit_pair(empty_bar(slot_t >> 3), 3);  // both producers and the metadata warps may refill the stage
-                        if (kb_t == last_kb) {
-                            if (SKEW == 0) ptx::tc_commit_pair(acc_full_bar(0), 3);
-                            ptx::tc_commit_pair(acc_full_bar(1), 3);
-                        }
+                    const uint64_t a0 = ptx::desc_advance(a_desc0, off), a1 = ptx::desc_advance(a_desc0, off + Cfg::A_BLOCK), b = ptx::desc_advance(b_desc0, off);
+                    const uint32_t e = meta0 + slot;
+                    ptx::mma_sp_i8_pair(tmem_base, a0, b, e, idesc, kb != 0);
+                    ptx::mma_sp_i8_pair(tmem_base, ptx::desc_advance(a0, 32), ptx::desc_advance(b, 64), e + 2, idesc, 1u);
+                    ptx::mma_sp_i8_pair(tmem_base + BN, a1, b, e + 4, idesc, kb != 0);
+                    ptx::mma_sp_i8_pair(tmem_base + BN, ptx::desc_advance(a1, 32), ptx::desc_advance(b, 64), e + 6, idesc, 1u);
+                    ptx::tc_commit_pair(empty_bar(slot >> 3), 3);  // both producers and the metadata warps may refill the stage
+                    if (kb == last_kb) {
+                        ptx::tc_commit_pair(acc_full_bar(0), 3);
+                        ptx::tc_commit_pair(acc_full_bar(1), 3);
                     }
                     NM_TRACE_STAGE(g, 4);
                 }
-                if (g < total) {
-                    off_l += Cfg::STAGE; slot_l += Cfg::META_SLOT;
-                    if (slot_l == S * Cfg::META_SLOT) { off_l = 0; slot_l = 0; }
-                    kb_l = kb_l == last_kb ? 0 : kb_l + 1;
-                }
-                if (g >= (uint32_t)SKEW) {
-                    off_t += Cfg::STAGE; slot_t += Cfg::META_SLOT;
-                    if (slot_t == S * Cfg::META_SLOT) { off_t = 0; slot_t = 0; }
-                    kb_t = kb_t == last_kb ? 0 : kb_t + 1;
-                }
+                off += Cfg::STAGE; slot += Cfg::META_SLOT;
+                if (slot == S * Cfg::META_SLOT) { off = 0; slot = 0; }
+                kb = kb == last_kb ? 0 : kb + 1;
                 __syncwarp();
             }
             if (ptx::elect_one()) {  // everything issued has retired before TMEM is released
@@ -365,8 +342,8 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
         // ------------------------------ epilogue warps (both CTAs) --------------------------------
         // Warps 2-5 read block 0's accumulator, warps 6-9 block 1's; each its TMEM lane quarter, all BN columns.
         constexpr int CH = BN / 32;
-        // narrow outputs leave through staging tiles that a block's four warps share (narrow_tile); for 32-bit outputs that form (one
-        // 16 KB tile per block) was measured slower than a tile per warp (FFN2 alone 44.6 against 42.5 us)
+        // int8 outputs leave through staging tiles of each warp's own (narrow_tile), bfloat16 through tiles that a block's four warps share
+        // (narrow_group_tile); for 32-bit outputs a shared tile of 16 KB per block was measured slower than a tile per warp
         const int ew = warp - 2, q = warp & 3, blk = ew >> 2;
         const uint32_t acc_taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)blk * BN;
         uint32_t* my_stage = reinterpret_cast<uint32_t*>(store_stage + ew * 4096);
@@ -443,7 +420,7 @@ nm_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                         using OT = typename EpiOut<EPI>::type;
                         auto conv = [&](int j) -> OT {
                             float y_abs;
-                            const OT o = epi_convert<EPI>(r[c & (RB - 1)][j], c_n, b_n, p.sy, 0.0f, y_abs);
+                            const OT o = epi_convert<EPI>(r[c & (RB - 1)][j], c_n, b_n, y_abs);
                             if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
                             return o;
                         };

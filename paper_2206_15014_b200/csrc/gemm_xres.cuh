@@ -338,7 +338,7 @@ nm_gemm_xres_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
                         using OT = typename EpiOut<EPI>::type;
                         auto conv = [&](int j) -> OT {
                             float y_abs;
-                            const OT o = epi_convert<EPI>(r[ci & 1][j], c_n, b_n, p.sy, 0.0f, y_abs);
+                            const OT o = epi_convert<EPI>(r[ci & 1][j], c_n, b_n, y_abs);
                             if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
                             return o;
                         };
