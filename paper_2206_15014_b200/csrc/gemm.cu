@@ -64,13 +64,9 @@ template <int EPI> constexpr bool kF32 = EPI == EPI_F32 || EPI == EPI_F32MAX;
 template <int EPI> struct EpiOut { using type = uint32_t; };          // fp32 / int32 move as 32-bit patterns
 template <> struct EpiOut<EPI_Q8> { using type = uint8_t; };
 template <> struct EpiOut<EPI_BF16> { using type = uint16_t; };
-// Narrow outputs leave through [tokens][32 channels] tiles of the warp's own (narrow_tile), or [tokens][128 channels] tiles that the four warps of a
-// TMEM-lane-quarter group fill together (narrow_group_tile): there a named barrier per group orders the fills against the one warp
-// that issues the TMA store, kNarrowAgree + half makes the group take a timed-out wait together so that nobody is left alone on it.
-// EPI_Q8 without a branch per value: the code from the reciprocal rsy = RN(1 / sy), exact unless the product sits
+// EPI_Q8 a value at a time (split kernel, direct stores), without a branch: the code from the reciprocal rsy = RN(1 / sy), exact unless the product sits
 // within 2^-15 of a rounding tie (6 values in 100000), where only the IEEE division decides.  `worst` keeps the largest
-// distance of a product from its rounded integer over a run of values; beyond 0.49996948 the caller fills the run again
-// with the exact quantiser.  The clamp to [-128.49, 127.49] before the add of 1.5 * 2^23 (whose own rounding rounds to
+// distance of a product from its rounded integer; beyond 0.49996948 the caller takes the code from the exact quantiser.  The clamp to [-128.49, 127.49] before the add of 1.5 * 2^23 (whose own rounding rounds to
 // the nearest-even integer) leaves nothing to clamp afterwards, and the low byte of the sum's bit pattern
 // 0x4B400000 + code is the code.
 __device__ __forceinline__ uint8_t epi_convert_q8_fast(uint32_t acc, float c_n, float b_n, float rsy, float& worst) {
@@ -85,6 +81,9 @@ __device__ __forceinline__ uint8_t epi_convert_q8_fast(uint32_t acc, float c_n, 
 // The exact quantiser as a call: the repair of near-ties runs for a few values in 10^5, its code stays out of the loops.
 __device__ __noinline__ int quantise8_exact_call(float y, float sy) { return quantise8_exact(y, sy); }
 
+// Narrow outputs leave through [tokens][32 channels] tiles of the warp's own (narrow_tile), or [tokens][128 channels] tiles that the four warps of a
+// TMEM-lane-quarter group fill together (narrow_group_tile): there a named barrier per group orders the fills against the one warp
+// that issues the TMA store, kNarrowAgree + half makes the group take a timed-out wait together so that nobody is left alone on it.
 template <int EPI> constexpr bool kNarrow = EPI == EPI_Q8 || EPI == EPI_BF16;
 constexpr uint32_t kNarrowGroup = 9, kNarrowAgree = 13;  // named barriers: one per group from kNarrowGroup on
 
@@ -1672,16 +1671,18 @@ static int launch_gemm_split(const LinearArgs& a, int splits) {
 
 // Where the kernel with resident activations is the faster pair kernel.  At least two output tiles (with one the activations
 // are not read twice), and then by measurement, this kernel / the other one in us:
-//  - dense weights, which the other kernel streams besides the activations: always (6144 tokens 768 -> 768 10.6 / 12.8, 768 -> 3072
-//    21.0 / 23.7, 12288 tokens 1024 -> 4096 bfloat16 47.7 / 51.4), except for narrow outputs whose rows are not 16-byte
-//    aligned (20000 tokens 1024 -> 1500 bfloat16 37.9 / 37.2);
-//  - 2:4 weights: up to 896 reduction elements (6144 tokens 768 -> 768 9.9 / 11.3, 768 -> 2304 15.4 / 16.8, 9000 tokens 512 -> 2048
-//    18.0 / 20.6, 40000 tokens 768 -> 3072 bfloat16 82.9 / 83.9); at 1024 only while a pair has few tiles, then the fill of the
-//    resident weights of the other kernel is what counts (5000 tokens 1024 -> 1024 10.4 / 12.1, 16384 tokens 1024 -> 3072, 14
-//    tiles, 47.2 / 48.7; 1024 -> 4096, 19 tiles, 62.0 / 60.2; bfloat16: 5000 tokens 1024 -> 4096, 6 tiles, 21.2 / 22.5; 49152
-//    tokens 1024 -> 1024, 14 tiles, 44.2 / 40.9);
-//  - int8 outputs of 2:4 weights, whose conversion sets the pace: a few tiles (3977 tokens 768 -> 3072, 3 tiles, 18.6 / 18.9; 12288
-//    tokens 768 -> 3072, 10 tiles, 43.5 / 42.5).
+//  - dense weights, which the other kernel streams besides the activations: always (6144 tokens 768 -> 768 9.3 / 9.9, 768 -> 3072
+//    19.2 / 21.7, 12288 tokens 1024 -> 4096 bfloat16 44.2 / 45.3), except for narrow outputs whose rows are not 16-byte
+//    aligned (20000 tokens 1024 -> 1500 bfloat16 30.5 / 30.2);
+//  - 2:4 weights: up to 896 reduction elements (6144 tokens 768 -> 768 7.7 / 8.6, 768 -> 2304 13.0 / 13.4, 9000 tokens 512 -> 2048
+//    14.8 / 16.0); at 1024 only while a pair has few tiles, then the fill of the resident weights of the other kernel is what counts
+//    (5000 tokens 1024 -> 1024 8.2 / 9.4; 16384 tokens 1024 -> 4096, 19 tiles, 64.0 / 56.8; 49152 tokens 1024 -> 1024 bfloat16, 14
+//    tiles, 43.6 / 40.0);
+//  - int8 outputs of 2:4 weights: a few tiles (3977 tokens 768 -> 3072, 3 tiles, 12.0 / 13.1).
+// The lines were drawn when a stage's MMAs took 430-550 clocks to issue (now 70-150, see elect_one); measured since over 432 shapes, either
+// kernel forced is no better than the rule in the mean (this one 1.002, the other 1.07), but it loses at 16384 tokens 1024 -> 3072
+// (45.8 / 43.2), 40000 tokens 768 -> 3072 bfloat16 (82.0 / 79.5), 49152 tokens 768 -> 1024 bfloat16 (37.3 / 33.8), and with int8 outputs of more
+// tiles (16384 tokens 768 -> 3072 34.7 / 36.1, 4096 tokens 1024 -> 4096 15.4 / 16.7).
 template <bool SPARSE, int EPI>
 static bool use_xres(const LinearArgs& a) {
     const nm_packed_t& W = *a.W;
@@ -1696,11 +1697,10 @@ static bool use_xres(const LinearArgs& a) {
 }
 
 // Whether the one-CTA kernel has at most one 192-token tile for every SM.  It then beats the pair kernels where their larger
-// tiles leave SMs idle or need a second round: 3977 tokens 3072 -> 768 (126 tiles of 128 x 192; 42 of 512 x 192) 14.9 against 17.9 us, packed 4-bit codes 20.2
-// against 27.6; 4500 tokens (144 tiles) 15.2 / 17.8; 5000 tokens 2560 -> 640 13.8 / 16.2.  With a second wave it loses: 5500 tokens 3072 ->
-// 768 (174 tiles) 22.5 / 18.3.  Against the 256-channel kernels: 5000 tokens 640 -> 640 (135 tiles; 81 of 256 x 192 on 74 pairs) 7.3 / 9.5,
-// dense 2560 -> 640 14.0 / 19.1, 9000 tokens 896 -> 384 8.6 / 10.6,
-// packed 4-bit codes 5000 tokens 640 -> 640 9.3 / 12.3.
+// tiles leave SMs idle or need a second round: 3977 tokens 3072 -> 768 (126 tiles of 128 x 192; 42 of 512 x 192) 11.6 against 14.6 us, packed 4-bit codes
+// 15.9 against 20.8; 4500 tokens (144 tiles) 11.4 / 14.6; 5000 tokens 2560 -> 640 10.1 / 13.1.  With a second wave it loses: 5500 tokens 3072 ->
+// 768 (174 tiles) 17.8 / 14.5.  Against the 256-channel kernels, before their MMAs were issued by an elected lane: 5000 tokens 640 -> 640 (135 tiles; 81
+// of 256 x 192 on 74 pairs) 7.3 / 9.5, dense 2560 -> 640 14.0 / 19.1, 9000 tokens 896 -> 384 8.6 / 10.6, packed 4-bit codes 5000 tokens 640 -> 640 9.3 / 12.3.
 static bool one_wave(const LinearArgs& a) {
     const long long tiles = (long long)((a.W->out + kBM - 1) / kBM) * ((a.tokens + 191) / 192);
     return tiles <= sm_count() && a.W->in / 32 <= kTmemCols - 2 * 192;
@@ -1708,8 +1708,11 @@ static bool one_wave(const LinearArgs& a) {
 
 // Token-tile width of the wide kernel: the one whose slowest pair has the least to do (tiles per pair, rounded
 // up, times the tile width); 0 = the wide kernel does not apply (short reductions keep their weights resident in
-// the 256-channel kernel; a matrix of at most 256 channels would leave one of the two blocks idle; narrow outputs
-// and small problems stay on the other kernels).
+// the 256-channel kernel; a matrix of at most 256 channels would leave one of the two blocks idle; small problems stay on the other
+// kernels).  It / the 256-channel kernel in us: 16384 tokens 4096 -> 1024 fp32 40.8 / 49.2, bfloat16 35.8 / 44.6, int8 36.7 / 52.1, packed 4-bit codes
+// 51.9 / 78.5; over 165 shapes the other takes 1.12 of its time.  The line of half the pairs is older than the present issue of the MMAs and
+// loses where the last round of its large tiles is nearly empty or few pairs have one: 9000 tokens 3072 -> 768 24.6 / 17.2, 16384 tokens 2048 -> 4096
+// int8 94.6 / 76.9, 4096 tokens 4096 -> 4096 64 / 55.
 static int wide_bn(const LinearArgs& a) {
     if (g_opt.no_wide || g_opt.no_pair) return 0;
     const nm_packed_t& W = *a.W;

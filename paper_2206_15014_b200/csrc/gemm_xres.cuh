@@ -9,8 +9,10 @@
 // The index metadata changes with every tile: four metadata warps (one per TMEM lane quarter, both CTAs) keep a ring of
 // four buffers of 32 TMEM columns filled, one tile's reduction each.  A token tile's slices are replaced one by one as the
 // last output tile's MMAs are done with them.
-// What bounds it: the epilogue.  A stage takes 370-480 clocks for 384 of MMAs (800-1100 while the MMAs' operands were built per thread, see
-// elect_one), a tile 3.4-5 k: fp32 by its stores, int8 by its conversion.  16384 tokens 768 -> 3072: bfloat16 31.7 -> 28.9 us
+// What bounds it: the epilogue, and with it the loads, which wait behind its stores.  1024 -> 4096, 16384 tokens, time stamps: a stage's MMAs
+// take 100-140 clocks to issue (640-830 while their operands were built per thread, see elect_one) and are handed over every 525-566, a tile of four
+// stages follows the other after 5.3 k clocks with fp32 outputs, 3.7 k with bfloat16, 4.4 k with int8, of which its epilogue takes 4.7, 3.0 and
+// 3.8 k; a load takes 3.7-5.3 k from issue to arrival.  16384 tokens 768 -> 3072: bfloat16 31.7 -> 28.9 us
 // with staging tiles of each warp's own (narrow_tile).  Measured without gain: two MMAs of half the
 // width, alternating accumulators, weights in 64-byte rows (16384 tokens 1024 -> 4096 64.6 / 62.0 us).
 #pragma once

@@ -189,8 +189,8 @@ __device__ __forceinline__ unsigned keep_mask(const float* a) {
 //
 // A row spans `wpr` warps; the partial sums of its warps are added in a fixed order, so the result is
 // deterministic.  85 M weights at 2:4 / 4 bit and 32 candidates, search and projection: 461 us with all candidates in single precision,
-// 297 so (398 shapes and formats 0.71 in the geometric mean, 1.05 at the worst, a
-// matrix of 1 M weights of dense 4 bit).  What bounds it now: instructions (61 % of the issue slots), their fetching among the stalls.
+// 281 so (80 shapes and formats from 64 to 4096 rows 0.40 to 0.95).  What bounds it: instructions (61 % of the issue slots in an earlier
+// state), their fetching among the stalls.
 // ---------------------------------------------------------------------------------------------
 template <int N, int M>
 __device__ __forceinline__ void kept_values(const float* v, float* sel) {
