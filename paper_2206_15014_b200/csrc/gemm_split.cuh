@@ -227,45 +227,44 @@ nm_gemm_split_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_co
         __syncwarp();
         ptx::cluster_arrive();
         ptx::cluster_wait();
-        if (*abort_flag == 0u) {
-            const float rsy = EPI == EPI_Q8 ? __frcp_rn(p.sy) : 0.0f;
-            float amax = 0.0f;
-            using OT = typename EpiOut<EPI>::type;
-            OT* const Y = reinterpret_cast<OT*>(kF32<EPI> ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW);
-            for (int ch = half; ch < chunks; ch += 2) {
-                const int col = rank * slice + ch * 8, t = t0 + col;
-                if (t >= p.tokens) break;
-                uint32_t r[8];
-                ptx::tmem_ld_32x8(lane_taddr + col, r);
-                ptx::tmem_ld_wait();
-                for (int d = 0; d < splits - 1; ++d) {
-                    const uint4* part = reinterpret_cast<const uint4*>(recv) + (size_t)((d * chunks + ch) * 2) * kBM + row;
-                    const uint4 a = part[0], b = part[kBM];
-                    r[0] += a.x; r[1] += a.y; r[2] += a.z; r[3] += a.w;
-                    r[4] += b.x; r[5] += b.y; r[6] += b.z; r[7] += b.w;
-                }
-                const int jmax = n < p.out ? min(8, p.tokens - t) : 0;
-                OT* dst = Y + (size_t)t * p.out + n;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    OT o;
-                    if constexpr (EPI == EPI_Q8) {
-                        float worst = 0.0f;
-                        o = epi_convert_q8_fast(r[j], c_n, b_n, rsy, worst);
-                        if (!(worst <= 0.49996948f)) o = (OT)(int8_t)quantise8_exact_call(__fmaf_rn((float)(int)r[j], c_n, b_n), p.sy);
-                    } else {
-                        float y_abs;
-                        o = epi_convert<EPI>(r[j], c_n, b_n, y_abs);
-                        if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
-                    }
-                    if (j < jmax) dst[(size_t)j * p.out] = o;
-                }
+        const bool whole = *abort_flag == 0u;  // every CTA has sent its sums; otherwise nothing is stored
+        const float rsy = EPI == EPI_Q8 ? __frcp_rn(p.sy) : 0.0f;
+        float amax = 0.0f;
+        using OT = typename EpiOut<EPI>::type;
+        OT* const Y = reinterpret_cast<OT*>(kF32<EPI> ? (void*)p.Y : EPI == EPI_ACC ? (void*)p.ACC : p.NARROW);
+        for (int ch = half; ch < chunks; ch += 2) {
+            const int col = rank * slice + ch * 8, t = t0 + col;
+            if (t >= p.tokens) break;
+            uint32_t r[8];
+            ptx::tmem_ld_32x8(lane_taddr + col, r);
+            ptx::tmem_ld_wait();
+            for (int d = 0; d < splits - 1; ++d) {
+                const uint4* part = reinterpret_cast<const uint4*>(recv) + (size_t)((d * chunks + ch) * 2) * kBM + row;
+                const uint4 a = part[0], b = part[kBM];
+                r[0] += a.x; r[1] += a.y; r[2] += a.z; r[3] += a.w;
+                r[4] += b.x; r[5] += b.y; r[6] += b.z; r[7] += b.w;
             }
-            if (EPI == EPI_F32MAX) {
+            const int jmax = whole && n < p.out ? min(8, p.tokens - t) : 0;
+            OT* dst = Y + (size_t)t * p.out + n;
 #pragma unroll
-                for (int s = 16; s > 0; s >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, s));
-                if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(p.absmax), __float_as_uint(amax));
+            for (int j = 0; j < 8; ++j) {
+                OT o;
+                if constexpr (EPI == EPI_Q8) {
+                    float worst = 0.0f;
+                    o = epi_convert_q8_fast(r[j], c_n, b_n, rsy, worst);
+                    if (!(worst <= 0.49996948f)) o = (OT)(int8_t)quantise8_exact_call(__fmaf_rn((float)(int)r[j], c_n, b_n), p.sy);
+                } else {
+                    float y_abs;
+                    o = epi_convert<EPI>(r[j], c_n, b_n, y_abs);
+                    if constexpr (EPI == EPI_F32MAX) amax = fmaxf(amax, j < jmax ? y_abs : 0.0f);
+                }
+                if (j < jmax) dst[(size_t)j * p.out] = o;
             }
+        }
+        if (EPI == EPI_F32MAX) {
+#pragma unroll
+            for (int s = 16; s > 0; s >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, s));
+            if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(p.absmax), __float_as_uint(amax));
         }
     }
     if (warp < 2 || warp >= kSplitThreads / 32) {  // the cluster's barriers of the others; apart, so that the builders hold nothing of the epilogue's
